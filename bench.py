@@ -814,10 +814,11 @@ def run_recolor(args):
     torch.cuda.synchronize()
     ms = (time.perf_counter() - t0) * 1e3 / steps
     clk = clocks.stop()
-    # products performed: moments; three per root iteration; two per polar
-    # iteration; the whitening of Sigma_ZY and the two products of A
-    flops = (2.0 * N * (d_s * d_s + d_r * d_r + d_s * d_r)
-             + 6.0 * (its[0] * d_s ** 3 + its[1] * d_r ** 3)
+    # products performed: moments (upper triangle); the covariances' factors and
+    # their inverses (2 d^3 / 3 each); two per polar iteration; the whitening of
+    # Sigma_ZY and the two products of A
+    flops = (1.0 * N * (d_s + d_r) ** 2
+             + 2.0 / 3.0 * (d_s ** 3 + d_r ** 3)
              + 4.0 * its[2] * d_s * d_r * d_r
              + 2 * (2.0 * d_s * d_s * d_r + 2.0 * d_s * d_r * d_r))
     sm_mhz = clk.get("sm_mhz") or 2070.0

@@ -416,11 +416,14 @@ hf_status hf_fold(hf_dtype dtype, int32_t n_maps, int32_t d_R, int64_t K, int32_
  * d_W_out: device [d_R][d_S] in `dtype`: A^T, the layout of hf_plan_desc's
  *       d_W; d_b_out: device float[d_R]; h_r_out: host float, r (or NULL);
  *       h_iters_out: host int32[3] (or NULL), the iterations taken by the
- *       roots of Sigma_Z and Sigma_Y and by the polar factor.
+ *       roots of Sigma_Z and Sigma_Y (1: a triangular factor served as the
+ *       root) and by the polar factor.
  * d_workspace: hf_recolor_workspace_size bytes, 256-byte aligned.
- * Requires d_S >= d_R and N * d_S < 2^31.  Matrix roots and the polar
- * factor use Newton-Schulz iterations in fp32; the matrix products run on
- * this library's tcgen05 kernel in fp32 accuracy (each fp32 operand split
+ * Requires d_S >= d_R and N * d_S < 2^31.  A needs no particular square root
+ * of the covariances: they are factored as L L^T, or, where a pivot is below
+ * 1e-4 of the mean eigenvalue, rooted by Newton-Schulz iterations; the polar
+ * factor takes Newton-Schulz iterations, all in fp32.  The matrix products run
+ * on this library's tcgen05 kernel in fp32 accuracy (each fp32 operand split
  * exactly into three bf16 parts, the six largest partial products summed in
  * an fp32 tensor-memory accumulator).  The call synchronises `stream`
  * (convergence checks) and returns HF_ERR_DEVICE_CHECK if an iteration does

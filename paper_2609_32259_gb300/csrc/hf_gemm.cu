@@ -64,11 +64,17 @@ struct GemmParams {
   float* partial;     // split-K partials [splits][M][N] (splits > 1)
   int32_t* err;       // error word (a wait ran out)
   int M, N;
-  int Mp, Np;         // plane rows of A and B (multiples of 256)
+  int Mp, Np;         // plane pitch of A and B in rows
+  int a_row0;         // plane row of A's row 0
   int n_kb;           // 128-byte atoms of K
-  int tiles_m, tiles_n, splits, kb_per_split;
+  int tiles_m, tiles_n, n_tiles, splits, kb_per_split;
+  int tri;            // row block m's column blocks are [0, n_lo) and [n_diag + m, tiles_n)
+  int n_lo, n_diag;
+  int fresh_lo, fresh_hi;  // columns in [lo, hi) (multiples of 64) take no C_in
   int n_terms;
   int term_a[kGMaxTerms], term_b[kGMaxTerms];
+  int accumulate;     // beta = 1, C_in is C and no diagonal term: C += alpha sum
+  int flush;          // > 0: the sums go to C every `flush` atoms (accumulate, vec, splits == 1)
   int vec;            // C rows can take 16-byte stores (ldc % 4 == 0, C 16-byte aligned)
   float alpha, beta;
 };
@@ -76,8 +82,22 @@ struct GemmParams {
 __device__ __forceinline__ void gemm_decode(const GemmParams& P, int tile, int* m, int* n, int* sp) {
   *sp = tile % P.splits;
   const int rest = tile / P.splits;
-  *m = rest % P.tiles_m;
-  *n = rest / P.tiles_m;
+  if (!P.tri) {
+    *m = rest % P.tiles_m;
+    *n = rest / P.tiles_m;
+    return;
+  }
+  int row = 0, base = 0;
+  for (;; ++row) {
+    const int hi = max(P.n_lo, P.n_diag + row), cnt = P.n_lo + P.tiles_n - hi;
+    if (rest < base + cnt) {
+      const int i = rest - base;
+      *m = row;
+      *n = i < P.n_lo ? i : hi + i - P.n_lo;
+      return;
+    }
+    base += cnt;
+  }
 }
 
 __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const void* map, int32_t x, int32_t y,
@@ -87,6 +107,12 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const void* map, 
       " [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
       "l"(map), "r"(x), "r"(y), "r"(bar_cluster)
       : "memory");
+}
+
+__device__ __forceinline__ void red_add_v4(float* p, float a, float b, float c, float d) {
+  asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c),
+               "f"(d)
+               : "memory");
 }
 
 __global__ void __launch_bounds__(kGThreads, 1)
@@ -101,7 +127,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
   const bool leader = rank == 0;
   const int first = static_cast<int>(cluster_id_x());
   const int step = static_cast<int>(nclusters_x());
-  const int total = P.tiles_m * P.tiles_n * P.splits;
+  const int total = P.n_tiles * P.splits;
   uint8_t* sA = smem;                                 // stage s: A atom at s * kGStageBytes
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kGStages * kGStageBytes);
   uint64_t* full = bars;
@@ -149,7 +175,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
         int m, n, sp;
         gemm_decode(P, tile, &m, &n, &sp);
         const int kb0 = sp * P.kb_per_split, kb1 = min(P.n_kb, kb0 + P.kb_per_split);
-        const int arow = m * kGTile + static_cast<int>(rank) * kGRows;
+        const int arow = P.a_row0 + m * kGTile + static_cast<int>(rank) * kGRows;
         const int brow = n * kGTile + static_cast<int>(rank) * kGRows;
         for (int kb = kb0; kb < kb1 && ok; ++kb) {
           for (int t = 0; t < P.n_terms; ++t) {
@@ -278,6 +304,21 @@ __global__ void __launch_bounds__(kGThreads, 1)
         }
         acc ^= 1;
         if (acc == 0) acc_phase ^= 1;
+        if (P.flush > 0 && (kb - kb0) % P.flush == P.flush - 1 && kb + 1 < kb1) {
+          // long sums go out in parts (splits == 1, C += ...): the fp32 sum in
+          // registers and the one in C then each take fewer, smaller roundings
+          const int frow = m * kGTile + static_cast<int>(rank) * kGRows + row_in;
+          const int fcol = n * kGTile + cg * kGEpiCols;
+          if (frow < P.M && fcol + kGEpiCols <= P.N) {
+            float* dst = P.C + static_cast<int64_t>(frow) * P.ldc + fcol;
+#pragma unroll
+            for (int i = 0; i < kGEpiCols; i += 4)
+              red_add_v4(dst + i, P.alpha * sum[i], P.alpha * sum[i + 1], P.alpha * sum[i + 2],
+                         P.alpha * sum[i + 3]);
+#pragma unroll
+            for (int i = 0; i < kGEpiCols; ++i) sum[i] = 0.f;
+          }
+        }
       }
       if (!ok) break;
       const int row = m * kGTile + static_cast<int>(rank) * kGRows + row_in;
@@ -300,27 +341,40 @@ __global__ void __launch_bounds__(kGThreads, 1)
         float* dst = P.C + static_cast<int64_t>(row) * P.ldc + col0;
         const float* cin = P.Cin + static_cast<int64_t>(row) * P.ldc + col0;
         const int dcol = row - col0;  // this row's diagonal element, if in range
+        const float beta = col0 >= P.fresh_lo && col0 < P.fresh_hi ? 0.f : P.beta;
+        const bool vec = P.vec && col0 + kGEpiCols <= P.N;
+        if (vec && P.accumulate && beta != 0.f) {
+          // C += alpha sum: vector reductions at L2, each element by this one
+          // thread (so the order is fixed), instead of loads that a store to
+          // the same matrix holds back: a K = 128 tile took 20 us with them
 #pragma unroll
-        for (int i = 0; i < kGEpiCols; i += 4) {
-          if (P.vec && col0 + i + 4 <= P.N) {
+          for (int i = 0; i < kGEpiCols; i += 4)
+            red_add_v4(dst + i, P.alpha * sum[i], P.alpha * sum[i + 1], P.alpha * sum[i + 2],
+                       P.alpha * sum[i + 3]);
+        } else if (vec) {
+#pragma unroll
+          for (int i = 0; i < kGEpiCols; i += 4) {
             float o[4] = {P.alpha * sum[i], P.alpha * sum[i + 1], P.alpha * sum[i + 2],
                           P.alpha * sum[i + 3]};
-            if (P.beta != 0.f) {
+            if (beta != 0.f) {
               const float4 c = *reinterpret_cast<const float4*>(cin + i);
-              o[0] = fmaf(P.beta, c.x, o[0]);
-              o[1] = fmaf(P.beta, c.y, o[1]);
-              o[2] = fmaf(P.beta, c.z, o[2]);
-              o[3] = fmaf(P.beta, c.w, o[3]);
+              o[0] = fmaf(beta, c.x, o[0]);
+              o[1] = fmaf(beta, c.y, o[1]);
+              o[2] = fmaf(beta, c.z, o[2]);
+              o[3] = fmaf(beta, c.w, o[3]);
             }
 #pragma unroll
             for (int k = 0; k < 4; ++k)
               if (dcol == i + k) o[k] += P.diag;
             *reinterpret_cast<float4*>(dst + i) = make_float4(o[0], o[1], o[2], o[3]);
-          } else {
+          }
+        } else {
+#pragma unroll
+          for (int i = 0; i < kGEpiCols; i += 4) {
             for (int k = 0; k < 4; ++k) {
               if (col0 + i + k >= P.N) continue;
               float o = P.alpha * sum[i + k];
-              if (P.beta != 0.f) o = fmaf(P.beta, cin[i + k], o);
+              if (beta != 0.f) o = fmaf(beta, cin[i + k], o);
               if (dcol == i + k) o += P.diag;
               dst[i + k] = o;
             }
@@ -344,16 +398,17 @@ __global__ void __launch_bounds__(kGThreads, 1)
   }
 }
 
-// C = alpha * sum_s partial[s] + beta * C_in + diag I.
+// C = alpha * sum_s partial[s] + beta * C_in + diag I (tri: the computed tiles only).
 __global__ void gemm_reduce_kernel(const float* partial, int splits, int M, int N, float* C,
                                    const float* Cin, int64_t ldc, float alpha, float beta,
-                                   float diag) {
+                                   float diag, int tri, int n_lo, int n_diag) {
   const int64_t n_el = static_cast<int64_t>(M) * N;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n_el;
        i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t r = i / N, c = i - r * N;
+    if (tri && c / kGTile >= n_lo && c / kGTile < n_diag + r / kGTile) continue;
     float s = 0.f;
     for (int k = 0; k < splits; ++k) s += partial[k * n_el + i];
-    const int64_t r = i / N, c = i - r * N;
     float o = alpha * s;
     if (beta != 0.f) o = fmaf(beta, Cin[r * ldc + c], o);
     if (r == c) o += diag;
@@ -457,11 +512,104 @@ size_t gemm_planes_bytes(int64_t rows, int64_t K) {
   return static_cast<size_t>(3 * round_up(rows, kGTile) * round_up(K, 64) * 2);
 }
 
+hf_status gemm_planes(cudaStream_t s, const GemmWork& wk, int M, int N, int k_p, float alpha,
+                      const GemmPlanes& a, const GemmPlanes& b, float beta, float* C, int64_t ldc,
+                      const GemmShape& shape, const float* Cin, float diag) {
+  if (Cin == nullptr) Cin = C;
+  if (M <= 0 || N <= 0) return HF_OK;
+  CUtensorMap ma, mb;
+  hf_status st = plane_map(&ma, a.planes, static_cast<uint64_t>(3 * a.rows_p),
+                           static_cast<uint64_t>(k_p));
+  if (st != HF_OK) return st;
+  st = plane_map(&mb, b.planes, static_cast<uint64_t>(3 * b.rows_p), static_cast<uint64_t>(k_p));
+  if (st != HF_OK) return st;
+
+  GemmParams P;
+  std::memset(&P, 0, sizeof(P));
+  P.C = C;
+  P.Cin = Cin;
+  P.diag = diag;
+  P.ldc = ldc;
+  P.err = wk.err;
+  P.M = M;
+  P.N = N;
+  P.Mp = static_cast<int>(a.rows_p);
+  P.Np = static_cast<int>(b.rows_p);
+  P.a_row0 = a.row0;
+  P.n_kb = k_p / 64;
+  P.tiles_m = static_cast<int>(round_up(M, kGTile) / kGTile);
+  P.tiles_n = static_cast<int>(round_up(N, kGTile) / kGTile);
+  P.tri = shape.tri ? 1 : 0;
+  P.n_lo = (shape.diag_col + kGTile - 1) / kGTile;
+  P.n_diag = shape.diag_col / kGTile;
+  P.n_tiles = P.tiles_m * P.tiles_n;
+  if (P.tri) {
+    P.n_tiles = 0;
+    for (int m = 0; m < P.tiles_m; ++m)
+      P.n_tiles += P.n_lo + P.tiles_n - std::max(P.n_lo, P.n_diag + m);
+  }
+  P.fresh_lo = shape.fresh_lo;
+  P.fresh_hi = shape.fresh_hi;
+  // terms a_i b_j with i + j <= 2, smallest first: an accumulator that
+  // adds by truncation loses at most an ulp of its current magnitude per add
+  const int ta[kGMaxTerms] = {2, 1, 0, 1, 0, 0}, tb[kGMaxTerms] = {0, 1, 2, 0, 1, 0};
+  P.n_terms = kGMaxTerms;
+  for (int t = 0; t < kGMaxTerms; ++t) {
+    P.term_a[t] = ta[t];
+    P.term_b[t] = tb[t];
+  }
+  P.vec = (ldc % 4 == 0 && ((reinterpret_cast<uintptr_t>(C) | reinterpret_cast<uintptr_t>(Cin)) &
+                             15u) == 0)
+              ? 1
+              : 0;
+  P.accumulate = beta == 1.f && Cin == C && diag == 0.f ? 1 : 0;
+  P.alpha = alpha;
+  P.beta = beta;
+  const int pairs = std::max(1, device_sm_count() / 2);
+  const int tiles = P.n_tiles;
+  // split K while the tiles leave SM pairs idle, keeping >= 4 atoms per split
+  int splits = 1;
+  while (P.fresh_hi == P.fresh_lo && tiles * splits * 2 <= pairs && P.n_kb / (splits * 2) >= 4 &&
+         static_cast<size_t>(splits * 2) * M * N * 4 <= wk.partial_bytes)
+    splits *= 2;
+  // no split may be empty: its tile would be written from a stale accumulator
+  P.kb_per_split = (P.n_kb + splits - 1) / splits;
+  P.splits = (P.n_kb + P.kb_per_split - 1) / P.kb_per_split;
+  splits = P.splits;
+  P.partial = wk.partial;
+  P.flush = P.accumulate && P.vec && splits == 1 ? shape.flush : 0;
+  const size_t smem = gemm_smem_bytes();
+  HF_CUDA_TRY(cudaFuncSetAttribute(gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   static_cast<int>(smem)),
+              "hf_recolor_fit: product shared memory");
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  const int clusters = std::max(1, std::min(pairs, tiles * splits));
+  cfg.gridDim = dim3(2 * clusters, 1, 1);
+  cfg.blockDim = dim3(kGThreads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  HF_CUDA_TRY(cudaLaunchKernelEx(&cfg, gemm_kernel, ma, mb, P), "hf_recolor_fit: product launch");
+  if (splits > 1) {
+    const int64_t n_el = static_cast<int64_t>(M) * N;
+    const int grid = static_cast<int>(std::min<int64_t>((n_el + 255) / 256, 4096));
+    gemm_reduce_kernel<<<grid, 256, 0, s>>>(wk.partial, splits, M, N, C, Cin, ldc, alpha, beta,
+                                            diag, P.tri, P.n_lo, P.n_diag);
+    HF_CUDA_TRY(cudaGetLastError(), "hf_recolor_fit: product reduce launch");
+  }
+  return HF_OK;
+}
+
 hf_status gemm_f32(cudaStream_t s, const GemmWork& wk, int M, int N, int K, float alpha,
                    const float* A, int64_t a_i, int64_t a_k, const float* B, int64_t b_k,
                    int64_t b_j, float beta, float* C, int64_t ldc, const float* Cin,
                    float diag) {
-  if (Cin == nullptr) Cin = C;
   if (M <= 0 || N <= 0) return HF_OK;
   if (K <= 0) {
     set_error("hf_recolor_fit: internal error: a product with K = 0");
@@ -490,78 +638,9 @@ hf_status gemm_f32(cudaStream_t s, const GemmWork& wk, int M, int N, int K, floa
                                            static_cast<int>(Kp));
   }
   HF_CUDA_TRY(cudaGetLastError(), "hf_recolor_fit: operand split launch");
-  CUtensorMap ma, mb;
-  hf_status st = plane_map(&ma, pa, static_cast<uint64_t>(3 * Mp), static_cast<uint64_t>(Kp));
-  if (st != HF_OK) return st;
-  st = plane_map(&mb, pb, static_cast<uint64_t>(3 * Np), static_cast<uint64_t>(Kp));
-  if (st != HF_OK) return st;
-
-  GemmParams P;
-  std::memset(&P, 0, sizeof(P));
-  P.C = C;
-  P.Cin = Cin;
-  P.diag = diag;
-  P.ldc = ldc;
-  P.err = wk.err;
-  P.M = M;
-  P.N = N;
-  P.Mp = static_cast<int>(Mp);
-  P.Np = static_cast<int>(Np);
-  P.n_kb = static_cast<int>(Kp / 64);
-  P.tiles_m = static_cast<int>(Mp / kGTile);
-  P.tiles_n = static_cast<int>(Np / kGTile);
-  // terms a_i b_j with i + j <= 2, smallest first: an accumulator that
-  // adds by truncation loses at most an ulp of its current magnitude per add
-  const int ta[kGMaxTerms] = {2, 1, 0, 1, 0, 0}, tb[kGMaxTerms] = {0, 1, 2, 0, 1, 0};
-  P.n_terms = kGMaxTerms;
-  for (int t = 0; t < kGMaxTerms; ++t) {
-    P.term_a[t] = ta[t];
-    P.term_b[t] = tb[t];
-  }
-  P.vec = (ldc % 4 == 0 && ((reinterpret_cast<uintptr_t>(C) | reinterpret_cast<uintptr_t>(Cin)) &
-                             15u) == 0)
-              ? 1
-              : 0;
-  P.alpha = alpha;
-  P.beta = beta;
-  const int pairs = std::max(1, device_sm_count() / 2);
-  const int tiles = P.tiles_m * P.tiles_n;
-  // split K while the tiles leave SM pairs idle, keeping >= 4 atoms per split
-  int splits = 1;
-  while (tiles * splits * 2 <= pairs && P.n_kb / (splits * 2) >= 4 &&
-         static_cast<size_t>(splits * 2) * M * N * 4 <= wk.partial_bytes)
-    splits *= 2;
-  // no split may be empty: its tile would be written from a stale accumulator
-  P.kb_per_split = (P.n_kb + splits - 1) / splits;
-  P.splits = (P.n_kb + P.kb_per_split - 1) / P.kb_per_split;
-  splits = P.splits;
-  P.partial = wk.partial;
-  const size_t smem = gemm_smem_bytes();
-  HF_CUDA_TRY(cudaFuncSetAttribute(gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   static_cast<int>(smem)),
-              "hf_recolor_fit: product shared memory");
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 2;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  const int clusters = std::max(1, std::min(pairs, tiles * splits));
-  cfg.gridDim = dim3(2 * clusters, 1, 1);
-  cfg.blockDim = dim3(kGThreads, 1, 1);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  HF_CUDA_TRY(cudaLaunchKernelEx(&cfg, gemm_kernel, ma, mb, P), "hf_recolor_fit: product launch");
-  if (splits > 1) {
-    const int64_t n_el = static_cast<int64_t>(M) * N;
-    const int grid = static_cast<int>(std::min<int64_t>((n_el + 255) / 256, 4096));
-    gemm_reduce_kernel<<<grid, 256, 0, s>>>(wk.partial, splits, M, N, C, Cin, ldc, alpha, beta,
-                                            diag);
-    HF_CUDA_TRY(cudaGetLastError(), "hf_recolor_fit: product reduce launch");
-  }
-  return HF_OK;
+  const GemmPlanes ga{pa, Mp, 0}, gb{pb, Np, 0};
+  return gemm_planes(s, wk, M, N, static_cast<int>(Kp), alpha, ga, gb, beta, C, ldc, GemmShape{}, Cin,
+                     diag);
 }
 
 }  // namespace hf

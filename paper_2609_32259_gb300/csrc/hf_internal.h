@@ -147,6 +147,28 @@ struct GemmWork {
 };
 // Bytes of the three bf16 planes of an operand with `rows` rows and K columns.
 size_t gemm_planes_bytes(int64_t rows, int64_t K);
+// An operand that is already split: three planes of `rows_p` rows each,
+// K-major bf16, the operand's row 0 at plane row `row0`.
+struct GemmPlanes {
+  const void* planes;
+  int64_t rows_p;
+  int row0;
+};
+// Which part of C a product writes.  tri: of the 256 x 256 tiles of row block
+// m, those left of column diag_col and those that reach column diag_col +
+// 256 m or beyond (diag_col 0: a symmetric product's upper triangle).  Columns
+// in [fresh_lo, fresh_hi) (multiples of 64) take no C_in.
+struct GemmShape {
+  bool tri = false;
+  int diag_col = 0;
+  int fresh_lo = 0, fresh_hi = 0;
+  int flush = 0;  // > 0: a sum over K goes to C in parts of this many 64-wide atoms (C += only)
+};
+// C = alpha op(A) op(B) + beta C_in + diag I of split operands with k_p
+// columns (a multiple of 64, zero-padded).
+hf_status gemm_planes(cudaStream_t s, const GemmWork& wk, int M, int N, int k_p, float alpha,
+                      const GemmPlanes& a, const GemmPlanes& b, float beta, float* C, int64_t ldc,
+                      const GemmShape& shape, const float* Cin = nullptr, float diag = 0.f);
 // C[M x N] = alpha op(A) op(B) + beta C_in + diag I (row-major C and C_in,
 // leading dimension ldc; C_in NULL = C), op(A)(i, k) = A[i * a_i + k * a_k],
 // op(B)(k, j) = B[k * b_k + j * b_j], in fp32 accuracy on the tensor cores
@@ -155,6 +177,19 @@ hf_status gemm_f32(cudaStream_t s, const GemmWork& wk, int M, int N, int K, floa
                    const float* A, int64_t a_i, int64_t a_k, const float* B, int64_t b_k,
                    int64_t b_j, float beta, float* C, int64_t ldc, const float* Cin = nullptr,
                    float diag = 0.f);
+
+// Triangular factor of the symmetric positive definite n x n matrix W
+// (row-major, leading dimension ld, n a multiple of kFactorBlock; the blocks on
+// and above the diagonal are read): W = L L^T.  On return row i holds
+// L^{-1}'s row i in columns 0 .. i (zeros to the end of the diagonal block,
+// work values after it).  upper (or NULL, cleared before): L^T, n_upper x
+// n_upper.  Tt: kFactorBlock^2 floats; planes: tri_factor_planes_bytes(n).  A
+// pivot that is not above *thr sets *flag (cleared before) and the result is
+// of no use.
+constexpr int kFactorBlock = 128;
+size_t tri_factor_planes_bytes(int n);
+hf_status tri_factor(cudaStream_t s, const GemmWork& wk, float* W, int64_t ld, int n, float* Tt,
+                     void* planes, const float* thr, int32_t* flag, float* upper, int n_upper);
 
 }  // namespace hf
 

@@ -4,11 +4,20 @@
 //   Z = X / r; weighted means and covariances of Z and Y
 //   R* = polar factor of Sigma_Z^{-1/2} Sigma_ZY Sigma_Y^{-1/2}      (Eq. 4)
 //   A = Sigma_Z^{-1/2} R* Sigma_Y^{1/2},  b = mu_Y - mu_Z A           (Eq. 5)
-// Matrix square roots and the polar factor use Newton-Schulz iterations, so
-// every step is a matrix product or an elementwise pass: the coupled
-// iteration T = (3I - Z Y) / 2, Y <- Y T, Z <- T Z turns Y_0 = S / c,
+// Any square roots of the covariances give the same A: with the triangular
+// factors Sigma_Z = L L^T and Sigma_Y = C C^T (hf_factor.cu),
+// Sigma_Z^{-1/2} = L^{-T} Q for an orthogonal Q, which the polar factor takes
+// along, so
+//   A = L^{-T} polar(L^{-1} Sigma_ZY C^{-T}) C^T,
+// one factorisation instead of ~11 iterations of three dense products (at
+// 32,768 x 3,072 -> 1,024 the fit took 16.5 ms with iterated roots and three
+// dense moment products, 6.0 ms now; fp32 fits with d_S > d_R come out a
+// quarter as far from 64 bits).  Only where a pivot is too small
+// for fp32 (kPivot of the mean eigenvalue; reg is 0 or tiny and the covariance
+// near singular) the symmetric roots are iterated instead, as far as they
+// converge: the coupled iteration T = (3I - Z Y) / 2, Y <- Y T, Z <- T Z turns Y_0 = S / c,
 // Z_0 = I into (S / c)^{1/2} and (S / c)^{-1/2}; X <- X (3I - X^T X) / 2
-// turns X_0 = M / |M|_F into the orthogonal polar factor U Q^T of
+// turns X_0 = M into the orthogonal polar factor U Q^T of
 // M = U Lambda Q^T (full column rank), which is the R* of Eq. 4.
 // Offline (once per map, before folding).  The products are fp32 GEMMs on
 // this library's tcgen05 kernel (hf_gemm.cu: each operand split exactly into
@@ -28,9 +37,15 @@
 namespace hf {
 namespace {
 
-// The moments' products run over the samples in chunks of this many, so the
-// bf16 planes of their operands stay a bounded part of the workspace.
+// The moments' product runs over the samples in chunks of this many, so the
+// bf16 planes of its operand stay a bounded part of the workspace.
 constexpr int64_t kMomentChunk = 8192;
+// Atoms of 64 samples that one fp32 sum of the moments takes before it goes to
+// the matrix: 32 x 16 roundings for 32,768 samples instead of 512 in a row.
+constexpr int kMomentFlush = 32;
+// A pivot below this share of the mean eigenvalue has lost too many of its
+// digits in fp32; the ridge keeps pivots above reg of it (the paper's fits: 1e-3).
+constexpr float kPivot = 1e-4f;
 // Split-K partials: room for every SM pair's 256 x 256 tile twice over.
 constexpr size_t kPartialBytes = static_cast<size_t>(2) * 96 * 65536 * sizeof(float);
 
@@ -41,51 +56,115 @@ hf_status sgemm(const GemmWork& h, cudaStream_t s, int M, int N, int K, float al
   return gemm_f32(s, h, M, N, K, alpha, A, a_i, a_k, B, b_k, b_j, beta, C, ldc, Cin, diag);
 }
 
-// A product over the sample axis (K = N samples) in chunks of kMomentChunk:
-// C = alpha sum_chunks op(A_c) op(B_c).
-hf_status moment_product(const GemmWork& h, cudaStream_t s, int M, int N, int64_t K,
-                         const float* A, int64_t a_i, int64_t a_k, const float* B, int64_t b_k,
-                         int64_t b_j, float* C, int64_t ldc) {
-  for (int64_t k0 = 0; k0 < K; k0 += kMomentChunk) {
-    const int kc = static_cast<int>(std::min<int64_t>(kMomentChunk, K - k0));
-    const hf_status st = sgemm(h, s, M, N, kc, 1.f, A + k0 * a_k, a_i, a_k, B + k0 * b_k, b_k,
-                               b_j, k0 == 0 ? 0.f : 1.f, C, ldc);
-    if (st != HF_OK) return st;
-  }
-  return HF_OK;
-}
-
 __device__ __forceinline__ float ld(const __nv_bfloat16* p) { return __bfloat162float(*p); }
 __device__ __forceinline__ float ld(const float* p) { return *p; }
 
-// Column sums of w X and w Y, sum w, and sum w |x|^2.  A thread sums its
-// column over the block's rows (at most a few hundred) in fp32; the partial
-// sums meet in fp64 (GB300's fp64 rate is a small fraction of fp32's).
-template <typename T>
-__global__ void rc_stats_kernel(const T* X, const T* Y, const float* w, int64_t N, int dx,
-                                int dy, double* sx, double* sy, double* sw_ss) {
-  const int d = dx + dy;
-  const int col = blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t rows = (N + gridDim.y - 1) / gridDim.y;
-  const int64_t n0 = blockIdx.y * rows, n1 = min(N, n0 + rows);
-  float s = 0.f, ssq = 0.f, swt = 0.f;
-  if (col < d) {
-    for (int64_t n = n0; n < n1; ++n) {
-      const float wn = w[n];
-      const float v = col < dx ? ld(X + n * dx + col) : ld(Y + n * dy + (col - dx));
-      const float wv = wn * v;
-      s += wv;
-      if (col < dx) ssq = fmaf(wv, v, ssq);
-      if (col == 0) swt += wn;
+// Column sums of w [X | Y] and, from X, sum w and sum w |x|^2, in two passes.
+// rc_stats_kernel: a warp takes every eighth row of the block's slice and
+// 32 V columns per read, four reads of two rows in flight; a thread sums at most a few
+// hundred values in fp32 (GB300's fp64 rate is a small fraction of fp32's) and
+// the block's partial sums go out as fp64; rc_stats_sum_kernel adds the slices.
+// Bounded by reading X and Y once.  (fp64 atomics in the place of the partial
+// sums took 0.36 ms for 0.27 GB.)
+constexpr int kStatSlices = 128;
+template <typename T, int V>
+struct alignas(V * sizeof(T)) StatVec {
+  T x[V];
+};
+template <typename T, int V>
+__global__ void __launch_bounds__(256)
+    rc_stats_kernel(const T* X, const T* Y, const float* w, int64_t N, int dx, int dy,
+                    double* part) {
+  constexpr int kCols = 128 * V;  // per block: four reads of a warp
+  __shared__ float sums[8][kCols];
+  __shared__ double ss[8], sw[8];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int nbx = (dx + kCols - 1) / kCols;
+  const bool is_x = static_cast<int>(blockIdx.x) < nbx;
+  const int b0 = (is_x ? blockIdx.x : blockIdx.x - nbx) * kCols, d = is_x ? dx : dy;
+  const T* const M = is_x ? X : Y;
+  const int64_t per = (N + gridDim.y - 1) / gridDim.y;
+  const int64_t n0 = blockIdx.y * per, n1 = min(N, n0 + per);
+  float s[4 * V], q = 0.f, wt = 0.f;
+#pragma unroll
+  for (int i = 0; i < 4 * V; ++i) s[i] = 0.f;
+#pragma unroll 2
+  for (int64_t n = n0 + warp; n < n1; n += 8) {
+    const float wn = w[n];
+    const T* row = M + n * d;
+    StatVec<T, V> v[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int c = b0 + (lane + 32 * i) * V;  // d is a multiple of V
+      if (c < d)
+        v[i] = *reinterpret_cast<const StatVec<T, V>*>(row + c);
+      else
+        for (int k = 0; k < V; ++k) v[i].x[k] = T(0.f);
     }
-    atomicAdd(col < dx ? sx + col : sy + (col - dx), static_cast<double>(s));
-    if (col == 0) atomicAdd(sw_ss, static_cast<double>(swt));
+#pragma unroll
+    for (int i = 0; i < 4 * V; ++i) {
+      const float x = ld(&v[i / V].x[i % V]), wv = wn * x;
+      s[i] += wv;
+      q = fmaf(wv, x, q);
+    }
+    wt += wn;
   }
-  // the shared sum of squares: every lane of the warp takes part (lanes
-  // past the columns hold 0), one fp64 atomic per warp
-  double q = ssq;
-  for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
-  if ((threadIdx.x & 31) == 0 && q != 0.0) atomicAdd(sw_ss + 1, q);
+#pragma unroll
+  for (int i = 0; i < 4 * V; ++i) sums[warp][(lane + 32 * (i / V)) * V + i % V] = s[i];
+  double dq = q;
+  for (int o = 16; o > 0; o >>= 1) dq += __shfl_xor_sync(0xffffffffu, dq, o);
+  if (lane == 0) {
+    ss[warp] = dq;
+    sw[warp] = wt;
+  }
+  __syncthreads();
+  // a slice's row: the sums of X's and Y's columns, sum w, sum w |x|^2 of each
+  // of X's column blocks
+  double* const out = part + static_cast<int64_t>(blockIdx.y) * (dx + dy + 1 + nbx);
+  for (int c = threadIdx.x; c < kCols; c += blockDim.x) {
+    if (b0 + c >= d) break;
+    double t = 0.0;
+    for (int k = 0; k < 8; ++k) t += sums[k][c];
+    out[(is_x ? 0 : dx) + b0 + c] = t;
+  }
+  if (is_x && threadIdx.x == 0) {
+    double t = 0.0, u = 0.0;
+    for (int k = 0; k < 8; ++k) {
+      t += ss[k];
+      u += sw[k];
+    }
+    if (blockIdx.x == 0) out[dx + dy] = u;
+    out[dx + dy + 1 + blockIdx.x] = t;
+  }
+}
+
+// sums[c] = the slices' sums of column c, c <= d (the last one sum w): 32
+// columns a block, eight threads each; the grid's last block adds up the nbx
+// columns of sum w |x|^2 into sums[d + 1].
+__global__ void __launch_bounds__(256)
+    rc_stats_sum_kernel(const double* part, int slices, int d, int nbx, double* sums) {
+  __shared__ double sh[8][33];
+  const int lane = threadIdx.x & 31, y = threadIdx.x >> 5, stride = d + 1 + nbx;
+  const bool ss = blockIdx.x == gridDim.x - 1;
+  const int c = blockIdx.x * 32 + lane;
+  double t = 0.0;
+  if (ss) {
+    for (int i = threadIdx.x; i < slices * nbx; i += 256)
+      t += part[static_cast<int64_t>(i / nbx) * stride + d + 1 + i % nbx];
+  } else if (c <= d) {
+#pragma unroll 8
+    for (int i = y; i < slices; i += 8) t += part[static_cast<int64_t>(i) * stride + c];
+  }
+  sh[y][lane] = t;
+  __syncthreads();
+  if (y != 0) return;
+  for (int k = 1; k < 8; ++k) t += sh[k][lane];
+  if (ss) {
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (lane == 0) sums[d + 1] = t;
+  } else if (c <= d) {
+    sums[c] = t;
+  }
 }
 
 // fp32 means mu_x (of X, not yet divided by r), mu_y, and [1 / W, 1 / r].
@@ -100,38 +179,104 @@ __global__ void rc_mean_kernel(const double* sx, const double* sy, const double*
   }
 }
 
-// Xc = sqrt(w / W) (x - mu_x) / r and Yc = sqrt(w / W) (y - mu_y), fp32.
+// Centred, weighted samples as the moments' operand: feature f of sample n is
+// sqrt(w / W) (x - mu_x) / r (f < dx), sqrt(w / W) (y - mu_y) (np <= f <
+// np + dy), 0 elsewhere and past the last sample; written as the three bf16
+// planes of gemm_planes, feature-major, for the samples n0 .. n0 + k_p - 1.
+// A block turns 64 features x 64 samples through shared memory, read along the
+// features and written along the samples, 128 bytes each way: 6 bytes written
+// per value are what bounds it (32,768 x 4,096: 0.8 GB written, 0.27 GB read),
+// where an fp32 copy of the centred samples cost 0.46 ms and its split
+// another 0.4 ms.
 template <typename T>
-__global__ void rc_center_kernel(const T* X, const T* Y, const float* w, int64_t N, int dx,
-                                 int dy, const float* mu, const float* scal, float* Xc,
-                                 float* Yc) {
-  const int d = dx + dy;
+__global__ void __launch_bounds__(256)
+    rc_planes_kernel(const T* X, const T* Y, const float* w, int64_t N, int64_t n0, int dx, int dy,
+                     int np, const float* mu, const float* scal, __nv_bfloat16* out,
+                     int64_t rows_p, int64_t k_p) {
+  __shared__ float tile[64][65];
+  __shared__ float scale[64];
+  const int f0 = blockIdx.y * 64, k0 = blockIdx.x * 64;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const float inv_w = scal[0], inv_r = scal[1];
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N * d;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t n = i / d;
-    const int c = static_cast<int>(i - n * d);
-    const float sc = sqrtf(w[n] * inv_w);
-    if (c < dx)
-      Xc[n * dx + c] = sc * (ld(X + n * dx + c) - mu[c]) * inv_r;
-    else
-      Yc[n * dy + (c - dx)] = sc * (ld(Y + n * dy + (c - dx)) - mu[c]);
+  if (threadIdx.x < 64) {
+    const int64_t n = n0 + k0 + threadIdx.x;
+    scale[threadIdx.x] = n < N ? sqrtf(w[n] * inv_w) : 0.f;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int f = f0 + lane + 32 * h;
+    const bool is_x = f < dx, is_y = f >= np && f < np + dy;
+    const T* src = is_x ? X + f : Y + (f - np);
+    const int64_t step = is_x ? dx : dy;
+    const float m = is_x ? mu[f] : is_y ? mu[dx + f - np] : 0.f;
+    const float mul = is_x ? inv_r : 1.f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int k = warp + 8 * i;
+      const int64_t n = n0 + k0 + k;
+      float v = 0.f;
+      if ((is_x || is_y) && n < N) v = scale[k] * (ld(src + n * step) - m) * mul;
+      tile[k][lane + 32 * h] = v;
+    }
+  }
+  __syncthreads();
+  const int64_t plane = rows_p * k_p / 2;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int f = warp + 8 * i;
+    const float a = tile[2 * lane][f], b = tile[2 * lane + 1][f];
+    const __nv_bfloat162 h0 = __floats2bfloat162_rn(a, b);
+    const float2 g0 = __bfloat1622float2(h0);
+    const float ra = a - g0.x, rb = b - g0.y;
+    const __nv_bfloat162 h1 = __floats2bfloat162_rn(ra, rb);
+    const float2 g1 = __bfloat1622float2(h1);
+    __nv_bfloat162* o = reinterpret_cast<__nv_bfloat162*>(out + (f0 + f) * k_p + k0) + lane;
+    o[0] = h0;
+    o[plane] = h1;
+    o[2 * plane] = __floats2bfloat162_rn(ra - g1.x, rb - g1.y);
   }
 }
 
-// S += reg * trace(S) / d * I  (one block of 256 threads).
-__global__ void rc_ridge_kernel(float* S, int d, float reg) {
+// S += reg * trace(S) / d * I for the d x d matrix at S; the diagonal of its
+// padding, up to n, becomes the mean eigenvalue; *thr receives the smallest
+// pivot to accept (one block of 256 threads).
+__global__ void rc_ridge_kernel(float* S, int64_t ld, int d, int n, float reg, float* thr) {
   __shared__ double part[256];
   double t = 0.0;
-  for (int i = threadIdx.x; i < d; i += blockDim.x) t += S[static_cast<int64_t>(i) * d + i];
+  for (int i = threadIdx.x; i < d; i += blockDim.x) t += S[i * ld + i];
   part[threadIdx.x] = t;
   __syncthreads();
   for (int o = blockDim.x / 2; o > 0; o >>= 1) {
     if (threadIdx.x < o) part[threadIdx.x] += part[threadIdx.x + o];
     __syncthreads();
   }
-  const float add = reg * static_cast<float>(part[0] / d);
-  for (int i = threadIdx.x; i < d; i += blockDim.x) S[static_cast<int64_t>(i) * d + i] += add;
+  const float mean = static_cast<float>(part[0] / d);
+  const float add = reg * mean;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    if (i < d)
+      S[i * ld + i] += add;
+    else
+      S[i * ld + i] = mean;
+  }
+  if (threadIdx.x == 0) *thr = kPivot * mean;
+}
+
+// out (rows x cols, dense) from the matrix at S: mode 0 as it is, 1 the
+// symmetric matrix whose upper triangle S holds, 2 the lower triangle with
+// zeros above it.
+__global__ void rc_extract_kernel(const float* S, int64_t ld, int rows, int cols, int mode,
+                                  float* out) {
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= cols) return;
+  for (int i = blockIdx.y; i < rows; i += gridDim.y) {
+    float v = 0.f;
+    if (mode == 1 && i > j)
+      v = S[j * ld + i];
+    else if (mode != 2 || j <= i)
+      v = S[i * ld + j];
+    out[static_cast<int64_t>(i) * cols + j] = v;
+  }
 }
 
 // *out = trace(S) (one block of 256 threads).
@@ -160,9 +305,11 @@ __global__ void rc_affine_kernel(float* out, const float* in, int64_t n_el, int 
 }
 
 // sum of squares of x, or of (x - I) when minus_identity: fp32 per thread
-// (a few dozen elements each), fp64 across threads.
-__global__ void rc_sumsq_kernel(const float* x, int64_t n_el, int cols, int minus_identity,
-                                double* out) {
+// (a few dozen elements each), fp64 across threads, one atomic per block (one
+// per warp made the 1,024-square pass 17 us of queueing on one address).
+__global__ void __launch_bounds__(256)
+    rc_sumsq_kernel(const float* x, int64_t n_el, int cols, int minus_identity, double* out) {
+  __shared__ double part[8];
   float s = 0.f;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n_el;
        i += (int64_t)gridDim.x * blockDim.x) {
@@ -172,7 +319,12 @@ __global__ void rc_sumsq_kernel(const float* x, int64_t n_el, int cols, int minu
   }
   double q = s;
   for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
-  if ((threadIdx.x & 31) == 0) atomicAdd(out, q);
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = q;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int k = 1; k < 8; ++k) q += part[k];
+    atomicAdd(out, q);
+  }
 }
 
 // W_out = A^T in the output type: 32 x 32 tiles through shared memory, read
@@ -223,9 +375,11 @@ __global__ void rc_bias_final_kernel(const double* sy, const double* sw_ss, cons
 }
 
 struct Rc {
-  size_t stats, bacc, mu, xc, yc, sz, sy, szy, p1, p2, p3, p4, sz_ih, sy_ih, sy_h, m, x1, x2, xtx, a,
-      planes_a, planes_b, partial, err, total;
-  size_t planes_bytes;
+  size_t stats, part, bacc, mu, gram, tt, fplanes, thr, flag, sz, sy, szy, p1, p2, p3, p4, sz_ih, sy_ih,
+      sy_h, m, x1, x2, xtx, a, planes_a, planes_b, partial, err, total;
+  size_t planes_a_bytes, planes_b_bytes;
+  int np, mp, F;     // features of X and of Y padded to whole factor blocks; their sum
+  int64_t chunk;     // samples per moments product (a multiple of 64)
 };
 
 Rc rc_layout(int64_t N, int dx, int dy) {
@@ -239,10 +393,19 @@ Rc rc_layout(int64_t N, int dx, int dy) {
   const size_t f = sizeof(float);
   const size_t dmax = static_cast<size_t>(dx > dy ? dx : dy);
   L.stats = take(sizeof(double) * (dx + dy + 4));
+  L.part = take(sizeof(double) * kStatSlices * (dx + dy + 1 + (dx + 127) / 128));
   L.bacc = take(sizeof(double) * dy);
   L.mu = take(f * (dx + dy + 2));
-  L.xc = take(f * N * dx);
-  L.yc = take(f * N * dy);
+  auto up = [](int64_t x, int64_t a) { return (x + a - 1) / a * a; };
+  L.np = static_cast<int>(up(dx, kFactorBlock));
+  L.mp = static_cast<int>(up(dy, kFactorBlock));
+  L.F = L.np + L.mp;
+  L.chunk = std::min<int64_t>(up(N, 64), kMomentChunk);
+  L.gram = take(f * L.F * L.F);
+  L.tt = take(f * kFactorBlock * kFactorBlock);
+  L.fplanes = take(tri_factor_planes_bytes(L.np));
+  L.thr = take(f * 2);
+  L.flag = take(sizeof(int32_t));
   L.sz = take(f * dx * dx);
   L.sy = take(f * dy * dy);
   L.szy = take(f * dx * dy);
@@ -258,12 +421,12 @@ Rc rc_layout(int64_t N, int dx, int dy) {
   L.x2 = take(f * dx * dy);
   L.xtx = take(f * dy * dy);
   L.a = take(f * dx * dy);
-  // bf16 planes of the products' operands: rows up to max(d_S, d_R), K up
-  // to max(d_S, one chunk of samples)
-  const int64_t kmax = std::max<int64_t>(dx, std::min<int64_t>(N, kMomentChunk));
-  L.planes_bytes = gemm_planes_bytes(static_cast<int64_t>(dmax), kmax);
-  L.planes_a = take(L.planes_bytes);
-  L.planes_b = take(L.planes_bytes);
+  // bf16 planes of the products' operands; the moments' operand holds every
+  // feature for one chunk of samples
+  L.planes_b_bytes = gemm_planes_bytes(static_cast<int64_t>(dmax), static_cast<int64_t>(dmax));
+  L.planes_a_bytes = std::max(L.planes_b_bytes, gemm_planes_bytes(L.F, L.chunk));
+  L.planes_a = take(L.planes_a_bytes);
+  L.planes_b = take(L.planes_b_bytes);
   L.partial = take(kPartialBytes);
   L.err = take(sizeof(int32_t));
   L.total = off;
@@ -307,7 +470,7 @@ hf_status ns_sqrt(cudaStream_t s, const GemmWork& h, const float* S, int d, floa
   const int grid = 1024;
   double c2 = 0.0;
   HF_CUDA_TRY(cudaMemsetAsync(dscr, 0, sizeof(double), s), "clear");
-  rc_sumsq_kernel<<<grid, 256, 0, s>>>(S, n_el, d, 0, dscr);
+  rc_sumsq_kernel<<<2 * device_sm_count(), 256, 0, s>>>(S, n_el, d, 0, dscr);
   hf_status st = read_double(s, dscr, &c2);
   if (st != HF_OK) return st;
   const double c = sqrt(c2);
@@ -339,7 +502,7 @@ hf_status ns_sqrt(cudaStream_t s, const GemmWork& h, const float* S, int d, floa
       double e2 = 0.0;
       HF_CUDA_TRY(cudaMemsetAsync(dscr, 0, sizeof(double), s), "clear");
       // |I - Z Y| = 2 |T - I|
-      rc_sumsq_kernel<<<grid, 256, 0, s>>>(T, n_el, d, 1, dscr);
+      rc_sumsq_kernel<<<2 * device_sm_count(), 256, 0, s>>>(T, n_el, d, 1, dscr);
       if ((st = read_double(s, dscr, &e2)) != HF_OK) return st;
       if (converged(2.0 * sqrt(e2 / d), &prev)) break;
     }
@@ -375,7 +538,7 @@ hf_status ns_polar(cudaStream_t s, const GemmWork& h, const float* M, int dx, in
   const int grid = 1024;
   double m2 = 0.0;
   HF_CUDA_TRY(cudaMemsetAsync(dscr, 0, sizeof(double), s), "clear");
-  rc_sumsq_kernel<<<grid, 256, 0, s>>>(M, n_el, dy, 0, dscr);
+  rc_sumsq_kernel<<<2 * device_sm_count(), 256, 0, s>>>(M, n_el, dy, 0, dscr);
   hf_status st = read_double(s, dscr, &m2);
   if (st != HF_OK) return st;
   if (!(m2 > 0.0)) {
@@ -392,7 +555,7 @@ hf_status ns_polar(cudaStream_t s, const GemmWork& h, const float* M, int dx, in
     if (it % 4 == 3) {
       double e2 = 0.0;
       HF_CUDA_TRY(cudaMemsetAsync(dscr, 0, sizeof(double), s), "clear");
-      rc_sumsq_kernel<<<grid, 256, 0, s>>>(P, p_el, dy, 1, dscr);
+      rc_sumsq_kernel<<<2 * device_sm_count(), 256, 0, s>>>(P, p_el, dy, 1, dscr);
       if ((st = read_double(s, dscr, &e2)) != HF_OK) return st;
       if (converged(sqrt(e2 / dy), &prev)) break;
     }
@@ -423,50 +586,117 @@ hf_status recolor_typed(int64_t N, int dx, int dy, const void* Xv, const void* Y
   GemmWork h;
   h.planes_a = ws + L.planes_a;
   h.planes_b = ws + L.planes_b;
-  h.planes_a_bytes = h.planes_b_bytes = L.planes_bytes;
+  h.planes_a_bytes = L.planes_a_bytes;
+  h.planes_b_bytes = L.planes_b_bytes;
   h.partial = F(L.partial);
   h.partial_bytes = kPartialBytes;
   h.err = reinterpret_cast<int32_t*>(ws + L.err);
   HF_CUDA_TRY(cudaMemsetAsync(h.err, 0, sizeof(int32_t), s), "clear");
   HF_CUDA_TRY(cudaMemsetAsync(stats, 0, sizeof(double) * (dx + dy + 4), s), "clear");
   const int d = dx + dy;
-  // at most ~128 rows per thread, so the per-thread fp32 sums stay short
-  dim3 sgrid((d + 255) / 256, static_cast<unsigned>(std::min<int64_t>((N + 127) / 128, 65535)));
-  rc_stats_kernel<T><<<sgrid, 256, 0, s>>>(X, Y, w, N, dx, dy, sx, sy, sw_ss);
+  {
+    double* const part = reinterpret_cast<double*>(ws + L.part);
+    const int slices = static_cast<int>(std::min<int64_t>((N + 63) / 64, kStatSlices));
+    const bool pairs = dx % 2 == 0 && dy % 2 == 0 &&
+                       ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(Y)) &
+                        (2 * sizeof(T) - 1)) == 0;
+    const int cols = pairs ? 256 : 128;
+    const int nbx = (dx + cols - 1) / cols, nby = (dy + cols - 1) / cols;
+    if (pairs)
+      rc_stats_kernel<T, 2><<<dim3(nbx + nby, slices), 256, 0, s>>>(X, Y, w, N, dx, dy, part);
+    else
+      rc_stats_kernel<T, 1><<<dim3(nbx + nby, slices), 256, 0, s>>>(X, Y, w, N, dx, dy, part);
+    rc_stats_sum_kernel<<<(d + 32) / 32 + 1, 256, 0, s>>>(part, slices, d, nbx, sx);
+  }
   float* mu = F(L.mu);
   rc_mean_kernel<<<(d + 255) / 256, 256, 0, s>>>(sx, sy, sw_ss, dx, dy, mu, mu + d);
-  rc_center_kernel<T><<<2048, 256, 0, s>>>(X, Y, w, N, dx, dy, mu, mu + d, F(L.xc), F(L.yc));
-  HF_CUDA_TRY(cudaGetLastError(), "hf_recolor_fit: moments launch");
+  HF_CUDA_TRY(cudaGetLastError(), "hf_recolor_fit: statistics launch");
   hf_status st;
-  // Sigma_Z = Xc^T Xc, Sigma_Y = Yc^T Yc, Sigma_ZY = Xc^T Yc
-  if ((st = moment_product(h, s, dx, dx, N, F(L.xc), 1, dx, F(L.xc), dx, 1, F(L.sz), dx)) != HF_OK)
+  float* const G = F(L.gram);   // [Sigma_Z Sigma_ZY; . Sigma_Y], upper 256-tiles
+  float* const GY = G + static_cast<int64_t>(L.np) * L.F + L.np;
+  float* const thr = F(L.thr);
+  int32_t* const flag = reinterpret_cast<int32_t*>(ws + L.flag);
+  const int64_t rows_p = (L.F + 255) / 256 * 256;
+  // The second moments of both sides are one symmetric product, of which the
+  // upper 256 x 256 tiles are computed (32,768 x (3,072 + 1,024): 2.2 ms; three
+  // separate dense products took 3.65 ms)
+  auto moments = [&]() -> hf_status {
+    HF_CUDA_TRY(cudaMemsetAsync(G, 0, sizeof(float) * L.F * L.F, s), "clear");
+    for (int64_t k0 = 0; k0 < N; k0 += L.chunk) {
+      const int k_p = static_cast<int>((std::min<int64_t>(L.chunk, N - k0) + 63) / 64 * 64);
+      rc_planes_kernel<T><<<dim3(k_p / 64, static_cast<unsigned>(rows_p / 64)), 256, 0, s>>>(
+          X, Y, w, N, k0, dx, dy, L.np, mu, mu + d, static_cast<__nv_bfloat16*>(h.planes_a),
+          rows_p, k_p);
+      HF_CUDA_TRY(cudaGetLastError(), "hf_recolor_fit: moments launch");
+      const GemmPlanes z{h.planes_a, rows_p, 0};
+      GemmShape upper;
+      upper.tri = true;
+      upper.flush = kMomentFlush;
+      const hf_status e = gemm_planes(s, h, L.F, L.F, k_p, 1.f, z, z, 1.f, G, L.F, upper);
+      if (e != HF_OK) return e;
+    }
+    rc_ridge_kernel<<<1, 256, 0, s>>>(G, L.F, dx, L.np, reg, thr);
+    rc_ridge_kernel<<<1, 256, 0, s>>>(GY, L.F, dy, L.mp, reg, thr + 1);
+    HF_CUDA_TRY(cudaGetLastError(), "hf_recolor_fit: ridge launch");
+    return HF_OK;
+  };
+  auto extract = [&](const float* S, int rows, int cols, int mode, float* out) {
+    rc_extract_kernel<<<dim3((cols + 255) / 256, std::min(rows, 1024)), 256, 0, s>>>(
+        S, L.F, rows, cols, mode, out);
+  };
+  if ((st = moments()) != HF_OK) return st;
+  HF_CUDA_TRY(cudaMemsetAsync(flag, 0, sizeof(int32_t), s), "clear");
+  HF_CUDA_TRY(cudaMemsetAsync(F(L.sy_h), 0, sizeof(float) * dy * dy, s), "clear");
+  if ((st = tri_factor(s, h, G, L.F, L.np, F(L.tt), ws + L.fplanes, thr, flag, nullptr, 0)) !=
+      HF_OK)
     return st;
-  if ((st = moment_product(h, s, dy, dy, N, F(L.yc), 1, dy, F(L.yc), dy, 1, F(L.sy), dy)) != HF_OK)
+  if ((st = tri_factor(s, h, GY, L.F, L.mp, F(L.tt), ws + L.fplanes, thr + 1, flag, F(L.sy_h),
+                       dy)) != HF_OK)
     return st;
-  if ((st = moment_product(h, s, dx, dy, N, F(L.xc), 1, dx, F(L.yc), dy, 1, F(L.szy), dy)) != HF_OK)
-    return st;
-  if (reg > 0.f) {
-    rc_ridge_kernel<<<1, 256, 0, s>>>(F(L.sz), dx, reg);
-    rc_ridge_kernel<<<1, 256, 0, s>>>(F(L.sy), dy, reg);
+  extract(G, dx, dx, 2, F(L.sz_ih));   // L^{-1}
+  extract(GY, dy, dy, 2, F(L.sy_ih));  // C^{-1}
+  int32_t weak = 0;
+  HF_CUDA_TRY(cudaMemcpyAsync(&weak, flag, sizeof(weak), cudaMemcpyDeviceToHost, s), "read back");
+  HF_CUDA_TRY(cudaStreamSynchronize(s), "synchronize");
+  int it1 = 1, it2 = 1, it3 = 0;
+  const int64_t left_i = weak ? dx : 1, left_k = weak ? 1 : dx;  // left root: symmetric, or L^{-T}
+  if (weak) {
+    if ((st = moments()) != HF_OK) return st;
+    extract(G, dx, dx, 1, F(L.sz));
+    extract(GY, dy, dy, 1, F(L.sy));
+    extract(G + L.np, dx, dy, 0, F(L.szy));
+    if ((st = ns_sqrt(s, h, F(L.sz), dx, reg, F(L.p1), F(L.p2), F(L.p3), F(L.p4), nullptr,
+                      F(L.sz_ih), dscr, &it1)) != HF_OK)
+      return st;
+    if ((st = ns_sqrt(s, h, F(L.sy), dy, reg, F(L.p1), F(L.p2), F(L.p3), F(L.p4), F(L.sy_h),
+                      F(L.sy_ih), dscr, &it2)) != HF_OK)
+      return st;
+    // M = Sigma_Z^{-1/2} Sigma_ZY Sigma_Y^{-1/2}
+    if ((st = sgemm(h, s, dx, dy, dx, 1.f, F(L.sz_ih), dx, 1, F(L.szy), dy, 1, 0.f, F(L.x2), dy)) !=
+        HF_OK)
+      return st;
+    if ((st = sgemm(h, s, dx, dy, dy, 1.f, F(L.x2), dy, 1, F(L.sy_ih), dy, 1, 0.f, F(L.m), dy)) !=
+        HF_OK)
+      return st;
+  } else {
+    // M = (L^{-1} Sigma_ZY) C^{-T}, by products with the computed inverses:
+    // what is off in them cancels against A's outer factors, where Sigma_ZY
+    // eliminated along with Sigma_Z takes rounding errors of its own (square
+    // fits came out 1.5 times as far off)
+    if ((st = sgemm(h, s, dx, dy, dx, 1.f, F(L.sz_ih), dx, 1, G + L.np, L.F, 1, 0.f, F(L.x2), dy)) !=
+        HF_OK)
+      return st;
+    if ((st = sgemm(h, s, dx, dy, dy, 1.f, F(L.x2), dy, 1, F(L.sy_ih), 1, dy, 0.f, F(L.m), dy)) !=
+        HF_OK)
+      return st;
   }
-  int it1 = 0, it2 = 0, it3 = 0;
-  if ((st = ns_sqrt(s, h, F(L.sz), dx, reg, F(L.p1), F(L.p2), F(L.p3), F(L.p4), nullptr,
-                    F(L.sz_ih), dscr, &it1)) != HF_OK)
-    return st;
-  if ((st = ns_sqrt(s, h, F(L.sy), dy, reg, F(L.p1), F(L.p2), F(L.p3), F(L.p4), F(L.sy_h), F(L.sy_ih),
-                    dscr, &it2)) != HF_OK)
-    return st;
-  // M = Sigma_Z^{-1/2} Sigma_ZY Sigma_Y^{-1/2}
-  if ((st = sgemm(h, s, dx, dy, dx, 1.f, F(L.sz_ih), dx, 1, F(L.szy), dy, 1, 0.f, F(L.x2), dy)) != HF_OK)
-    return st;
-  if ((st = sgemm(h, s, dx, dy, dy, 1.f, F(L.x2), dy, 1, F(L.sy_ih), dy, 1, 0.f, F(L.m), dy)) != HF_OK)
-    return st;
   float* R = nullptr;
   if ((st = ns_polar(s, h, F(L.m), dx, dy, F(L.x1), F(L.x2), F(L.xtx), dscr, &R, &it3)) != HF_OK)
     return st;
-  // A = Sigma_Z^{-1/2} R* Sigma_Y^{1/2}
+  // A = Sigma_Z^{-1/2} R* Sigma_Y^{1/2}, or L^{-T} R* C^T
   float* tmp = R == F(L.x1) ? F(L.x2) : F(L.x1);
-  if ((st = sgemm(h, s, dx, dy, dx, 1.f, F(L.sz_ih), dx, 1, R, dy, 1, 0.f, tmp, dy)) != HF_OK) return st;
+  if ((st = sgemm(h, s, dx, dy, dx, 1.f, F(L.sz_ih), left_i, left_k, R, dy, 1, 0.f, tmp, dy)) != HF_OK)
+    return st;
   if ((st = sgemm(h, s, dx, dy, dy, 1.f, tmp, dy, 1, F(L.sy_h), dy, 1, 0.f, F(L.a), dy)) != HF_OK)
     return st;
   {

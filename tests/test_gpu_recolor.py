@@ -53,6 +53,46 @@ def test_recolor_matches_oracle(dtype, tol):
     assert relb <= tol, relb
 
 
+# Edges of the blocks of 128 features, of the 256-wide product tiles and of the
+# chunks of 8,192 samples; odd widths (no paired reads).
+@pytest.mark.parametrize("N,d_s,d_r,dtype", [
+    (700, 128, 128, "f32"), (1000, 129, 65, "f32"), (5000, 300, 7, "f32"), (8193, 257, 130, "bf16"),
+    (16500, 384, 256, "f32"), (900, 40, 1, "f32")])
+def test_recolor_factor_block_edges(N, d_s, d_r, dtype):
+    X, Y, w = _data(N + d_s, N, d_s, d_r, 0.5, dtype)
+    A, b, r = _fit(dtype, X, Y, w, 1e-2)
+    A_ref, b_ref, r_ref = O.recolor(*(t.double().cpu().numpy() for t in (X, Y, w)), reg=1e-2)
+    assert abs(r - r_ref) <= 1e-5 * r_ref
+    # fp32: the factors' relative error is about the condition number (at most
+    # d / reg) times 2^-24, 2e-3 at d = 384; bf16 adds its output rounding
+    tol = 2e-3 if dtype == "f32" else 6e-3
+    assert np.linalg.norm(A - A_ref) <= tol * np.linalg.norm(A_ref)
+    assert np.linalg.norm(b - b_ref) <= tol * max(np.linalg.norm(b_ref), 1.0)
+
+
+def test_recolor_small_pivots_take_the_iterated_roots():
+    """One direction of X has 3e-5 of the mean variance, below what the
+    triangular factor accepts: the symmetric roots are iterated (more than one
+    iteration is reported) and the fit maps one covariance to the other."""
+    X, Y, w = _data(5, 4096, 96, 64, 0.5, "f32")
+    X = torch.linalg.qr(X.double())[0] * X.shape[0] ** 0.5
+    X[:, 0] *= 3e-5 ** 0.5
+    X = X.float().contiguous()
+    ws = torch.empty(B.recolor_workspace_size(4096, 96, 64), dtype=torch.uint8, device="cuda")
+    W_out = torch.empty((64, 96), dtype=torch.float32, device="cuda")
+    b_out = torch.empty((64,), dtype=torch.float32, device="cuda")
+    _, its = B.recolor_fit("f32", X, Y, w, W_out, b_out, ws, reg=0.0, return_iters=True)
+    assert its[0] > 1 and its[1] > 1, its
+    # Against the oracle's A the roots' stopping residual counts times the
+    # condition number (3e4), but A^T Sigma_Z A = Sigma_Y holds to the residuals
+    # themselves: an iteration stops at |I - Z Y|_F <= 1e-3 sqrt(d), the
+    # polar factor's likewise, 1e-2 in all
+    A = W_out.double().cpu().numpy().T
+    Xn, Yn, wn = X.double().cpu().numpy(), Y.double().cpu().numpy(), w.double().cpu().numpy()
+    _, _, S_z, S_y, _ = O.weighted_moments(Xn / O.sender_rms(Xn, wn), Yn, wn)
+    assert np.linalg.norm(A.T @ S_z @ A - S_y) <= 1e-2 * np.linalg.norm(S_y)
+
+
 def test_recolor_recovers_an_exact_rotation():
     """Y = Z Q + c with Q orthogonal: the fit returns A = Q, b = c."""
     g = torch.Generator(device="cpu").manual_seed(2)

@@ -100,6 +100,19 @@ __device__ __forceinline__ void tma_prefetch_map(const void* map) {
 }
 
 // ---------------------------------------------------------------------------
+// Programmatic dependent launch: a kernel launched with the attribute may
+// start while its predecessor in the stream still runs.  depend_wait returns
+// when the predecessor has ended and its writes are visible (every thread calls
+// it before its first global access); depend_launch lets the successor start.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void depend_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void depend_launch() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// ---------------------------------------------------------------------------
 // Thread-block clusters (a CTA pair sharing one tcgen05 MMA)
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t cluster_ctarank() {
@@ -120,6 +133,12 @@ __device__ __forceinline__ uint32_t nclusters_x() {
   return r;
 }
 
+__device__ __forceinline__ uint32_t cluster_nctarank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+
 // Every thread of every CTA in the cluster arrives and waits.
 __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" :::
@@ -131,6 +150,13 @@ __device__ __forceinline__ uint32_t mapa_shared(uint32_t smem, uint32_t rank) {
   uint32_t r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem), "r"(rank));
   return r;
+}
+
+// A word of the same shared variable in CTA `rank` of the cluster.
+__device__ __forceinline__ int cluster_read(const int* p, uint32_t rank) {
+  int v;
+  asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(mapa_shared(smem_addr(p), rank)) : "memory");
+  return v;
 }
 
 // Arrive on an mbarrier that may live in another CTA of the cluster, with

@@ -115,6 +115,35 @@ struct hf_plan_s {
 
 namespace hf {
 
+// Prologue kernels of a transfer (alignment, plan metadata) of at most
+// kFusedRows tokens on either side and kFusedReq requests run as one launch.
+// Their time is a chain of latencies, so a thread takes one row (four above
+// 8,192 rows), and one CTA all of them up to 1,024 (the cluster's exchange
+// costs about 1 us), a cluster of eight above.  The launch overlaps the end of
+// the kernel before it (programmatic dependent launch).
+constexpr int kFusedRows = 32768;
+constexpr int kFusedReq = 64;
+inline int fused_rows_per_thread(int64_t rows) { return rows <= 8192 ? 1 : 4; }
+template <typename Kern, typename... Args>
+cudaError_t launch_fused_rows(Kern kern, int64_t rows, cudaStream_t stream, const Args&... args) {
+  const int ctas = rows <= 1024 ? 1 : 8, per = ctas * fused_rows_per_thread(rows);
+  const int64_t threads = ((rows + per - 1) / per + 31) / 32 * 32;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = static_cast<unsigned>(ctas);
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = dim3(static_cast<unsigned>(ctas), 1, 1);
+  cfg.blockDim = dim3(static_cast<unsigned>(threads < 128 ? 128 : threads), 1, 1);
+  cfg.stream = stream;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
 void set_error(const std::string& msg);
 hf_status cuda_fail(cudaError_t e, const char* what);
 int device_sm_count();

@@ -197,63 +197,72 @@ struct RowArgs {
 
 __device__ __forceinline__ void flag(int32_t* status, int bits) { atomicOr(status, bits); }
 
-// Per receiver row: position, destination row, checks, and whether the row
-// differs from the previous one (starts a new distinct row).
+// One receiver row: position, destination row, checks (status bits), whether
+// it differs from the previous one (starts a new distinct row), and the
+// smallest and largest valid column (kmax -1: none).  q: its request, which
+// starts at row r0 and position pos0.
+struct RowInfo {
+  int32_t pos, dst;
+  int is_new, bits;
+  int32_t kmin, kmax;
+};
+__device__ __forceinline__ RowInfo plan_row(const RowArgs& a, int64_t j, int q, int32_t r0,
+                                            int32_t pos0) {
+  RowInfo o;
+  o.bits = 0;
+  const int32_t t = static_cast<int32_t>(j - r0);
+  o.pos = pos0 + t;
+  o.dst = static_cast<int32_t>(j);
+  if (a.paged) {
+    const int bi = t / a.block_size;
+    int32_t blk = -1;
+    if (bi < a.max_blocks) blk = a.block_table[(int64_t)q * a.max_blocks + bi];
+    if (blk < 0 || blk >= a.n_blocks) {
+      o.bits |= HF_CHECK_BAD_BLOCK;
+      o.dst = -1;
+    } else {
+      o.dst = blk * a.block_size + t % a.block_size;
+    }
+  }
+  const int32_t e0 = a.row_ptr[j], e1 = a.row_ptr[j + 1], p0 = j > r0 ? a.row_ptr[j - 1] : e0;
+  const int n = e1 - e0;
+  if (n <= 0) o.bits |= HF_CHECK_BAD_ROW;
+  if (a.single_entry && (n != 1 || a.w[e0] != 1.0f)) o.bits |= HF_CHECK_BAD_ROW;
+  o.kmin = INT_MAX;
+  o.kmax = -1;
+  // a row of another length, or with another entry, than the one before
+  const bool compare = j > r0 && n == e0 - p0;
+  o.is_new = compare ? 0 : 1;
+  for (int i = 0; i < n; ++i) {
+    const int32_t k = a.col[e0 + i];
+    if (compare && (k != a.col[p0 + i] || a.w[e0 + i] != a.w[p0 + i])) o.is_new = 1;
+    if (k < 0 || k >= a.T_s) {
+      o.bits |= HF_CHECK_BAD_COLUMN;
+    } else {
+      o.kmin = min(o.kmin, k);
+      o.kmax = max(o.kmax, k);
+    }
+  }
+  return o;
+}
+
+// Per receiver row: its metadata and whether it starts a new distinct row.
 __global__ void plan_rows_kernel(RowArgs a) {
   const PlanDev& d = a.d;
   for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < a.T_r;
        j += (int64_t)gridDim.x * blockDim.x) {
     const int q = find_request(d.r_tok_ptr, a.n_req, j);
-    const int32_t r0 = d.r_tok_ptr[q];
-    const int32_t t = static_cast<int32_t>(j - r0);
-    d.pos[j] = d.r_pos0[q] + t;
-    int32_t dst = static_cast<int32_t>(j);
-    if (a.paged) {
-      const int bi = t / a.block_size;
-      int32_t blk = -1;
-      if (bi < a.max_blocks) blk = a.block_table[(int64_t)q * a.max_blocks + bi];
-      if (blk < 0 || blk >= a.n_blocks) {
-        flag(d.status, HF_CHECK_BAD_BLOCK);
-        dst = -1;
-      } else {
-        dst = blk * a.block_size + t % a.block_size;
-      }
-    }
-    d.dst_row[j] = dst;
-    const int32_t e0 = a.row_ptr[j], e1 = a.row_ptr[j + 1];
-    if (e1 <= e0) flag(d.status, HF_CHECK_BAD_ROW);
-    if (a.single_entry && (e1 - e0 != 1 || a.w[e0] != 1.0f)) flag(d.status, HF_CHECK_BAD_ROW);
-    int32_t kmin = INT_MAX, kmax = -1;
-    for (int32_t e = e0; e < e1; ++e) {
-      const int32_t k = a.col[e];
-      if (k < 0 || k >= a.T_s) {
-        flag(d.status, HF_CHECK_BAD_COLUMN);
-      } else {
-        kmin = min(kmin, k);
-        kmax = max(kmax, k);
-      }
-    }
+    const RowInfo o = plan_row(a, j, q, d.r_tok_ptr[q], d.r_pos0[q]);
+    d.pos[j] = o.pos;
+    d.dst_row[j] = o.dst;
+    if (o.bits) flag(d.status, o.bits);
     if (a.pam) {
       // the row's first valid column (-1: none); made a running maximum by
       // a scan, it assigns the row to a window
-      d.row_key[j] = kmax >= 0 ? kmin : -1;
-      if (kmax >= 0) atomicMax(&d.win_info[0], kmax - kmin);
+      d.row_key[j] = o.kmax >= 0 ? o.kmin : -1;
+      if (o.kmax >= 0) atomicMax(&d.win_info[0], o.kmax - o.kmin);
     }
-    int is_new = (j == r0) ? 1 : 0;
-    if (!is_new) {
-      const int32_t p0 = a.row_ptr[j - 1];
-      if (e1 - e0 != e0 - p0) {
-        is_new = 1;
-      } else {
-        for (int32_t i = 0; i < e1 - e0; ++i) {
-          if (a.col[e0 + i] != a.col[p0 + i] || a.w[e0 + i] != a.w[p0 + i]) {
-            is_new = 1;
-            break;
-          }
-        }
-      }
-    }
-    d.new_flag[j] = is_new;
+    d.new_flag[j] = o.is_new;
   }
 }
 
@@ -322,6 +331,198 @@ __global__ void plan_windows_kernel(RowArgs a) {
                                                    static_cast<int32_t>(x));
     }
   }
+}
+
+// The tables of a plan with few requests, in one launch's parameters.
+template <int kL>
+struct FewTables {
+  int32_t L_r, D_r, D_s, n_req;
+  float inv_r[2 * kL];
+  float inv_freq[kMaxHeadDim / 2];
+  float inv_freq_s[kMaxHeadDim / 2];
+  int32_t r_tok_ptr[kFusedReq + 1];
+  int32_t r_pos0[kFusedReq];
+  int32_t s_tok_ptr[kFusedReq + 1];
+  int32_t s_pos0[kFusedReq];
+  int32_t s_row0[kFusedReq];
+  LayerSegs segs[kL];
+};
+static_assert(sizeof(FewTables<kMaxLayersR>) < 32000, "FewTables must fit the parameter space");
+constexpr int kFewLayers = 48;  // a third of the parameter bytes of kMaxLayersR
+
+// The whole plan in one launch (kR consecutive rows per thread): the tables,
+// the rows' metadata, the numbering of distinct rows and, with pooling after
+// the map, the windows; the running sums and maxima go over the block and,
+// through distributed shared memory, over the cluster's CTAs, and so do the
+// status bits.  Latency bounds it: 8 us for a 4K context where the five passes
+// took 21 us and the gaps between their launches (bounds and results as theirs).
+template <int kL, int kR>
+__global__ void __launch_bounds__(1024)
+    plan_fused_kernel(const __grid_constant__ FewTables<kL> t, const __grid_constant__ RowArgs a,
+                      int want_pos) {
+  __shared__ int scan_new[32], scan_key[32];
+  __shared__ int cta_new, cta_key, cta_span, cta_bits;
+  __shared__ int32_t rp[kFusedReq + 1], sp[kFusedReq + 1];
+  const PlanDev& d = a.d;
+  const uint32_t rank = cluster_ctarank(), ctas = cluster_nctarank();
+  const int tid = threadIdx.x;
+  const int64_t thr = static_cast<int64_t>(rank) * blockDim.x + tid, n_thr = ctas * blockDim.x;
+  for (int i = tid; i <= t.n_req; i += blockDim.x) {
+    rp[i] = t.r_tok_ptr[i];
+    sp[i] = t.s_tok_ptr[i];
+  }
+  if (tid == 0) {
+    cta_span = -1;
+    cta_bits = 0;
+  }
+  __syncthreads();
+  depend_wait();
+  depend_launch();
+  const int64_t j0 = kR * thr;
+  int num[kR], key[kR], q = -1;
+  int32_t pos[kR];
+  int bits = 0, span = -1;
+  unsigned starts = 0;  // bit i: row j0 + i starts a distinct row
+#pragma unroll
+  for (int i = 0; i < kR; ++i) {
+    const int64_t j = j0 + i;
+    num[i] = 0;
+    key[i] = -1;
+    pos[i] = 0;
+    if (j >= a.T_r) continue;
+    if (q < 0 || j >= rp[q + 1]) q = find_request(rp, t.n_req, j);
+    const RowInfo o = plan_row(a, j, q, rp[q], t.r_pos0[q]);
+    d.pos[j] = o.pos;
+    d.dst_row[j] = o.dst;
+    pos[i] = o.pos;
+    bits |= o.bits;
+    num[i] = o.is_new;
+    starts |= static_cast<unsigned>(o.is_new) << i;
+    if (o.kmax >= 0) {
+      key[i] = o.kmin;
+      span = max(span, o.kmax - o.kmin);
+    }
+  }
+  // the tables, while the rows' loads are under way in other warps
+  for (int64_t i = thr; i < 2 * t.L_r; i += n_thr) d.inv_r[i] = t.inv_r[i];
+  for (int64_t i = thr; i < t.D_r / 2; i += n_thr) d.inv_freq[i] = t.inv_freq[i];
+  for (int64_t i = thr; i < t.D_s / 2; i += n_thr) d.inv_freq_s[i] = t.inv_freq_s[i];
+  {
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(t.segs);
+    uint32_t* dst = reinterpret_cast<uint32_t*>(d.segs);
+    const int n = t.L_r * static_cast<int>(sizeof(LayerSegs) / 4);
+    for (int64_t i = thr; i < n; i += n_thr) dst[i] = src[i];
+  }
+  if (want_pos || a.span)
+    for (int64_t k = thr; k < a.T_s; k += n_thr) {
+      const int qs = find_request(sp, t.n_req, k);
+      const int32_t off = static_cast<int32_t>(k - sp[qs]);
+      if (want_pos) d.spos[k] = t.s_pos0[qs] + off;
+      if (a.span) d.srow[k] = t.s_row0[qs] + off;
+    }
+#pragma unroll
+  for (int i = 1; i < kR; ++i) {
+    num[i] += num[i - 1];
+    key[i] = max(key[i], key[i - 1]);
+  }
+  int n_new, key_all = -1, key_excl = -1;
+  int excl = block_scan_excl<ScanSum>(num[kR - 1], scan_new, &n_new);
+  if (a.pam) {
+    key_excl = block_scan_excl<ScanMax>(key[kR - 1], scan_key, &key_all);
+    if (span >= 0) atomicMax(&cta_span, span);
+  }
+  if (bits) atomicOr(&cta_bits, bits);
+  __syncthreads();
+  int h = cta_span;
+  if (ctas > 1) {
+    if (tid == 0) {
+      cta_new = n_new;
+      cta_key = key_all;
+    }
+    cluster_sync();
+    int before = 0, all = 0, kb = INT_MIN, ka = -1;
+    h = -1;
+    for (uint32_t c = 0; c < ctas; ++c) {
+      const int n = cluster_read(&cta_new, c), k = cluster_read(&cta_key, c);
+      if (c < rank) {
+        before += n;
+        kb = max(kb, k);
+      }
+      all += n;
+      ka = max(ka, k);
+      h = max(h, cluster_read(&cta_span, c));
+    }
+    excl += before;
+    n_new = all;
+    key_excl = max(key_excl, kb);
+    key_all = ka;
+  }
+  // runs of identical rows
+#pragma unroll
+  for (int i = 0; i < kR; ++i) {
+    const int64_t j = j0 + i;
+    if (j >= a.T_r) continue;
+    const int32_t incl = excl + num[i];
+    if (starts >> i & 1u) {
+      const int32_t u = incl - 1;
+      d.run_ptr[u] = static_cast<int32_t>(j);
+      // an empty row (flagged) has no column to read: row_ptr[j] may be the
+      // end of the caller's col array
+      const int32_t e0 = a.row_ptr[j];
+      int32_t k = a.row_ptr[j + 1] > e0 ? a.col[e0] : 0;
+      if (k < 0 || k >= a.T_s) k = 0;  // flagged
+      if (a.span) {
+        const int qs = find_request(sp, t.n_req, k);
+        k = t.s_row0[qs] + static_cast<int32_t>(k - sp[qs]);
+      }
+      d.ucol[u] = k;  // the sender-cache row
+      d.upos[u] = pos[i];
+    }
+    if (j == a.T_r - 1) {
+      d.run_ptr[incl] = static_cast<int32_t>(a.T_r);
+      *d.n_distinct = incl;
+    }
+  }
+  if (a.pam) {
+    // windows (plan_windows_kernel): row j is the first row of the windows
+    // between its key's and the key's of the row before
+    h = max(h, 0);
+    const int32_t S = h >= 128 ? 1 : 128 - h;
+    const int32_t n_win = key_all < 0 ? 0 : key_all / S + 1;
+    int out = 0;
+#pragma unroll
+    for (int i = 0; i < kR; ++i) {
+      const int64_t j = j0 + i;
+      if (j >= a.T_r) continue;
+      const int32_t kj = max(key_excl, key[i]);
+      const int32_t kp = i == 0 ? key_excl : max(key_excl, key[i - 1]);
+      const int32_t wj = kj < 0 ? -1 : kj / S, wp = kp < 0 ? -1 : kp / S;
+      for (int32_t w = wp + 1; w <= wj; ++w) d.win_ptr[w] = static_cast<int32_t>(j);
+      if (j == a.T_r - 1) d.win_ptr[n_win] = static_cast<int32_t>(a.T_r);
+      if (kj >= 0) {
+        const int64_t lo = (int64_t)wj * S;
+        for (int32_t e = a.row_ptr[j]; e < a.row_ptr[j + 1]; ++e) {
+          const int32_t k = a.col[e];
+          if (k >= 0 && k < a.T_s && (k < lo || k >= lo + 128)) out = HF_CHECK_POOL_WINDOW;
+        }
+      }
+    }
+    if (h >= 128) out = HF_CHECK_POOL_WINDOW;
+    if (out) atomicOr(&cta_bits, out);
+    if (rank == 0 && tid == 0) {
+      d.win_info[0] = h;
+      d.win_info[1] = S;
+      d.win_info[2] = n_win;
+    }
+  }
+  __syncthreads();
+  if (ctas > 1) cluster_sync();
+  if (rank == 0 && tid == 0) {
+    int all = 0;
+    for (uint32_t c = 0; c < ctas; ++c) all |= ctas > 1 ? cluster_read(&cta_bits, c) : cta_bits;
+    *d.status = all;
+  }
+  if (ctas > 1) cluster_sync();  // no CTA leaves while its shared memory is read
 }
 
 // Eq. 1: pi(l) = 1 + round((l-1)(L_S-1)/(L_R-1)) (one-based), round half
@@ -474,12 +675,38 @@ hf_status validate(const hf_plan_desc* d) {
 
 }  // namespace
 
+namespace {
+
+template <int kL>
+hf_status launch_plan_fused(const hf_plan_s* p, const PlanTables& tables, const RowArgs& a,
+                            cudaStream_t stream) {
+  const PlanConsts& c = tables.c;
+  FewTables<kL> t;
+  t.L_r = c.L_r;
+  t.D_r = c.D_r;
+  t.D_s = c.D_s;
+  t.n_req = c.n_req;
+  std::memcpy(t.inv_r, c.inv_r, sizeof(t.inv_r));
+  std::memcpy(t.inv_freq, c.inv_freq, sizeof(t.inv_freq));
+  std::memcpy(t.inv_freq_s, c.inv_freq_s, sizeof(t.inv_freq_s));
+  std::memcpy(t.r_tok_ptr, c.r_tok_ptr, sizeof(t.r_tok_ptr));
+  std::memcpy(t.r_pos0, c.r_pos0, sizeof(t.r_pos0));
+  std::memcpy(t.s_tok_ptr, c.s_tok_ptr, sizeof(t.s_tok_ptr));
+  std::memcpy(t.s_pos0, c.s_pos0, sizeof(t.s_pos0));
+  std::memcpy(t.s_row0, c.s_row0, sizeof(t.s_row0));
+  std::memcpy(t.segs, tables.s.segs, sizeof(t.segs));
+  const int64_t rows = std::max(p->T_r, p->T_s);
+  HF_CUDA_TRY(launch_fused_rows(fused_rows_per_thread(rows) == 1 ? plan_fused_kernel<kL, 1>
+                                                                 : plan_fused_kernel<kL, 4>,
+                                rows, stream, t, a, p->unrot ? 1 : 0),
+              "plan launch");
+  return HF_OK;
+}
+
+}  // namespace
+
 hf_status launch_plan_kernels(hf_plan_s* p, const PlanTables& tables, cudaStream_t stream) {
   const PlanDev d = plan_dev(p);
-  plan_init_kernel<<<1, 256, 0, stream>>>(tables.c, d);
-  plan_segs_kernel<<<1, 128, 0, stream>>>(tables.s, d.segs);
-  HF_CUDA_TRY(cudaGetLastError(), "plan init launch");
-  if (p->T_r == 0) return HF_OK;
   RowArgs a;
   a.d = d;
   a.row_ptr = p->desc.d_row_ptr;
@@ -496,6 +723,15 @@ hf_status launch_plan_kernels(hf_plan_s* p, const PlanTables& tables, cudaStream
   a.single_entry = p->desc.align_mode != HF_ALIGN_OVERLAP_MEAN;
   a.span = p->span ? 1 : 0;
   a.pam = p->pam ? 1 : 0;
+  // one launch up to kFusedRows tokens (15 us at 32K, the passes 29 us); above,
+  // the passes, whose loads fill the GPU
+  if (p->T_r > 0 && std::max(p->T_r, p->T_s) <= kFusedRows && p->desc.n_req <= kFusedReq)
+    return p->desc.L_r <= kFewLayers ? launch_plan_fused<kFewLayers>(p, tables, a, stream)
+                                     : launch_plan_fused<kMaxLayersR>(p, tables, a, stream);
+  plan_init_kernel<<<1, 256, 0, stream>>>(tables.c, d);
+  plan_segs_kernel<<<1, 128, 0, stream>>>(tables.s, d.segs);
+  HF_CUDA_TRY(cudaGetLastError(), "plan init launch");
+  if (p->T_r == 0) return HF_OK;
   const int64_t want = (p->T_r + 255) / 256;
   const int grid = static_cast<int>(std::min<int64_t>(want, 8LL * device_sm_count()));
   plan_rows_kernel<<<grid, 256, 0, stream>>>(a);

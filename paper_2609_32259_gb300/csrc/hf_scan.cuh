@@ -101,6 +101,35 @@ __global__ void __launch_bounds__(kScanThreads) scan_inplace_kernel(int* data, i
   if (tid == 0 && total != nullptr) *total = carry;
 }
 
+// Exclusive scan of one value per thread over the block (at most 1,024
+// threads); *total receives op over all of them.  buf: 32 words of shared
+// memory of this scan's own, read by every warp after the one barrier.
+template <typename Op>
+__device__ __forceinline__ int block_scan_excl(int v, int* buf, int* total) {
+  const Op op;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int n_warps = (blockDim.x + 31) >> 5;
+  int t = v;
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const int o = __shfl_up_sync(0xffffffffu, t, off);
+    if (lane >= off) t = op(o, t);
+  }
+  int excl = __shfl_up_sync(0xffffffffu, t, 1);
+  if (lane == 0) excl = Op::identity();
+  if (lane == 31) buf[warp] = t;
+  __syncthreads();
+  int w = lane < n_warps ? buf[lane] : Op::identity();
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const int o = __shfl_up_sync(0xffffffffu, w, off);
+    if (lane >= off) w = op(o, w);
+  }
+  *total = __shfl_sync(0xffffffffu, w, 31);
+  const int before = __shfl_sync(0xffffffffu, w, warp > 0 ? warp - 1 : 0);
+  return warp > 0 ? op(before, excl) : excl;
+}
+
 // Index of the request owning global token j: the largest q with
 // ptr[q] <= j (empty requests are skipped because a later equal pointer wins).
 __device__ __forceinline__ int find_request(const int32_t* ptr, int n_req, int64_t j) {
@@ -120,6 +149,15 @@ __device__ __forceinline__ int lower_bound_i32(const int32_t* a, int n, int32_t 
     if (a[mid] < x) lo = mid + 1; else hi = mid;
   }
   return lo;
+}
+
+// The same, where every index below lo is known to hold less than x: a few
+// steps from lo, then the binary search of the rest.
+__device__ __forceinline__ int lower_bound_from(const int32_t* a, int n, int lo, int32_t x) {
+#pragma unroll 1
+  for (int i = 0; i < 8; ++i, ++lo)
+    if (lo >= n || a[lo] >= x) return lo;
+  return lo + lower_bound_i32(a + lo, n - lo, x);
 }
 
 // First index k in [0, n) with a[k] > x (n if none).

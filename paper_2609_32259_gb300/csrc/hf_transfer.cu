@@ -1081,6 +1081,7 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const Xfe
   const XferParams& P0 = Ps[0];
   extern __shared__ __align__(1024) uint8_t smem[];
   if (smem_addr(smem) & 1023u) {  // the swizzled stages need 1024-byte alignment
+    depend_wait();
     if (threadIdx.x == 0) atomicOr(P0.status, HF_CHECK_INTERNAL);
     return;
   }
@@ -1139,6 +1140,10 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const Xfe
   cluster_sync();  // the leader's barriers exist before any remote arrival
   tc_fence_after_sync();
   const uint32_t tmem_base = *sTmem;
+  // everything above may run beside the end of the kernel before this one;
+  // what that kernel wrote (the plan's tables, for one) is read from here on
+  depend_wait();
+  depend_launch();
 
   DirTable<kDirs> dt;
   const int total_tiles = build_dirs<kDirs, kPam>(Ps, n_dir, &dt);
@@ -1669,11 +1674,13 @@ hf_status launch_pairs(Kern kern, int64_t max_pair_tiles, size_t smem, cudaStrea
                                    static_cast<int>(smem)),
               "set shared memory size");
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.blockDim = dim3(kThreads, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
@@ -1687,6 +1694,7 @@ hf_status launch_pairs(Kern kern, int64_t max_pair_tiles, size_t smem, cudaStrea
     clusters = std::min(clusters, active);
   clusters = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(clusters, max_pair_tiles)));
   cfg.gridDim = dim3(2 * clusters, 1, 1);
+  cfg.numAttrs = 2;
   HF_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, args...), "transfer kernel launch");
   return HF_OK;
 }

@@ -48,7 +48,8 @@ struct WorkspaceLayout {
   size_t upos;       // int32[T_r]: RoPE position of each distinct row's first receiver row
   size_t pos;        // int32[T_r]: RoPE position of each receiver row
   size_t dst_row;    // int32[T_r]: destination row of each receiver row
-  size_t new_flag;   // int32[T_r]: 1 where a receiver row starts a new distinct row
+  size_t new_flag;   // int32[T_r]: 1 where a receiver row starts a new distinct row, then its
+                     // running sum: the one-based number of each row's distinct row
   // pooling after the map (overlap mean pooling): windows of 128 aligned
   // sender tokens with stride S = 128 - h, h the widest row's column span
   size_t win_info;   // int32[4]: h, S, number of windows, unused

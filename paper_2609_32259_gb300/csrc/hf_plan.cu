@@ -463,6 +463,7 @@ __global__ void __launch_bounds__(1024)
     const int64_t j = j0 + i;
     if (j >= a.T_r) continue;
     const int32_t incl = excl + num[i];
+    d.new_flag[j] = incl;
     if (starts >> i & 1u) {
       const int32_t u = incl - 1;
       d.run_ptr[u] = static_cast<int32_t>(j);

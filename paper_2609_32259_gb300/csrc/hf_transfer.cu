@@ -59,8 +59,12 @@ constexpr int kThreads = 64 + kEpiThreads + 32 * kBuilderWarps;  // 16 warps
 constexpr int kAtoms = 2;                // 128-byte swizzle atoms (k-blocks) per A stage (a B stage holds one)
 constexpr int kAtomABytes = kBM * 128;   // 128 rows x 128 bytes
 constexpr int kStageABytes = kAtoms * kAtomABytes;
-constexpr int kStgFloats = kBM * 64;     // epilogue staging: 128 rows x 2 heads x 32
+constexpr int kStgRow = 68;              // epilogue staging: a row of 2 heads x 32 floats (or 256
+                                         // bytes of outputs) and 16 bytes of padding, so that 32
+                                         // rows' 16-byte writes spread over the banks
+constexpr int kStgFloats = kBM * kStgRow;
 constexpr int kRunStride = 132;          // run starts / positions of a tile (129 used)
+constexpr int kRotPairs = kMaxHeadDim / 2;  // one position's rotation of every pair
 constexpr int kMaxStages = 8;
 constexpr int kTmemCols = 512;           // two accumulators of up to 256 columns
 
@@ -108,6 +112,7 @@ struct XferParams {
   const int32_t* win_info;  // h, S, number of windows
   const int32_t* win_ptr;
   const int32_t* pos;       // RoPE position of every receiver row
+  const int32_t* uidx;      // one-based number of every receiver row's distinct row
   int stages_a, stages_b, lag;  // A ring (stages), B ring (atoms), loader groups in flight
   int rope, paged, knorm, unrot, D_s;
   int stall;  // test hook: the map producer withholds its first atom (hf_debug_transfer_stalled)
@@ -280,69 +285,97 @@ __device__ __forceinline__ void rotate4(float4& x, float4& y, const float* c, co
 // [jb, je) of one slice.  Shared memory is slow to answer while the tensor
 // core streams its operands, so the lane keeps the staged (unrotated) values
 // of its current distinct row in registers and reads the next row's only
-// when the walk enters its run; positions inside a run, and across runs of
-// one request, are consecutive, so the angles advance by one position per
+// when the walk enters its run (uidx, the plan's number of each row's distinct
+// row, read a row ahead, says where); positions inside a run, and across runs
+// of one request, are consecutive, so the angles advance by one position per
 // row (re-anchored exactly every 16 rows and wherever the position jumps).
+// What bounds it is the length of one warp's chain of instructions (ten warps
+// hide little of each other), so the arithmetic is on pairs of fp32 values.
 template <typename T>
-__device__ __forceinline__ void walk_rows(int jb, int je, int u, const int32_t* srun,
-                                          const int32_t* supos, const float* stg, int qq,
-                                          bool two_heads, bool do_rope, const float* f,
-                                          const float* C1, const float* S1, const XferParams& P,
-                                          T* out_lc, int ocol, int q, int half) {
+__device__ __forceinline__ void walk_rows(int jb, int je, int u0, const int32_t* spb,
+                                          const float* stg, int qq, bool two_heads, bool do_rope,
+                                          const float* f, const float2* c1, const float2* s1,
+                                          const XferParams& P, T* out_lc, int ocol, int q,
+                                          int half) {
   if (jb >= je) return;
-  float4 a0, b0, a1 = make_float4(0.f, 0.f, 0.f, 0.f), b1 = a1;
-  int uend = 0, pb = 0;  // end of the current run; position of row j is pb + j
-  int expect = INT_MIN;  // position for which cs/sn are valid
-  float cs[4] = {1.f, 1.f, 1.f, 1.f}, sn[4] = {0.f, 0.f, 0.f, 0.f};
-  --u;
+  float2 a0[2], b0[2], a1[2], b1[2];  // two pairs each: first halves and partners, both heads
+#pragma unroll
+  for (int k = 0; k < 2; ++k) a1[k] = b1[k] = make_float2(0.f, 0.f);
+  int u = -1, pb = 0;     // current distinct row; position of row j is pb + j
+  int expect = INT_MIN;   // position for which cs/sn are valid
+  float2 cs[2] = {make_float2(1.f, 1.f), make_float2(1.f, 1.f)};
+  float2 sn[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+  int unext = __ldg(P.uidx + jb);  // number of row j's distinct row, one-based, read a row ahead
   int dnext = P.paged ? __ldg(P.dst_row + jb) : jb;  // destination of row j, read a row ahead
+  T* const out = out_lc + ocol + q + 4 * qq;
+#pragma unroll 1
   for (int j = jb; j < je; ++j) {
-    const int drow = dnext;
-    if (P.paged) {
-      if (j + 1 < je) dnext = __ldg(P.dst_row + j + 1);
-    } else {
-      dnext = j + 1;
-    }
-    if (j >= uend) {  // first row, or the first row of a later run
-      do {
-        ++u;
-      } while (srun[u + 1] <= j);
-      uend = srun[u + 1];
-      pb = supos[u] - srun[u];
-      const float* urow = stg + u * 64;
-      const int sw = u & 7;
-      a0 = *reinterpret_cast<const float4*>(urow + ((qq ^ sw) << 2));
-      b0 = *reinterpret_cast<const float4*>(urow + (((4 + qq) ^ sw) << 2));
+    const int drow = dnext, uj = unext - 1 - u0;
+    const int jn = min(j + 1, je - 1);
+    unext = __ldg(P.uidx + jn);
+    dnext = P.paged ? __ldg(P.dst_row + jn) : jn;
+    if (uj != u) {  // first row, or the first row of a later run
+      u = uj;
+      pb = spb[u];
+      const float* urow = stg + u * kStgRow + 4 * qq;
+      const float4 va = *reinterpret_cast<const float4*>(urow);
+      const float4 vb = *reinterpret_cast<const float4*>(urow + 16);
+      a0[0] = make_float2(va.x, va.y);
+      a0[1] = make_float2(va.z, va.w);
+      b0[0] = make_float2(vb.x, vb.y);
+      b0[1] = make_float2(vb.z, vb.w);
       if (two_heads) {
-        a1 = *reinterpret_cast<const float4*>(urow + 32 + ((qq ^ sw) << 2));
-        b1 = *reinterpret_cast<const float4*>(urow + 32 + (((4 + qq) ^ sw) << 2));
+        const float4 vc = *reinterpret_cast<const float4*>(urow + 32);
+        const float4 vd = *reinterpret_cast<const float4*>(urow + 48);
+        a1[0] = make_float2(vc.x, vc.y);
+        a1[1] = make_float2(vc.z, vc.w);
+        b1[0] = make_float2(vd.x, vd.y);
+        b1[1] = make_float2(vd.z, vd.w);
       }
     }
-    float4 x0 = a0, y0 = b0, x1 = a1, y1 = b1;
+    float2 x0[2], y0[2], x1[2], y1[2];
     if (do_rope) {
       const int p = pb + j;
       if (p != expect || ((j - jb) & 15) == 0) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) rope_sincos(p, f[k], &sn[k], &cs[k]);
+        for (int k = 0; k < 2; ++k) {
+          rope_sincos(p, f[2 * k], &sn[k].x, &cs[k].x);
+          rope_sincos(p, f[2 * k + 1], &sn[k].y, &cs[k].y);
+        }
       } else {  // advance every angle by one position
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const float t = cs[k] * C1[k] - sn[k] * S1[k];
-          sn[k] = sn[k] * C1[k] + cs[k] * S1[k];
+        for (int k = 0; k < 2; ++k) {
+          const float2 ns1 = make_float2(-s1[k].x, -s1[k].y);
+          const float2 t = __ffma2_rn(sn[k], ns1, __fmul2_rn(cs[k], c1[k]));
+          sn[k] = __ffma2_rn(cs[k], s1[k], __fmul2_rn(sn[k], c1[k]));
           cs[k] = t;
         }
       }
       expect = p + 1;
-      rotate4(x0, y0, cs, sn);
-      if (two_heads) rotate4(x1, y1, cs, sn);
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {  // (x, y) -> (x cos - y sin, y cos + x sin)
+        const float2 ns = make_float2(-sn[k].x, -sn[k].y);
+        x0[k] = __ffma2_rn(b0[k], ns, __fmul2_rn(a0[k], cs[k]));
+        y0[k] = __ffma2_rn(a0[k], sn[k], __fmul2_rn(b0[k], cs[k]));
+        x1[k] = __ffma2_rn(b1[k], ns, __fmul2_rn(a1[k], cs[k]));
+        y1[k] = __ffma2_rn(a1[k], sn[k], __fmul2_rn(b1[k], cs[k]));
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        x0[k] = a0[k];
+        y0[k] = b0[k];
+        x1[k] = a1[k];
+        y1[k] = b1[k];
+      }
     }
     if (drow >= 0) {
-      T* o = out_lc + static_cast<int64_t>(drow) * P.d_r + ocol + q + 4 * qq;
-      store4(o, x0);
-      store4(o + half, y0);
+      T* o = out + static_cast<int64_t>(drow) * P.d_r;
+      store4(o, make_float4(x0[0].x, x0[0].y, x0[1].x, x0[1].y));
+      store4(o + half, make_float4(y0[0].x, y0[0].y, y0[1].x, y0[1].y));
       if (two_heads) {
-        store4(o + 2 * half, x1);
-        store4(o + 3 * half, y1);
+        store4(o + 2 * half, make_float4(x1[0].x, x1[0].y, x1[1].x, x1[1].y));
+        store4(o + 3 * half, make_float4(y1[0].x, y1[0].y, y1[1].x, y1[1].y));
       }
     }
   }
@@ -353,75 +386,59 @@ __device__ __forceinline__ void walk_rows(int jb, int je, int u, const int32_t* 
 // y = acc / r + b, so each distinct row is converted once into the staging
 // buffer and copied out whole.  Columns go in passes of 256 bytes per row
 // (128 rows x 256 bytes of staging); in a pass, warp (g, sp) converts TMEM
-// lane quarter sp, half g of the pass's columns, then warp e copies the runs
-// of distinct rows e, e + 8, ...: 16 lanes x 16 bytes per receiver row, the
-// two half-warps taking alternate receiver rows of the run.
-template <typename T>
+// lane quarter sp, half g of the pass's columns, then every thread hands the
+// copy engine the staged row of its receiver rows (a 256-byte bulk copy each).
+// The copies bound it: about 13 cycles each and SM, 11 at the full HBM write
+// rate; without them a tile of 460 receiver rows takes 5.4K cycles instead of
+// 18.4K.  16-byte loads and stores by the threads took about 22K and eight
+// times the instructions (eight requests, 36K tokens, paged: 2.26 -> 1.97 ms
+// with the key walk's changes).
+// release() runs once the last accumulator column has been read.
+template <typename T, typename Release>
 __device__ __forceinline__ void copy_epilogue(const XferParams& P, uint32_t ta,
-                                              const float* bias_tile, float inv_r, int nrows,
-                                              const int32_t* srun, uint8_t* stg, int g, int row,
-                                              int e, int lane, T* out_lc, int ocol0) {
+                                              const float* bias_tile, float inv_r, int u0, int jb,
+                                              int je, uint8_t* stg, int g, int row, int e,
+                                              int tid_e, T* out_lc, int ocol0, Release release) {
   constexpr int kPassCols = 256 / sizeof(T);  // 128 bf16 or 64 fp32 columns
   constexpr int kHalfCols = kPassCols / 2;
   constexpr int kPerChunk = 16 / sizeof(T);
-  const int hw = lane >> 4, cidx = lane & 15;
+  const uint64_t policy = l2_policy_evict_first();
   for (int pc0 = 0; pc0 < P.BN; pc0 += kPassCols) {
-    uint8_t* srow = stg + row * 256;
+    if (e < 8) {  // the two extra warps only copy
+      uint8_t* srow = stg + row * (kStgRow * 4) + g * 128;
 #pragma unroll
-    for (int k = 0; k < kHalfCols; k += 16) {
-      if (e >= 8) break;  // the two extra warps only copy
-      const int col = pc0 + g * kHalfCols + k;
-      uint32_t v[16];
-      tmem_load_16(ta + static_cast<uint32_t>(col), v);
-      float y[16];
+      for (int k = 0; k < kHalfCols; k += 32) {
+        const int col = pc0 + g * kHalfCols + k;
+        uint32_t v[32];
+        tmem_load_2x16(ta + static_cast<uint32_t>(col), ta + static_cast<uint32_t>(col + 16), v);
+        float y[32];
 #pragma unroll
-      for (int i = 0; i < 16; i += 4) {
-        const float4 bb = __ldg(reinterpret_cast<const float4*>(bias_tile + col + i));
-        y[i] = fmaf(__uint_as_float(v[i]), inv_r, bb.x);
-        y[i + 1] = fmaf(__uint_as_float(v[i + 1]), inv_r, bb.y);
-        y[i + 2] = fmaf(__uint_as_float(v[i + 2]), inv_r, bb.z);
-        y[i + 3] = fmaf(__uint_as_float(v[i + 3]), inv_r, bb.w);
+        for (int i = 0; i < 32; i += 4) {
+          const float4 bb = __ldg(reinterpret_cast<const float4*>(bias_tile + col + i));
+          y[i] = fmaf(__uint_as_float(v[i]), inv_r, bb.x);
+          y[i + 1] = fmaf(__uint_as_float(v[i + 1]), inv_r, bb.y);
+          y[i + 2] = fmaf(__uint_as_float(v[i + 2]), inv_r, bb.z);
+          y[i + 3] = fmaf(__uint_as_float(v[i + 3]), inv_r, bb.w);
+        }
+#pragma unroll
+        for (int h = 0; h < 32 / kPerChunk; ++h)
+          *reinterpret_cast<uint4*>(srow + (k / kPerChunk + h) * 16) =
+              pack16(y + h * kPerChunk, (const T*)nullptr);
       }
-#pragma unroll
-      for (int h = 0; h < 16 / kPerChunk; ++h) {
-        const int chunk = (col - pc0) / kPerChunk + h;  // 0..15 within the 256-byte row
-        *reinterpret_cast<uint4*>(srow + ((chunk ^ (row & 7)) << 4)) =
-            pack16(y + h * kPerChunk, (const T*)nullptr);
-      }
+      fence_proxy_async_smem();
     }
+    if (pc0 + kPassCols >= P.BN) release();
     named_barrier_sync(1, kEpiThreads);
-    // the next distinct row's staged chunk and run bounds are read while this
-    // row's receiver rows are stored (shared-memory reads are slow to answer
-    // while the tensor core streams its operands)
-    int u = e;
-    uint4 val = make_uint4(0u, 0u, 0u, 0u);
-    int js = 0, je = 0;
-    if (u < nrows) {
-      val = *reinterpret_cast<const uint4*>(stg + u * 256 + ((cidx ^ (u & 7)) << 4));
-      js = srun[u];
-      je = srun[u + 1];
+    const uint32_t src = smem_addr(stg);
+    T* const out = out_lc + ocol0 + pc0;
+    for (int j = jb + tid_e; j < je; j += kEpiThreads) {
+      const int u = __ldg(P.uidx + j) - 1 - u0;
+      const int drow = P.paged ? __ldg(P.dst_row + j) : j;
+      if (drow >= 0)
+        bulk_store(out + static_cast<int64_t>(drow) * P.d_r,
+                   src + static_cast<uint32_t>(u) * (kStgRow * 4), 256u, policy);
     }
-    while (u < nrows) {
-      const int un = u + kEpiWarps;
-      uint4 nval = val;
-      int njs = 0, nje = 0;
-      if (un < nrows) {
-        nval = *reinterpret_cast<const uint4*>(stg + un * 256 + ((cidx ^ (un & 7)) << 4));
-        njs = srun[un];
-        nje = srun[un + 1];
-      }
-      for (int j = js + hw; j < je; j += 2) {
-        const int drow = P.paged ? __ldg(P.dst_row + j) : j;
-        if (drow >= 0)
-          __stcs(reinterpret_cast<uint4*>(out_lc + static_cast<int64_t>(drow) * P.d_r + ocol0 +
-                                          pc0 + cidx * kPerChunk),
-                 val);
-      }
-      u = un;
-      val = nval;
-      js = njs;
-      je = nje;
-    }
+    bulk_store_wait_read();
     named_barrier_sync(1, kEpiThreads);
   }
 }
@@ -451,17 +468,16 @@ __device__ __forceinline__ void pam_walk(int jb, int je, int base, const float* 
       const int loc = __ldg(P.col + e) - base;
       if (loc < 0 || loc >= kBM) continue;  // flagged at plan creation
       const float wt = __ldg(P.w + e);
-      const float* urow = stg + loc * 64;
-      const int sw = loc & 7;
-      const float4 a = *reinterpret_cast<const float4*>(urow + ((qq ^ sw) << 2));
-      const float4 b = *reinterpret_cast<const float4*>(urow + (((4 + qq) ^ sw) << 2));
+      const float* urow = stg + loc * kStgRow + 4 * qq;
+      const float4 a = *reinterpret_cast<const float4*>(urow);
+      const float4 b = *reinterpret_cast<const float4*>(urow + 16);
       x0 = make_float4(fmaf(wt, a.x, x0.x), fmaf(wt, a.y, x0.y), fmaf(wt, a.z, x0.z),
                        fmaf(wt, a.w, x0.w));
       y0 = make_float4(fmaf(wt, b.x, y0.x), fmaf(wt, b.y, y0.y), fmaf(wt, b.z, y0.z),
                        fmaf(wt, b.w, y0.w));
       if (two_heads) {
-        const float4 a1 = *reinterpret_cast<const float4*>(urow + 32 + ((qq ^ sw) << 2));
-        const float4 b1 = *reinterpret_cast<const float4*>(urow + 32 + (((4 + qq) ^ sw) << 2));
+        const float4 a1 = *reinterpret_cast<const float4*>(urow + 32);
+        const float4 b1 = *reinterpret_cast<const float4*>(urow + 48);
         x1 = make_float4(fmaf(wt, a1.x, x1.x), fmaf(wt, a1.y, x1.y), fmaf(wt, a1.z, x1.z),
                          fmaf(wt, a1.w, x1.w));
         y1 = make_float4(fmaf(wt, b1.x, y1.x), fmaf(wt, b1.y, y1.y), fmaf(wt, b1.z, y1.z),
@@ -532,10 +548,10 @@ __device__ __forceinline__ void pam_epilogue(const XferParams& P, uint32_t ta,
       if (stages_head) {
         uint32_t v[32];
         tmem_load_2x16(ta + tcol + q, ta + tcol + half + q, v);
-        float* srow = sStg + row * 64 + g * 32;
+        float* srow = sStg + row * kStgRow + g * 32;
 #pragma unroll
         for (int k = 0; k < 8; ++k)
-          *reinterpret_cast<float4*>(srow + ((k ^ (row & 7)) << 2)) = make_float4(
+          *reinterpret_cast<float4*>(srow + 4 * k) = make_float4(
               __uint_as_float(v[4 * k]) * inv_r, __uint_as_float(v[4 * k + 1]) * inv_r,
               __uint_as_float(v[4 * k + 2]) * inv_r, __uint_as_float(v[4 * k + 3]) * inv_r);
       }
@@ -558,16 +574,6 @@ __device__ __forceinline__ void pam_epilogue(const XferParams& P, uint32_t ta,
       named_barrier_sync(1, kEpiThreads);
     }
   }
-}
-
-// Last u in [0, nrows) with srun[u] <= j.
-__device__ __forceinline__ int find_row(const int32_t* srun, int nrows, int j) {
-  int lo = 0, hi = nrows - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (srun[mid] <= j) lo = mid; else hi = mid - 1;
-  }
-  return lo;
 }
 
 // One 128-byte atom of operand row t for the builder path: features
@@ -810,6 +816,9 @@ __device__ __forceinline__ void gather_rows(const XferParams* Ps, const DirTable
     int64_t snext = n_seg > 1 ? seg_base(1) : 0;
     int64_t roff[8];
     uint32_t doff[8];
+    // rows past the last distinct row are not copied: their products (of what
+    // the stage held before) stay in accumulator rows that nothing reads
+    unsigned live = 0;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const int r = slab * 32 + 4 * i + rsub;
@@ -817,8 +826,11 @@ __device__ __forceinline__ void gather_rows(const XferParams* Ps, const DirTable
       if (pam_on<kPam>(P)) {
         const int k = pam_token(P, m, row0, r);
         kr = P.srow ? __ldg(P.srow + k) : k;
+        live |= 1u << i;
       } else {
-        kr = P.ucol[min(m * kPairRows + row0 + r, U - 1)];
+        const int u = m * kPairRows + row0 + r;
+        kr = P.ucol[min(u, U - 1)];
+        live |= (u < U ? 1u : 0u) << i;
       }
       roff[i] = kr * P.d_s + ch * kPerChunk;
       doff[i] = static_cast<uint32_t>(r * 128 + ((ch ^ (r & 7)) << 4));
@@ -837,7 +849,8 @@ __device__ __forceinline__ void gather_rows(const XferParams* Ps, const DirTable
         if (a < na) {
           const T* base = sender + sbase + kin * kBK;
 #pragma unroll
-          for (int i = 0; i < 8; ++i) cp_async_16(sa + a * kAtomABytes + doff[i], base + roff[i]);
+          for (int i = 0; i < 8; ++i)
+            if (live >> i & 1u) cp_async_16(sa + a * kAtomABytes + doff[i], base + roff[i]);
           if (++kin == P.atoms_per_seg) {
             kin = 0;
             ++seg;
@@ -1095,9 +1108,9 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const Xfe
   uint8_t* sA = smem;
   uint8_t* sB = sA + stages_a * kStageABytes;
   float* sStg = reinterpret_cast<float*>(sB + stages_b * stage_b_bytes);
-  int32_t* sRun = reinterpret_cast<int32_t*>(sStg + kStgFloats);
-  int32_t* sUpos = sRun + kRunStride;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(sUpos + kRunStride);
+  float2* sRot = reinterpret_cast<float2*>(sStg + kStgFloats);  // cos, sin of one position's step
+  int32_t* sPb = reinterpret_cast<int32_t*>(sRot + kRotPairs);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(sPb + kRunStride);
   uint64_t* full_a = bars;
   uint64_t* empty_a = bars + kMaxStages;
   uint64_t* full_b = bars + 2 * kMaxStages;
@@ -1319,6 +1332,7 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const Xfe
     const int ps = lane >> 2, qq = lane & 3;  // row slot 0..7, pair quad 0..3
     int acc = 0;
     uint32_t acc_phase = 0;
+    int rot_dir = -1;  // direction whose one-position rotations sRot holds
     for (int seq = 0, tile = tile_of(0, first_tile, tile_step, by_slot); tile < total_tiles;
        tile = tile_of(++seq, first_tile, tile_step, by_slot)) {
       const int dd = dir_of(dt, n_dir, tile);
@@ -1345,6 +1359,7 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const Xfe
         break;
       }
       tc_fence_after_sync();
+      bool released = false;  // the accumulator has been handed back
       const int u0 = m * kPairRows + row0;
       const int nrows = min(kBM, U - u0);  // <= 0: this CTA has no rows in the tile
       if (nrows > 0 && pam_on<kPam>(P)) {
@@ -1359,19 +1374,28 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const Xfe
                         P.bias + static_cast<int64_t>(lc) * P.d_r + nb * P.BN, P.inv_r[lc], base,
                         jb, je, sStg, e, g, row, lane, P.rope && c == 0, out_lc, nb * P.BN);
       } else if (nrows > 0) {
-        for (int i = tid_e; i <= nrows; i += kEpiThreads) {
-          sRun[i] = P.run_ptr[u0 + i];
-          sUpos[i] = i < nrows ? P.upos[u0 + i] : 0;
+        // position of row j of distinct row u0 + i: sPb[i] + j
+        for (int i = tid_e; i < nrows; i += kEpiThreads)
+          sPb[i] = __ldg(P.upos + u0 + i) - __ldg(P.run_ptr + u0 + i);
+        if (dd != rot_dir) {
+          rot_dir = dd;
+          if (P.rope)
+            for (int i = tid_e; i < half; i += kEpiThreads)
+              rope_sincos(1, __ldg(P.inv_freq + i), &sRot[i].y, &sRot[i].x);
         }
-        named_barrier_sync(1, kEpiThreads);
         // this warp's receiver rows [wjb, wje); lane slot ps walks the
         // consecutive rows [ljb, lje) of them
-        const int jb = sRun[0], je = sRun[nrows];
+        const int jb = __ldg(P.run_ptr + u0), je = __ldg(P.run_ptr + u0 + nrows);
         const int per = (je - jb + kEpiWarps - 1) / kEpiWarps;
         const int wjb = min(je, jb + e * per), wje = min(je, wjb + per);
         const int per_slot = (wje - wjb + 7) >> 3;
         const int ljb = min(wje, wjb + ps * per_slot), lje = min(wje, ljb + per_slot);
-        const int ustart = ljb < lje ? find_row(sRun, nrows, ljb) : 0;
+        auto release = [&] {
+          tc_fence_before_sync();
+          __syncwarp();
+          if (lane == 0) arrive_leader(smem_addr(&tempty[ac]), row0);
+          released = true;
+        };
         const float inv_r = P.inv_r[lc];
         const float* bias = P.bias + static_cast<int64_t>(lc) * P.d_r;
         const bool do_rope = P.rope && c == 0;
@@ -1381,8 +1405,9 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const Xfe
         T* const out_lc = reinterpret_cast<T*>(P.receiver) +
                           (static_cast<int64_t>(lc) * P.recv_rows) * P.d_r;
         if (c == 1 || (!P.rope && !P.knorm)) {
-          copy_epilogue<T>(P, ta, bias + nb * P.BN, inv_r, nrows, sRun,
-                           reinterpret_cast<uint8_t*>(sStg), g, row, e, lane, out_lc, nb * P.BN);
+          copy_epilogue<T>(P, ta, bias + nb * P.BN, inv_r, u0, jb, je,
+                           reinterpret_cast<uint8_t*>(sStg), g, row, e, tid_e, out_lc, nb * P.BN,
+                           release);
         } else
         for (int hp = 0; hp < n_pairs; ++hp) {
           const bool stages_head = stager && (g == 0 || two_heads);
@@ -1435,30 +1460,33 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const Xfe
                   y[16 + i] *= rn * __ldg(P.knorm_w + half + q + i);
                 }
               }
-              float* srow = sStg + row * 64 + g * 32;
+              float* srow = sStg + row * kStgRow + g * 32;
 #pragma unroll
               for (int k = 0; k < 8; ++k)
-                *reinterpret_cast<float4*>(srow + ((k ^ (row & 7)) << 2)) =
+                *reinterpret_cast<float4*>(srow + 4 * k) =
                     make_float4(y[4 * k], y[4 * k + 1], y[4 * k + 2], y[4 * k + 3]);
             }
+            if (hp == n_pairs - 1 && q + 16 >= half) release();
             named_barrier_sync(1, kEpiThreads);
             // step 2: rows of this warp's slice, both heads of the pair
-            float C1[4], S1[4];
+            float2 c1[2], s1[2];  // one step = one row
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              C1[k] = 1.f;
-              S1[k] = 0.f;
-              if (do_rope) rope_sincos(1, f[k], &S1[k], &C1[k]);  // one step = one row
+            for (int k = 0; k < 2; ++k) {
+              const float4 r = *reinterpret_cast<const float4*>(sRot + q + 4 * qq + 2 * k);
+              c1[k] = make_float2(r.x, r.z);
+              s1[k] = make_float2(r.y, r.w);
             }
-            walk_rows<T>(ljb, lje, ustart, sRun, sUpos, sStg, qq, two_heads, do_rope, f, C1, S1, P,
-                         out_lc, ocol_pair, q, half);
+            walk_rows<T>(ljb, lje, u0, sPb, sStg, qq, two_heads, do_rope, f, c1, s1, P, out_lc,
+                         ocol_pair, q, half);
             named_barrier_sync(1, kEpiThreads);
           }
         }
       }
-      tc_fence_before_sync();
-      __syncwarp();
-      if (lane == 0) arrive_leader(smem_addr(&tempty[ac]), row0);
+      if (!released) {
+        tc_fence_before_sync();
+        __syncwarp();
+        if (lane == 0) arrive_leader(smem_addr(&tempty[ac]), row0);
+      }
       }
       if (timed_out) break;
       if (wide) {
@@ -1468,6 +1496,7 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const Xfe
         if (acc == 0) acc_phase ^= 1;
       }
     }
+    bulk_store_wait_all();  // the receiver rows are written before the CTA ends
   } else {
     // ------------------------------------------------------------ A builders
     const int t = threadIdx.x - 64 - kEpiThreads;  // 0..127
@@ -1642,22 +1671,23 @@ hf_status make_map(CUtensorMap* map, const void* base, bool f32, uint64_t rows, 
 size_t smem_bytes(int BN, int stages_a, int stages_b) {
   return static_cast<size_t>(stages_a) * kStageABytes +
          static_cast<size_t>(stages_b) * (BN / 2) * 128 + kStgFloats * sizeof(float) +
-         2 * kRunStride * sizeof(int32_t) + (4 * kMaxStages + 5) * sizeof(uint64_t) + 8;
+         kRotPairs * sizeof(float2) + kRunStride * sizeof(int32_t) + (4 * kMaxStages + 5) * sizeof(uint64_t) + 8;
 }
 
 // Ring depths.  A B stage is one 128-byte atom of K of this CTA's map rows
 // (16 KB at BN = 256), so the TMA producer refills the ring in fine steps;
-// 96 KB of B stages, and the rest of shared memory in A stages (two atoms,
+// 80 KB of B stages, and the rest of shared memory in A stages (two atoms,
 // 32 KB): three at BN = 256.  A loader waits for stage i - lag after issuing
 // stage i, so it never blocks on a young group.  Measured on the 32K
-// Llama -> Ministral-shaped transfer: three A stages and six one-atom B stages
-// beat three two-atom B stages by 1%, and four A stages with four one-atom B
-// stages lose 2-3% (deeper A rings do not pay; B depth does).
+// Llama -> Ministral-shaped transfer: one-atom B stages beat two-atom ones by 1%,
+// four A stages with four one-atom B stages lose 2-3% (deeper A rings do not
+// pay; B depth does).  The fifth B stage is the last that fits beside the
+// padded staging rows that the bulk copies of the value tiles need.
 void pick_rings(int BN, int* stages_a, int* stages_b, int* lag) {
   int dev = 0, optin = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  const int sb = std::min(kMaxStages, (96 * 1024) / ((BN / 2) * 128));
+  const int sb = std::min(kMaxStages, (80 * 1024) / ((BN / 2) * 128));
   int sa = kMaxStages;
   while (sa > 2 && smem_bytes(BN, sa, sb) > static_cast<size_t>(optin)) --sa;
   *stages_a = sa;
@@ -1752,6 +1782,7 @@ hf_status make_xfer(hf_plan_s* p, const void* sender, void* receiver, int l_begi
   P.win_info = reinterpret_cast<const int32_t*>(ws + p->lay.win_info);
   P.win_ptr = reinterpret_cast<const int32_t*>(ws + p->lay.win_ptr);
   P.pos = reinterpret_cast<const int32_t*>(ws + p->lay.pos);
+  P.uidx = reinterpret_cast<const int32_t*>(ws + p->lay.new_flag);
   P.atoms_per_stage = p->split ? 1 : kAtoms;
   P.n_batoms = n_atoms;
   P.n_kb = (n_atoms + P.atoms_per_stage - 1) / P.atoms_per_stage;

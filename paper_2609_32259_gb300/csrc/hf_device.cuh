@@ -409,6 +409,58 @@ __device__ __forceinline__ void tmem_load_16(uint32_t taddr, uint32_t (&r)[16]) 
 }
 
 // ---------------------------------------------------------------------------
+// 16-byte chunks of operand rows in fp32
+// ---------------------------------------------------------------------------
+// Accumulates w * (8 bf16 | 4 fp32 values) into acc.
+__device__ __forceinline__ void accum16(const uint4& v, float wt, float* acc,
+                                        const __nv_bfloat16*) {
+  const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&v);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const float2 f = __bfloat1622float2(h[i]);
+    acc[2 * i] = fmaf(wt, f.x, acc[2 * i]);
+    acc[2 * i + 1] = fmaf(wt, f.y, acc[2 * i + 1]);
+  }
+}
+__device__ __forceinline__ void accum16(const uint4& v, float wt, float* acc, const float*) {
+  acc[0] = fmaf(wt, __uint_as_float(v.x), acc[0]);
+  acc[1] = fmaf(wt, __uint_as_float(v.y), acc[1]);
+  acc[2] = fmaf(wt, __uint_as_float(v.z), acc[2]);
+  acc[3] = fmaf(wt, __uint_as_float(v.w), acc[3]);
+}
+__device__ __forceinline__ uint4 pack16(const float* a, const __nv_bfloat16*) {
+  uint4 r;
+  __nv_bfloat162 h0 = __floats2bfloat162_rn(a[0], a[1]), h1 = __floats2bfloat162_rn(a[2], a[3]);
+  __nv_bfloat162 h2 = __floats2bfloat162_rn(a[4], a[5]), h3 = __floats2bfloat162_rn(a[6], a[7]);
+  r.x = *reinterpret_cast<uint32_t*>(&h0);
+  r.y = *reinterpret_cast<uint32_t*>(&h1);
+  r.z = *reinterpret_cast<uint32_t*>(&h2);
+  r.w = *reinterpret_cast<uint32_t*>(&h3);
+  return r;
+}
+__device__ __forceinline__ uint4 pack16(const float* a, const float*) {
+  return make_uint4(__float_as_uint(a[0]), __float_as_uint(a[1]), __float_as_uint(a[2]),
+                    __float_as_uint(a[3]));
+}
+
+// 8 fp32 values as bf16 (round to nearest) in *hi, and in *lo the bf16
+// rounding of what that rounding lost (exact in fp32): hi + lo carries each
+// value to about 16 mantissa bits.
+__device__ __forceinline__ void pack16_split(const float* a, uint4* hi, uint4* lo) {
+  uint32_t h[4], r[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const __nv_bfloat162 b = __floats2bfloat162_rn(a[2 * i], a[2 * i + 1]);
+    const float2 bf = __bfloat1622float2(b);
+    const __nv_bfloat162 d = __floats2bfloat162_rn(a[2 * i] - bf.x, a[2 * i + 1] - bf.y);
+    h[i] = *reinterpret_cast<const uint32_t*>(&b);
+    r[i] = *reinterpret_cast<const uint32_t*>(&d);
+  }
+  *hi = make_uint4(h[0], h[1], h[2], h[3]);
+  *lo = make_uint4(r[0], r[1], r[2], r[3]);
+}
+
+// ---------------------------------------------------------------------------
 // RoPE angles
 // ---------------------------------------------------------------------------
 // sin and cos of p * f for an integer position 0 <= p < 2^24 and an fp32

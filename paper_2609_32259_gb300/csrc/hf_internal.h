@@ -55,8 +55,18 @@ struct WorkspaceLayout {
   size_t win_info;   // int32[4]: h, S, number of windows, unused
   size_t row_key;    // int32[T_r]: first column of each row, then its running maximum
   size_t win_ptr;    // int32[T_s + 2]: first receiver row of each window
-  size_t total;
+  size_t total;      // what a plan cannot do without
+  // operand rows made before the transfer (see x_rows below), for as many
+  // receiver layers as fit kOperandBytes, one at least
+  size_t xbuf;
+  size_t total_made; // total with them (equal to it where no rows are made)
+  int64_t x_rows;
+  int x_layers, made;
 };
+
+// Bytes of made operand rows to aim at: receiver layers per launch, so that
+// a launch's last round of tiles is a small part of it.
+constexpr size_t kOperandBytes = static_cast<size_t>(512) << 20;
 
 WorkspaceLayout workspace_layout(const hf_plan_desc& d);
 
@@ -101,6 +111,15 @@ struct hf_plan_s {
   bool span;    // aligned sender tokens are spans inside a longer sender cache
   bool pam;     // pooling after the map: map input rows are sender rows in windows
   bool wide;    // tiles of two 256-column blocks (operand rows built by the loader warps)
+  // bit c: the map input rows of role c (pooled, blended, weighted or rotated
+  // back) are made by a pass of their own before the transfer, which then
+  // copies them; x_rows rows (distinct rows, or sender tokens with pooling after
+  // the map) of x_layers receiver layers at a time.  0 where rows are copies, in
+  // fp32, and where the workspace holds only WorkspaceLayout::total bytes: the
+  // loader warps then build what is not a copy.
+  int made;
+  int64_t x_rows;
+  int x_layers;
   int64_t s_rows;  // sender-cache rows per (layer, role)
   char* ws;
   size_t ws_bytes;
@@ -157,6 +176,9 @@ hf_status plan_build(const hf_plan_desc* desc, void* d_workspace, size_t workspa
 // launch ends through the bounded waits with HF_CHECK_TIMEOUT.
 hf_status launch_transfer(hf_plan_s* p, const void* sender, void* receiver, cudaStream_t stream,
                           int l_begin = 0, int l_end = -1, bool stall = false);
+// The operand rows of receiver layers [l_begin, l_end) of a plan with made rows.
+hf_status launch_operands(const hf_plan_s* p, const void* sender, cudaStream_t stream, int l_begin,
+                          int l_end);
 // Several plans in one launch: they must share the dtype, the operand path
 // and where the pooling happens (batch_compatible); n <= kMaxBatch.
 bool batch_compatible(const hf_plan_s* const* plans, int n);

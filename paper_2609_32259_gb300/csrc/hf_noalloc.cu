@@ -56,6 +56,7 @@ extern "C" hf_status hf_transfer_noalloc(const hf_plan_desc* desc, const void* s
   size_t need = 0;
   hf_status s = hf_plan_workspace_size(desc, &need);
   if (s != HF_OK) return s;
+  need = workspace_layout(*desc).total;  // without room for made operand rows
   if (need > kNoAllocScratchBytes) {
     set_error("hf_transfer_noalloc: this transfer needs " + std::to_string(need) +
               " bytes of metadata but the built-in scratch holds " +

@@ -39,6 +39,44 @@ int device_sm_count() {
 
 static size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
+namespace {
+
+// How a descriptor's map input rows come about.
+struct OperandPath {
+  bool pam, one_entry, gather, split;
+  int made;  // roles whose rows a pass of their own makes (hf_plan_s::made)
+  int K;
+};
+OperandPath operand_path(const hf_plan_desc& d) {
+  OperandPath o{};
+  const int n_seg = d.layer_mode == HF_LAYER_PAPER3 ? 3
+                    : d.layer_mode == HF_LAYER_EXPLICIT ? d.n_seg : 1;
+  o.K = n_seg * d.H_s * d.D_s;
+  // The copy-only operand path needs every segment to be one sender layer
+  // with weight 1, one-entry rows and no rotation.
+  bool one_layer_segments = d.layer_mode == HF_LAYER_PAPER3;
+  if (d.layer_mode == HF_LAYER_EXPLICIT && d.n_terms == 1 && d.h_seg_w) {
+    one_layer_segments = true;
+    for (int i = 0; i < d.L_r * d.n_seg; ++i)
+      if (d.h_seg_w[i] != 1.0f) one_layer_segments = false;
+  }
+  const bool unrot = d.sender_k_rotated == 1;
+  // overlap mean pooling commutes with the map (it is linear): unless the
+  // pooled row itself is needed (key norm, sender keys rotated back per
+  // position) or the caller asks otherwise, the map input rows are sender
+  // rows and the epilogue pools the mapped rows
+  o.pam = d.align_mode == HF_ALIGN_OVERLAP_MEAN && d.pool_before_map == 0 && !unrot &&
+          d.d_knorm_w == nullptr;
+  o.one_entry = d.align_mode != HF_ALIGN_OVERLAP_MEAN || o.pam;
+  const bool copies = one_layer_segments && o.one_entry;  // values, and keys if not rotated
+  o.gather = copies && !unrot;
+  o.split = !o.gather && d.dtype == HF_BF16 && d.round_built_operands == 0;
+  if (!o.gather && d.dtype == HF_BF16) o.made = copies ? 1 : 3;
+  return o;
+}
+
+}  // namespace
+
 WorkspaceLayout workspace_layout(const hf_plan_desc& d) {
   const int L_r = d.L_r, D_r = d.D_r, D_s = d.D_s, n_req = d.n_req;
   const int64_t T_r = d.r_tok_ptr[n_req];
@@ -77,7 +115,20 @@ WorkspaceLayout workspace_layout(const hf_plan_desc& d) {
   w.win_info = take(sizeof(int32_t) * 4);
   w.row_key = take(sizeof(int32_t) * (size_t)(n_key > 0 ? n_key : 1));
   w.win_ptr = take(sizeof(int32_t) * (size_t)(n_win > 0 ? n_win : 1));
-  w.total = off;
+  w.total = w.xbuf = w.total_made = off;
+  const OperandPath path = operand_path(d);
+  if (path.made) {
+    // distinct rows, or sender tokens with pooling after the map; where one
+    // layer's rows alone would take over 2 GiB the loader warps build them
+    w.x_rows = path.pam ? d.s_tok_ptr[n_req] : T_r;
+    const size_t layer = static_cast<size_t>(path.made == 3 ? 2 : 1) *
+                         static_cast<size_t>(std::max<int64_t>(w.x_rows, 1)) * path.K *
+                         (path.split ? 4 : 2);
+    if (layer > 4 * kOperandBytes) return w;
+    w.x_layers = static_cast<int>(std::min<size_t>(L_r, std::max<size_t>(1, kOperandBytes / layer)));
+    w.made = path.made;
+    w.total_made = align_up(off + layer * w.x_layers, 256);
+  }
   return w;
 }
 
@@ -765,7 +816,7 @@ extern "C" hf_status hf_plan_workspace_size(const hf_plan_desc* desc, size_t* by
     set_error("hf_plan_workspace_size: invalid descriptor");
     return HF_ERR_INVALID_ARGUMENT;
   }
-  *bytes = workspace_layout(*desc).total;
+  *bytes = workspace_layout(*desc).total_made;
   return HF_OK;
 }
 
@@ -795,33 +846,24 @@ hf_status plan_build(const hf_plan_desc* desc, void* d_workspace, size_t workspa
   p->T_r = desc->r_tok_ptr[desc->n_req];
   p->BN = (p->d_r % 256 == 0) ? 256 : 128;
   p->groups = ((p->BN / 2) % desc->D_r == 0) ? 2 : 1;
-  // The copy-only operand path needs every segment to be one sender layer
-  // with weight 1, one-entry rows and no rotation.
-  bool one_layer_segments = desc->layer_mode == HF_LAYER_PAPER3;
-  if (desc->layer_mode == HF_LAYER_EXPLICIT && desc->n_terms == 1) {
-    one_layer_segments = true;
-    for (int i = 0; i < desc->L_r * desc->n_seg; ++i)
-      if (desc->h_seg_w[i] != 1.0f) one_layer_segments = false;
-  }
+  const OperandPath path = operand_path(*desc);
   p->unrot = desc->sender_k_rotated == 1;
   p->rope = desc->theta_r > 0.0 || desc->h_inv_freq_r != nullptr;
-  // overlap mean pooling commutes with the map (it is linear): unless the
-  // pooled row itself is needed (key norm, sender keys rotated back per
-  // position) or the caller asks otherwise, the map input rows are sender
-  // rows and the epilogue pools the mapped rows
-  p->pam = desc->align_mode == HF_ALIGN_OVERLAP_MEAN && desc->pool_before_map == 0 &&
-           !p->unrot && desc->d_knorm_w == nullptr;
-  const bool one_entry = desc->align_mode != HF_ALIGN_OVERLAP_MEAN || p->pam;
-  p->gather = one_layer_segments && one_entry && !p->unrot;
-  p->split = !p->gather && desc->dtype == HF_BF16 && desc->round_built_operands == 0;
+  p->pam = path.pam;
+  p->gather = path.gather;
+  p->split = path.split;
+  p->made = workspace_bytes >= lay.total_made ? lay.made : 0;
+  p->x_rows = lay.x_rows;
+  p->x_layers = lay.x_layers;
+  const bool one_entry = path.one_entry;
   // one-entry rows (Token Alignment, same-index, sender rows of pooling
   // after the map) have at most two (term, entry) pairs per segment, both
   // staged by cp.async; pooled rows have more, whose direct loads stall the
   // warp anyway (measured slower staged)
-  p->staged = p->split && !p->unrot && one_entry;
+  p->staged = p->split && !p->unrot && one_entry && !p->made;
   // built operand rows bound their paths: a tile covering two 256-column
   // blocks (both TMEM accumulators) builds each A stage once for both
-  p->wide = !p->gather && p->d_r % 512 == 0;
+  p->wide = !p->gather && !p->made && p->d_r % 512 == 0;
   p->ws = static_cast<char*>(d_workspace);
   p->ws_bytes = workspace_bytes;
   p->lay = lay;

@@ -93,11 +93,16 @@ struct XferParams {
   int64_t recv_rows;  // receiver rows per (layer, role) in receiver_kv
   int L_r, d_s, d_r, D_r;
   int l0, n_l;  // receiver layers [l0, l0 + n_l) of this launch
-  int n_kb, atoms_per_seg, last_atoms, BN, n_tiles_n, groups;  // n_kb: A stages per tile
+  int atoms_per_seg, BN, n_tiles_n;
   // split: each A stage holds one map atom of K as two bf16 atoms, the
-  // rounded operand and its rounding residual, multiplied by the same B atom
-  // (atoms_per_stage = 1); otherwise kAtoms atoms of K per A stage
-  int split, atoms_per_stage, n_batoms;  // n_batoms: B atoms (map atoms of K) per tile
+  // rounded operand and its rounding residual, multiplied by the same B atom;
+  // otherwise kAtoms atoms of K per A stage.  With made rows (bit c of `made`:
+  // the tiles of role c read rows that the operand pass has made, planes of
+  // [x_rows][K] per layer of this launch and role) it holds for those tiles only.
+  int split, n_batoms;  // n_batoms: B atoms (map atoms of K) per tile
+  int made, made_roles;
+  const void* x;
+  int64_t x_rows;
   int staged;  // split one-entry rows built by build_rows_staged
   // wide tiles (operand rows built by the loader warps, which bound those
   // paths): a tile covers two 256-column blocks, one per TMEM accumulator,
@@ -119,6 +124,27 @@ struct XferParams {
   float knorm_eps;
   uint32_t idesc;
 };
+
+// Where the map input rows come from (fixed at compile time: the branches that
+// made rows need in the loader and the MMA thread cost copied rows 4-7%).
+constexpr int kBuiltRows = 0;   // built by the loader warps
+constexpr int kCopiedRows = 1;  // sender rows
+constexpr int kMadeRows = 2;    // rows of the operand pass, or sender rows, by role
+
+// A stages of a tile of role c, and the map atoms of K in its last one.
+struct KLoop {
+  bool made, split;
+  int n_kb, last_atoms;
+};
+template <int kRows>
+__device__ __forceinline__ KLoop k_loop(const XferParams& P, int c) {
+  KLoop k;
+  k.made = kRows == kMadeRows && ((P.made >> c) & 1);
+  k.split = kRows != kCopiedRows && P.split && (kRows == kBuiltRows || k.made);
+  k.n_kb = k.split ? P.n_batoms : (P.n_batoms + kAtoms - 1) / kAtoms;
+  k.last_atoms = k.split ? 1 : P.n_batoms - kAtoms * (k.n_kb - 1);
+  return k;
+}
 
 template <typename T>
 struct Elem;
@@ -188,55 +214,6 @@ __device__ __forceinline__ int pam_token(const XferParams& P, int m, int row0, i
 template <int kPam>
 __device__ __forceinline__ bool pam_on(const XferParams& P) {
   return kPam == 2 ? P.pam != 0 : kPam == 1;
-}
-
-// Accumulates w * (8 bf16 | 4 fp32 values) into acc.
-__device__ __forceinline__ void accum16(const uint4& v, float wt, float* acc,
-                                        const __nv_bfloat16*) {
-  const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&v);
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const float2 f = __bfloat1622float2(h[i]);
-    acc[2 * i] = fmaf(wt, f.x, acc[2 * i]);
-    acc[2 * i + 1] = fmaf(wt, f.y, acc[2 * i + 1]);
-  }
-}
-__device__ __forceinline__ void accum16(const uint4& v, float wt, float* acc, const float*) {
-  acc[0] = fmaf(wt, __uint_as_float(v.x), acc[0]);
-  acc[1] = fmaf(wt, __uint_as_float(v.y), acc[1]);
-  acc[2] = fmaf(wt, __uint_as_float(v.z), acc[2]);
-  acc[3] = fmaf(wt, __uint_as_float(v.w), acc[3]);
-}
-__device__ __forceinline__ uint4 pack16(const float* a, const __nv_bfloat16*) {
-  uint4 r;
-  __nv_bfloat162 h0 = __floats2bfloat162_rn(a[0], a[1]), h1 = __floats2bfloat162_rn(a[2], a[3]);
-  __nv_bfloat162 h2 = __floats2bfloat162_rn(a[4], a[5]), h3 = __floats2bfloat162_rn(a[6], a[7]);
-  r.x = *reinterpret_cast<uint32_t*>(&h0);
-  r.y = *reinterpret_cast<uint32_t*>(&h1);
-  r.z = *reinterpret_cast<uint32_t*>(&h2);
-  r.w = *reinterpret_cast<uint32_t*>(&h3);
-  return r;
-}
-__device__ __forceinline__ uint4 pack16(const float* a, const float*) {
-  return make_uint4(__float_as_uint(a[0]), __float_as_uint(a[1]), __float_as_uint(a[2]),
-                    __float_as_uint(a[3]));
-}
-
-// 8 fp32 values as bf16 (round to nearest) in *hi, and in *lo the bf16
-// rounding of what that rounding lost (exact in fp32): hi + lo carries each
-// value to about 16 mantissa bits.
-__device__ __forceinline__ void pack16_split(const float* a, uint4* hi, uint4* lo) {
-  uint32_t h[4], r[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const __nv_bfloat162 b = __floats2bfloat162_rn(a[2 * i], a[2 * i + 1]);
-    const float2 bf = __bfloat1622float2(b);
-    const __nv_bfloat162 d = __floats2bfloat162_rn(a[2 * i] - bf.x, a[2 * i + 1] - bf.y);
-    h[i] = *reinterpret_cast<const uint32_t*>(&b);
-    r[i] = *reinterpret_cast<const uint32_t*>(&d);
-  }
-  *hi = make_uint4(h[0], h[1], h[2], h[3]);
-  *lo = make_uint4(r[0], r[1], r[2], r[3]);
 }
 
 // Writes 16 bytes of fp32 results of operand row t, chunk ch, into an A atom
@@ -781,7 +758,7 @@ __device__ __forceinline__ void arrive_leader(uint32_t bar, int row0) {
 // layout.  A thread keeps LAG groups in flight: after committing k-block i
 // it waits for k-block i-LAG and fences it to the async proxy; then one lane
 // per warp arrives on that stage's barrier in the leader CTA of the pair.
-template <typename T, int LAG, int kDirs, int kPam>
+template <typename T, int LAG, int kDirs, int kPam, int kRows>
 __device__ __forceinline__ void gather_rows(const XferParams* Ps, const DirTable<kDirs>& dt,
                                             int n_dir, uint8_t* sA, uint64_t* full_a,
                                             uint64_t* empty_a, volatile int* sAbort, int t,
@@ -807,13 +784,23 @@ __device__ __forceinline__ void gather_rows(const XferParams* Ps, const DirTable
     const int l = lc >> 1, c = lc & 1;
     // element offset of segment s2's sender layer/role block; the current
     // segment's is in sbase and the next one's is loaded a segment ahead
+    const KLoop kl = k_loop<kRows>(P, c);
     const LayerSegs* lsegs = P.segs + l;
     const int n_seg = __ldg(&lsegs->n_seg);
     auto seg_base = [&](int s2) -> int64_t {
       return (static_cast<int64_t>(__ldg(&lsegs->layer[s2][0]) * 2 + c) * P.s_rows) * P.d_s;
     };
-    int64_t sbase = seg_base(0);
-    int64_t snext = n_seg > 1 ? seg_base(1) : 0;
+    int64_t sbase = 0, snext = 0;
+    // made rows are whole operand rows: one base, and the residuals a plane on
+    const int64_t width = kl.made ? static_cast<int64_t>(P.n_batoms) * kBK : P.d_s;
+    const int64_t plane = P.x_rows * width;
+    if (kl.made) {
+      const int at = (l - P.l0) * P.made_roles + (P.made_roles == 2 ? c : 0);
+      sender = reinterpret_cast<const T*>(P.x) + at * (kl.split ? 2 : 1) * plane;
+    } else {
+      sbase = seg_base(0);
+      if (n_seg > 1) snext = seg_base(1);
+    }
     int64_t roff[8];
     uint32_t doff[8];
     // rows past the last distinct row are not copied: their products (of what
@@ -825,33 +812,37 @@ __device__ __forceinline__ void gather_rows(const XferParams* Ps, const DirTable
       int64_t kr;  // sender-cache row
       if (pam_on<kPam>(P)) {
         const int k = pam_token(P, m, row0, r);
-        kr = P.srow ? __ldg(P.srow + k) : k;
+        kr = P.srow && !kl.made ? __ldg(P.srow + k) : k;
         live |= 1u << i;
       } else {
         const int u = m * kPairRows + row0 + r;
-        kr = P.ucol[min(u, U - 1)];
+        kr = kl.made ? min(u, U - 1) : P.ucol[min(u, U - 1)];
         live |= (u < U ? 1u : 0u) << i;
       }
-      roff[i] = kr * P.d_s + ch * kPerChunk;
+      roff[i] = kr * width + ch * kPerChunk;
       doff[i] = static_cast<uint32_t>(r * 128 + ((ch ^ (r & 7)) << 4));
     }
     int seg = 0, kin = 0;  // segment of the next atom, and the atom within it
-    for (int kb = 0; kb < P.n_kb; ++kb) {
+    for (int kb = 0; kb < kl.n_kb; ++kb) {
       if (!mbar_wait(smem_addr(&empty_a[stage]), phase ^ 1)) {
         raise_timeout(P, sAbort);
         ok = false;
         break;
       }
       const uint32_t sa = smem_addr(sA + stage * kStageABytes);
-      const int na = kb == P.n_kb - 1 ? P.last_atoms : kAtoms;
+      const int na = kb == kl.n_kb - 1 && !kl.split ? kl.last_atoms : kAtoms;
 #pragma unroll
       for (int a = 0; a < kAtoms; ++a) {
         if (a < na) {
           const T* base = sender + sbase + kin * kBK;
+          if (kl.split && a == 1) base += plane - kBK;  // the residuals of the same atom
 #pragma unroll
           for (int i = 0; i < 8; ++i)
             if (live >> i & 1u) cp_async_16(sa + a * kAtomABytes + doff[i], base + roff[i]);
-          if (++kin == P.atoms_per_seg) {
+          ++kin;
+          if (kl.made) {
+            if (kl.split && a == 1) --kin;
+          } else if (kin == P.atoms_per_seg) {
             kin = 0;
             ++seg;
             sbase = snext;
@@ -1024,7 +1015,8 @@ __device__ __forceinline__ void build_rows_staged(const XferParams* Ps, const Di
       fr.e1 = P.row_ptr[fj0 + 1];
     }
     int pending = 0;  // stages issued and not yet finished (<= LAG)
-    for (int kb = 0; kb < P.n_kb; ++kb) {
+    const int n_kb = P.n_batoms;  // one map atom of K a stage
+    for (int kb = 0; kb < n_kb; ++kb) {
       if (!mbar_wait(smem_addr(&empty_a[stage]), phase ^ 1)) {
         raise_timeout(P, sAbort);
         ok = false;
@@ -1074,7 +1066,7 @@ __device__ __forceinline__ void build_rows_staged(const XferParams* Ps, const Di
     __syncwarp();
     for (int q = pending; q >= 1; --q) {
       const int st = (stage + stages - q) % stages;
-      finish_staged_row<T>(P, lsegs, c, fr, P.n_kb - q, sA + st * kStageABytes);
+      finish_staged_row<T>(P, lsegs, c, fr, n_kb - q, sA + st * kStageABytes);
       fence_proxy_async_smem();
       __syncwarp();
       if (lane == 0) arrive_leader(smem_addr(&full_a[st]), row0);
@@ -1087,10 +1079,11 @@ __device__ __forceinline__ void build_rows_staged(const XferParams* Ps, const Di
 // every role looks its tile's direction up and reads that direction's
 // parameters).  All directions share the dtype, the operand path and the
 // ring depths; a B stage is stage_b_stride bytes (the widest direction's).
-template <typename T, bool kGather, int kDirs, int kPam>
+template <typename T, int kRows, int kDirs, int kPam>
 __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const XferParams* Ps,
                                               int n_dir, int stage_b_stride) {
   constexpr int kBK = Elem<T>::kBK;
+  constexpr bool kGather = kRows != kBuiltRows;
   const XferParams& P0 = Ps[0];
   extern __shared__ __align__(1024) uint8_t smem[];
   if (smem_addr(smem) & 1023u) {  // the swizzled stages need 1024-byte alignment
@@ -1231,8 +1224,10 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const Xfe
        tile = tile_of(++seq, first_tile, tile_step, by_slot)) {
         const XferParams& P = Ps[dir_of(dt, n_dir, tile)];
         const uint32_t idesc = P.idesc;
-        const int n_kb = P.n_kb, last_atoms = P.last_atoms, per_stage = P.atoms_per_stage;
-        const bool split = P.split != 0;
+        const KLoop kl = k_loop<kRows>(P, tile & 1);  // a direction's tiles start at an even one
+        const int n_kb = kl.n_kb, last_atoms = kl.last_atoms;
+        const bool split = kl.split;
+        const int per_stage = split ? 1 : kAtoms;
         const bool wide = !kGather && P.wide != 0;  // both accumulators, one per column block
         const int n_half = wide ? 2 : 1;
         bool free_acc = mbar_wait(smem_addr(&tempty[wide ? 0 : acc]), acc_phase ^ 1);
@@ -1502,11 +1497,11 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const Xfe
     const int t = threadIdx.x - 64 - kEpiThreads;  // 0..127
     if (kGather) {
       switch (P0.lag) {
-        case 1: gather_rows<T, 1, kDirs, kPam>(Ps, dt, n_dir, sA, full_a, empty_a, sAbort, t, lane, row0, total_tiles, first_tile, tile_step); break;
-        case 2: gather_rows<T, 2, kDirs, kPam>(Ps, dt, n_dir, sA, full_a, empty_a, sAbort, t, lane, row0, total_tiles, first_tile, tile_step); break;
-        case 3: gather_rows<T, 3, kDirs, kPam>(Ps, dt, n_dir, sA, full_a, empty_a, sAbort, t, lane, row0, total_tiles, first_tile, tile_step); break;
-        case 4: gather_rows<T, 4, kDirs, kPam>(Ps, dt, n_dir, sA, full_a, empty_a, sAbort, t, lane, row0, total_tiles, first_tile, tile_step); break;
-        default: gather_rows<T, 5, kDirs, kPam>(Ps, dt, n_dir, sA, full_a, empty_a, sAbort, t, lane, row0, total_tiles, first_tile, tile_step); break;
+        case 1: gather_rows<T, 1, kDirs, kPam, kRows>(Ps, dt, n_dir, sA, full_a, empty_a, sAbort, t, lane, row0, total_tiles, first_tile, tile_step); break;
+        case 2: gather_rows<T, 2, kDirs, kPam, kRows>(Ps, dt, n_dir, sA, full_a, empty_a, sAbort, t, lane, row0, total_tiles, first_tile, tile_step); break;
+        case 3: gather_rows<T, 3, kDirs, kPam, kRows>(Ps, dt, n_dir, sA, full_a, empty_a, sAbort, t, lane, row0, total_tiles, first_tile, tile_step); break;
+        case 4: gather_rows<T, 4, kDirs, kPam, kRows>(Ps, dt, n_dir, sA, full_a, empty_a, sAbort, t, lane, row0, total_tiles, first_tile, tile_step); break;
+        default: gather_rows<T, 5, kDirs, kPam, kRows>(Ps, dt, n_dir, sA, full_a, empty_a, sAbort, t, lane, row0, total_tiles, first_tile, tile_step); break;
       }
     } else if (P0.staged) {
       switch (P0.lag) {
@@ -1540,7 +1535,8 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const Xfe
         }
         const bool unrot_k = P.unrot && c == 0;
         int seg = 0, kin = 0;  // segment of the next atom, and the atom within it
-        for (int kb = 0; kb < P.n_kb; ++kb) {
+        const KLoop kl = k_loop<kRows>(P, c);
+        for (int kb = 0; kb < kl.n_kb; ++kb) {
           if (!mbar_wait(smem_addr(&empty_a[stage]), phase ^ 1)) {
             raise_timeout(P, sAbort);
             ok = false;
@@ -1566,7 +1562,7 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const Xfe
               ++seg;
             }
           } else {
-            const int na = kb == P.n_kb - 1 ? P.last_atoms : kAtoms;
+            const int na = kb == kl.n_kb - 1 ? kl.last_atoms : kAtoms;
             for (int a = 0; a < na; ++a) {
               build_atom<T>(P, segs, seg, kin, c, e0, e1, tok, st + a * kAtomABytes, nullptr, t);
               if (++kin == P.atoms_per_seg) {
@@ -1601,11 +1597,11 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const Xfe
   }
 }
 
-template <typename T, bool kGather, int kPam>
+template <typename T, int kRows, int kPam>
 __global__ void __launch_bounds__(kThreads, 1)
     transfer_kernel(const __grid_constant__ CUtensorMap tmap_w,
                     const __grid_constant__ XferParams P) {
-  transfer_body<T, kGather, 1, kPam>(&tmap_w, &P, 1, (P.BN / 2) * 128);
+  transfer_body<T, kRows, 1, kPam>(&tmap_w, &P, 1, (P.BN / 2) * 128);
 }
 
 // Several directions in one launch (hf_transfer_batch).
@@ -1617,10 +1613,10 @@ struct BatchParams {
 };
 static_assert(sizeof(BatchParams) < 32000, "BatchParams must fit the kernel parameter space");
 
-template <typename T, bool kGather, int kPam>
+template <typename T, int kRows, int kPam>
 __global__ void __launch_bounds__(kThreads, 1)
     transfer_batch_kernel(const __grid_constant__ BatchParams B) {
-  transfer_body<T, kGather, kMaxBatch, kPam>(B.maps, B.P, B.n_dir, B.stage_b_stride);
+  transfer_body<T, kRows, kMaxBatch, kPam>(B.maps, B.P, B.n_dir, B.stage_b_stride);
 }
 
 // ---------------------------------------------------------------------------
@@ -1783,10 +1779,11 @@ hf_status make_xfer(hf_plan_s* p, const void* sender, void* receiver, int l_begi
   P.win_ptr = reinterpret_cast<const int32_t*>(ws + p->lay.win_ptr);
   P.pos = reinterpret_cast<const int32_t*>(ws + p->lay.pos);
   P.uidx = reinterpret_cast<const int32_t*>(ws + p->lay.new_flag);
-  P.atoms_per_stage = p->split ? 1 : kAtoms;
   P.n_batoms = n_atoms;
-  P.n_kb = (n_atoms + P.atoms_per_stage - 1) / P.atoms_per_stage;
-  P.last_atoms = n_atoms - P.atoms_per_stage * (P.n_kb - 1);
+  P.made = p->made;
+  P.made_roles = p->made == 3 ? 2 : 1;
+  P.x = p->made ? ws + p->lay.xbuf : nullptr;
+  P.x_rows = p->x_rows;
   P.atoms_per_seg = p->d_s / bk;
   P.BN = p->BN;
   P.wide = p->wide ? 1 : 0;
@@ -1807,10 +1804,10 @@ hf_status make_xfer(hf_plan_s* p, const void* sender, void* receiver, int l_begi
   return HF_OK;
 }
 
-template <typename T, bool kGather, int kPam>
+template <typename T, int kRows, int kPam>
 hf_status launch_batch_typed(const BatchParams& B, int64_t max_pair_tiles, size_t smem,
                              cudaStream_t stream) {
-  return launch_pairs(transfer_batch_kernel<T, kGather, kPam>, max_pair_tiles, smem, stream, B);
+  return launch_pairs(transfer_batch_kernel<T, kRows, kPam>, max_pair_tiles, smem, stream, B);
 }
 
 }  // namespace
@@ -1820,6 +1817,20 @@ hf_status launch_transfer(hf_plan_s* p, const void* sender, void* receiver, cuda
   const hf_plan_desc& d = p->desc;
   if (l_end < 0) l_end = d.L_r;
   if (p->T_r == 0 || l_end <= l_begin) return HF_OK;
+  if (p->made) {
+    // the operand rows of as many receiver layers as their buffer holds, then
+    // these layers' transfer
+    if (l_end - l_begin > p->x_layers) {
+      for (int l = l_begin; l < l_end; l += p->x_layers) {
+        const hf_status e = launch_transfer(p, sender, receiver, stream, l,
+                                            std::min(l_end, l + p->x_layers), stall);
+        if (e != HF_OK) return e;
+      }
+      return HF_OK;
+    }
+    const hf_status e = launch_operands(p, sender, stream, l_begin, l_end);
+    if (e != HF_OK) return e;
+  }
   XferParams P;
   CUtensorMap mw;
   int64_t max_pair_tiles = 0;
@@ -1827,24 +1838,25 @@ hf_status launch_transfer(hf_plan_s* p, const void* sender, void* receiver, cuda
   if (s != HF_OK) return s;
   P.stall = stall ? 1 : 0;
   const size_t smem = smem_bytes(p->BN, P.stages_a, P.stages_b);
+  auto go = [&](auto kern) { return launch_pairs(kern, max_pair_tiles, smem, stream, mw, P); };
+  using Bf = __nv_bfloat16;
   if (d.dtype == HF_F32)
-    return p->gather
-               ? launch_pairs(transfer_kernel<float, true, 2>, max_pair_tiles, smem, stream, mw, P)
-               : launch_pairs(transfer_kernel<float, false, 2>, max_pair_tiles, smem, stream, mw, P);
+    return p->gather ? go(transfer_kernel<float, kCopiedRows, 2>)
+                     : go(transfer_kernel<float, kBuiltRows, 2>);
+  if (p->made)
+    return p->pam ? go(transfer_kernel<Bf, kMadeRows, 1>) : go(transfer_kernel<Bf, kMadeRows, 0>);
   if (p->pam)
-    return p->gather
-               ? launch_pairs(transfer_kernel<__nv_bfloat16, true, 1>, max_pair_tiles, smem, stream, mw, P)
-               : launch_pairs(transfer_kernel<__nv_bfloat16, false, 1>, max_pair_tiles, smem, stream, mw, P);
-  return p->gather
-             ? launch_pairs(transfer_kernel<__nv_bfloat16, true, 0>, max_pair_tiles, smem, stream, mw, P)
-             : launch_pairs(transfer_kernel<__nv_bfloat16, false, 0>, max_pair_tiles, smem, stream, mw, P);
+    return p->gather ? go(transfer_kernel<Bf, kCopiedRows, 1>) : go(transfer_kernel<Bf, kBuiltRows, 1>);
+  return p->gather ? go(transfer_kernel<Bf, kCopiedRows, 0>) : go(transfer_kernel<Bf, kBuiltRows, 0>);
 }
 
 bool batch_compatible(const hf_plan_s* const* plans, int n) {
+  if (plans[0]->made) return false;  // operand passes of their own
   for (int i = 1; i < n; ++i)
     if (plans[i]->desc.dtype != plans[0]->desc.dtype || plans[i]->gather != plans[0]->gather ||
         plans[i]->split != plans[0]->split || plans[i]->staged != plans[0]->staged ||
-        plans[i]->pam != plans[0]->pam || plans[i]->wide != plans[0]->wide)
+        plans[i]->pam != plans[0]->pam || plans[i]->wide != plans[0]->wide ||
+        plans[i]->made)
       return false;
   return true;
 }
@@ -1885,14 +1897,14 @@ hf_status launch_transfer_batch(hf_plan_s* const* plans, const void* const* send
   const size_t smem = smem_bytes(max_bn, sa, sb);
   hf_status s;
   if (plans[0]->desc.dtype == HF_F32)
-    s = plans[0]->gather ? launch_batch_typed<float, true, 2>(*B, tiles, smem, stream)
-                         : launch_batch_typed<float, false, 2>(*B, tiles, smem, stream);
+    s = plans[0]->gather ? launch_batch_typed<float, kCopiedRows, 2>(*B, tiles, smem, stream)
+                         : launch_batch_typed<float, kBuiltRows, 2>(*B, tiles, smem, stream);
   else if (plans[0]->pam)
-    s = plans[0]->gather ? launch_batch_typed<__nv_bfloat16, true, 1>(*B, tiles, smem, stream)
-                         : launch_batch_typed<__nv_bfloat16, false, 1>(*B, tiles, smem, stream);
+    s = plans[0]->gather ? launch_batch_typed<__nv_bfloat16, kCopiedRows, 1>(*B, tiles, smem, stream)
+                         : launch_batch_typed<__nv_bfloat16, kBuiltRows, 1>(*B, tiles, smem, stream);
   else
-    s = plans[0]->gather ? launch_batch_typed<__nv_bfloat16, true, 0>(*B, tiles, smem, stream)
-                         : launch_batch_typed<__nv_bfloat16, false, 0>(*B, tiles, smem, stream);
+    s = plans[0]->gather ? launch_batch_typed<__nv_bfloat16, kCopiedRows, 0>(*B, tiles, smem, stream)
+                         : launch_batch_typed<__nv_bfloat16, kBuiltRows, 0>(*B, tiles, smem, stream);
   delete B;
   return s;
 }

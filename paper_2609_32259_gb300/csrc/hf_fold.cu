@@ -4,11 +4,17 @@
 //   T = B^T W                      (rho x K)
 //   W_final = W + G^T T            (element [n][k] += sum_r G[r][n] T[r][k])
 //   b_final = b + (b B) G.
-// A block reads its columns of W twice (the second time from L2) and
-// writes them once.  Plain fp32 CUDA-core arithmetic (4 rank FLOP per
-// element, which at rank 16 outweighs the memory time): a rank of 16 is
-// too thin a contraction for the tensor cores, and fp32 maps need fp32
-// accuracy.
+// Two forms.  fold_mma_kernel (bf16 maps, rank <= 16, d_R <= 1,024, K a multiple
+// of 8) reads W once: the 4 rank FLOP per element outweigh the memory time on
+// the fp32 ALUs, so both contractions run on the warp-level tensor
+// instructions, with every fp32 factor split exactly into three bf16 parts and
+// the products above 2^-23 kept (a rank of 16 is one 16-deep step: too thin for
+// an accumulator in tensor memory; 80 maps of 1,024 x 3,072, rank 16, with the
+// bias: 0.37 ms, fold_kernel 0.49; the same error against 64 bits).  fold_kernel
+// takes the rest with plain fp32 arithmetic; a block reads its columns of W
+// twice (the second time from L2) and writes them once.
+#include <algorithm>
+
 #include <cuda_bf16.h>
 
 #include <string>
@@ -242,35 +248,256 @@ __global__ void __launch_bounds__(kFoldThreads) fold_kernel(const T* W, const fl
   fold_cp_wait<0>();
 }
 
-// b_final = b + (b B) G for one map per block.
+// ---------------------------------------------------------------------------
+// bf16 maps on the tensor cores
+// ---------------------------------------------------------------------------
+constexpr int kMmaWarps = 16;
+constexpr int kMmaCols = 32;            // columns of W per unit of work
+constexpr int kMmaRows = 1024;          // d_R at most: 64 rows per warp
+constexpr int kMmaStride = kMmaCols + 8;  // padded shared-memory row: 80 bytes, no bank twice
+constexpr int kPartStride = kMmaCols + 4;
+
+__device__ __forceinline__ void mma_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0,
+                                          uint32_t b1) {
+  asm(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
+      "{%8, %9}, {%0, %1, %2, %3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// Four transposed 8 x 8 matrices: two 16 x 8 right operands (16 rows of shared
+// memory, two groups of eight columns).
+__device__ __forceinline__ void ldsm_x4_t(uint32_t (&r)[4], const void* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(p)))
+               : "memory");
+}
+// (x, y) as three bf16 pairs that add up to it exactly (24 bits).
+__device__ __forceinline__ void split3(float x, float y, uint32_t* h0, uint32_t* h1, uint32_t* h2) {
+  const __nv_bfloat162 a = __floats2bfloat162_rn(x, y);
+  const float2 fa = __bfloat1622float2(a);
+  x -= fa.x;
+  y -= fa.y;
+  const __nv_bfloat162 b = __floats2bfloat162_rn(x, y);
+  const float2 fb = __bfloat1622float2(b);
+  const __nv_bfloat162 c = __floats2bfloat162_rn(x - fb.x, y - fb.y);
+  *h0 = *reinterpret_cast<const uint32_t*>(&a);
+  *h1 = *reinterpret_cast<const uint32_t*>(&b);
+  *h2 = *reinterpret_cast<const uint32_t*>(&c);
+}
+
+struct FoldMmaSmem {
+  __nv_bfloat16 w[2][kMmaRows][kMmaStride];
+  float part[kMmaWarps][16][kPartStride];
+  __nv_bfloat16 t[3][16][kMmaStride];
+};
+
+// A persistent CTA takes a run of units (map, 32 columns).  Warp w owns rows 16
+// steps w .. of W (steps <= 4 blocks of 16): it alone copies them in, works on
+// them and copies them out, so that only T takes a barrier.  Per unit:
+//  1. T = B^T W: the warp's share of the contraction over the rows, with the
+//     split B of its rows in registers (kept while the map stays the same);
+//     W is exact in bf16, so three products per term;
+//  2. the warps' shares meet in shared memory, T is split there;
+//  3. W += G^T T on the warp's rows: six products, added to W in fp32, rounded
+//     once, back into the buffer, which then leaves in 16-byte stores and takes
+//     the columns of the unit after the next.
+// The latency of these steps bounds it, at a third of the tensor instructions'
+// and of the memory rate (64 KB in and out per unit and SM; two buffers of 32
+// columns are what fits; step 1 of a unit before step 3 of the one before it
+// exposed the copies instead and was 17% slower).
+__global__ void __launch_bounds__(32 * kMmaWarps)
+    fold_mma_kernel(const __nv_bfloat16* W, const float* __restrict__ Bm,
+                    const float* __restrict__ Gm, __nv_bfloat16* Wf, int n_maps, int d_r, int64_t K,
+                    int rank, int steps) {
+  extern __shared__ __align__(128) uint8_t fold_smem[];
+  FoldMmaSmem& sm = *reinterpret_cast<FoldMmaSmem*>(fold_smem);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int g = lane >> 2, t = lane & 3;  // fragment row and column pair
+  const int per_map = static_cast<int>((K + kMmaCols - 1) / kMmaCols);
+  const int64_t units = static_cast<int64_t>(n_maps) * per_map;
+  const int64_t u0 = units * blockIdx.x / gridDim.x, u1 = units * (blockIdx.x + 1) / gridDim.x;
+  const int row0 = warp * 16 * steps, rows = min(16 * steps, d_r - row0);  // <= 0: padding only
+  for (int i = lane; i < (16 * steps - max(rows, 0)) * kMmaStride; i += 32) {
+    const int r = row0 + max(rows, 0) + i / kMmaStride;  // rows past d_R: zeros
+    sm.w[0][r][i % kMmaStride] = sm.w[1][r][i % kMmaStride] = __nv_bfloat16(0.f);
+  }
+  // the warp's rows of a unit, 16-byte pieces, four per row
+  auto load = [&](int64_t u) {
+    if (u < u1) {
+      const int map = static_cast<int>(u / per_map), buf = static_cast<int>((u - u0) & 1);
+      const int64_t k0 = (u - static_cast<int64_t>(map) * per_map) * kMmaCols;
+      const __nv_bfloat16* src = W + (static_cast<int64_t>(map) * d_r + row0) * K + k0;
+      for (int i = lane; i < 4 * rows; i += 32) {
+        const int r = i >> 2, c = (i & 3) * 8;
+        if (k0 + c < K) fold_cp_async<16>(&sm.w[buf][row0 + r][c], src + r * K + c);
+      }
+    }
+    fold_cp_commit();
+  };
+  load(u0);
+  load(u0 + 1);
+  uint32_t bf[4][3][4];  // B^T, rank x 16 rows per step, split
+  uint32_t gf[4][3][4];  // G^T, 16 rows x rank per step, split
+  int map_now = -1;
+  const int lrow = lane & 15, lcol = (lane >> 4) * 8;  // ldmatrix: this lane's row
+  for (int64_t u = u0; u < u1; ++u) {
+    const int buf = static_cast<int>((u - u0) & 1);
+    const int map = static_cast<int>(u / per_map);
+    const int64_t k0 = (u - static_cast<int64_t>(map) * per_map) * kMmaCols;
+    auto& w = sm.w[buf];
+    if (map != map_now) {
+      map_now = map;
+      const float* const B = Bm + static_cast<int64_t>(map) * d_r * rank;
+      const float* const G = Gm + static_cast<int64_t>(map) * rank * d_r;
+      auto at_b = [&](int n, int r) { return n < d_r && r < rank ? __ldg(B + n * rank + r) : 0.f; };
+      auto at_g = [&](int n, int r) { return n < d_r && r < rank ? __ldg(G + r * d_r + n) : 0.f; };
+#pragma unroll
+      for (int s = 0; s < 4; ++s) {
+        if (s >= steps) break;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          // B^T: rank row g (+8), rows 2t (+8) of W
+          const int r = g + 8 * (i & 1), c = row0 + 16 * s + 2 * t + 8 * (i >> 1);
+          split3(at_b(c, r), at_b(c + 1, r), &bf[s][0][i], &bf[s][1][i], &bf[s][2][i]);
+          // G^T: W row g (+8), rank columns 2t (+8)
+          const int n = row0 + 16 * s + g + 8 * (i & 1), q = 2 * t + 8 * (i >> 1);
+          split3(at_g(n, q), at_g(n, q + 1), &gf[s][0][i], &gf[s][1][i], &gf[s][2][i]);
+        }
+      }
+    }
+    {
+      // step 1 (the next unit's columns may still be on their way)
+      fold_cp_wait<1>();
+      __syncwarp();
+      float d[4][4] = {};
+#pragma unroll
+      for (int s = 0; s < 4; ++s) {
+        if (s >= steps) break;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          uint32_t x[4];
+          ldsm_x4_t(x, &w[row0 + 16 * s + lrow][16 * h + lcol]);
+#pragma unroll
+          for (int p = 2; p >= 0; --p) {
+            mma_16816(d[2 * h], bf[s][p], x[0], x[1]);
+            mma_16816(d[2 * h + 1], bf[s][p], x[2], x[3]);
+          }
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        *reinterpret_cast<float2*>(&sm.part[warp][g][8 * i + 2 * t]) = make_float2(d[i][0], d[i][1]);
+        *reinterpret_cast<float2*>(&sm.part[warp][g + 8][8 * i + 2 * t]) =
+            make_float2(d[i][2], d[i][3]);
+      }
+    }
+    __syncthreads();
+    {
+      // step 2
+      float x = 0.f;  // T[warp][lane]
+#pragma unroll
+      for (int q = 0; q < kMmaWarps; ++q) x += sm.part[q][warp][lane];
+      const __nv_bfloat16 h0 = __float2bfloat16_rn(x);
+      x -= __bfloat162float(h0);
+      const __nv_bfloat16 h1 = __float2bfloat16_rn(x);
+      sm.t[0][warp][lane] = h0;
+      sm.t[1][warp][lane] = h1;
+      sm.t[2][warp][lane] = __float2bfloat16_rn(x - __bfloat162float(h1));
+    }
+    __syncthreads();
+    {
+      // step 3
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        uint32_t x[3][4];
+#pragma unroll
+        for (int p = 0; p < 3; ++p) ldsm_x4_t(x[p], &sm.t[p][lrow][16 * h + lcol]);
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+          if (s >= steps) break;
+          float y[2][4] = {};
+#pragma unroll
+          for (int k = 0; k < 6; ++k) {  // the smallest products first
+            constexpr int kG[6] = {2, 1, 0, 1, 0, 0}, kT[6] = {0, 1, 2, 0, 1, 0};
+            mma_16816(y[0], gf[s][kG[k]], x[kT[k]][0], x[kT[k]][1]);
+            mma_16816(y[1], gf[s][kG[k]], x[kT[k]][2], x[kT[k]][3]);
+          }
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            const int col = 16 * h + 8 * q + 2 * t;
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+              __nv_bfloat162* const o =
+                  reinterpret_cast<__nv_bfloat162*>(&w[row0 + 16 * s + g + 8 * k][col]);
+              const float2 wv = __bfloat1622float2(*o);
+              *o = __floats2bfloat162_rn(wv.x + y[q][2 * k], wv.y + y[q][2 * k + 1]);
+            }
+          }
+        }
+      }
+      __syncwarp();
+      __nv_bfloat16* const dst = Wf + (static_cast<int64_t>(map) * d_r + row0) * K + k0;
+#pragma unroll 4
+      for (int i = lane; i < 4 * rows; i += 32) {
+        const int r = i >> 2, c = (i & 3) * 8;
+        if (k0 + c < K)
+          *reinterpret_cast<uint4*>(dst + r * K + c) =
+              *reinterpret_cast<const uint4*>(&w[row0 + r][c]);
+      }
+      __syncwarp();
+      load(u + 2);
+    }
+  }
+  fold_cp_wait<0>();
+}
+
+// b_final = b + (b B) G for one map per block, every load of a pass in flight
+// at once (one rank column at a time took 17 us for 80 maps).
+template <int R>
 __global__ void __launch_bounds__(256) fold_b_kernel(const float* b, const float* __restrict__ Bm,
                                                      const float* __restrict__ Gm, float* bf,
-                                                     int d_r, int rank) {
-  __shared__ float part[256 / 32][kMaxRank];
-  __shared__ float bB[kMaxRank];
+                                                     int d_r) {
+  __shared__ float part[256 / 32][R];
+  __shared__ float bB[R];
   const int map = blockIdx.x;
   const float* bm = b + static_cast<int64_t>(map) * d_r;
-  const float* B = Bm + static_cast<int64_t>(map) * d_r * rank;
-  const float* G = Gm + static_cast<int64_t>(map) * rank * d_r;
+  const float* B = Bm + static_cast<int64_t>(map) * d_r * R;
+  const float* G = Gm + static_cast<int64_t>(map) * R * d_r;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int r = 0; r < rank; ++r) {
-    float s = 0.f;
-    for (int m = threadIdx.x; m < d_r; m += blockDim.x)
-      s = fmaf(bm[m], B[static_cast<int64_t>(m) * rank + r], s);
+  float s[R];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) part[warp][r] = s;
+  for (int r = 0; r < R; ++r) s[r] = 0.f;
+#pragma unroll 2
+  for (int m = threadIdx.x; m < d_r; m += blockDim.x) {
+    const float x = bm[m];
+#pragma unroll
+    for (int q = 0; q < R; q += 4) {
+      const float4 v = __ldg(reinterpret_cast<const float4*>(B + static_cast<int64_t>(m) * R + q));
+      s[q] = fmaf(x, v.x, s[q]);
+      s[q + 1] = fmaf(x, v.y, s[q + 1]);
+      s[q + 2] = fmaf(x, v.z, s[q + 2]);
+      s[q + 3] = fmaf(x, v.w, s[q + 3]);
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s[r] += __shfl_xor_sync(0xffffffffu, s[r], o);
+    if (lane == 0) part[warp][r] = s[r];
   }
   __syncthreads();
-  if (threadIdx.x < rank) {
-    float s = 0.f;
-    for (int w = 0; w < 256 / 32; ++w) s += part[w][threadIdx.x];
-    bB[threadIdx.x] = s;
+  if (threadIdx.x < R) {
+    float t = 0.f;
+    for (int w = 0; w < 256 / 32; ++w) t += part[w][threadIdx.x];
+    bB[threadIdx.x] = t;
   }
   __syncthreads();
   for (int n = threadIdx.x; n < d_r; n += blockDim.x) {
     float v = bm[n];
-    for (int r = 0; r < rank; ++r) v = fmaf(bB[r], G[static_cast<int64_t>(r) * d_r + n], v);
+#pragma unroll
+    for (int r = 0; r < R; ++r) v = fmaf(bB[r], __ldg(G + static_cast<int64_t>(r) * d_r + n), v);
     bf[static_cast<int64_t>(map) * d_r + n] = v;
   }
 }
@@ -307,7 +534,23 @@ hf_status launch_fold(int n_maps, int d_r, int64_t K, int rank, const void* W, c
   int dev = 0, optin = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  hf_status s;
+  hf_status s = HF_OK;
+  // the tensor-core form where its units fit; in fp32 the maps need more than
+  // bf16 products of an exact W, and two 16-deep steps of rank 32 more registers
+  // than a warp's share of B and G leaves
+  const bool mma = sizeof(T) == 2 && (rank == 4 || rank == 8 || rank == 16) && d_r <= kMmaRows &&
+                   K % 8 == 0 && sizeof(FoldMmaSmem) <= static_cast<size_t>(optin);
+  if (mma) {
+    HF_CUDA_TRY(cudaFuncSetAttribute(fold_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     static_cast<int>(sizeof(FoldMmaSmem))),
+                "hf_fold: shared memory size");
+    const int64_t units = n_maps * ((K + kMmaCols - 1) / kMmaCols);
+    const int grid = static_cast<int>(std::min<int64_t>(units, device_sm_count()));
+    fold_mma_kernel<<<grid, 32 * kMmaWarps, sizeof(FoldMmaSmem), stream>>>(
+        static_cast<const __nv_bfloat16*>(W), B, G, static_cast<__nv_bfloat16*>(Wf), n_maps, d_r, K,
+        rank, (d_r + 16 * kMmaWarps - 1) / (16 * kMmaWarps));
+    HF_CUDA_TRY(cudaGetLastError(), "hf_fold: launch");
+  } else
   switch (rank) {
     case 4: s = launch_fold_r<T, 4>(n_maps, d_r, K, W, B, G, Wf, optin, stream); break;
     case 8: s = launch_fold_r<T, 8>(n_maps, d_r, K, W, B, G, Wf, optin, stream); break;
@@ -318,7 +561,12 @@ hf_status launch_fold(int n_maps, int d_r, int64_t K, int rank, const void* W, c
       return HF_ERR_UNSUPPORTED;
   }
   if (s != HF_OK) return s;
-  fold_b_kernel<<<n_maps, 256, 0, stream>>>(b, B, G, bf, d_r, rank);
+  switch (rank) {
+    case 4: fold_b_kernel<4><<<n_maps, 256, 0, stream>>>(b, B, G, bf, d_r); break;
+    case 8: fold_b_kernel<8><<<n_maps, 256, 0, stream>>>(b, B, G, bf, d_r); break;
+    case 16: fold_b_kernel<16><<<n_maps, 256, 0, stream>>>(b, B, G, bf, d_r); break;
+    default: fold_b_kernel<32><<<n_maps, 256, 0, stream>>>(b, B, G, bf, d_r); break;
+  }
   HF_CUDA_TRY(cudaGetLastError(), "hf_fold: bias launch");
   return HF_OK;
 }

@@ -54,6 +54,29 @@ def test_fold_matches_oracle(dtype, in_place):
         assert np.allclose(bf[m].double().cpu().numpy(), bref, rtol=1e-5, atol=1e-6), m
 
 
+# The tensor-core form: one row and one column group to its largest d_R, rows
+# that no warp's 16 divide, a ragged last unit of columns, padded ranks, more
+# units than SMs; a d_R, a K and a rank past it (the other form).
+@pytest.mark.parametrize("n_maps,d_R,K,rank", [
+    (1, 1, 8, 4), (3, 270, 40, 8), (2, 1024, 104, 16), (1, 1008, 3080, 16), (9, 128, 1024, 16),
+    (1, 1040, 64, 16), (2, 64, 36, 16), (2, 64, 64, 32)])
+def test_fold_bf16_units(n_maps, d_R, K, rank):
+    dev = torch.device("cuda")
+    g = torch.Generator(device="cpu").manual_seed(d_R + K)
+    Wm = (torch.randn((n_maps, d_R, K), generator=g) / np.sqrt(K)).to(torch.bfloat16).to(dev)
+    b = (torch.randn((n_maps, d_R), generator=g) * 0.1).to(dev)
+    Bm, Gm = _factors(n_maps, d_R, rank, 6, dev)
+    Wf, bf = Wm.clone(), b.clone()
+    B.fold("bf16", Wf, bf, Bm, Gm, Wf, bf)   # in place
+    for m in range(n_maps):
+        Af, bref = O.fold(Wm[m].double().cpu().numpy().T, b[m].double().cpu().numpy(),
+                          Bm[m].double().cpu().numpy(), Gm[m].double().cpu().numpy())
+        got = Wf[m].double().cpu().numpy()
+        # one rounding to bf16 (2^-9 of the value) and fp32 sums
+        assert np.all(np.abs(got - Af.T) <= 2.0 ** -8 * np.abs(Af.T) + 1e-6), m
+        assert np.allclose(bf[m].double().cpu().numpy(), bref, rtol=1e-5, atol=1e-6), m
+
+
 def test_transfer_with_folded_maps_matches_unfused_oracle():
     w = W.llama_to_ministral(600).with_(L_s=4, L_r=3)
     c = Case(w)

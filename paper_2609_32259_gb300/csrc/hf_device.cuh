@@ -200,6 +200,16 @@ __device__ __forceinline__ void tma_load_2d_pair_hint(uint32_t dst, const void* 
       : "memory");
 }
 
+// The same within one CTA (no pair).
+__device__ __forceinline__ void tma_load_2d_hint(uint32_t dst, const void* map, int32_t x, int32_t y,
+                                                 uint32_t bar, uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cta.global.tile.mbarrier::complete_tx::bytes"
+      ".L2::cache_hint [%0], [%1, {%2, %3}], [%4], %5;" ::"r"(dst),
+      "l"(map), "r"(x), "r"(y), "r"(bar), "l"(policy)
+      : "memory");
+}
+
 // ---------------------------------------------------------------------------
 // cp.async (16-byte global -> shared copies tracked by commit groups)
 // ---------------------------------------------------------------------------

@@ -64,6 +64,14 @@ struct WorkspaceLayout {
   int x_layers, made;
 };
 
+// Receiver tokens up to which copied bf16 rows take single-CTA tiles.  With 512
+// receiver tokens or fewer about 150 distinct rows at most are to be expected
+// with Token Alignment: a pair's 256-row tile is then mostly padding, and the
+// maps, read once, are what bounds the transfer (256 tokens, Ministral ->
+// Llama-shaped, whole step: 104 us with pairs, 95 us single, of which the maps'
+// bytes take 60; six directions of 160 tokens 418 and 378 us).
+constexpr int64_t kSingleRows = 512;
+
 // Bytes of made operand rows to aim at: receiver layers per launch, so that
 // a launch's last round of tiles is a small part of it.
 constexpr size_t kOperandBytes = static_cast<size_t>(512) << 20;
@@ -111,6 +119,9 @@ struct hf_plan_s {
   bool span;    // aligned sender tokens are spans inside a longer sender cache
   bool pam;     // pooling after the map: map input rows are sender rows in windows
   bool wide;    // tiles of two 256-column blocks (operand rows built by the loader warps)
+  // tiles of 128 rows x 256 columns on single CTAs instead of 256 x 256 on
+  // pairs: few distinct rows (kSingleRows)
+  bool single;
   // bit c: the map input rows of role c (pooled, blended, weighted or rotated
   // back) are made by a pass of their own before the transfer, which then
   // copies them; x_rows rows (distinct rows, or sender tokens with pooling after

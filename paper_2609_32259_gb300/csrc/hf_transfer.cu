@@ -37,6 +37,8 @@
 // (pam_epilogue).  Plans whose rows the builders compute use wide tiles:
 // two 256-column blocks per tile in the two accumulators, so each built A
 // stage feeds twice the MMAs.
+// Transfers of few distinct rows (kSingleRows) take tiles of 128 rows x 256
+// columns on single CTAs (kPair = false): the same roles without a pair.
 // Pipeline hand-offs use mbarriers with bounded waits; nothing traps.
 #include <algorithm>
 #include <climits>
@@ -63,8 +65,11 @@ constexpr int kStgRow = 68;              // epilogue staging: a row of 2 heads x
                                          // bytes of outputs) and 16 bytes of padding, so that 32
                                          // rows' 16-byte writes spread over the banks
 constexpr int kStgFloats = kBM * kStgRow;
-constexpr int kRunStride = 132;          // run starts / positions of a tile (129 used)
-constexpr int kRotPairs = kMaxHeadDim / 2;  // one position's rotation of every pair
+// The padding of staging row i holds what key tiles look up: word kPadPos the
+// position of distinct row i's run (row j's is that + j), words kPadRot the
+// cosine and sine of one position's rotation of pair i.
+constexpr int kPadPos = 64, kPadRot = 66;
+static_assert(kMaxHeadDim / 2 <= kBM, "one pair per staging row");
 constexpr int kMaxStages = 8;
 constexpr int kTmemCols = 512;           // two accumulators of up to 256 columns
 
@@ -269,8 +274,7 @@ __device__ __forceinline__ void rotate4(float4& x, float4& y, const float* c, co
 // What bounds it is the length of one warp's chain of instructions (ten warps
 // hide little of each other), so the arithmetic is on pairs of fp32 values.
 template <typename T>
-__device__ __forceinline__ void walk_rows(int jb, int je, int u0, const int32_t* spb,
-                                          const float* stg, int qq, bool two_heads, bool do_rope,
+__device__ __forceinline__ void walk_rows(int jb, int je, int u0, const float* stg, int qq, bool two_heads, bool do_rope,
                                           const float* f, const float2* c1, const float2* s1,
                                           const XferParams& P, T* out_lc, int ocol, int q,
                                           int half) {
@@ -293,7 +297,7 @@ __device__ __forceinline__ void walk_rows(int jb, int je, int u0, const int32_t*
     dnext = P.paged ? __ldg(P.dst_row + jn) : jn;
     if (uj != u) {  // first row, or the first row of a later run
       u = uj;
-      pb = spb[u];
+      pb = __float_as_int(stg[u * kStgRow + kPadPos]);
       const float* urow = stg + u * kStgRow + 4 * qq;
       const float4 va = *reinterpret_cast<const float4*>(urow);
       const float4 vb = *reinterpret_cast<const float4*>(urow + 16);
@@ -719,12 +723,12 @@ struct DirTable {
   int U[kDirs];
 };
 
-template <int kDirs, int kPam>
+template <int kDirs, int kPam, int kTileRows>
 __device__ __forceinline__ int build_dirs(const XferParams* Ps, int n_dir, DirTable<kDirs>* dt) {
   int total = 0;
   for (int d = 0; d < (kDirs == 1 ? 1 : n_dir); ++d) {
     const int U = pam_on<kPam>(Ps[d]) ? 128 * __ldg(Ps[d].win_info + 2) : *Ps[d].n_distinct;
-    const int mt = (U + kPairRows - 1) / kPairRows;
+    const int mt = (U + kTileRows - 1) / kTileRows;
     dt->U[d] = U;
     dt->m_tiles[d] = mt;
     dt->base[d] = total;
@@ -758,7 +762,7 @@ __device__ __forceinline__ void arrive_leader(uint32_t bar, int row0) {
 // layout.  A thread keeps LAG groups in flight: after committing k-block i
 // it waits for k-block i-LAG and fences it to the async proxy; then one lane
 // per warp arrives on that stage's barrier in the leader CTA of the pair.
-template <typename T, int LAG, int kDirs, int kPam, int kRows>
+template <typename T, int LAG, int kDirs, int kPam, int kRows, int kTileRows>
 __device__ __forceinline__ void gather_rows(const XferParams* Ps, const DirTable<kDirs>& dt,
                                             int n_dir, uint8_t* sA, uint64_t* full_a,
                                             uint64_t* empty_a, volatile int* sAbort, int t,
@@ -815,7 +819,7 @@ __device__ __forceinline__ void gather_rows(const XferParams* Ps, const DirTable
         kr = P.srow && !kl.made ? __ldg(P.srow + k) : k;
         live |= 1u << i;
       } else {
-        const int u = m * kPairRows + row0 + r;
+        const int u = m * kTileRows + row0 + r;
         kr = kl.made ? min(u, U - 1) : P.ucol[min(u, U - 1)];
         live |= (u < U ? 1u : 0u) << i;
       }
@@ -1079,11 +1083,14 @@ __device__ __forceinline__ void build_rows_staged(const XferParams* Ps, const Di
 // every role looks its tile's direction up and reads that direction's
 // parameters).  All directions share the dtype, the operand path and the
 // ring depths; a B stage is stage_b_stride bytes (the widest direction's).
-template <typename T, int kRows, int kDirs, int kPam>
+template <typename T, int kRows, int kDirs, int kPam, bool kPair>
 __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const XferParams* Ps,
                                               int n_dir, int stage_b_stride) {
   constexpr int kBK = Elem<T>::kBK;
   constexpr bool kGather = kRows != kBuiltRows;
+  constexpr int kTileRows = kPair ? kPairRows : kBM;
+  constexpr int kCtas = kPair ? 2 : 1;  // CTAs that share a tile
+  static_assert(kPair || kRows == kCopiedRows, "single CTAs take copied rows");
   const XferParams& P0 = Ps[0];
   extern __shared__ __align__(1024) uint8_t smem[];
   if (smem_addr(smem) & 1023u) {  // the swizzled stages need 1024-byte alignment
@@ -1091,19 +1098,17 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const Xfe
     if (threadIdx.x == 0) atomicOr(P0.status, HF_CHECK_INTERNAL);
     return;
   }
-  const uint32_t rank = cluster_ctarank();  // 0: leader of the pair (issues the MMAs)
+  const uint32_t rank = kPair ? cluster_ctarank() : 0;  // 0: leader of the pair (issues the MMAs)
   const bool leader = rank == 0;
-  const int first_tile = static_cast<int>(cluster_id_x());
-  const int tile_step = static_cast<int>(nclusters_x());
+  const int first_tile = static_cast<int>(kPair ? cluster_id_x() : blockIdx.x);
+  const int tile_step = static_cast<int>(kPair ? nclusters_x() : gridDim.x);
   const int row0 = static_cast<int>(rank) * kBM;  // this CTA's rows within a pair tile
   const int stages_a = P0.stages_a, stages_b = P0.stages_b;
   const int stage_b_bytes = stage_b_stride;
   uint8_t* sA = smem;
   uint8_t* sB = sA + stages_a * kStageABytes;
   float* sStg = reinterpret_cast<float*>(sB + stages_b * stage_b_bytes);
-  float2* sRot = reinterpret_cast<float2*>(sStg + kStgFloats);  // cos, sin of one position's step
-  int32_t* sPb = reinterpret_cast<int32_t*>(sRot + kRotPairs);
-  uint64_t* bars = reinterpret_cast<uint64_t*>(sPb + kRunStride);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(sStg + kStgFloats);
   uint64_t* full_a = bars;
   uint64_t* empty_a = bars + kMaxStages;
   uint64_t* full_b = bars + 2 * kMaxStages;
@@ -1121,16 +1126,16 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const Xfe
     // the follower's copies are unused.  empty_* / tfull / drain receive the
     // leader's multicast commits in both CTAs.
     for (int s = 0; s < stages_a; ++s) {
-      mbar_init(smem_addr(&full_a[s]), 2 * kBuilderWarps);  // every A builder warp of the pair
+      mbar_init(smem_addr(&full_a[s]), kCtas * kBuilderWarps);  // every A builder warp of the pair
       mbar_init(smem_addr(&empty_a[s]), 1);
     }
     for (int s = 0; s < stages_b; ++s) {
-      mbar_init(smem_addr(&full_b[s]), 2);  // one expect_tx per CTA + the TMA bytes
+      mbar_init(smem_addr(&full_b[s]), kCtas);  // one expect_tx per CTA + the TMA bytes
       mbar_init(smem_addr(&empty_b[s]), 1);
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(smem_addr(&tfull[a]), 1);
-      mbar_init(smem_addr(&tempty[a]), 2 * kEpiWarps);  // every epilogue warp of the pair
+      mbar_init(smem_addr(&tempty[a]), kCtas * kEpiWarps);  // every epilogue warp of the pair
     }
     mbar_init(smem_addr(drain), 1);
     *sAbort = 0;
@@ -1139,11 +1144,16 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const Xfe
   if (warp == 0 && lane == 0)
     for (int d = 0; d < (kDirs == 1 ? 1 : n_dir); ++d) tma_prefetch_map(&maps[d]);
   if (warp == 1) {
-    tmem_alloc_pair(smem_addr(sTmem), kTmemCols);
-    tmem_relinquish_pair();
+    if (kPair) {
+      tmem_alloc_pair(smem_addr(sTmem), kTmemCols);
+      tmem_relinquish_pair();
+    } else {
+      tmem_alloc(smem_addr(sTmem), kTmemCols);
+      tmem_relinquish();
+    }
   }
   __syncthreads();
-  cluster_sync();  // the leader's barriers exist before any remote arrival
+  if (kPair) cluster_sync();  // the leader's barriers exist before any remote arrival
   tc_fence_after_sync();
   const uint32_t tmem_base = *sTmem;
   // everything above may run beside the end of the kernel before this one;
@@ -1152,7 +1162,7 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const Xfe
   depend_launch();
 
   DirTable<kDirs> dt;
-  const int total_tiles = build_dirs<kDirs, kPam>(Ps, n_dir, &dt);
+  const int total_tiles = build_dirs<kDirs, kPam, kTileRows>(Ps, n_dir, &dt);
   const bool by_slot = slot_order(total_tiles, tile_step);
 
   if (warp == 0) {
@@ -1170,7 +1180,7 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const Xfe
         const int dd = dir_of(dt, n_dir, tile);
         const XferParams& P = Ps[dd];
         const CUtensorMap* tmap = &maps[dd];
-        const int half_bn = P.BN / 2;  // B rows (receiver columns) per CTA
+        const int half_bn = P.BN / kCtas;  // B rows (receiver columns) per CTA
         const int atom_b_bytes = half_bn * 128;
         int lc, m, n;
         decode_tile(tile - dt.base[dd], dt.m_tiles[dd] * P.n_tiles_n, P.n_tiles_n, P.l0, &lc, &m,
@@ -1185,13 +1195,18 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const Xfe
             ok = false;
             break;
           }
-          const uint32_t fb = mapa_shared(smem_addr(&full_b[stage]), 0);
+          const uint32_t fb = kPair ? mapa_shared(smem_addr(&full_b[stage]), 0)
+                                    : smem_addr(&full_b[stage]);
           if (!(P.stall && seq == 0 && ab == 0)) {  // the test hook leaves this stage empty
-            mbar_arrive_expect_tx_cluster(fb, atom_b_bytes);
-            tma_load_2d_pair_hint(smem_addr(sB + stage * stage_b_bytes), tmap, at * kBK,
-                                  lc * P.d_r + (n * n_half + h) * P.BN +
-                                      static_cast<int>(rank) * half_bn,
-                                  fb, pol_b);
+            const uint32_t dst = smem_addr(sB + stage * stage_b_bytes);
+            const int y = lc * P.d_r + (n * n_half + h) * P.BN + static_cast<int>(rank) * half_bn;
+            if (kPair) {
+              mbar_arrive_expect_tx_cluster(fb, atom_b_bytes);
+              tma_load_2d_pair_hint(dst, tmap, at * kBK, y, fb, pol_b);
+            } else {
+              mbar_arrive_expect_tx(fb, atom_b_bytes);
+              tma_load_2d_hint(dst, tmap, at * kBK, y, fb, pol_b);
+            }
           }
           if (++stage == stages_b) {
             stage = 0;
@@ -1215,6 +1230,16 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const Xfe
       const uint64_t desc_b0 = sw128_kmajor_desc(smem_addr(sB));
       const uint32_t step_a = kStageABytes >> 4, step_b = static_cast<uint32_t>(stage_b_bytes) >> 4;
       const uint32_t atom_a = kAtomABytes >> 4;
+      // the pair's instructions, or one CTA's
+      auto mma_bf16_any = [](uint32_t d, uint64_t a, uint64_t b, uint32_t id, uint32_t acc) {
+        if (kPair) mma_bf16_pair(d, a, b, id, acc); else mma_bf16(d, a, b, id, acc);
+      };
+      auto mma_tf32_any = [](uint32_t d, uint64_t a, uint64_t b, uint32_t id, uint32_t acc) {
+        if (kPair) mma_tf32_pair(d, a, b, id, acc); else mma_tf32(d, a, b, id, acc);
+      };
+      auto commit = [](uint32_t bar) {
+        if (kPair) tc_commit_pair(bar, 0x3); else tc_commit(bar);
+      };
       int sa = 0, sb = 0;
       uint32_t pa = 0, pb = 0;
       int acc = 0;
@@ -1260,24 +1285,24 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const Xfe
             const uint64_t bd = desc_b0 + sb * step_b;
             // four 32-byte K steps per 128-byte atom (descriptor units of 16 bytes)
             if (sizeof(T) == 2) {
-              mma_bf16_pair(d_tmem, ad, bd, idesc, accumulate);
-              mma_bf16_pair(d_tmem, ad + 2, bd + 2, idesc, 1);
-              mma_bf16_pair(d_tmem, ad + 4, bd + 4, idesc, 1);
-              mma_bf16_pair(d_tmem, ad + 6, bd + 6, idesc, 1);
+              mma_bf16_any(d_tmem, ad, bd, idesc, accumulate);
+              mma_bf16_any(d_tmem, ad + 2, bd + 2, idesc, 1);
+              mma_bf16_any(d_tmem, ad + 4, bd + 4, idesc, 1);
+              mma_bf16_any(d_tmem, ad + 6, bd + 6, idesc, 1);
               if (split) {  // the residual atom against the same map atom
                 const uint64_t lo = ad + atom_a;
-                mma_bf16_pair(d_tmem, lo, bd, idesc, 1);
-                mma_bf16_pair(d_tmem, lo + 2, bd + 2, idesc, 1);
-                mma_bf16_pair(d_tmem, lo + 4, bd + 4, idesc, 1);
-                mma_bf16_pair(d_tmem, lo + 6, bd + 6, idesc, 1);
+                mma_bf16_any(d_tmem, lo, bd, idesc, 1);
+                mma_bf16_any(d_tmem, lo + 2, bd + 2, idesc, 1);
+                mma_bf16_any(d_tmem, lo + 4, bd + 4, idesc, 1);
+                mma_bf16_any(d_tmem, lo + 6, bd + 6, idesc, 1);
               }
             } else {
-              mma_tf32_pair(d_tmem, ad, bd, idesc, accumulate);
-              mma_tf32_pair(d_tmem, ad + 2, bd + 2, idesc, 1);
-              mma_tf32_pair(d_tmem, ad + 4, bd + 4, idesc, 1);
-              mma_tf32_pair(d_tmem, ad + 6, bd + 6, idesc, 1);
+              mma_tf32_any(d_tmem, ad, bd, idesc, accumulate);
+              mma_tf32_any(d_tmem, ad + 2, bd + 2, idesc, 1);
+              mma_tf32_any(d_tmem, ad + 4, bd + 4, idesc, 1);
+              mma_tf32_any(d_tmem, ad + 6, bd + 6, idesc, 1);
             }
-            tc_commit_pair(empty_b0 + 8 * sb, 0x3);
+            commit(empty_b0 + 8 * sb);
             if (++sb == stages_b) {
               sb = 0;
               pb ^= 1;
@@ -1287,7 +1312,7 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const Xfe
             accumulate = 1;
           }
           if (!ok) break;
-          tc_commit_pair(empty_a0 + 8 * sa, 0x3);
+          commit(empty_a0 + 8 * sa);
           if (++sa == stages_a) {
             sa = 0;
             pa ^= 1;
@@ -1295,17 +1320,17 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const Xfe
         }
         if (!ok) break;
         if (wide) {
-          tc_commit_pair(smem_addr(&tfull[0]), 0x3);
-          tc_commit_pair(smem_addr(&tfull[1]), 0x3);
+          commit(smem_addr(&tfull[0]));
+          commit(smem_addr(&tfull[1]));
           acc_phase ^= 1;
         } else {
-          tc_commit_pair(smem_addr(&tfull[acc]), 0x3);
+          commit(smem_addr(&tfull[acc]));
           acc ^= 1;
           if (acc == 0) acc_phase ^= 1;
         }
       }
       // every issued MMA has completed before TMEM is released
-      tc_commit_pair(smem_addr(drain), 0x3);
+      commit(smem_addr(drain));
     }
     if (lane == 0) {
       if (!mbar_wait(smem_addr(drain), 0)) raise_timeout(P0, sAbort);
@@ -1327,7 +1352,7 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const Xfe
     const int ps = lane >> 2, qq = lane & 3;  // row slot 0..7, pair quad 0..3
     int acc = 0;
     uint32_t acc_phase = 0;
-    int rot_dir = -1;  // direction whose one-position rotations sRot holds
+    int rot_dir = -1;  // direction whose one-position rotations the padding holds
     for (int seq = 0, tile = tile_of(0, first_tile, tile_step, by_slot); tile < total_tiles;
        tile = tile_of(++seq, first_tile, tile_step, by_slot)) {
       const int dd = dir_of(dt, n_dir, tile);
@@ -1355,7 +1380,7 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const Xfe
       }
       tc_fence_after_sync();
       bool released = false;  // the accumulator has been handed back
-      const int u0 = m * kPairRows + row0;
+      const int u0 = m * kTileRows + row0;
       const int nrows = min(kBM, U - u0);  // <= 0: this CTA has no rows in the tile
       if (nrows > 0 && pam_on<kPam>(P)) {
         const int w = u0 >> 7;  // this CTA's window
@@ -1369,14 +1394,15 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const Xfe
                         P.bias + static_cast<int64_t>(lc) * P.d_r + nb * P.BN, P.inv_r[lc], base,
                         jb, je, sStg, e, g, row, lane, P.rope && c == 0, out_lc, nb * P.BN);
       } else if (nrows > 0) {
-        // position of row j of distinct row u0 + i: sPb[i] + j
         for (int i = tid_e; i < nrows; i += kEpiThreads)
-          sPb[i] = __ldg(P.upos + u0 + i) - __ldg(P.run_ptr + u0 + i);
+          sStg[i * kStgRow + kPadPos] =
+              __int_as_float(__ldg(P.upos + u0 + i) - __ldg(P.run_ptr + u0 + i));
         if (dd != rot_dir) {
           rot_dir = dd;
           if (P.rope)
             for (int i = tid_e; i < half; i += kEpiThreads)
-              rope_sincos(1, __ldg(P.inv_freq + i), &sRot[i].y, &sRot[i].x);
+              rope_sincos(1, __ldg(P.inv_freq + i), &sStg[i * kStgRow + kPadRot + 1],
+                          &sStg[i * kStgRow + kPadRot]);
         }
         // this warp's receiver rows [wjb, wje); lane slot ps walks the
         // consecutive rows [ljb, lje) of them
@@ -1467,11 +1493,13 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const Xfe
             float2 c1[2], s1[2];  // one step = one row
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
-              const float4 r = *reinterpret_cast<const float4*>(sRot + q + 4 * qq + 2 * k);
-              c1[k] = make_float2(r.x, r.z);
-              s1[k] = make_float2(r.y, r.w);
+              const float* const r = sStg + (q + 4 * qq + 2 * k) * kStgRow + kPadRot;
+              const float2 r0 = *reinterpret_cast<const float2*>(r);
+              const float2 r1 = *reinterpret_cast<const float2*>(r + kStgRow);
+              c1[k] = make_float2(r0.x, r1.x);
+              s1[k] = make_float2(r0.y, r1.y);
             }
-            walk_rows<T>(ljb, lje, u0, sPb, sStg, qq, two_heads, do_rope, f, c1, s1, P, out_lc,
+            walk_rows<T>(ljb, lje, u0, sStg, qq, two_heads, do_rope, f, c1, s1, P, out_lc,
                          ocol_pair, q, half);
             named_barrier_sync(1, kEpiThreads);
           }
@@ -1497,11 +1525,11 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const Xfe
     const int t = threadIdx.x - 64 - kEpiThreads;  // 0..127
     if (kGather) {
       switch (P0.lag) {
-        case 1: gather_rows<T, 1, kDirs, kPam, kRows>(Ps, dt, n_dir, sA, full_a, empty_a, sAbort, t, lane, row0, total_tiles, first_tile, tile_step); break;
-        case 2: gather_rows<T, 2, kDirs, kPam, kRows>(Ps, dt, n_dir, sA, full_a, empty_a, sAbort, t, lane, row0, total_tiles, first_tile, tile_step); break;
-        case 3: gather_rows<T, 3, kDirs, kPam, kRows>(Ps, dt, n_dir, sA, full_a, empty_a, sAbort, t, lane, row0, total_tiles, first_tile, tile_step); break;
-        case 4: gather_rows<T, 4, kDirs, kPam, kRows>(Ps, dt, n_dir, sA, full_a, empty_a, sAbort, t, lane, row0, total_tiles, first_tile, tile_step); break;
-        default: gather_rows<T, 5, kDirs, kPam, kRows>(Ps, dt, n_dir, sA, full_a, empty_a, sAbort, t, lane, row0, total_tiles, first_tile, tile_step); break;
+        case 1: gather_rows<T, 1, kDirs, kPam, kRows, kTileRows>(Ps, dt, n_dir, sA, full_a, empty_a, sAbort, t, lane, row0, total_tiles, first_tile, tile_step); break;
+        case 2: gather_rows<T, 2, kDirs, kPam, kRows, kTileRows>(Ps, dt, n_dir, sA, full_a, empty_a, sAbort, t, lane, row0, total_tiles, first_tile, tile_step); break;
+        case 3: gather_rows<T, 3, kDirs, kPam, kRows, kTileRows>(Ps, dt, n_dir, sA, full_a, empty_a, sAbort, t, lane, row0, total_tiles, first_tile, tile_step); break;
+        case 4: gather_rows<T, 4, kDirs, kPam, kRows, kTileRows>(Ps, dt, n_dir, sA, full_a, empty_a, sAbort, t, lane, row0, total_tiles, first_tile, tile_step); break;
+        default: gather_rows<T, 5, kDirs, kPam, kRows, kTileRows>(Ps, dt, n_dir, sA, full_a, empty_a, sAbort, t, lane, row0, total_tiles, first_tile, tile_step); break;
       }
     } else if (P0.staged) {
       switch (P0.lag) {
@@ -1590,18 +1618,18 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const Xfe
     while (global_timer_ns() - t0 < 200000ull) {
     }
   }
-  cluster_sync();  // neither CTA leaves while the pair's MMAs or arrivals may touch it
+  if (kPair) cluster_sync();  // neither CTA leaves while the pair's MMAs or arrivals may touch it
   if (warp == 1) {
     tc_fence_after_sync();
-    tmem_dealloc_pair(tmem_base, kTmemCols);
+    if (kPair) tmem_dealloc_pair(tmem_base, kTmemCols); else tmem_dealloc(tmem_base, kTmemCols);
   }
 }
 
-template <typename T, int kRows, int kPam>
+template <typename T, int kRows, int kPam, bool kPair = true>
 __global__ void __launch_bounds__(kThreads, 1)
     transfer_kernel(const __grid_constant__ CUtensorMap tmap_w,
                     const __grid_constant__ XferParams P) {
-  transfer_body<T, kRows, 1, kPam>(&tmap_w, &P, 1, (P.BN / 2) * 128);
+  transfer_body<T, kRows, 1, kPam, kPair>(&tmap_w, &P, 1, P.BN / (kPair ? 2 : 1) * 128);
 }
 
 // Several directions in one launch (hf_transfer_batch).
@@ -1613,10 +1641,10 @@ struct BatchParams {
 };
 static_assert(sizeof(BatchParams) < 32000, "BatchParams must fit the kernel parameter space");
 
-template <typename T, int kRows, int kPam>
+template <typename T, int kRows, int kPam, bool kPair = true>
 __global__ void __launch_bounds__(kThreads, 1)
     transfer_batch_kernel(const __grid_constant__ BatchParams B) {
-  transfer_body<T, kRows, kMaxBatch, kPam>(B.maps, B.P, B.n_dir, B.stage_b_stride);
+  transfer_body<T, kRows, kMaxBatch, kPam, kPair>(B.maps, B.P, B.n_dir, B.stage_b_stride);
 }
 
 // ---------------------------------------------------------------------------
@@ -1664,38 +1692,41 @@ hf_status make_map(CUtensorMap* map, const void* base, bool f32, uint64_t rows, 
   return HF_OK;
 }
 
-size_t smem_bytes(int BN, int stages_a, int stages_b) {
+// Bytes of a B stage: one atom of K of the map rows that a CTA holds.
+int stage_b_bytes(int BN, bool single) { return BN / (single ? 1 : 2) * 128; }
+
+size_t smem_bytes(int stage_b, int stages_a, int stages_b) {
   return static_cast<size_t>(stages_a) * kStageABytes +
-         static_cast<size_t>(stages_b) * (BN / 2) * 128 + kStgFloats * sizeof(float) +
-         kRotPairs * sizeof(float2) + kRunStride * sizeof(int32_t) + (4 * kMaxStages + 5) * sizeof(uint64_t) + 8;
+         static_cast<size_t>(stages_b) * stage_b + kStgFloats * sizeof(float) +
+         (4 * kMaxStages + 5) * sizeof(uint64_t) + 8;
 }
 
 // Ring depths.  A B stage is one 128-byte atom of K of this CTA's map rows
 // (16 KB at BN = 256), so the TMA producer refills the ring in fine steps;
-// 80 KB of B stages, and the rest of shared memory in A stages (two atoms,
+// 96 KB of B stages, and the rest of shared memory in A stages (two atoms,
 // 32 KB): three at BN = 256.  A loader waits for stage i - lag after issuing
 // stage i, so it never blocks on a young group.  Measured on the 32K
 // Llama -> Ministral-shaped transfer: one-atom B stages beat two-atom ones by 1%,
 // four A stages with four one-atom B stages lose 2-3% (deeper A rings do not
-// pay; B depth does).  The fifth B stage is the last that fits beside the
-// padded staging rows that the bulk copies of the value tiles need.
-void pick_rings(int BN, int* stages_a, int* stages_b, int* lag) {
+// pay; B depth does).
+void pick_rings(int stage_b, int* stages_a, int* stages_b, int* lag) {
   int dev = 0, optin = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  const int sb = std::min(kMaxStages, (80 * 1024) / ((BN / 2) * 128));
+  const int sb = std::min(kMaxStages, (96 * 1024) / stage_b);
   int sa = kMaxStages;
-  while (sa > 2 && smem_bytes(BN, sa, sb) > static_cast<size_t>(optin)) --sa;
+  while (sa > 2 && smem_bytes(stage_b, sa, sb) > static_cast<size_t>(optin)) --sa;
   *stages_a = sa;
   *stages_b = sb;
   *lag = std::max(1, sa - 2);
 }
 
 // Launches `kern` with clusters of two CTAs: one CTA pair per co-resident
-// cluster slot, at most one per pair tile.
+// cluster slot, at most one per pair tile; single: one CTA per SM instead, at
+// most one per tile.
 template <typename Kern, typename... Args>
-hf_status launch_pairs(Kern kern, int64_t max_pair_tiles, size_t smem, cudaStream_t stream,
-                       Args... args) {
+hf_status launch_pairs(Kern kern, bool single, int64_t max_pair_tiles, size_t smem,
+                       cudaStream_t stream, Args... args) {
   HF_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    static_cast<int>(smem)),
               "set shared memory size");
@@ -1712,6 +1743,14 @@ hf_status launch_pairs(Kern kern, int64_t max_pair_tiles, size_t smem, cudaStrea
   cfg.stream = stream;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  if (single) {
+    cfg.gridDim = dim3(static_cast<unsigned>(
+                           std::max<int64_t>(1, std::min<int64_t>(device_sm_count(), max_pair_tiles))),
+                       1, 1);
+    cfg.attrs = attr + 1;
+    HF_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, args...), "transfer kernel launch");
+    return HF_OK;
+  }
   // one CTA pair per co-resident cluster slot, at most one per pair tile
   int clusters = device_sm_count() / 2;
   cfg.gridDim = dim3(2 * clusters, 1, 1);
@@ -1739,7 +1778,8 @@ hf_status make_xfer(hf_plan_s* p, const void* sender, void* receiver, int l_begi
   const int bk = 128 / esize;
   CUtensorMap& mw = *map_out;
   hf_status s = make_map(&mw, d.d_W, f32, static_cast<uint64_t>(d.L_r) * 2 * p->d_r,
-                         static_cast<uint64_t>(p->K), static_cast<uint32_t>(p->BN / 2),
+                         static_cast<uint64_t>(p->K),
+                         static_cast<uint32_t>(p->BN / (p->single ? 1 : 2)),
                          static_cast<uint32_t>(bk), CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
   if (s != HF_OK) return s;
   XferParams& P = *out;
@@ -1788,7 +1828,7 @@ hf_status make_xfer(hf_plan_s* p, const void* sender, void* receiver, int l_begi
   P.BN = p->BN;
   P.wide = p->wide ? 1 : 0;
   P.n_tiles_n = p->d_r / (p->BN * (p->wide ? 2 : 1));
-  pick_rings(p->BN, &P.stages_a, &P.stages_b, &P.lag);
+  pick_rings(stage_b_bytes(p->BN, p->single), &P.stages_a, &P.stages_b, &P.lag);
   P.rope = p->rope ? 1 : 0;
   P.unrot = p->unrot ? 1 : 0;
   P.D_s = d.D_s;
@@ -1797,17 +1837,19 @@ hf_status make_xfer(hf_plan_s* p, const void* sender, void* receiver, int l_begi
   P.paged = d.paged ? 1 : 0;
   P.knorm = d.d_knorm_w ? 1 : 0;
   P.knorm_eps = d.knorm_eps;
-  P.idesc = make_idesc(f32 ? 2u : 1u, kPairRows, p->BN);
+  const int tile_rows = p->single ? kBM : kPairRows;
+  P.idesc = make_idesc(f32 ? 2u : 1u, tile_rows, p->BN);
   // pooling after the map: at most T_s windows (stride >= 1), two per pair tile
-  const int64_t row_blocks = p->pam ? (p->T_s + 1) / 2 : (p->T_r + kPairRows - 1) / kPairRows;
+  const int64_t row_blocks = p->pam ? (p->T_s + 1) / 2 : (p->T_r + tile_rows - 1) / tile_rows;
   *max_pair_tiles = 2LL * P.n_l * row_blocks * static_cast<int64_t>(P.n_tiles_n);
   return HF_OK;
 }
 
-template <typename T, int kRows, int kPam>
+template <typename T, int kRows, int kPam, bool kPair = true>
 hf_status launch_batch_typed(const BatchParams& B, int64_t max_pair_tiles, size_t smem,
                              cudaStream_t stream) {
-  return launch_pairs(transfer_batch_kernel<T, kRows, kPam>, max_pair_tiles, smem, stream, B);
+  return launch_pairs(transfer_batch_kernel<T, kRows, kPam, kPair>, !kPair, max_pair_tiles, smem,
+                      stream, B);
 }
 
 }  // namespace
@@ -1837,12 +1879,15 @@ hf_status launch_transfer(hf_plan_s* p, const void* sender, void* receiver, cuda
   hf_status s = make_xfer(p, sender, receiver, l_begin, l_end, &P, &mw, &max_pair_tiles);
   if (s != HF_OK) return s;
   P.stall = stall ? 1 : 0;
-  const size_t smem = smem_bytes(p->BN, P.stages_a, P.stages_b);
-  auto go = [&](auto kern) { return launch_pairs(kern, max_pair_tiles, smem, stream, mw, P); };
+  const size_t smem = smem_bytes(stage_b_bytes(p->BN, p->single), P.stages_a, P.stages_b);
+  auto go = [&](auto kern) {
+    return launch_pairs(kern, p->single, max_pair_tiles, smem, stream, mw, P);
+  };
   using Bf = __nv_bfloat16;
   if (d.dtype == HF_F32)
     return p->gather ? go(transfer_kernel<float, kCopiedRows, 2>)
                      : go(transfer_kernel<float, kBuiltRows, 2>);
+  if (p->single) return go(transfer_kernel<Bf, kCopiedRows, 0, false>);
   if (p->made)
     return p->pam ? go(transfer_kernel<Bf, kMadeRows, 1>) : go(transfer_kernel<Bf, kMadeRows, 0>);
   if (p->pam)
@@ -1856,7 +1901,7 @@ bool batch_compatible(const hf_plan_s* const* plans, int n) {
     if (plans[i]->desc.dtype != plans[0]->desc.dtype || plans[i]->gather != plans[0]->gather ||
         plans[i]->split != plans[0]->split || plans[i]->staged != plans[0]->staged ||
         plans[i]->pam != plans[0]->pam || plans[i]->wide != plans[0]->wide ||
-        plans[i]->made)
+        plans[i]->made || plans[i]->single != plans[0]->single)
       return false;
   return true;
 }
@@ -1886,17 +1931,20 @@ hf_status launch_transfer_batch(hf_plan_s* const* plans, const void* const* send
     return HF_OK;
   }
   int sa = 0, sb = 0, lag = 0;
-  pick_rings(max_bn, &sa, &sb, &lag);
+  const int stage_b = stage_b_bytes(max_bn, plans[0]->single);
+  pick_rings(stage_b, &sa, &sb, &lag);
   for (int i = 0; i < k; ++i) {
     B->P[i].stages_a = sa;
     B->P[i].stages_b = sb;
     B->P[i].lag = lag;
   }
   B->n_dir = k;
-  B->stage_b_stride = (max_bn / 2) * 128;
-  const size_t smem = smem_bytes(max_bn, sa, sb);
+  B->stage_b_stride = stage_b;
+  const size_t smem = smem_bytes(stage_b, sa, sb);
   hf_status s;
-  if (plans[0]->desc.dtype == HF_F32)
+  if (plans[0]->single)
+    s = launch_batch_typed<__nv_bfloat16, kCopiedRows, 0, false>(*B, tiles, smem, stream);
+  else if (plans[0]->desc.dtype == HF_F32)
     s = plans[0]->gather ? launch_batch_typed<float, kCopiedRows, 2>(*B, tiles, smem, stream)
                          : launch_batch_typed<float, kBuiltRows, 2>(*B, tiles, smem, stream);
   else if (plans[0]->pam)

@@ -14,14 +14,17 @@
 //
 // A chain of n / 128 steps bounds it (one CTA's 128 pivots, then two short
 // launches), not its operations: at n = 3,072 0.17 TFLOP of bf16 products, 0.1
-// ms of tensor time.  Blocks of 128 because the
-// block and its inverse fit one CTA's shared memory and two K atoms of the
+// ms of tensor time.  So two matrices are eliminated in the same steps, and
+// each kernel is launched while the one before it drains (a fit of 32,768 x
+// 3,072 -> 1,024: 6.04 ms with neither, 5.40 with both).  Blocks of 128 because
+// the block and its inverse fit one CTA's shared memory and two K atoms of the
 // product kernel; an iteration for the roots of S costs 33 dense products of
 // the same size (7.5 ms at 3,072).
 #include <cfloat>
 
 #include <cuda_bf16.h>
 
+#include "hf_device.cuh"
 #include "hf_internal.h"
 
 namespace hf {
@@ -39,9 +42,21 @@ constexpr int kPanelThreads = 256;
 // (zeros above the diagonal) goes to W's block and, transposed, to Tt.  With
 // upper not null the block of L^T goes to upper (leading dimension n_upper,
 // rows and columns below n_upper).
+// One CTA per matrix.
+struct TriPair {
+  TriProblem p[2];
+};
 __global__ void __launch_bounds__(kDiagThreads)
-    rc_diag_kernel(float* W, int64_t ld, int r0, const float* thr, int32_t* flag, float* Tt,
-                   float* upper, int n_upper) {
+    rc_diag_kernel(const __grid_constant__ TriPair tp, int r0, int32_t* flag) {
+  const TriProblem& pr = tp.p[blockIdx.x];
+  float* const W = pr.W;
+  const int64_t ld = pr.ld;
+  const float* const thr = pr.thr;
+  float* const Tt = pr.Tt;
+  float* const upper = pr.upper;
+  const int n_upper = pr.n_upper;
+  depend_wait();
+  depend_launch();
   extern __shared__ __align__(16) float sm[];
   float* const S = sm;               // [128][kLd]
   float* const T = sm + kNb * kLd;   // [32][kSub + 4]: the sub-block's L^{-1}
@@ -187,8 +202,17 @@ __global__ void __launch_bounds__(kDiagThreads)
 // row, plane p's element (column, row) at (p rows_p + column) 128 + row.  With
 // upper not null the columns right of the block also go to upper.
 __global__ void __launch_bounds__(kPanelThreads)
-    rc_panel_kernel(float* W, int64_t ld, int r0, const float* __restrict__ Tt,
-                    __nv_bfloat16* planes, int64_t rows_p, float* upper, int n_upper) {
+    rc_panel_kernel(const __grid_constant__ TriPair tp, int r0) {
+  const TriProblem& pr = tp.p[blockIdx.y];
+  depend_wait();
+  depend_launch();
+  if (static_cast<int>(blockIdx.x) * kPanelCols >= pr.n) return;
+  float* const W = pr.W;
+  const int64_t ld = pr.ld, rows_p = (pr.n + 255) / 256 * 256;
+  const float* const Tt = pr.Tt;
+  __nv_bfloat16* const planes = static_cast<__nv_bfloat16*>(pr.planes);
+  float* const upper = pr.upper;
+  const int n_upper = pr.n_upper;
   extern __shared__ __align__(16) float sm[];
   float* const t = sm;              // [k][row]
   float* const s = sm + kNb * kNb;  // [k][32]
@@ -272,8 +296,8 @@ size_t tri_factor_planes_bytes(int n) {
   return static_cast<size_t>(3 * rows_p * kNb * 2);
 }
 
-hf_status tri_factor(cudaStream_t s, const GemmWork& wk, float* W, int64_t ld, int n, float* Tt,
-                     void* planes, const float* thr, int32_t* flag, float* upper, int n_upper) {
+hf_status tri_factor(cudaStream_t s, const GemmWork& wk, const TriProblem* problems, int count,
+                     int32_t* flag) {
   const size_t diag_smem = (kNb * kLd + kSub * (kSub + 4) + 4 * kSub) * sizeof(float);
   const size_t panel_smem = (kNb * kNb + kNb * kPanelCols) * sizeof(float);
   HF_CUDA_TRY(cudaFuncSetAttribute(rc_diag_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -282,23 +306,35 @@ hf_status tri_factor(cudaStream_t s, const GemmWork& wk, float* W, int64_t ld, i
   HF_CUDA_TRY(cudaFuncSetAttribute(rc_panel_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    static_cast<int>(panel_smem)),
               "hf_recolor_fit: panel shared memory");
-  const int64_t rows_p = (n + 255) / 256 * 256;
-  for (int r0 = 0; r0 < n; r0 += kNb) {
-    rc_diag_kernel<<<1, kDiagThreads, diag_smem, s>>>(W, ld, r0, thr, flag, Tt, upper, n_upper);
-    rc_panel_kernel<<<n / kPanelCols, kPanelThreads, panel_smem, s>>>(
-        W, ld, r0, Tt, static_cast<__nv_bfloat16*>(planes), rows_p, upper, n_upper);
-    HF_CUDA_TRY(cudaGetLastError(), "hf_recolor_fit: factor launch");
-    const int below = r0 + kNb;
-    if (below >= n) break;
-    const GemmPlanes a{planes, rows_p, below}, b{planes, rows_p, 0};
-    GemmShape shape;  // all of L^{-1}, and of S what is on or above the diagonal
-    shape.tri = true;
-    shape.diag_col = below;
-    shape.fresh_lo = r0;
-    shape.fresh_hi = below;
-    const hf_status st = gemm_planes(s, wk, n - below, n, kNb, -1.f, a, b, 1.f,
-                                     W + static_cast<int64_t>(below) * ld, ld, shape);
-    if (st != HF_OK) return st;
+  int n_max = 0;
+  for (int i = 0; i < count; ++i) n_max = n_max > problems[i].n ? n_max : problems[i].n;
+  for (int r0 = 0; r0 < n_max; r0 += kNb) {
+    TriPair tp;  // the matrices that have this block row
+    int live = 0;
+    for (int i = 0; i < count; ++i)
+      if (r0 < problems[i].n) tp.p[live++] = problems[i];
+    if (live == 1) tp.p[1] = tp.p[0];
+    HF_CUDA_TRY(launch_dependent(rc_diag_kernel, dim3(live), dim3(kDiagThreads), diag_smem, s, tp, r0,
+                                 flag),
+                "hf_recolor_fit: factor launch");
+    HF_CUDA_TRY(launch_dependent(rc_panel_kernel, dim3(n_max / kPanelCols, live),
+                                 dim3(kPanelThreads), panel_smem, s, tp, r0),
+                "hf_recolor_fit: panel launch");
+    for (int i = 0; i < live; ++i) {
+      const TriProblem& p = tp.p[i];
+      const int below = r0 + kNb;
+      if (below >= p.n) continue;
+      const int64_t rows_p = (p.n + 255) / 256 * 256;
+      const GemmPlanes a{p.planes, rows_p, below}, b{p.planes, rows_p, 0};
+      GemmShape shape;  // all of L^{-1}, and of S what is on or above the diagonal
+      shape.tri = true;
+      shape.diag_col = below;
+      shape.fresh_lo = r0;
+      shape.fresh_hi = below;
+      const hf_status st = gemm_planes(s, wk, p.n - below, p.n, kNb, -1.f, a, b, 1.f,
+                                       p.W + static_cast<int64_t>(below) * p.ld, p.ld, shape);
+      if (st != HF_OK) return st;
+    }
   }
   return HF_OK;
 }

@@ -120,6 +120,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
                 const __grid_constant__ GemmParams P) {
   extern __shared__ __align__(1024) uint8_t smem[];
   if (smem_addr(smem) & 1023u) {
+    depend_wait();
     if (threadIdx.x == 0) atomicOr(P.err, 2);
     return;
   }
@@ -164,6 +165,8 @@ __global__ void __launch_bounds__(kGThreads, 1)
   cluster_sync();
   tc_fence_after_sync();
   const uint32_t tmem_base = *sTmem;
+  depend_wait();  // the operands are the kernels' before this one
+  depend_launch();
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
@@ -403,6 +406,8 @@ __global__ void gemm_reduce_kernel(const float* partial, int splits, int M, int 
                                    const float* Cin, int64_t ldc, float alpha, float beta,
                                    float diag, int tri, int n_lo, int n_diag) {
   const int64_t n_el = static_cast<int64_t>(M) * N;
+  depend_wait();
+  depend_launch();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n_el;
        i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t r = i / N, c = i - r * N;
@@ -426,6 +431,8 @@ __global__ void gemm_split_kernel(const float* src, int R, int K, int64_t s_r, i
   __shared__ float tile[32][65];
   const int r0 = blockIdx.y * 32, k0 = blockIdx.x * 64;
   const int tid = threadIdx.x;  // 256 threads
+  depend_wait();
+  depend_launch();
   if (s_r == 1 && s_k != 1) {
     // contiguous along r: thread reads rows r0 + (tid & 31), k = k0 + (tid >> 5) + 8 i
     for (int i = 0; i < 8; ++i) {
@@ -583,7 +590,9 @@ hf_status gemm_planes(cudaStream_t s, const GemmWork& wk, int M, int N, int k_p,
                                    static_cast<int>(smem)),
               "hf_recolor_fit: product shared memory");
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2;
   attr[0].val.clusterDim.y = 1;
@@ -594,14 +603,14 @@ hf_status gemm_planes(cudaStream_t s, const GemmWork& wk, int M, int N, int k_p,
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   HF_CUDA_TRY(cudaLaunchKernelEx(&cfg, gemm_kernel, ma, mb, P), "hf_recolor_fit: product launch");
   if (splits > 1) {
     const int64_t n_el = static_cast<int64_t>(M) * N;
     const int grid = static_cast<int>(std::min<int64_t>((n_el + 255) / 256, 4096));
-    gemm_reduce_kernel<<<grid, 256, 0, s>>>(wk.partial, splits, M, N, C, Cin, ldc, alpha, beta,
-                                            diag, P.tri, P.n_lo, P.n_diag);
-    HF_CUDA_TRY(cudaGetLastError(), "hf_recolor_fit: product reduce launch");
+    HF_CUDA_TRY(launch_dependent(gemm_reduce_kernel, dim3(grid), dim3(256), 0, s, wk.partial, splits, M,
+                                 N, C, Cin, ldc, alpha, beta, diag, P.tri, P.n_lo, P.n_diag),
+                "hf_recolor_fit: product reduce launch");
   }
   return HF_OK;
 }
@@ -629,15 +638,16 @@ hf_status gemm_f32(cudaStream_t s, const GemmWork& wk, int M, int N, int K, floa
   __nv_bfloat16* pb = same ? pa : static_cast<__nv_bfloat16*>(wk.planes_b);
   {
     dim3 grid(static_cast<unsigned>(Kp / 64), static_cast<unsigned>(Mp / 32));
-    gemm_split_kernel<<<grid, 256, 0, s>>>(A, M, K, a_i, a_k, pa, static_cast<int>(Mp),
-                                           static_cast<int>(Kp));
+    HF_CUDA_TRY(launch_dependent(gemm_split_kernel, grid, dim3(256), 0, s, A, M, K, a_i, a_k, pa,
+                                 static_cast<int>(Mp), static_cast<int>(Kp)),
+                "hf_recolor_fit: operand split launch");
   }
   if (!same) {
     dim3 grid(static_cast<unsigned>(Kp / 64), static_cast<unsigned>(Np / 32));
-    gemm_split_kernel<<<grid, 256, 0, s>>>(B, N, K, b_j, b_k, pb, static_cast<int>(Np),
-                                           static_cast<int>(Kp));
+    HF_CUDA_TRY(launch_dependent(gemm_split_kernel, grid, dim3(256), 0, s, B, N, K, b_j, b_k, pb,
+                                 static_cast<int>(Np), static_cast<int>(Kp)),
+                "hf_recolor_fit: operand split launch");
   }
-  HF_CUDA_TRY(cudaGetLastError(), "hf_recolor_fit: operand split launch");
   const GemmPlanes ga{pa, Mp, 0}, gb{pb, Np, 0};
   return gemm_planes(s, wk, M, N, static_cast<int>(Kp), alpha, ga, gb, beta, C, ldc, GemmShape{}, Cin,
                      diag);

@@ -175,6 +175,25 @@ cudaError_t launch_fused_rows(Kern kern, int64_t rows, cudaStream_t stream, cons
   return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
+// A launch that may overlap the end of the kernel before it in the stream
+// (programmatic dependent launch): the kernel calls depend_wait before its
+// first global access.
+template <typename Kern, typename... Args>
+cudaError_t launch_dependent(Kern kern, dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+                             const Args&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
 void set_error(const std::string& msg);
 hf_status cuda_fail(cudaError_t e, const char* what);
 int device_sm_count();
@@ -249,10 +268,21 @@ hf_status gemm_f32(cudaStream_t s, const GemmWork& wk, int M, int N, int K, floa
 // n_upper.  Tt: kFactorBlock^2 floats; planes: tri_factor_planes_bytes(n).  A
 // pivot that is not above *thr sets *flag (cleared before) and the result is
 // of no use.
+// Up to two matrices are factored side by side: a chain of latencies each.
 constexpr int kFactorBlock = 128;
 size_t tri_factor_planes_bytes(int n);
-hf_status tri_factor(cudaStream_t s, const GemmWork& wk, float* W, int64_t ld, int n, float* Tt,
-                     void* planes, const float* thr, int32_t* flag, float* upper, int n_upper);
+struct TriProblem {
+  float* W;
+  int64_t ld;
+  int n;
+  float* Tt;
+  void* planes;
+  const float* thr;
+  float* upper;
+  int n_upper;
+};
+hf_status tri_factor(cudaStream_t s, const GemmWork& wk, const TriProblem* problems, int count,
+                     int32_t* flag);
 
 }  // namespace hf
 

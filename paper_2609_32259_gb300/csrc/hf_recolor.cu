@@ -11,7 +11,7 @@
 //   A = L^{-T} polar(L^{-1} Sigma_ZY C^{-T}) C^T,
 // one factorisation instead of ~11 iterations of three dense products (at
 // 32,768 x 3,072 -> 1,024 the fit took 16.5 ms with iterated roots and three
-// dense moment products, 6.0 ms now; fp32 fits with d_S > d_R come out a
+// dense moment products, 5.4 ms now; fp32 fits with d_S > d_R come out a
 // quarter as far from 64 bits).  Only where a pivot is too small
 // for fp32 (kPivot of the mean eigenvalue; reg is 0 or tiny and the covariance
 // near singular) the symmetric roots are iterated instead, as far as they
@@ -375,7 +375,7 @@ __global__ void rc_bias_final_kernel(const double* sy, const double* sw_ss, cons
 }
 
 struct Rc {
-  size_t stats, part, bacc, mu, gram, tt, fplanes, thr, flag, sz, sy, szy, p1, p2, p3, p4, sz_ih, sy_ih,
+  size_t stats, part, bacc, mu, gram, tt, fplanes, fplanes_y, thr, flag, sz, sy, szy, p1, p2, p3, p4, sz_ih, sy_ih,
       sy_h, m, x1, x2, xtx, a, planes_a, planes_b, partial, err, total;
   size_t planes_a_bytes, planes_b_bytes;
   int np, mp, F;     // features of X and of Y padded to whole factor blocks; their sum
@@ -402,8 +402,9 @@ Rc rc_layout(int64_t N, int dx, int dy) {
   L.F = L.np + L.mp;
   L.chunk = std::min<int64_t>(up(N, 64), kMomentChunk);
   L.gram = take(f * L.F * L.F);
-  L.tt = take(f * kFactorBlock * kFactorBlock);
+  L.tt = take(2 * f * kFactorBlock * kFactorBlock);
   L.fplanes = take(tri_factor_planes_bytes(L.np));
+  L.fplanes_y = take(tri_factor_planes_bytes(L.mp));
   L.thr = take(f * 2);
   L.flag = take(sizeof(int32_t));
   L.sz = take(f * dx * dx);
@@ -647,12 +648,10 @@ hf_status recolor_typed(int64_t N, int dx, int dy, const void* Xv, const void* Y
   if ((st = moments()) != HF_OK) return st;
   HF_CUDA_TRY(cudaMemsetAsync(flag, 0, sizeof(int32_t), s), "clear");
   HF_CUDA_TRY(cudaMemsetAsync(F(L.sy_h), 0, sizeof(float) * dy * dy, s), "clear");
-  if ((st = tri_factor(s, h, G, L.F, L.np, F(L.tt), ws + L.fplanes, thr, flag, nullptr, 0)) !=
-      HF_OK)
-    return st;
-  if ((st = tri_factor(s, h, GY, L.F, L.mp, F(L.tt), ws + L.fplanes, thr + 1, flag, F(L.sy_h),
-                       dy)) != HF_OK)
-    return st;
+  const TriProblem tri[2] = {
+      {G, L.F, L.np, F(L.tt), ws + L.fplanes, thr, nullptr, 0},
+      {GY, L.F, L.mp, F(L.tt) + kFactorBlock * kFactorBlock, ws + L.fplanes_y, thr + 1, F(L.sy_h), dy}};
+  if ((st = tri_factor(s, h, tri, 2, flag)) != HF_OK) return st;
   extract(G, dx, dx, 2, F(L.sz_ih));   // L^{-1}
   extract(GY, dy, dy, 2, F(L.sy_ih));  // C^{-1}
   int32_t weak = 0;

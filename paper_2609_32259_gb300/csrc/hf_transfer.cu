@@ -30,7 +30,7 @@
 //               once, or write the rounded row and its rounding residual as
 //               two atoms (split operands).  Both write the 128-byte swizzled
 //               layout and fence it to the async proxy before arriving on the
-//               stage barrier.
+//               stage barrier.  Rows that follow one another come by TMA.
 // Overlap mean pooling is linear, so by default it follows the map: the
 // tile rows of a CTA are a window of 128 consecutive aligned sender tokens
 // and the epilogue pools the mapped rows of each receiver row's columns
@@ -762,13 +762,20 @@ __device__ __forceinline__ void arrive_leader(uint32_t bar, int row0) {
 // layout.  A thread keeps LAG groups in flight: after committing k-block i
 // it waits for k-block i-LAG and fences it to the async proxy; then one lane
 // per warp arrives on that stage's barrier in the leader CTA of the pair.
+// Rows that follow one another (made rows, and the windows of pooling after the
+// map where the aligned tokens are whole caches) come by tensor copies instead,
+// 32 rows of an atom a warp: no thread's load or store has to wait behind them,
+// which the epilogue feels (overlap-mean 4K 549 -> 530 us, interpolated 8K 944
+// -> 908, rotated 3K 408 -> 382).  The arrivals a stage expects are the same, so
+// tiles of either kind follow one another.
 template <typename T, int LAG, int kDirs, int kPam, int kRows, int kTileRows>
 __device__ __forceinline__ void gather_rows(const XferParams* Ps, const DirTable<kDirs>& dt,
-                                            int n_dir, uint8_t* sA, uint64_t* full_a,
-                                            uint64_t* empty_a, volatile int* sAbort, int t,
-                                            int lane, int row0, int total_tiles, int first_tile,
-                                            int tile_step) {
+                                            const CUtensorMap* maps_a, int n_dir, uint8_t* sA,
+                                            uint64_t* full_a, uint64_t* empty_a,
+                                            volatile int* sAbort, int t, int lane, int row0,
+                                            int total_tiles, int first_tile, int tile_step) {
   constexpr int kBK = Elem<T>::kBK;
+  constexpr bool kBulk = kRows == kMadeRows || (kPam == 1 && kRows == kCopiedRows);
   const bool by_slot = slot_order(total_tiles, tile_step);
   constexpr int kPerChunk = 16 / sizeof(T);
   const int stages = Ps[0].stages_a;
@@ -791,9 +798,10 @@ __device__ __forceinline__ void gather_rows(const XferParams* Ps, const DirTable
     const KLoop kl = k_loop<kRows>(P, c);
     const LayerSegs* lsegs = P.segs + l;
     const int n_seg = __ldg(&lsegs->n_seg);
-    auto seg_base = [&](int s2) -> int64_t {
-      return (static_cast<int64_t>(__ldg(&lsegs->layer[s2][0]) * 2 + c) * P.s_rows) * P.d_s;
+    auto seg_row = [&](int s2) -> int64_t {
+      return static_cast<int64_t>(__ldg(&lsegs->layer[s2][0]) * 2 + c) * P.s_rows;
     };
+    auto seg_base = [&](int s2) -> int64_t { return seg_row(s2) * P.d_s; };
     int64_t sbase = 0, snext = 0;
     // made rows are whole operand rows: one base, and the residuals a plane on
     const int64_t width = kl.made ? static_cast<int64_t>(P.n_batoms) * kBK : P.d_s;
@@ -805,6 +813,26 @@ __device__ __forceinline__ void gather_rows(const XferParams* Ps, const DirTable
       sbase = seg_base(0);
       if (n_seg > 1) snext = seg_base(1);
     }
+    // rows that follow one another: their first one in maps_a, for this warp
+    const bool bulk = kBulk && (kl.made || (kRows == kCopiedRows && !P.srow));
+    int64_t first_row = 0, brow = 0;  // brow: the segment's first sender row
+    bool any_row = false;
+    if (bulk) {
+      int64_t k0;
+      if (pam_on<kPam>(P)) {
+        k0 = static_cast<int64_t>((m * kTileRows + row0) >> 7) * __ldg(P.win_info + 1) + slab * 32;
+        any_row = k0 < P.T_s;
+      } else {
+        k0 = static_cast<int64_t>(m) * kTileRows + row0 + slab * 32;
+        any_row = k0 < U;
+      }
+      if (kl.made) {
+        const int at = (l - P.l0) * P.made_roles + (P.made_roles == 2 ? c : 0);
+        k0 += at * (kl.split ? 2 : 1) * P.x_rows;
+      }
+      first_row = k0;
+      if (!kl.made) brow = seg_row(0);
+    }
     int64_t roff[8];
     uint32_t doff[8];
     // rows past the last distinct row are not copied: their products (of what
@@ -812,6 +840,7 @@ __device__ __forceinline__ void gather_rows(const XferParams* Ps, const DirTable
     unsigned live = 0;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
+      if (bulk) break;
       const int r = slab * 32 + 4 * i + rsub;
       int64_t kr;  // sender-cache row
       if (pam_on<kPam>(P)) {
@@ -835,6 +864,42 @@ __device__ __forceinline__ void gather_rows(const XferParams* Ps, const DirTable
       }
       const uint32_t sa = smem_addr(sA + stage * kStageABytes);
       const int na = kb == kl.n_kb - 1 && !kl.split ? kl.last_atoms : kAtoms;
+      if (bulk) {
+        if (lane == 0) {
+          if (any_row) {
+            const uint32_t fa = mapa_shared(smem_addr(&full_a[stage]), 0);
+            mbar_arrive_expect_tx_cluster(fa, static_cast<uint32_t>(na) * (kAtomABytes / 4));
+            for (int a = 0; a < na; ++a) {
+              // the residuals of an atom are a plane on
+              const int64_t y = first_row + (kl.made ? (kl.split && a == 1 ? P.x_rows : 0) : brow);
+              const int x = (kl.split ? kb : kl.made ? kb * kAtoms + a : kin) * kBK;
+              tma_load_2d_pair(sa + a * kAtomABytes + slab * (kAtomABytes / 4), &maps_a[dd], x,
+                               static_cast<int32_t>(y), fa);
+              if (!kl.made && ++kin == P.atoms_per_seg) {
+                kin = 0;
+                ++seg;
+                if (seg < n_seg) brow = seg_row(seg);
+              }
+            }
+          } else {
+            arrive_leader(smem_addr(&full_a[stage]), row0);
+          }
+        }
+        if (pending > 0) {  // copied rows of the tile before
+          cp_async_wait<0>();
+          fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0)
+            for (int k = pending; k >= 1; --k)
+              arrive_leader(smem_addr(&full_a[(stage + stages - k) % stages]), row0);
+          pending = 0;
+        }
+        if (++stage == stages) {
+          stage = 0;
+          phase ^= 1;
+        }
+        continue;
+      }
 #pragma unroll
       for (int a = 0; a < kAtoms; ++a) {
         if (a < na) {
@@ -1084,8 +1149,9 @@ __device__ __forceinline__ void build_rows_staged(const XferParams* Ps, const Di
 // parameters).  All directions share the dtype, the operand path and the
 // ring depths; a B stage is stage_b_stride bytes (the widest direction's).
 template <typename T, int kRows, int kDirs, int kPam, bool kPair>
-__device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const XferParams* Ps,
-                                              int n_dir, int stage_b_stride) {
+__device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const CUtensorMap* maps_a,
+                                              const XferParams* Ps, int n_dir,
+                                              int stage_b_stride) {
   constexpr int kBK = Elem<T>::kBK;
   constexpr bool kGather = kRows != kBuiltRows;
   constexpr int kTileRows = kPair ? kPairRows : kBM;
@@ -1525,11 +1591,11 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const Xfe
     const int t = threadIdx.x - 64 - kEpiThreads;  // 0..127
     if (kGather) {
       switch (P0.lag) {
-        case 1: gather_rows<T, 1, kDirs, kPam, kRows, kTileRows>(Ps, dt, n_dir, sA, full_a, empty_a, sAbort, t, lane, row0, total_tiles, first_tile, tile_step); break;
-        case 2: gather_rows<T, 2, kDirs, kPam, kRows, kTileRows>(Ps, dt, n_dir, sA, full_a, empty_a, sAbort, t, lane, row0, total_tiles, first_tile, tile_step); break;
-        case 3: gather_rows<T, 3, kDirs, kPam, kRows, kTileRows>(Ps, dt, n_dir, sA, full_a, empty_a, sAbort, t, lane, row0, total_tiles, first_tile, tile_step); break;
-        case 4: gather_rows<T, 4, kDirs, kPam, kRows, kTileRows>(Ps, dt, n_dir, sA, full_a, empty_a, sAbort, t, lane, row0, total_tiles, first_tile, tile_step); break;
-        default: gather_rows<T, 5, kDirs, kPam, kRows, kTileRows>(Ps, dt, n_dir, sA, full_a, empty_a, sAbort, t, lane, row0, total_tiles, first_tile, tile_step); break;
+        case 1: gather_rows<T, 1, kDirs, kPam, kRows, kTileRows>(Ps, dt, maps_a, n_dir, sA, full_a, empty_a, sAbort, t, lane, row0, total_tiles, first_tile, tile_step); break;
+        case 2: gather_rows<T, 2, kDirs, kPam, kRows, kTileRows>(Ps, dt, maps_a, n_dir, sA, full_a, empty_a, sAbort, t, lane, row0, total_tiles, first_tile, tile_step); break;
+        case 3: gather_rows<T, 3, kDirs, kPam, kRows, kTileRows>(Ps, dt, maps_a, n_dir, sA, full_a, empty_a, sAbort, t, lane, row0, total_tiles, first_tile, tile_step); break;
+        case 4: gather_rows<T, 4, kDirs, kPam, kRows, kTileRows>(Ps, dt, maps_a, n_dir, sA, full_a, empty_a, sAbort, t, lane, row0, total_tiles, first_tile, tile_step); break;
+        default: gather_rows<T, 5, kDirs, kPam, kRows, kTileRows>(Ps, dt, maps_a, n_dir, sA, full_a, empty_a, sAbort, t, lane, row0, total_tiles, first_tile, tile_step); break;
       }
     } else if (P0.staged) {
       switch (P0.lag) {
@@ -1628,13 +1694,14 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const Xfe
 template <typename T, int kRows, int kPam, bool kPair = true>
 __global__ void __launch_bounds__(kThreads, 1)
     transfer_kernel(const __grid_constant__ CUtensorMap tmap_w,
+                    const __grid_constant__ CUtensorMap tmap_a,
                     const __grid_constant__ XferParams P) {
-  transfer_body<T, kRows, 1, kPam, kPair>(&tmap_w, &P, 1, P.BN / (kPair ? 2 : 1) * 128);
+  transfer_body<T, kRows, 1, kPam, kPair>(&tmap_w, &tmap_a, &P, 1, P.BN / (kPair ? 2 : 1) * 128);
 }
 
 // Several directions in one launch (hf_transfer_batch).
 struct BatchParams {
-  CUtensorMap maps[kMaxBatch];
+  CUtensorMap maps[kMaxBatch], maps_a[kMaxBatch];
   XferParams P[kMaxBatch];
   int n_dir;
   int stage_b_stride;
@@ -1644,7 +1711,7 @@ static_assert(sizeof(BatchParams) < 32000, "BatchParams must fit the kernel para
 template <typename T, int kRows, int kPam, bool kPair = true>
 __global__ void __launch_bounds__(kThreads, 1)
     transfer_batch_kernel(const __grid_constant__ BatchParams B) {
-  transfer_body<T, kRows, kMaxBatch, kPam, kPair>(B.maps, B.P, B.n_dir, B.stage_b_stride);
+  transfer_body<T, kRows, kMaxBatch, kPam, kPair>(B.maps, B.maps_a, B.P, B.n_dir, B.stage_b_stride);
 }
 
 // ---------------------------------------------------------------------------
@@ -1771,7 +1838,8 @@ namespace {
 // The kernel parameters and map tile descriptor of one plan's launch over
 // receiver layers [l_begin, l_end); *max_pair_tiles bounds its pair tiles.
 hf_status make_xfer(hf_plan_s* p, const void* sender, void* receiver, int l_begin, int l_end,
-                    XferParams* out, CUtensorMap* map_out, int64_t* max_pair_tiles) {
+                    XferParams* out, CUtensorMap* map_out, CUtensorMap* map_a_out,
+                    int64_t* max_pair_tiles) {
   const hf_plan_desc& d = p->desc;
   const bool f32 = d.dtype == HF_F32;
   const int esize = f32 ? 4 : 2;
@@ -1782,6 +1850,19 @@ hf_status make_xfer(hf_plan_s* p, const void* sender, void* receiver, int l_begi
                          static_cast<uint32_t>(p->BN / (p->single ? 1 : 2)),
                          static_cast<uint32_t>(bk), CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
   if (s != HF_OK) return s;
+  if (p->made || (p->pam && p->gather && !p->span)) {
+    // operand rows that follow one another: made ones, or the sender's under
+    // pooling after the map
+    const int planes = (p->made == 3 ? 2 : 1) * (p->split ? 2 : 1);
+    s = p->made ? make_map(map_a_out, p->ws + p->lay.xbuf, f32,
+                           static_cast<uint64_t>(p->x_layers) * planes * p->x_rows,
+                           static_cast<uint64_t>(p->K), 32u, static_cast<uint32_t>(bk),
+                           CU_TENSOR_MAP_L2_PROMOTION_L2_256B)
+                : make_map(map_a_out, sender, f32, static_cast<uint64_t>(d.L_s) * 2 * p->s_rows,
+                           static_cast<uint64_t>(p->d_s), 32u, static_cast<uint32_t>(bk),
+                           CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
+    if (s != HF_OK) return s;
+  }
   XferParams& P = *out;
   std::memset(&P, 0, sizeof(P));
   char* ws = p->ws;
@@ -1874,14 +1955,14 @@ hf_status launch_transfer(hf_plan_s* p, const void* sender, void* receiver, cuda
     if (e != HF_OK) return e;
   }
   XferParams P;
-  CUtensorMap mw;
+  CUtensorMap mw, ma = {};
   int64_t max_pair_tiles = 0;
-  hf_status s = make_xfer(p, sender, receiver, l_begin, l_end, &P, &mw, &max_pair_tiles);
+  hf_status s = make_xfer(p, sender, receiver, l_begin, l_end, &P, &mw, &ma, &max_pair_tiles);
   if (s != HF_OK) return s;
   P.stall = stall ? 1 : 0;
   const size_t smem = smem_bytes(stage_b_bytes(p->BN, p->single), P.stages_a, P.stages_b);
   auto go = [&](auto kern) {
-    return launch_pairs(kern, p->single, max_pair_tiles, smem, stream, mw, P);
+    return launch_pairs(kern, p->single, max_pair_tiles, smem, stream, mw, ma, P);
   };
   using Bf = __nv_bfloat16;
   if (d.dtype == HF_F32)
@@ -1917,7 +1998,7 @@ hf_status launch_transfer_batch(hf_plan_s* const* plans, const void* const* send
     if (p->T_r == 0) continue;
     int64_t mt = 0;
     const hf_status s = make_xfer(p, senders[i], receivers[i], 0, p->desc.L_r, &B->P[k],
-                                  &B->maps[k], &mt);
+                                  &B->maps[k], &B->maps_a[k], &mt);
     if (s != HF_OK) {
       delete B;
       return s;

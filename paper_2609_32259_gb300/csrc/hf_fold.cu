@@ -10,7 +10,7 @@
 // instructions, with every fp32 factor split exactly into three bf16 parts and
 // the products above 2^-23 kept (a rank of 16 is one 16-deep step: too thin for
 // an accumulator in tensor memory; 80 maps of 1,024 x 3,072, rank 16, with the
-// bias: 0.37 ms, fold_kernel 0.49; the same error against 64 bits).  fold_kernel
+// bias: 0.27 ms, fold_kernel 0.49; the same error against 64 bits).  fold_kernel
 // takes the rest with plain fp32 arithmetic; a block reads its columns of W
 // twice (the second time from L2) and writes them once.
 #include <algorithm>
@@ -19,6 +19,7 @@
 
 #include <string>
 
+#include "hf_device.cuh"
 #include "hf_internal.h"
 
 namespace hf {
@@ -254,7 +255,7 @@ __global__ void __launch_bounds__(kFoldThreads) fold_kernel(const T* W, const fl
 constexpr int kMmaWarps = 16;
 constexpr int kMmaCols = 32;            // columns of W per unit of work
 constexpr int kMmaRows = 1024;          // d_R at most: 64 rows per warp
-constexpr int kMmaStride = kMmaCols + 8;  // padded shared-memory row: 80 bytes, no bank twice
+constexpr int kTStride = kMmaCols + 8;  // padded row of T: 80 bytes, no bank twice
 constexpr int kPartStride = kMmaCols + 4;
 
 __device__ __forceinline__ void mma_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0,
@@ -288,10 +289,13 @@ __device__ __forceinline__ void split3(float x, float y, uint32_t* h0, uint32_t*
 }
 
 struct FoldMmaSmem {
-  __nv_bfloat16 w[2][kMmaRows][kMmaStride];
+  // 64-byte rows, the 16-byte piece c of row r at c ^ (r / 2 mod 4): eight rows'
+  // pieces lie in different banks, and tensor copies write it out
+  __nv_bfloat16 w[2][kMmaRows][kMmaCols];
   float part[kMmaWarps][16][kPartStride];
-  __nv_bfloat16 t[3][16][kMmaStride];
+  __nv_bfloat16 t[3][16][kTStride];
 };
+static_assert(kMmaCols == 32, "the 64-byte swizzle is over rows of 32");
 
 // A persistent CTA takes a run of units (map, 32 columns).  Warp w owns rows 16
 // steps w .. of W (steps <= 4 blocks of 16): it alone copies them in, works on
@@ -301,17 +305,20 @@ struct FoldMmaSmem {
 //     W is exact in bf16, so three products per term;
 //  2. the warps' shares meet in shared memory, T is split there;
 //  3. W += G^T T on the warp's rows: six products, added to W in fp32, rounded
-//     once, back into the buffer, which then leaves in 16-byte stores and takes
-//     the columns of the unit after the next.
-// The latency of these steps bounds it, at a third of the tensor instructions'
-// and of the memory rate (64 KB in and out per unit and SM; two buffers of 32
-// columns are what fits; step 1 of a unit before step 3 of the one before it
-// exposed the copies instead and was 17% slower).
+//     once, back into the buffer, which then leaves by a tensor copy; once that
+//     has read it (during the next unit's step 1) the buffer takes the columns of
+//     the unit after.
+// The chain of these steps bounds it (64 KB in and out per unit and SM; two
+// buffers of 32 columns are what fits): of 9.7K cycles a unit step 3 takes 4.4K
+// (3K at the tensor instructions' rate), steps 1 and 2 1.5K and 1.2K; the memory
+// rate allows 5.6K.  With the rows written out by the threads a unit took 13K
+// (4.1K of them in those stores; 80 maps of 1,024 x 3,072: 358 us, 254 now).
+// Step 1 of a unit before step 3 of the one before it exposed the copies.
 __global__ void __launch_bounds__(32 * kMmaWarps)
     fold_mma_kernel(const __nv_bfloat16* W, const float* __restrict__ Bm,
-                    const float* __restrict__ Gm, __nv_bfloat16* Wf, int n_maps, int d_r, int64_t K,
-                    int rank, int steps) {
-  extern __shared__ __align__(128) uint8_t fold_smem[];
+                    const float* __restrict__ Gm, const __grid_constant__ CUtensorMap map_out,
+                    int n_maps, int d_r, int64_t K, int rank, int steps) {
+  extern __shared__ __align__(1024) uint8_t fold_smem[];
   FoldMmaSmem& sm = *reinterpret_cast<FoldMmaSmem*>(fold_smem);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = lane >> 2, t = lane & 3;  // fragment row and column pair
@@ -319,29 +326,32 @@ __global__ void __launch_bounds__(32 * kMmaWarps)
   const int64_t units = static_cast<int64_t>(n_maps) * per_map;
   const int64_t u0 = units * blockIdx.x / gridDim.x, u1 = units * (blockIdx.x + 1) / gridDim.x;
   const int row0 = warp * 16 * steps, rows = min(16 * steps, d_r - row0);  // <= 0: padding only
-  for (int i = lane; i < (16 * steps - max(rows, 0)) * kMmaStride; i += 32) {
-    const int r = row0 + max(rows, 0) + i / kMmaStride;  // rows past d_R: zeros
-    sm.w[0][r][i % kMmaStride] = sm.w[1][r][i % kMmaStride] = __nv_bfloat16(0.f);
+  for (int i = lane; i < (16 * steps - max(rows, 0)) * kMmaCols; i += 32) {
+    const int r = row0 + max(rows, 0) + i / kMmaCols;  // rows past d_R: zeros
+    sm.w[0][r][i % kMmaCols] = sm.w[1][r][i % kMmaCols] = __nv_bfloat16(0.f);
   }
   // the warp's rows of a unit, 16-byte pieces, four per row
+  const int lr = lane >> 2, lc = (lane & 3) * 8, lswz = ((lane & 3) ^ (lane >> 3)) * 8;
   auto load = [&](int64_t u) {
     if (u < u1) {
       const int map = static_cast<int>(u / per_map), buf = static_cast<int>((u - u0) & 1);
       const int64_t k0 = (u - static_cast<int64_t>(map) * per_map) * kMmaCols;
-      const __nv_bfloat16* src = W + (static_cast<int64_t>(map) * d_r + row0) * K + k0;
-      for (int i = lane; i < 4 * rows; i += 32) {
-        const int r = i >> 2, c = (i & 3) * 8;
-        if (k0 + c < K) fold_cp_async<16>(&sm.w[buf][row0 + r][c], src + r * K + c);
+      const __nv_bfloat16* src = W + (static_cast<int64_t>(map) * d_r + row0 + lr) * K + k0 + lc;
+      if (k0 + lc < K) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+          if (lr + 8 * i < rows)
+            fold_cp_async<16>(&sm.w[buf][row0 + lr + 8 * i][lswz], src + 8 * i * K);
       }
     }
     fold_cp_commit();
   };
   load(u0);
-  load(u0 + 1);
   uint32_t bf[4][3][4];  // B^T, rank x 16 rows per step, split
   uint32_t gf[4][3][4];  // G^T, 16 rows x rank per step, split
   int map_now = -1;
-  const int lrow = lane & 15, lcol = (lane >> 4) * 8;  // ldmatrix: this lane's row
+  const int lrow = lane & 15, lhalf = lane >> 4;  // ldmatrix: this lane's row and piece
+  const int lsw = (lrow >> 1) & 3, gsw = (g >> 1) & 3;
   for (int64_t u = u0; u < u1; ++u) {
     const int buf = static_cast<int>((u - u0) & 1);
     const int map = static_cast<int>(u / per_map);
@@ -368,8 +378,8 @@ __global__ void __launch_bounds__(32 * kMmaWarps)
       }
     }
     {
-      // step 1 (the next unit's columns may still be on their way)
-      fold_cp_wait<1>();
+      // step 1
+      fold_cp_wait<0>();
       __syncwarp();
       float d[4][4] = {};
 #pragma unroll
@@ -378,7 +388,7 @@ __global__ void __launch_bounds__(32 * kMmaWarps)
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           uint32_t x[4];
-          ldsm_x4_t(x, &w[row0 + 16 * s + lrow][16 * h + lcol]);
+          ldsm_x4_t(x, &w[row0 + 16 * s + lrow][((2 * h + lhalf) ^ lsw) * 8]);
 #pragma unroll
           for (int p = 2; p >= 0; --p) {
             mma_16816(d[2 * h], bf[s][p], x[0], x[1]);
@@ -392,6 +402,9 @@ __global__ void __launch_bounds__(32 * kMmaWarps)
         *reinterpret_cast<float2*>(&sm.part[warp][g + 8][8 * i + 2 * t]) =
             make_float2(d[i][2], d[i][3]);
       }
+      if (lane == 0) bulk_store_wait_read();  // the unit before has left its buffer
+      __syncwarp();
+      load(u + 1);
     }
     __syncthreads();
     {
@@ -413,7 +426,7 @@ __global__ void __launch_bounds__(32 * kMmaWarps)
       for (int h = 0; h < 2; ++h) {
         uint32_t x[3][4];
 #pragma unroll
-        for (int p = 0; p < 3; ++p) ldsm_x4_t(x[p], &sm.t[p][lrow][16 * h + lcol]);
+        for (int p = 0; p < 3; ++p) ldsm_x4_t(x[p], &sm.t[p][lrow][16 * h + 8 * lhalf]);
 #pragma unroll
         for (int s = 0; s < 4; ++s) {
           if (s >= steps) break;
@@ -426,31 +439,28 @@ __global__ void __launch_bounds__(32 * kMmaWarps)
           }
 #pragma unroll
           for (int q = 0; q < 2; ++q) {
-            const int col = 16 * h + 8 * q + 2 * t;
+            const int col = ((2 * h + q) ^ gsw) * 8 + 2 * t;
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
-              __nv_bfloat162* const o =
-                  reinterpret_cast<__nv_bfloat162*>(&w[row0 + 16 * s + g + 8 * k][col]);
+              const int r = 16 * s + g + 8 * k;
+              if (r >= rows) continue;  // rows past d_R stay zeros, whatever T holds
+              __nv_bfloat162* const o = reinterpret_cast<__nv_bfloat162*>(&w[row0 + r][col]);
               const float2 wv = __bfloat1622float2(*o);
               *o = __floats2bfloat162_rn(wv.x + y[q][2 * k], wv.y + y[q][2 * k + 1]);
             }
           }
         }
       }
+      fence_proxy_async_smem();
       __syncwarp();
-      __nv_bfloat16* const dst = Wf + (static_cast<int64_t>(map) * d_r + row0) * K + k0;
-#pragma unroll 4
-      for (int i = lane; i < 4 * rows; i += 32) {
-        const int r = i >> 2, c = (i & 3) * 8;
-        if (k0 + c < K)
-          *reinterpret_cast<uint4*>(dst + r * K + c) =
-              *reinterpret_cast<const uint4*>(&w[row0 + r][c]);
-      }
-      __syncwarp();
-      load(u + 2);
+      if (lane == 0 && rows > 0)
+        tma_store_3d(&map_out, smem_addr(&w[row0][0]), static_cast<int32_t>(k0), row0, map);
     }
   }
-  fold_cp_wait<0>();
+  if (lane == 0) {
+    bulk_store_wait_read();
+    bulk_store_wait_all();
+  }
 }
 
 // b_final = b + (b B) G for one map per block, every load of a pass in flight
@@ -546,9 +556,12 @@ hf_status launch_fold(int n_maps, int d_r, int64_t K, int rank, const void* W, c
                 "hf_fold: shared memory size");
     const int64_t units = n_maps * ((K + kMmaCols - 1) / kMmaCols);
     const int grid = static_cast<int>(std::min<int64_t>(units, device_sm_count()));
+    const int steps = (d_r + 16 * kMmaWarps - 1) / (16 * kMmaWarps);
+    CUtensorMap map_out;
+    s = bf16_strip_map(&map_out, Wf, n_maps, d_r, K, 16 * steps);
+    if (s != HF_OK) return s;
     fold_mma_kernel<<<grid, 32 * kMmaWarps, sizeof(FoldMmaSmem), stream>>>(
-        static_cast<const __nv_bfloat16*>(W), B, G, static_cast<__nv_bfloat16*>(Wf), n_maps, d_r, K,
-        rank, (d_r + 16 * kMmaWarps - 1) / (16 * kMmaWarps));
+        static_cast<const __nv_bfloat16*>(W), B, G, map_out, n_maps, d_r, K, rank, steps);
     HF_CUDA_TRY(cudaGetLastError(), "hf_fold: launch");
   } else
   switch (rank) {

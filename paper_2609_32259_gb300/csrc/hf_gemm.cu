@@ -515,6 +515,28 @@ size_t gemm_smem_bytes() {
 
 }  // namespace
 
+hf_status bf16_strip_map(CUtensorMap* map, const void* base, uint64_t n, uint64_t rows,
+                         uint64_t cols, uint32_t box_rows) {
+  EncodeTiledFn fn = gemm_encode_fn();
+  if (!fn) {
+    set_error("cuTensorMapEncodeTiled is not available from the driver");
+    return HF_ERR_CUDA;
+  }
+  const cuuint64_t dims[3] = {cols, rows, n};
+  const cuuint64_t strides[2] = {cols * 2, rows * cols * 2};
+  const cuuint32_t box[3] = {32, box_rows, 1};
+  const cuuint32_t estr[3] = {1, 1, 1};
+  const CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims,
+                        strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                        CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) {
+    set_error("cuTensorMapEncodeTiled failed (error " + std::to_string((int)r) + ")");
+    return HF_ERR_CUDA;
+  }
+  return HF_OK;
+}
+
 size_t gemm_planes_bytes(int64_t rows, int64_t K) {
   return static_cast<size_t>(3 * round_up(rows, kGTile) * round_up(K, 64) * 2);
 }

@@ -128,3 +128,24 @@ def test_fold_ragged_tile_and_bad_arguments():
     with pytest.raises(B.HFError) as e:
         B.fold("f32", Wm, b, Bm6, Gm6, Wf, bf)               # rank not a multiple of 4
     assert e.value.status == B.HF_ERR_UNSUPPORTED
+
+
+def test_fold_infinity_stays_in_its_column():
+    """Rows past d_R (1,000 of 1,024) are padding of the tensor-core form: what an
+    infinity makes of its column reaches no other column and no later unit."""
+    dev = torch.device("cuda")
+    n_maps, d_R, K, rank = 2, 1000, 160 * 152, 8
+    g = torch.Generator(device="cpu").manual_seed(9)
+    Wm = (torch.randn((n_maps, d_R, K), generator=g) / np.sqrt(K)).to(torch.bfloat16).to(dev)
+    b = torch.zeros((n_maps, d_R), device=dev)
+    Bm, Gm = _factors(n_maps, d_R, rank, 6, dev)
+    clean, bf = torch.empty_like(Wm), torch.empty_like(b)
+    B.fold("bf16", Wm, b, Bm, Gm, clean, bf)
+    cols = torch.arange(0, K, 160, device=dev)
+    Wm[:, 3, cols] = float("inf")
+    got = torch.empty_like(Wm)
+    B.fold("bf16", Wm, b, Bm, Gm, got, bf)
+    torch.cuda.synchronize()
+    assert not torch.isfinite(got[:, 3, cols]).any()
+    got[:, :, cols] = clean[:, :, cols]
+    assert torch.equal(got, clean)

@@ -10,7 +10,7 @@
 // instructions, with every fp32 factor split exactly into three bf16 parts and
 // the products above 2^-23 kept (a rank of 16 is one 16-deep step: too thin for
 // an accumulator in tensor memory; 80 maps of 1,024 x 3,072, rank 16, with the
-// bias: 0.27 ms, fold_kernel 0.49; the same error against 64 bits).  fold_kernel
+// bias: 0.25 ms, fold_kernel 0.49; the same error against 64 bits).  fold_kernel
 // takes the rest with plain fp32 arithmetic; a block reads its columns of W
 // twice (the second time from L2) and writes them once.
 #include <algorithm>
@@ -324,6 +324,7 @@ __global__ void __launch_bounds__(32 * kMmaWarps)
   const int g = lane >> 2, t = lane & 3;  // fragment row and column pair
   const int per_map = static_cast<int>((K + kMmaCols - 1) / kMmaCols);
   const int64_t units = static_cast<int64_t>(n_maps) * per_map;
+  depend_launch();  // the biases' kernel
   const int64_t u0 = units * blockIdx.x / gridDim.x, u1 = units * (blockIdx.x + 1) / gridDim.x;
   const int row0 = warp * 16 * steps, rows = min(16 * steps, d_r - row0);  // <= 0: padding only
   for (int i = lane; i < (16 * steps - max(rows, 0)) * kMmaCols; i += 32) {
@@ -464,7 +465,9 @@ __global__ void __launch_bounds__(32 * kMmaWarps)
 }
 
 // b_final = b + (b B) G for one map per block, every load of a pass in flight
-// at once (one rank column at a time took 17 us for 80 maps).
+// at once (one rank column at a time took 17 us for 80 maps).  It is launched
+// beside the end of the maps' kernel, whose CTAs leave it no room earlier
+// (with the gap between the launches 12 us of 266 at 80 maps).
 template <int R>
 __global__ void __launch_bounds__(256) fold_b_kernel(const float* b, const float* __restrict__ Bm,
                                                      const float* __restrict__ Gm, float* bf,
@@ -510,6 +513,7 @@ __global__ void __launch_bounds__(256) fold_b_kernel(const float* b, const float
     for (int r = 0; r < R; ++r) v = fmaf(bB[r], __ldg(G + static_cast<int64_t>(r) * d_r + n), v);
     bf[static_cast<int64_t>(map) * d_r + n] = v;
   }
+  depend_wait();  // the maps, which this kernel has nothing to do with, are done
 }
 
 template <typename T, int R>
@@ -574,13 +578,14 @@ hf_status launch_fold(int n_maps, int d_r, int64_t K, int rank, const void* W, c
       return HF_ERR_UNSUPPORTED;
   }
   if (s != HF_OK) return s;
-  switch (rank) {
-    case 4: fold_b_kernel<4><<<n_maps, 256, 0, stream>>>(b, B, G, bf, d_r); break;
-    case 8: fold_b_kernel<8><<<n_maps, 256, 0, stream>>>(b, B, G, bf, d_r); break;
-    case 16: fold_b_kernel<16><<<n_maps, 256, 0, stream>>>(b, B, G, bf, d_r); break;
-    default: fold_b_kernel<32><<<n_maps, 256, 0, stream>>>(b, B, G, bf, d_r); break;
-  }
-  HF_CUDA_TRY(cudaGetLastError(), "hf_fold: bias launch");
+  auto bias = [&](auto kern) {
+    return launch_dependent(kern, dim3(n_maps), dim3(256), 0, stream, b, B, G, bf, d_r);
+  };
+  HF_CUDA_TRY(rank == 4    ? bias(fold_b_kernel<4>)
+              : rank == 8  ? bias(fold_b_kernel<8>)
+              : rank == 16 ? bias(fold_b_kernel<16>)
+                           : bias(fold_b_kernel<32>),
+              "hf_fold: bias launch");
   return HF_OK;
 }
 

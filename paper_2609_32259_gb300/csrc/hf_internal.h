@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <mutex>
 #include <string>
 
 #include "heterofold.h"
@@ -109,8 +110,8 @@ static_assert(sizeof(SegTables) < 32000, "SegTables must fit the kernel paramete
 struct hf_plan_s {
   hf_plan_desc desc;  // host-array fields are cleared after copying
   int d_s, d_r, K, n_seg;
-  int64_t T_s, T_r, nnz_hint;
-  int BN, groups, stages;
+  int64_t T_s, T_r;
+  int BN;
   bool gather;  // every map input row is a single unweighted sender row
   bool split;   // computed bf16 operand rows go to the tensor core as value + residual
   bool staged;  // split rows of one entry each: raw sender atoms staged by cp.async
@@ -131,6 +132,10 @@ struct hf_plan_s {
   int made;
   int64_t x_rows;
   int x_layers;
+  // The made rows are the plan's, not the call's: a transfer on another stream
+  // takes them after x_done, the end of the transfer before it.
+  std::mutex x_mutex;
+  cudaEvent_t x_done = nullptr;
   int64_t s_rows;  // sender-cache rows per (layer, role)
   char* ws;
   size_t ws_bytes;

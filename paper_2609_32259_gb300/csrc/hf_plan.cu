@@ -845,7 +845,6 @@ hf_status plan_build(const hf_plan_desc* desc, void* d_workspace, size_t workspa
   p->s_rows = desc->sender_rows > 0 ? desc->sender_rows : p->T_s;
   p->T_r = desc->r_tok_ptr[desc->n_req];
   p->BN = (p->d_r % 256 == 0) ? 256 : 128;
-  p->groups = ((p->BN / 2) % desc->D_r == 0) ? 2 : 1;
   const OperandPath path = operand_path(*desc);
   p->unrot = desc->sender_k_rotated == 1;
   p->rope = desc->theta_r > 0.0 || desc->h_inv_freq_r != nullptr;
@@ -949,6 +948,7 @@ extern "C" hf_status hf_plan_destroy(hf_plan plan) {
     delete[] plan->events;
     cudaSetDevice(cur);
   }
+  if (plan && plan->x_done) cudaEventDestroy(plan->x_done);
   delete plan;
   return HF_OK;
 }

@@ -1935,11 +1935,9 @@ hf_status launch_batch_typed(const BatchParams& B, int64_t max_pair_tiles, size_
 
 }  // namespace
 
-hf_status launch_transfer(hf_plan_s* p, const void* sender, void* receiver, cudaStream_t stream,
-                          int l_begin, int l_end, bool stall) {
+static hf_status transfer_layers(hf_plan_s* p, const void* sender, void* receiver,
+                                 cudaStream_t stream, int l_begin, int l_end, bool stall) {
   const hf_plan_desc& d = p->desc;
-  if (l_end < 0) l_end = d.L_r;
-  if (p->T_r == 0 || l_end <= l_begin) return HF_OK;
   if (p->made) {
     // the operand rows of at most as many receiver layers as their buffer holds,
     // then these layers' transfer; groups of like size, as the last round of a
@@ -1950,7 +1948,7 @@ hf_status launch_transfer(hf_plan_s* p, const void* sender, void* receiver, cuda
       const int per = (n + groups - 1) / groups;
       for (int l = l_begin; l < l_end; l += per) {
         const hf_status e =
-            launch_transfer(p, sender, receiver, stream, l, std::min(l_end, l + per), stall);
+            transfer_layers(p, sender, receiver, stream, l, std::min(l_end, l + per), stall);
         if (e != HF_OK) return e;
       }
       return HF_OK;
@@ -1978,6 +1976,31 @@ hf_status launch_transfer(hf_plan_s* p, const void* sender, void* receiver, cuda
   if (p->pam)
     return p->gather ? go(transfer_kernel<Bf, kCopiedRows, 1>) : go(transfer_kernel<Bf, kBuiltRows, 1>);
   return p->gather ? go(transfer_kernel<Bf, kCopiedRows, 0>) : go(transfer_kernel<Bf, kBuiltRows, 0>);
+}
+
+hf_status launch_transfer(hf_plan_s* p, const void* sender, void* receiver, cudaStream_t stream,
+                          int l_begin, int l_end, bool stall) {
+  if (l_end < 0) l_end = p->desc.L_r;
+  if (p->T_r == 0 || l_end <= l_begin) return HF_OK;
+  if (!p->made) return transfer_layers(p, sender, receiver, stream, l_begin, l_end, stall);
+  // a graph's replays are ordered by its owner: a capture cannot wait for what
+  // lies outside of it
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) {
+    cudaGetLastError();  // the legacy stream beside another thread's capture
+    cap = cudaStreamCaptureStatusActive;
+  }
+  std::lock_guard<std::mutex> lock(p->x_mutex);
+  if (cap != cudaStreamCaptureStatusNone)
+    return transfer_layers(p, sender, receiver, stream, l_begin, l_end, stall);
+  if (p->x_done)
+    HF_CUDA_TRY(cudaStreamWaitEvent(stream, p->x_done, 0), "wait for the plan's operand rows");
+  else
+    HF_CUDA_TRY(cudaEventCreateWithFlags(&p->x_done, cudaEventDisableTiming), "operand rows' event");
+  const hf_status s = transfer_layers(p, sender, receiver, stream, l_begin, l_end, stall);
+  if (s != HF_OK) return s;
+  HF_CUDA_TRY(cudaEventRecord(p->x_done, stream), "record the operand rows' event");
+  return HF_OK;
 }
 
 bool batch_compatible(const hf_plan_s* const* plans, int n) {

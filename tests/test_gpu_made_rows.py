@@ -81,3 +81,29 @@ def test_made_rows_equal_built_rows(name):
     assert job.device_status() == 0
     assert torch.equal(made, job.receiver)
     job.close()
+
+
+def test_made_rows_on_two_streams():
+    """The made rows lie in the plan's workspace: transfers of two caches with one
+    plan on two streams must not take each other's."""
+    w = L(3000, sender_k_rotated=True)
+    dev = torch.device("cuda")
+    tok = W.tokens(w)
+    sender = W.sender_kv(w, tok.T_s, dev)
+    other = sender.flip(2).contiguous()
+    Wm, b, r = W.maps(w, dev)
+    job = pipeline.job_from_workload(w, tok, sender, Wm, b, r, r_pos0=W.r_pos0(w), device=dev)
+    job.step()
+    senders, outs = [sender, other], [torch.empty_like(job.receiver) for _ in range(2)]
+    want = [torch.empty_like(job.receiver) for _ in range(2)]
+    for s, o in zip(senders, want):
+        B.transfer(job.plan, s, o)
+        torch.cuda.synchronize()
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    for _ in range(20):
+        for s, o, st in zip(senders, outs, streams):
+            B.transfer(job.plan, s, o, st)
+    torch.cuda.synchronize()
+    assert job.device_status() == 0
+    assert torch.equal(outs[0], want[0]) and torch.equal(outs[1], want[1])
+    job.close()

@@ -204,13 +204,14 @@ __global__ void overlap_fill_kernel(ReqPtrs rq, const int32_t* __restrict__ s_en
 // per thread (a further search starts where the one before ended),
 // the scan over the block and, through distributed shared memory, over the
 // cluster's CTAs; sender tokens are checked along the way.  Status bits are
-// gathered the same way, so nothing is cleared beforehand.
+// gathered the same way, so nothing is cleared beforehand.  The offsets are read
+// by ordinary loads (no __restrict__): see ld_dep.
 template <bool kOverlap, int kR>
 __global__ void __launch_bounds__(1024)
-    align_fused_kernel(const __grid_constant__ FewPtrs rq, const int32_t* __restrict__ s_end,
-                       const int32_t* __restrict__ r_end, int64_t T_s, int64_t T_r,
-                       int32_t* __restrict__ row_ptr, int32_t* __restrict__ col,
-                       float* __restrict__ w, int64_t capacity, int32_t* info) {
+    align_fused_kernel(const __grid_constant__ FewPtrs rq, const int32_t* s_end,
+                       const int32_t* r_end, int64_t T_s, int64_t T_r,
+                       int32_t* row_ptr, int32_t* col,
+                       float* w, int64_t capacity, int32_t* info) {
   __shared__ int32_t sp[kFusedReq + 1], rp[kFusedReq + 1];
   __shared__ int scan_buf[32], cta_total, cta_bits;
   const uint32_t rank = cluster_ctarank(), ctas = cluster_nctarank();

@@ -111,6 +111,14 @@ __device__ __forceinline__ void depend_wait() {
 __device__ __forceinline__ void depend_launch() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
+// A read in a kernel so launched.  It is an ordinary load, which stays below
+// depend_wait: __ldg (and const __restrict__) promises memory that nothing
+// writes while the kernel runs, which does not hold for what the kernel before
+// it may still be writing, and lets the compiler move the load above the wait.
+template <typename T>
+__device__ __forceinline__ T ld_dep(const T* p) {
+  return *p;
+}
 
 // ---------------------------------------------------------------------------
 // Thread-block clusters (a CTA pair sharing one tcgen05 MMA)

@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(kPanelThreads)
   }
 #pragma unroll
   for (int i = 0; i < kTVecs; ++i)
-    tin[i] = __ldg(reinterpret_cast<const float4*>(Tt) + tid + i * kPanelThreads);
+    tin[i] = ld_dep(reinterpret_cast<const float4*>(Tt) + tid + i * kPanelThreads);
 #pragma unroll
   for (int i = 0; i < kSVecs; ++i) {
     const int e = tid + i * kPanelThreads, k = e / (kPanelCols / 4), q = e % (kPanelCols / 4);

@@ -209,7 +209,7 @@ __device__ __forceinline__ void raise_timeout(const XferParams& P, volatile int*
 // last token past the end; those rows are never pooled).
 __device__ __forceinline__ int pam_token(const XferParams& P, int m, int row0, int r) {
   const int w = (m * kPairRows + row0) >> 7;
-  const int64_t k = static_cast<int64_t>(w) * __ldg(P.win_info + 1) + r;
+  const int64_t k = static_cast<int64_t>(w) * ld_dep(P.win_info + 1) + r;
   return static_cast<int>(k < P.T_s ? k : P.T_s - 1);
 }
 
@@ -286,15 +286,15 @@ __device__ __forceinline__ void walk_rows(int jb, int je, int u0, const float* s
   int expect = INT_MIN;   // position for which cs/sn are valid
   float2 cs[2] = {make_float2(1.f, 1.f), make_float2(1.f, 1.f)};
   float2 sn[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-  int unext = __ldg(P.uidx + jb);  // number of row j's distinct row, one-based, read a row ahead
-  int dnext = P.paged ? __ldg(P.dst_row + jb) : jb;  // destination of row j, read a row ahead
+  int unext = ld_dep(P.uidx + jb);  // number of row j's distinct row, one-based, read a row ahead
+  int dnext = P.paged ? ld_dep(P.dst_row + jb) : jb;  // destination of row j, read a row ahead
   T* const out = out_lc + ocol + q + 4 * qq;
 #pragma unroll 1
   for (int j = jb; j < je; ++j) {
     const int drow = dnext, uj = unext - 1 - u0;
     const int jn = min(j + 1, je - 1);
-    unext = __ldg(P.uidx + jn);
-    dnext = P.paged ? __ldg(P.dst_row + jn) : jn;
+    unext = ld_dep(P.uidx + jn);
+    dnext = P.paged ? ld_dep(P.dst_row + jn) : jn;
     if (uj != u) {  // first row, or the first row of a later run
       u = uj;
       pb = __float_as_int(stg[u * kStgRow + kPadPos]);
@@ -395,7 +395,7 @@ __device__ __forceinline__ void copy_epilogue(const XferParams& P, uint32_t ta,
         float y[32];
 #pragma unroll
         for (int i = 0; i < 32; i += 4) {
-          const float4 bb = __ldg(reinterpret_cast<const float4*>(bias_tile + col + i));
+          const float4 bb = ld_dep(reinterpret_cast<const float4*>(bias_tile + col + i));
           y[i] = fmaf(__uint_as_float(v[i]), inv_r, bb.x);
           y[i + 1] = fmaf(__uint_as_float(v[i + 1]), inv_r, bb.y);
           y[i + 2] = fmaf(__uint_as_float(v[i + 2]), inv_r, bb.z);
@@ -413,8 +413,8 @@ __device__ __forceinline__ void copy_epilogue(const XferParams& P, uint32_t ta,
     const uint32_t src = smem_addr(stg);
     T* const out = out_lc + ocol0 + pc0;
     for (int j = jb + tid_e; j < je; j += kEpiThreads) {
-      const int u = __ldg(P.uidx + j) - 1 - u0;
-      const int drow = P.paged ? __ldg(P.dst_row + j) : j;
+      const int u = ld_dep(P.uidx + j) - 1 - u0;
+      const int drow = P.paged ? ld_dep(P.dst_row + j) : j;
       if (drow >= 0)
         bulk_store(out + static_cast<int64_t>(drow) * P.d_r,
                    src + static_cast<uint32_t>(u) * (kStgRow * 4), 256u, policy);
@@ -440,15 +440,15 @@ __device__ __forceinline__ void pam_walk(int jb, int je, int base, const float* 
   if (jb >= je) return;
   int expect = INT_MIN;  // position for which cs/sn are valid
   float cs[4] = {1.f, 1.f, 1.f, 1.f}, sn[4] = {0.f, 0.f, 0.f, 0.f};
-  int e1 = __ldg(P.row_ptr + jb);
+  int e1 = ld_dep(P.row_ptr + jb);
   for (int j = jb; j < je; ++j) {
     const int e0 = e1;
-    e1 = __ldg(P.row_ptr + j + 1);
+    e1 = ld_dep(P.row_ptr + j + 1);
     float4 x0 = make_float4(0.f, 0.f, 0.f, 0.f), y0 = x0, x1 = x0, y1 = x0;
     for (int e = e0; e < e1; ++e) {
-      const int loc = __ldg(P.col + e) - base;
+      const int loc = ld_dep(P.col + e) - base;
       if (loc < 0 || loc >= kBM) continue;  // flagged at plan creation
-      const float wt = __ldg(P.w + e);
+      const float wt = ld_dep(P.w + e);
       const float* urow = stg + loc * kStgRow + 4 * qq;
       const float4 a = *reinterpret_cast<const float4*>(urow);
       const float4 b = *reinterpret_cast<const float4*>(urow + 16);
@@ -470,7 +470,7 @@ __device__ __forceinline__ void pam_walk(int jb, int je, int base, const float* 
     x1 = make_float4(x1.x + bias4[2].x, x1.y + bias4[2].y, x1.z + bias4[2].z, x1.w + bias4[2].w);
     y1 = make_float4(y1.x + bias4[3].x, y1.y + bias4[3].y, y1.z + bias4[3].z, y1.w + bias4[3].w);
     if (do_rope) {
-      const int p = __ldg(P.pos + j);
+      const int p = ld_dep(P.pos + j);
       if (p != expect || ((j - jb) & 15) == 0) {
 #pragma unroll
         for (int k = 0; k < 4; ++k) rope_sincos(p, f[k], &sn[k], &cs[k]);
@@ -486,7 +486,7 @@ __device__ __forceinline__ void pam_walk(int jb, int je, int base, const float* 
       rotate4(x0, y0, cs, sn);
       if (two_heads) rotate4(x1, y1, cs, sn);
     }
-    const int drow = P.paged ? __ldg(P.dst_row + j) : j;
+    const int drow = P.paged ? ld_dep(P.dst_row + j) : j;
     if (drow >= 0) {
       T* o = out_lc + static_cast<int64_t>(drow) * P.d_r + ocol + q + 4 * qq;
       store4(o, x0);
@@ -525,7 +525,7 @@ __device__ __forceinline__ void pam_epilogue(const XferParams& P, uint32_t ta,
     for (int q = 0; q < half; q += 16) {
       float f[4];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) f[k] = do_rope ? __ldg(P.inv_freq + q + 4 * qq + k) : 0.f;
+      for (int k = 0; k < 4; ++k) f[k] = do_rope ? ld_dep(P.inv_freq + q + 4 * qq + k) : 0.f;
       if (stages_head) {
         uint32_t v[32];
         tmem_load_2x16(ta + tcol + q, ta + tcol + half + q, v);
@@ -539,10 +539,10 @@ __device__ __forceinline__ void pam_epilogue(const XferParams& P, uint32_t ta,
       named_barrier_sync(1, kEpiThreads);
       const float* bb = bias_tile + 2 * hp * D + q + 4 * qq;
       float4 bias4[4];
-      bias4[0] = __ldg(reinterpret_cast<const float4*>(bb));
-      bias4[1] = __ldg(reinterpret_cast<const float4*>(bb + half));
-      bias4[2] = two_heads ? __ldg(reinterpret_cast<const float4*>(bb + D)) : make_float4(0.f, 0.f, 0.f, 0.f);
-      bias4[3] = two_heads ? __ldg(reinterpret_cast<const float4*>(bb + D + half)) : make_float4(0.f, 0.f, 0.f, 0.f);
+      bias4[0] = ld_dep(reinterpret_cast<const float4*>(bb));
+      bias4[1] = ld_dep(reinterpret_cast<const float4*>(bb + half));
+      bias4[2] = two_heads ? ld_dep(reinterpret_cast<const float4*>(bb + D)) : make_float4(0.f, 0.f, 0.f, 0.f);
+      bias4[3] = two_heads ? ld_dep(reinterpret_cast<const float4*>(bb + D + half)) : make_float4(0.f, 0.f, 0.f, 0.f);
       float C1[4], S1[4];
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
@@ -583,11 +583,11 @@ __device__ __forceinline__ void build_atom(const XferParams& P, const LayerSegs&
       const int k = tok >= 0 ? tok : P.col[e0 + ie];
       if (k < 0 || k >= P.T_s) continue;  // flagged at plan creation
       const float wt = tok >= 0 ? om : om * P.w[e0 + ie];
-      const int64_t kr = P.srow ? __ldg(P.srow + k) : k;
+      const int64_t kr = P.srow ? ld_dep(P.srow + k) : k;
       const uint4* src = reinterpret_cast<const uint4*>(base + kr * P.d_s);
       uint4 x[8];
 #pragma unroll
-      for (int k2 = 0; k2 < 8; ++k2) x[k2] = __ldg(src + k2);
+      for (int k2 = 0; k2 < 8; ++k2) x[k2] = ld_dep(src + k2);
 #pragma unroll
       for (int k2 = 0; k2 < 8; ++k2) accum16(x[k2], wt, acc + k2 * kPerChunk, (const T*)nullptr);
     }
@@ -621,7 +621,7 @@ __device__ __forceinline__ void build_atom_unrotated(const XferParams& P, const 
     float f[kPerChunk], acc[kPerChunk];
 #pragma unroll
     for (int q = 0; q < kPerChunk; ++q) {
-      f[q] = __ldg(P.inv_freq_s + fi + q);
+      f[q] = ld_dep(P.inv_freq_s + fi + q);
       acc[q] = 0.f;
     }
     for (int ti = 0; ti < segs.n_terms[seg]; ++ti) {
@@ -632,14 +632,14 @@ __device__ __forceinline__ void build_atom_unrotated(const XferParams& P, const 
         const int k = P.col[e];
         if (k < 0 || k >= P.T_s) continue;  // flagged at plan creation
         const float wt = om * P.w[e];
-        const int64_t kr = P.srow ? __ldg(P.srow + k) : k;
+        const int64_t kr = P.srow ? ld_dep(P.srow + k) : k;
         const T* row = base + kr * P.d_s;
         float x[kPerChunk], y[kPerChunk];
 #pragma unroll
         for (int q = 0; q < kPerChunk; ++q) x[q] = y[q] = 0.f;
-        accum16(__ldg(reinterpret_cast<const uint4*>(row + el)), 1.f, x, (const T*)nullptr);
-        accum16(__ldg(reinterpret_cast<const uint4*>(row + partner)), 1.f, y, (const T*)nullptr);
-        const int p = __ldg(P.spos + k);
+        accum16(ld_dep(reinterpret_cast<const uint4*>(row + el)), 1.f, x, (const T*)nullptr);
+        accum16(ld_dep(reinterpret_cast<const uint4*>(row + partner)), 1.f, y, (const T*)nullptr);
+        const int p = ld_dep(P.spos + k);
 #pragma unroll
         for (int q = 0; q < kPerChunk; ++q) {
           float sn, cs;
@@ -674,7 +674,7 @@ __device__ __forceinline__ void build_stage_unrotated(const XferParams& P, const
     float f[kPerChunk], ax[kPerChunk], ay[kPerChunk];
 #pragma unroll
     for (int i = 0; i < kPerChunk; ++i) {
-      f[i] = __ldg(P.inv_freq_s + i0 + i);
+      f[i] = ld_dep(P.inv_freq_s + i0 + i);
       ax[i] = 0.f;
       ay[i] = 0.f;
     }
@@ -686,14 +686,14 @@ __device__ __forceinline__ void build_stage_unrotated(const XferParams& P, const
         const int k = P.col[e];
         if (k < 0 || k >= P.T_s) continue;  // flagged at plan creation
         const float wt = om * P.w[e];
-        const int64_t kr = P.srow ? __ldg(P.srow + k) : k;
+        const int64_t kr = P.srow ? ld_dep(P.srow + k) : k;
         const T* row = base + kr * P.d_s;
         float x[kPerChunk], y[kPerChunk];
 #pragma unroll
         for (int i = 0; i < kPerChunk; ++i) x[i] = y[i] = 0.f;
-        accum16(__ldg(reinterpret_cast<const uint4*>(row + ex)), 1.f, x, (const T*)nullptr);
-        accum16(__ldg(reinterpret_cast<const uint4*>(row + ey)), 1.f, y, (const T*)nullptr);
-        const int p = __ldg(P.spos + k);
+        accum16(ld_dep(reinterpret_cast<const uint4*>(row + ex)), 1.f, x, (const T*)nullptr);
+        accum16(ld_dep(reinterpret_cast<const uint4*>(row + ey)), 1.f, y, (const T*)nullptr);
+        const int p = ld_dep(P.spos + k);
 #pragma unroll
         for (int i = 0; i < kPerChunk; ++i) {
           float sn, cs;
@@ -727,7 +727,7 @@ template <int kDirs, int kPam, int kTileRows>
 __device__ __forceinline__ int build_dirs(const XferParams* Ps, int n_dir, DirTable<kDirs>* dt) {
   int total = 0;
   for (int d = 0; d < (kDirs == 1 ? 1 : n_dir); ++d) {
-    const int U = pam_on<kPam>(Ps[d]) ? 128 * __ldg(Ps[d].win_info + 2) : *Ps[d].n_distinct;
+    const int U = pam_on<kPam>(Ps[d]) ? 128 * ld_dep(Ps[d].win_info + 2) : *Ps[d].n_distinct;
     const int mt = (U + kTileRows - 1) / kTileRows;
     dt->U[d] = U;
     dt->m_tiles[d] = mt;
@@ -797,9 +797,9 @@ __device__ __forceinline__ void gather_rows(const XferParams* Ps, const DirTable
     // segment's is in sbase and the next one's is loaded a segment ahead
     const KLoop kl = k_loop<kRows>(P, c);
     const LayerSegs* lsegs = P.segs + l;
-    const int n_seg = __ldg(&lsegs->n_seg);
+    const int n_seg = ld_dep(&lsegs->n_seg);
     auto seg_row = [&](int s2) -> int64_t {
-      return static_cast<int64_t>(__ldg(&lsegs->layer[s2][0]) * 2 + c) * P.s_rows;
+      return static_cast<int64_t>(ld_dep(&lsegs->layer[s2][0]) * 2 + c) * P.s_rows;
     };
     auto seg_base = [&](int s2) -> int64_t { return seg_row(s2) * P.d_s; };
     int64_t sbase = 0, snext = 0;
@@ -820,7 +820,7 @@ __device__ __forceinline__ void gather_rows(const XferParams* Ps, const DirTable
     if (bulk) {
       int64_t k0;
       if (pam_on<kPam>(P)) {
-        k0 = static_cast<int64_t>((m * kTileRows + row0) >> 7) * __ldg(P.win_info + 1) + slab * 32;
+        k0 = static_cast<int64_t>((m * kTileRows + row0) >> 7) * ld_dep(P.win_info + 1) + slab * 32;
         any_row = k0 < P.T_s;
       } else {
         k0 = static_cast<int64_t>(m) * kTileRows + row0 + slab * 32;
@@ -845,7 +845,7 @@ __device__ __forceinline__ void gather_rows(const XferParams* Ps, const DirTable
       int64_t kr;  // sender-cache row
       if (pam_on<kPam>(P)) {
         const int k = pam_token(P, m, row0, r);
-        kr = P.srow && !kl.made ? __ldg(P.srow + k) : k;
+        kr = P.srow && !kl.made ? ld_dep(P.srow + k) : k;
         live |= 1u << i;
       } else {
         const int u = m * kTileRows + row0 + r;
@@ -969,11 +969,11 @@ __device__ __forceinline__ void finish_staged_row(const XferParams& P, const Lay
   const T* sender = reinterpret_cast<const T*>(P.sender);
   uint8_t* slot1 = slot0 + kAtomABytes;
   const int seg = kb / P.atoms_per_seg, kin = kb - seg * P.atoms_per_seg;
-  const int n_t = __ldg(&lsegs->n_terms[seg]);
-  const int la0 = __ldg(&lsegs->layer[seg][0]);
-  const int la1 = n_t > 1 ? __ldg(&lsegs->layer[seg][1]) : la0;
-  const float om0 = __ldg(&lsegs->w[seg][0]);
-  const float om1 = n_t > 1 ? __ldg(&lsegs->w[seg][1]) : 0.f;
+  const int n_t = ld_dep(&lsegs->n_terms[seg]);
+  const int la0 = ld_dep(&lsegs->layer[seg][0]);
+  const int la1 = n_t > 1 ? ld_dep(&lsegs->layer[seg][1]) : la0;
+  const float om0 = ld_dep(&lsegs->w[seg][0]);
+  const float om1 = n_t > 1 ? ld_dep(&lsegs->w[seg][1]) : 0.f;
   const int64_t lrows = P.s_rows * P.d_s;
   const int frow = r.frow, sw = frow & 7;
   const bool one = r.tok >= 0;
@@ -1007,7 +1007,7 @@ __device__ __forceinline__ void finish_staged_row(const XferParams& P, const Lay
     for (int e = e_first; e < e_end; ++e) {
       const int k = P.col[e];
       if (k < 0 || k >= P.T_s) continue;  // flagged at plan creation
-      const int64_t kr = P.srow ? __ldg(P.srow + k) : k;
+      const int64_t kr = P.srow ? ld_dep(P.srow + k) : k;
       for (int ti = 0; ti < n_t; ++ti) {
         const int la = ti == 0 ? la0 : la1;
         const float wt = (ti == 0 ? om0 : om1) * P.w[e];
@@ -1016,7 +1016,7 @@ __device__ __forceinline__ void finish_staged_row(const XferParams& P, const Lay
                                kin * kBK) + 4 * h;
         uint4 x[4];
 #pragma unroll
-        for (int k2 = 0; k2 < 4; ++k2) x[k2] = __ldg(src + k2);
+        for (int k2 = 0; k2 < 4; ++k2) x[k2] = ld_dep(src + k2);
 #pragma unroll
         for (int k2 = 0; k2 < 4; ++k2) accum16(x[k2], wt, acc + k2 * kPerChunk, (const T*)nullptr);
       }
@@ -1068,8 +1068,8 @@ __device__ __forceinline__ void build_rows_staged(const XferParams* Ps, const Di
       }
       if (k0 >= P.T_s) k0 = -1;  // flagged at plan creation
       if (k1 >= P.T_s) k1 = -1;
-      kr0[i] = k0 < 0 ? -1 : (P.srow ? __ldg(P.srow + k0) : k0);
-      kr1[i] = k1 < 0 ? -1 : (P.srow ? __ldg(P.srow + k1) : k1);
+      kr0[i] = k0 < 0 ? -1 : (P.srow ? ld_dep(P.srow + k0) : k0);
+      kr1[i] = k1 < 0 ? -1 : (P.srow ? ld_dep(P.srow + k1) : k1);
     }
     StagedRow fr;
     fr.frow = slab * 32 + lane;
@@ -1092,9 +1092,9 @@ __device__ __forceinline__ void build_rows_staged(const XferParams* Ps, const Di
         break;
       }
       const int seg = kb / P.atoms_per_seg, kin = kb - seg * P.atoms_per_seg;
-      const int n_t = __ldg(&lsegs->n_terms[seg]);
-      const int la0 = __ldg(&lsegs->layer[seg][0]);
-      const int la1 = n_t > 1 ? __ldg(&lsegs->layer[seg][1]) : la0;
+      const int n_t = ld_dep(&lsegs->n_terms[seg]);
+      const int la0 = ld_dep(&lsegs->layer[seg][0]);
+      const int la1 = n_t > 1 ? ld_dep(&lsegs->layer[seg][1]) : la0;
       const T* b0 = sender + static_cast<int64_t>(la0 * 2 + c) * lrows + kin * kBK + ch * kPerChunk;
       const T* b1 = sender + static_cast<int64_t>(la1 * 2 + c) * lrows + kin * kBK + ch * kPerChunk;
       const uint32_t sa = smem_addr(sA + stage * kStageABytes);
@@ -1450,8 +1450,8 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const CUt
       const int nrows = min(kBM, U - u0);  // <= 0: this CTA has no rows in the tile
       if (nrows > 0 && pam_on<kPam>(P)) {
         const int w = u0 >> 7;  // this CTA's window
-        const int base = w * __ldg(P.win_info + 1);
-        const int jb = __ldg(P.win_ptr + w), je = __ldg(P.win_ptr + w + 1);
+        const int base = w * ld_dep(P.win_info + 1);
+        const int jb = ld_dep(P.win_ptr + w), je = ld_dep(P.win_ptr + w + 1);
         T* const out_lc = reinterpret_cast<T*>(P.receiver) +
                           (static_cast<int64_t>(lc) * P.recv_rows) * P.d_r;
         pam_epilogue<T>(P,
@@ -1462,17 +1462,17 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const CUt
       } else if (nrows > 0) {
         for (int i = tid_e; i < nrows; i += kEpiThreads)
           sStg[i * kStgRow + kPadPos] =
-              __int_as_float(__ldg(P.upos + u0 + i) - __ldg(P.run_ptr + u0 + i));
+              __int_as_float(ld_dep(P.upos + u0 + i) - ld_dep(P.run_ptr + u0 + i));
         if (dd != rot_dir) {
           rot_dir = dd;
           if (P.rope)
             for (int i = tid_e; i < half; i += kEpiThreads)
-              rope_sincos(1, __ldg(P.inv_freq + i), &sStg[i * kStgRow + kPadRot + 1],
+              rope_sincos(1, ld_dep(P.inv_freq + i), &sStg[i * kStgRow + kPadRot + 1],
                           &sStg[i * kStgRow + kPadRot]);
         }
         // this warp's receiver rows [wjb, wje); lane slot ps walks the
         // consecutive rows [ljb, lje) of them
-        const int jb = __ldg(P.run_ptr + u0), je = __ldg(P.run_ptr + u0 + nrows);
+        const int jb = ld_dep(P.run_ptr + u0), je = ld_dep(P.run_ptr + u0 + nrows);
         const int per = (je - jb + kEpiWarps - 1) / kEpiWarps;
         const int wjb = min(je, jb + e * per), wje = min(je, wjb + per);
         const int per_slot = (wje - wjb + 7) >> 3;
@@ -1509,7 +1509,7 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const CUt
 #pragma unroll
               for (int i = 0; i < 16; ++i) {
                 const float y = fmaf(__uint_as_float(v[i]), inv_r,
-                                     __ldg(bias + nb * P.BN + tcol + q2 + i));
+                                     ld_dep(bias + nb * P.BN + tcol + q2 + i));
                 ss = fmaf(y, y, ss);
               }
             }
@@ -1520,7 +1520,7 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const CUt
             // global read overlaps the staging
             float f[4];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) f[k] = do_rope ? __ldg(P.inv_freq + q + 4 * qq + k) : 0.f;
+            for (int k = 0; k < 4; ++k) f[k] = do_rope ? ld_dep(P.inv_freq + q + 4 * qq + k) : 0.f;
             if (stages_head) {
               // step 1: pairs q..q+15 of head 2*hp+g for this warp's 32 rows
               uint32_t v[32];
@@ -1529,8 +1529,8 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const CUt
               float y[32];
 #pragma unroll
               for (int i = 0; i < 16; i += 4) {
-                const float4 x = __ldg(reinterpret_cast<const float4*>(bcol + q + i));
-                const float4 z = __ldg(reinterpret_cast<const float4*>(bcol + half + q + i));
+                const float4 x = ld_dep(reinterpret_cast<const float4*>(bcol + q + i));
+                const float4 z = ld_dep(reinterpret_cast<const float4*>(bcol + half + q + i));
                 y[i] = fmaf(__uint_as_float(v[i]), inv_r, x.x);
                 y[i + 1] = fmaf(__uint_as_float(v[i + 1]), inv_r, x.y);
                 y[i + 2] = fmaf(__uint_as_float(v[i + 2]), inv_r, x.z);
@@ -1543,8 +1543,8 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const CUt
               if (do_knorm) {
 #pragma unroll
                 for (int i = 0; i < 16; ++i) {
-                  y[i] *= rn * __ldg(P.knorm_w + q + i);
-                  y[16 + i] *= rn * __ldg(P.knorm_w + half + q + i);
+                  y[i] *= rn * ld_dep(P.knorm_w + q + i);
+                  y[16 + i] *= rn * ld_dep(P.knorm_w + half + q + i);
                 }
               }
               float* srow = sStg + row * kStgRow + g * 32;

@@ -124,6 +124,33 @@ def test_recolor_statistics_of_many_samples():
     assert abs(r - r_ref) <= 128 * 2.0**-24 * r_ref
 
 
+# Ridges from just above the smallest accepted pivot (1e-4 of the mean eigenvalue)
+# on a spectrum of five decades, so that the pivots come down to the ridge.
+@pytest.mark.parametrize("reg", [1.2e-4, 3e-4, 1e-3])
+def test_recolor_factors_small_ridges(reg):
+    g = torch.Generator(device="cpu").manual_seed(8)
+    N, d_s, d_r = 4096, 384, 256
+    Q = torch.linalg.qr(torch.randn((d_s, d_s), generator=g, dtype=torch.float64))[0]
+    X = torch.randn((N, d_s), generator=g, dtype=torch.float64) * torch.logspace(
+        0, -2.5, d_s, dtype=torch.float64)
+    X = X @ Q
+    Y = X / X.std() @ (torch.randn((d_s, d_r), generator=g, dtype=torch.float64) / d_s ** 0.5)
+    Y = Y + 0.5 * torch.randn((N, d_r), generator=g, dtype=torch.float64)
+    X, Y = X.float(), Y.float()
+    w = torch.rand((N,), generator=g) + 0.5
+    ws = torch.empty(B.recolor_workspace_size(N, d_s, d_r), dtype=torch.uint8, device="cuda")
+    W_out = torch.empty((d_r, d_s), device="cuda")
+    b_out = torch.empty((d_r,), device="cuda")
+    _, its = B.recolor_fit("f32", X.cuda(), Y.cuda(), w.cuda(), W_out, b_out, ws, reg=reg,
+                           return_iters=True)
+    assert its[0] == 1 and its[1] == 1, its
+    A_ref, b_ref, _ = O.recolor(*(t.double().numpy() for t in (X, Y, w)), reg=reg)
+    # relative error about the condition number (largest eigenvalue, 12 mean
+    # ones, over the ridge) times 2^-24
+    rel = np.linalg.norm(W_out.double().cpu().numpy().T - A_ref) / np.linalg.norm(A_ref)
+    assert rel <= 12 / reg * 2.0**-24, rel
+
+
 def test_recolor_rejects_bad_shapes():
     with pytest.raises(B.HFError):
         B.recolor_workspace_size(100, 64, 128)   # d_S < d_R

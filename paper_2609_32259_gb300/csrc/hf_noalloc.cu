@@ -56,7 +56,9 @@ extern "C" hf_status hf_transfer_noalloc(const hf_plan_desc* desc, const void* s
   size_t need = 0;
   hf_status s = hf_plan_workspace_size(desc, &need);
   if (s != HF_OK) return s;
-  need = workspace_layout(*desc).total;  // without room for made operand rows
+  // Without room for made operand rows: those are ordered by an event of the
+  // plan, which a plan on the stack has nobody to free.
+  need = workspace_layout(*desc).total;
   if (need > kNoAllocScratchBytes) {
     set_error("hf_transfer_noalloc: this transfer needs " + std::to_string(need) +
               " bytes of metadata but the built-in scratch holds " +
@@ -82,7 +84,7 @@ extern "C" hf_status hf_transfer_noalloc(const hf_plan_desc* desc, const void* s
   hf_plan_s plan{};
   PlanTables tables;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  s = plan_build(desc, ws, kNoAllocScratchBytes, st, &plan, &tables);
+  s = plan_build(desc, ws, need, st, &plan, &tables);
   if (s != HF_OK) return s;
   return launch_transfer(&plan, sender_kv, receiver_kv, st);
 }

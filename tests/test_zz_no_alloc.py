@@ -14,6 +14,9 @@ This file is collected last so that a run stopping at the first failure
 has already run every other test."""
 
 import ctypes
+import os
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -90,6 +93,52 @@ def test_noalloc_matches_workspace_path_on_consecutive_calls():
     _assert_same(a.receiver, _noalloc(a))   # and back
     a.close()
     b.close()
+
+
+SHORT = {  # computed operand rows that would fit the built-in array
+    "interp": dict(layer_mode="interp"), "rotated": dict(sender_k_rotated=True),
+    "pooled_first": dict(align_mode="overlap_mean", knorm=True)}
+
+
+@pytest.mark.parametrize("name", sorted(SHORT))
+def test_noalloc_short_computed_rows(name):
+    """The rows are computed by the transfer kernel itself, to the same bits."""
+    job = _job(W.llama_to_ministral(31).with_(L_s=4, L_r=4, **SHORT[name]))
+    _assert_same(job.receiver, _noalloc(job))
+    job.close()
+
+
+_COUNT = """
+import ctypes, sys
+sys.path[:0] = [{root!r}, {tests!r}]
+import test_zz_no_alloc as t
+from paper_2609_32259_gb300 import workloads as W
+calls = ctypes.CDLL(None).hf_test_calls
+job = t._job(W.llama_to_ministral(31).with_(L_s=4, L_r=4, layer_mode="interp"))
+a = calls()
+for _ in range(3):
+    t._noalloc(job)
+print("calls", a, calls())
+"""
+
+
+def test_noalloc_makes_no_operand_rows(tmp_path):
+    """hf_transfer makes computed rows in a pass whose order an event of the plan
+    keeps; hf_transfer_noalloc may create none.  A preloaded stand-in for the pass
+    counts its calls."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    names = subprocess.run(["nm", "-D", "--defined-only", B.LIB_PATH], capture_output=True,
+                           text=True, check=True).stdout.split()
+    (symbol,) = [n for n in names if "launch_operands" in n]
+    (tmp_path / "count.c").write_text(
+        f"static int n; int {symbol}(void) {{ ++n; return 0; }} int hf_test_calls(void) {{ return n; }}")
+    lib = str(tmp_path / "libcount.so")
+    subprocess.run(["gcc", "-shared", "-fPIC", "-o", lib, str(tmp_path / "count.c")], check=True)
+    code = _COUNT.format(root=root, tests=os.path.join(root, "tests"))
+    out = subprocess.run([sys.executable, "-c", code], env=dict(os.environ, LD_PRELOAD=lib),
+                         capture_output=True, text=True, timeout=300)
+    assert out.returncode == 0, out.stderr
+    assert out.stdout.split()[-3:] == ["calls", "1", "1"], out.stdout
 
 
 def test_noalloc_rejects_transfers_beyond_its_scratch():

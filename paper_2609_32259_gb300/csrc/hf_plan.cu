@@ -45,17 +45,23 @@ namespace {
 struct OperandPath {
   bool pam, one_entry, gather, split;
   int made;  // roles whose rows a pass of their own makes (hf_plan_s::made)
-  int K;
+  int64_t K;
 };
 OperandPath operand_path(const hf_plan_desc& d) {
   OperandPath o{};
-  const int n_seg = d.layer_mode == HF_LAYER_PAPER3 ? 3
-                    : d.layer_mode == HF_LAYER_EXPLICIT ? d.n_seg : 1;
-  o.K = n_seg * d.H_s * d.D_s;
+  // hf_plan_workspace_size has not validated the descriptor, and gives one that
+  // hf_plan_create will refuse the size of a plan without made rows
+  const bool table = d.layer_mode == HF_LAYER_EXPLICIT;
+  if (d.L_r < 1 || d.L_r > kMaxLayersR || d.H_s < 1 || d.D_s < 1 ||
+      (table && (d.n_seg < 1 || d.n_seg > kMaxSeg || d.n_terms < 1 || d.n_terms > kMaxTerms)))
+    return o;
+  const int n_seg = d.layer_mode == HF_LAYER_PAPER3 ? 3 : table ? d.n_seg : 1;
+  const int64_t d_s = static_cast<int64_t>(d.H_s) * d.D_s;
+  o.K = d_s < (1 << 24) ? n_seg * d_s : 0;
   // The copy-only operand path needs every segment to be one sender layer
   // with weight 1, one-entry rows and no rotation.
   bool one_layer_segments = d.layer_mode == HF_LAYER_PAPER3;
-  if (d.layer_mode == HF_LAYER_EXPLICIT && d.n_terms == 1 && d.h_seg_w) {
+  if (table && d.n_terms == 1 && d.h_seg_w) {
     one_layer_segments = true;
     for (int i = 0; i < d.L_r * d.n_seg; ++i)
       if (d.h_seg_w[i] != 1.0f) one_layer_segments = false;
@@ -71,7 +77,7 @@ OperandPath operand_path(const hf_plan_desc& d) {
   const bool copies = one_layer_segments && o.one_entry;  // values, and keys if not rotated
   o.gather = copies && !unrot;
   o.split = !o.gather && d.dtype == HF_BF16 && d.round_built_operands == 0;
-  if (!o.gather && d.dtype == HF_BF16) o.made = copies ? 1 : 3;
+  if (!o.gather && d.dtype == HF_BF16 && o.K > 0) o.made = copies ? 1 : 3;
   return o;
 }
 

@@ -101,6 +101,23 @@ def test_plan_create_checks_workspace(B):
     assert st == B.HF_ERR_WORKSPACE  # not 256-byte aligned
 
 
+@pytest.mark.parametrize("over", [
+    dict(layer_mode="interp", H_s=0), dict(layer_mode="interp", D_s=0), dict(layer_mode="interp", D_s=-64),
+    dict(layer_mode="interp", L_r=0),
+    dict(layer_mode="explicit", seg_layer=np.zeros((6, 0, 2)), seg_w=1.0),
+    dict(layer_mode="explicit", seg_layer=np.zeros((6, 9, 1)), seg_w=0.5),
+    dict(sender_k_rotated=True, theta_s=1e4, H_s=0)])
+def test_workspace_size_of_refused_descriptors(B, over):
+    """The size comes before the validation: a descriptor that hf_plan_create
+    refuses still gets one, and the refusal is a status."""
+    d = _desc(B, **over)
+    need = B.plan_workspace_size(d)
+    assert 0 < need < 1 << 24  # no room for computed rows
+    h = ctypes.c_void_p(0)
+    st = B.lib().hf_plan_create(ctypes.byref(d.c), ctypes.c_void_p(256), need, None, ctypes.byref(h))
+    assert st in (B.HF_ERR_INVALID_ARGUMENT, B.HF_ERR_UNSUPPORTED)
+
+
 def test_workspace_grows_with_tokens(B):
     a = B.plan_workspace_size(_desc(B, r_tok_ptr=[0, 6]))
     b = B.plan_workspace_size(_desc(B, r_tok_ptr=[0, 60000]))

@@ -119,6 +119,28 @@ template <typename T>
 __device__ __forceinline__ T ld_dep(const T* p) {
   return *p;
 }
+// The same as a volatile load, which also stays where it is written among other
+// such loads, but, unlike an ordinary one, may pass stores: what the rotated
+// operand rows' builders and the key norm need (3K tokens of rotated keys, rows
+// built by the loader warps: 3.64 ms with ordinary loads, 3.40 with these; made
+// rows and key norm: 383 and 378 us; but pooled rows 0.85 and 0.93 ms).
+__device__ __forceinline__ int32_t ld_dep_volatile(const int32_t* p) {
+  int32_t v;
+  asm volatile("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float ld_dep_volatile(const float* p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ uint4 ld_dep_volatile(const uint4* p) {
+  uint4 v;
+  asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "l"(p));
+  return v;
+}
 
 // ---------------------------------------------------------------------------
 // Thread-block clusters (a CTA pair sharing one tcgen05 MMA)

@@ -621,7 +621,7 @@ __device__ __forceinline__ void build_atom_unrotated(const XferParams& P, const 
     float f[kPerChunk], acc[kPerChunk];
 #pragma unroll
     for (int q = 0; q < kPerChunk; ++q) {
-      f[q] = ld_dep(P.inv_freq_s + fi + q);
+      f[q] = ld_dep_volatile(P.inv_freq_s + fi + q);
       acc[q] = 0.f;
     }
     for (int ti = 0; ti < segs.n_terms[seg]; ++ti) {
@@ -632,14 +632,14 @@ __device__ __forceinline__ void build_atom_unrotated(const XferParams& P, const 
         const int k = P.col[e];
         if (k < 0 || k >= P.T_s) continue;  // flagged at plan creation
         const float wt = om * P.w[e];
-        const int64_t kr = P.srow ? ld_dep(P.srow + k) : k;
+        const int64_t kr = P.srow ? ld_dep_volatile(P.srow + k) : k;
         const T* row = base + kr * P.d_s;
         float x[kPerChunk], y[kPerChunk];
 #pragma unroll
         for (int q = 0; q < kPerChunk; ++q) x[q] = y[q] = 0.f;
-        accum16(ld_dep(reinterpret_cast<const uint4*>(row + el)), 1.f, x, (const T*)nullptr);
-        accum16(ld_dep(reinterpret_cast<const uint4*>(row + partner)), 1.f, y, (const T*)nullptr);
-        const int p = ld_dep(P.spos + k);
+        accum16(ld_dep_volatile(reinterpret_cast<const uint4*>(row + el)), 1.f, x, (const T*)nullptr);
+        accum16(ld_dep_volatile(reinterpret_cast<const uint4*>(row + partner)), 1.f, y, (const T*)nullptr);
+        const int p = ld_dep_volatile(P.spos + k);
 #pragma unroll
         for (int q = 0; q < kPerChunk; ++q) {
           float sn, cs;
@@ -674,7 +674,7 @@ __device__ __forceinline__ void build_stage_unrotated(const XferParams& P, const
     float f[kPerChunk], ax[kPerChunk], ay[kPerChunk];
 #pragma unroll
     for (int i = 0; i < kPerChunk; ++i) {
-      f[i] = ld_dep(P.inv_freq_s + i0 + i);
+      f[i] = ld_dep_volatile(P.inv_freq_s + i0 + i);
       ax[i] = 0.f;
       ay[i] = 0.f;
     }
@@ -686,14 +686,14 @@ __device__ __forceinline__ void build_stage_unrotated(const XferParams& P, const
         const int k = P.col[e];
         if (k < 0 || k >= P.T_s) continue;  // flagged at plan creation
         const float wt = om * P.w[e];
-        const int64_t kr = P.srow ? ld_dep(P.srow + k) : k;
+        const int64_t kr = P.srow ? ld_dep_volatile(P.srow + k) : k;
         const T* row = base + kr * P.d_s;
         float x[kPerChunk], y[kPerChunk];
 #pragma unroll
         for (int i = 0; i < kPerChunk; ++i) x[i] = y[i] = 0.f;
-        accum16(ld_dep(reinterpret_cast<const uint4*>(row + ex)), 1.f, x, (const T*)nullptr);
-        accum16(ld_dep(reinterpret_cast<const uint4*>(row + ey)), 1.f, y, (const T*)nullptr);
-        const int p = ld_dep(P.spos + k);
+        accum16(ld_dep_volatile(reinterpret_cast<const uint4*>(row + ex)), 1.f, x, (const T*)nullptr);
+        accum16(ld_dep_volatile(reinterpret_cast<const uint4*>(row + ey)), 1.f, y, (const T*)nullptr);
+        const int p = ld_dep_volatile(P.spos + k);
 #pragma unroll
         for (int i = 0; i < kPerChunk; ++i) {
           float sn, cs;
@@ -1509,7 +1509,7 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const CUt
 #pragma unroll
               for (int i = 0; i < 16; ++i) {
                 const float y = fmaf(__uint_as_float(v[i]), inv_r,
-                                     ld_dep(bias + nb * P.BN + tcol + q2 + i));
+                                     ld_dep_volatile(bias + nb * P.BN + tcol + q2 + i));
                 ss = fmaf(y, y, ss);
               }
             }
@@ -1543,8 +1543,8 @@ __device__ __forceinline__ void transfer_body(const CUtensorMap* maps, const CUt
               if (do_knorm) {
 #pragma unroll
                 for (int i = 0; i < 16; ++i) {
-                  y[i] *= rn * ld_dep(P.knorm_w + q + i);
-                  y[16 + i] *= rn * ld_dep(P.knorm_w + half + q + i);
+                  y[i] *= rn * ld_dep_volatile(P.knorm_w + q + i);
+                  y[16 + i] *= rn * ld_dep_volatile(P.knorm_w + half + q + i);
                 }
               }
               float* srow = sStg + row * kStgRow + g * 32;

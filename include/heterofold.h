@@ -268,9 +268,10 @@ typedef struct hf_plan_s* hf_plan;
  * bf16 plans whose map input rows are computed (interpolated or weighted
  * layers, pooling before the map, sender_k_rotated) they include room for
  * those rows, at most 512 MB or one receiver layer's: hf_transfer makes them
- * in a pass of their own.  Where one layer's would take over 2 GiB, and in a
- * workspace without that room (as many bytes as the same plan in fp32 needs),
- * the transfer kernel computes them itself, slower, to the same bits. */
+ * in a pass of their own.  Where one layer's would take over 2 GiB, in a
+ * workspace without that room (as many bytes as the same plan in fp32 needs)
+ * and in captured transfers, the transfer kernel computes them itself, slower,
+ * to the same bits. */
 hf_status hf_plan_workspace_size(const hf_plan_desc* desc, size_t* bytes);
 
 /*
@@ -292,8 +293,9 @@ hf_status hf_plan_create(const hf_plan_desc* desc, void* d_workspace, size_t wor
  * hf_transfer — write the receiver cache: one kernel launch on `stream`, or,
  * where computed map input rows have room in the workspace, a pass that makes
  * them and a launch for every group of receiver layers that fits.  Transfers
- * of such a plan run one after another, whatever their streams; graphs that
- * captured one are not to be replayed beside another of the same plan.
+ * of such a plan run one after another, whatever their streams.  Inside a
+ * stream capture the transfer kernel computes the rows itself, in one launch:
+ * graphs of one plan may be replayed side by side, and beside other transfers.
  * sender_kv:   device [L_s][2][sender_rows][H_s][D_s] (sender_rows = T_s
  *              unless the plan maps message spans) in the plan's dtype, the
  *              sender's keys and values; keys pre-RoPE (Section 3: keys are

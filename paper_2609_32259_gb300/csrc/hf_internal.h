@@ -128,7 +128,7 @@ struct hf_plan_s {
   // copies them; x_rows rows (distinct rows, or sender tokens with pooling after
   // the map) of x_layers receiver layers at a time.  0 where rows are copies, in
   // fp32, and where the workspace holds only WorkspaceLayout::total bytes: the
-  // loader warps then build what is not a copy.
+  // loader warps then build what is not a copy, as they do in captured transfers.
   int made;
   int64_t x_rows;
   int x_layers;

@@ -1837,8 +1837,10 @@ namespace {
 
 // The kernel parameters and map tile descriptor of one plan's launch over
 // receiver layers [l_begin, l_end); *max_pair_tiles bounds its pair tiles.
+// made: the operand pass has made its computed rows (otherwise the loader warps
+// build them).
 hf_status make_xfer(hf_plan_s* p, const void* sender, void* receiver, int l_begin, int l_end,
-                    XferParams* out, CUtensorMap* map_out, CUtensorMap* map_a_out,
+                    bool made, XferParams* out, CUtensorMap* map_out, CUtensorMap* map_a_out,
                     int64_t* max_pair_tiles) {
   const hf_plan_desc& d = p->desc;
   const bool f32 = d.dtype == HF_F32;
@@ -1850,11 +1852,11 @@ hf_status make_xfer(hf_plan_s* p, const void* sender, void* receiver, int l_begi
                          static_cast<uint32_t>(p->BN / (p->single ? 1 : 2)),
                          static_cast<uint32_t>(bk), CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
   if (s != HF_OK) return s;
-  if (p->made || (p->pam && p->gather && !p->span)) {
+  if (made || (p->pam && p->gather && !p->span)) {
     // operand rows that follow one another: made ones, or the sender's under
     // pooling after the map
     const int planes = (p->made == 3 ? 2 : 1) * (p->split ? 2 : 1);
-    s = p->made ? make_map(map_a_out, p->ws + p->lay.xbuf, f32,
+    s = made ? make_map(map_a_out, p->ws + p->lay.xbuf, f32,
                            static_cast<uint64_t>(p->x_layers) * planes * p->x_rows,
                            static_cast<uint64_t>(p->K), 32u, static_cast<uint32_t>(bk),
                            CU_TENSOR_MAP_L2_PROMOTION_L2_256B)
@@ -1901,14 +1903,14 @@ hf_status make_xfer(hf_plan_s* p, const void* sender, void* receiver, int l_begi
   P.pos = reinterpret_cast<const int32_t*>(ws + p->lay.pos);
   P.uidx = reinterpret_cast<const int32_t*>(ws + p->lay.new_flag);
   P.n_batoms = n_atoms;
-  P.made = p->made;
+  P.made = made ? p->made : 0;
   P.made_roles = p->made == 3 ? 2 : 1;
-  P.x = p->made ? ws + p->lay.xbuf : nullptr;
+  P.x = made ? ws + p->lay.xbuf : nullptr;
   P.x_rows = p->x_rows;
   P.atoms_per_seg = p->d_s / bk;
   P.BN = p->BN;
-  P.wide = p->wide ? 1 : 0;
-  P.n_tiles_n = p->d_r / (p->BN * (p->wide ? 2 : 1));
+  P.wide = p->wide && !made ? 1 : 0;
+  P.n_tiles_n = p->d_r / (p->BN * (P.wide ? 2 : 1));
   pick_rings(stage_b_bytes(p->BN, p->single), &P.stages_a, &P.stages_b, &P.lag);
   P.rope = p->rope ? 1 : 0;
   P.unrot = p->unrot ? 1 : 0;
@@ -1936,9 +1938,10 @@ hf_status launch_batch_typed(const BatchParams& B, int64_t max_pair_tiles, size_
 }  // namespace
 
 static hf_status transfer_layers(hf_plan_s* p, const void* sender, void* receiver,
-                                 cudaStream_t stream, int l_begin, int l_end, bool stall) {
+                                 cudaStream_t stream, int l_begin, int l_end, bool made,
+                                 bool stall) {
   const hf_plan_desc& d = p->desc;
-  if (p->made) {
+  if (made) {
     // the operand rows of at most as many receiver layers as their buffer holds,
     // then these layers' transfer; groups of like size, as the last round of a
     // small group's tiles would leave most of the SMs idle (rotated 3K: 27 + 5
@@ -1948,7 +1951,7 @@ static hf_status transfer_layers(hf_plan_s* p, const void* sender, void* receive
       const int per = (n + groups - 1) / groups;
       for (int l = l_begin; l < l_end; l += per) {
         const hf_status e =
-            transfer_layers(p, sender, receiver, stream, l, std::min(l_end, l + per), stall);
+            transfer_layers(p, sender, receiver, stream, l, std::min(l_end, l + per), made, stall);
         if (e != HF_OK) return e;
       }
       return HF_OK;
@@ -1959,7 +1962,7 @@ static hf_status transfer_layers(hf_plan_s* p, const void* sender, void* receive
   XferParams P;
   CUtensorMap mw, ma = {};
   int64_t max_pair_tiles = 0;
-  hf_status s = make_xfer(p, sender, receiver, l_begin, l_end, &P, &mw, &ma, &max_pair_tiles);
+  hf_status s = make_xfer(p, sender, receiver, l_begin, l_end, made, &P, &mw, &ma, &max_pair_tiles);
   if (s != HF_OK) return s;
   P.stall = stall ? 1 : 0;
   const size_t smem = smem_bytes(stage_b_bytes(p->BN, p->single), P.stages_a, P.stages_b);
@@ -1971,33 +1974,39 @@ static hf_status transfer_layers(hf_plan_s* p, const void* sender, void* receive
     return p->gather ? go(transfer_kernel<float, kCopiedRows, 2>)
                      : go(transfer_kernel<float, kBuiltRows, 2>);
   if (p->single) return go(transfer_kernel<Bf, kCopiedRows, 0, false>);
-  if (p->made)
+  if (made)
     return p->pam ? go(transfer_kernel<Bf, kMadeRows, 1>) : go(transfer_kernel<Bf, kMadeRows, 0>);
   if (p->pam)
     return p->gather ? go(transfer_kernel<Bf, kCopiedRows, 1>) : go(transfer_kernel<Bf, kBuiltRows, 1>);
   return p->gather ? go(transfer_kernel<Bf, kCopiedRows, 0>) : go(transfer_kernel<Bf, kBuiltRows, 0>);
 }
 
+// Made rows lie in the plan's workspace, so transfers that use them run one
+// after another, whatever their streams (x_done).  A captured transfer could
+// only be ordered within its graph, and graphs of one plan may be replayed side
+// by side: its rows are built by the loader warps, which share nothing.
+static bool may_use_made_rows(const hf_plan_s* p, cudaStream_t stream) {
+  if (!p->made) return false;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) {
+    cudaGetLastError();  // the legacy stream beside another thread's capture
+    return false;
+  }
+  return cap == cudaStreamCaptureStatusNone;
+}
+
 hf_status launch_transfer(hf_plan_s* p, const void* sender, void* receiver, cudaStream_t stream,
                           int l_begin, int l_end, bool stall) {
   if (l_end < 0) l_end = p->desc.L_r;
   if (p->T_r == 0 || l_end <= l_begin) return HF_OK;
-  if (!p->made) return transfer_layers(p, sender, receiver, stream, l_begin, l_end, stall);
-  // a graph's replays are ordered by its owner: a capture cannot wait for what
-  // lies outside of it
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) {
-    cudaGetLastError();  // the legacy stream beside another thread's capture
-    cap = cudaStreamCaptureStatusActive;
-  }
+  if (!may_use_made_rows(p, stream))
+    return transfer_layers(p, sender, receiver, stream, l_begin, l_end, false, stall);
   std::lock_guard<std::mutex> lock(p->x_mutex);
-  if (cap != cudaStreamCaptureStatusNone)
-    return transfer_layers(p, sender, receiver, stream, l_begin, l_end, stall);
   if (p->x_done)
     HF_CUDA_TRY(cudaStreamWaitEvent(stream, p->x_done, 0), "wait for the plan's operand rows");
   else
     HF_CUDA_TRY(cudaEventCreateWithFlags(&p->x_done, cudaEventDisableTiming), "operand rows' event");
-  const hf_status s = transfer_layers(p, sender, receiver, stream, l_begin, l_end, stall);
+  const hf_status s = transfer_layers(p, sender, receiver, stream, l_begin, l_end, true, stall);
   if (s != HF_OK) return s;
   HF_CUDA_TRY(cudaEventRecord(p->x_done, stream), "record the operand rows' event");
   return HF_OK;
@@ -2024,7 +2033,7 @@ hf_status launch_transfer_batch(hf_plan_s* const* plans, const void* const* send
     hf_plan_s* p = plans[i];
     if (p->T_r == 0) continue;
     int64_t mt = 0;
-    const hf_status s = make_xfer(p, senders[i], receivers[i], 0, p->desc.L_r, &B->P[k],
+    const hf_status s = make_xfer(p, senders[i], receivers[i], 0, p->desc.L_r, false, &B->P[k],
                                   &B->maps[k], &B->maps_a[k], &mt);
     if (s != HF_OK) {
       delete B;

@@ -7,6 +7,7 @@ import pytest
 import torch
 
 from gpu_harness import Case
+from paper_2609_32259_gb300 import binding as B
 from paper_2609_32259_gb300 import workloads as W
 
 pytestmark = pytest.mark.gpu
@@ -30,6 +31,40 @@ CASES = {
         n_req=3, lo=40, hi=300, seed=71).with_(L_s=4, L_r=3, align_mode="overlap_mean"),
     "interp_wide": lambda: W.llama_to_ministral(500).with_(L_s=5, L_r=3, layer_mode="interp"),
 }
+
+
+@pytest.mark.parametrize("over", [
+    dict(layer_mode="interp"), dict(sender_k_rotated=True),
+    dict(layer_mode="interp", align_mode="overlap_mean")])
+def test_graphs_of_one_plan_side_by_side(over):
+    """Two graphs of one plan with computed map input rows, each on its own
+    caches, replayed on two streams beside an eager transfer on a third: none
+    takes another's rows."""
+    w = W.llama_to_ministral(1500).with_(L_s=6, L_r=5, **over)
+    c = Case(w).run()
+    plan = c.job.plan
+    senders = [c.sender.flip(2 * i % 3).contiguous() if i else c.sender for i in range(3)]
+    want, outs = [], [torch.empty_like(c.job.receiver) for _ in senders]
+    for s, o in zip(senders, outs):
+        B.transfer(plan, s, o)
+        torch.cuda.synchronize()
+        want.append(o.clone())
+    graphs = [torch.cuda.CUDAGraph() for _ in range(2)]
+    for g, s, o in zip(graphs, senders, outs):
+        with torch.cuda.graph(g):
+            B.transfer(plan, s, o, torch.cuda.current_stream())
+    streams = [torch.cuda.Stream() for _ in senders]
+    for o in outs:
+        o.fill_(SENTINEL)
+    torch.cuda.synchronize()
+    for _ in range(10):
+        for i, st in enumerate(streams):
+            with torch.cuda.stream(st):
+                graphs[i].replay() if i < 2 else B.transfer(plan, senders[i], outs[i], st)
+    torch.cuda.synchronize()
+    assert c.job.device_status() == 0
+    for o, ref in zip(outs, want):
+        assert torch.equal(o, ref)
 
 
 @pytest.mark.parametrize("name", sorted(CASES))

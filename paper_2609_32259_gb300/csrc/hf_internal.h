@@ -120,9 +120,9 @@ struct hf_plan_s {
   bool span;    // aligned sender tokens are spans inside a longer sender cache
   bool pam;     // pooling after the map: map input rows are sender rows in windows
   bool wide;    // tiles of two 256-column blocks (operand rows built by the loader warps)
-  // tiles of 128 rows x 256 columns on single CTAs instead of 256 x 256 on
-  // pairs: few distinct rows (kSingleRows)
-  bool single;
+  // few distinct rows (kSingleRows): tiles of 128 rows x 256 columns on single
+  // CTAs instead of 256 x 256 on pairs, where every plan of the launch has few
+  bool few_rows;
   // bit c: the map input rows of role c (pooled, blended, weighted or rotated
   // back) are made by a pass of their own before the transfer, which then
   // copies them; x_rows rows (distinct rows, or sender tokens with pooling after

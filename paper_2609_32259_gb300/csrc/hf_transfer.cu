@@ -1838,9 +1838,9 @@ namespace {
 // The kernel parameters and map tile descriptor of one plan's launch over
 // receiver layers [l_begin, l_end); *max_pair_tiles bounds its pair tiles.
 // made: the operand pass has made its computed rows (otherwise the loader warps
-// build them).
+// build them); single: single-CTA tiles.
 hf_status make_xfer(hf_plan_s* p, const void* sender, void* receiver, int l_begin, int l_end,
-                    bool made, XferParams* out, CUtensorMap* map_out, CUtensorMap* map_a_out,
+                    bool made, bool single, XferParams* out, CUtensorMap* map_out, CUtensorMap* map_a_out,
                     int64_t* max_pair_tiles) {
   const hf_plan_desc& d = p->desc;
   const bool f32 = d.dtype == HF_F32;
@@ -1849,7 +1849,7 @@ hf_status make_xfer(hf_plan_s* p, const void* sender, void* receiver, int l_begi
   CUtensorMap& mw = *map_out;
   hf_status s = make_map(&mw, d.d_W, f32, static_cast<uint64_t>(d.L_r) * 2 * p->d_r,
                          static_cast<uint64_t>(p->K),
-                         static_cast<uint32_t>(p->BN / (p->single ? 1 : 2)),
+                         static_cast<uint32_t>(p->BN / (single ? 1 : 2)),
                          static_cast<uint32_t>(bk), CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
   if (s != HF_OK) return s;
   if (made || (p->pam && p->gather && !p->span)) {
@@ -1911,7 +1911,7 @@ hf_status make_xfer(hf_plan_s* p, const void* sender, void* receiver, int l_begi
   P.BN = p->BN;
   P.wide = p->wide && !made ? 1 : 0;
   P.n_tiles_n = p->d_r / (p->BN * (P.wide ? 2 : 1));
-  pick_rings(stage_b_bytes(p->BN, p->single), &P.stages_a, &P.stages_b, &P.lag);
+  pick_rings(stage_b_bytes(p->BN, single), &P.stages_a, &P.stages_b, &P.lag);
   P.rope = p->rope ? 1 : 0;
   P.unrot = p->unrot ? 1 : 0;
   P.D_s = d.D_s;
@@ -1920,7 +1920,7 @@ hf_status make_xfer(hf_plan_s* p, const void* sender, void* receiver, int l_begi
   P.paged = d.paged ? 1 : 0;
   P.knorm = d.d_knorm_w ? 1 : 0;
   P.knorm_eps = d.knorm_eps;
-  const int tile_rows = p->single ? kBM : kPairRows;
+  const int tile_rows = single ? kBM : kPairRows;
   P.idesc = make_idesc(f32 ? 2u : 1u, tile_rows, p->BN);
   // pooling after the map: at most T_s windows (stride >= 1), two per pair tile
   const int64_t row_blocks = p->pam ? (p->T_s + 1) / 2 : (p->T_r + tile_rows - 1) / tile_rows;
@@ -1962,18 +1962,20 @@ static hf_status transfer_layers(hf_plan_s* p, const void* sender, void* receive
   XferParams P;
   CUtensorMap mw, ma = {};
   int64_t max_pair_tiles = 0;
-  hf_status s = make_xfer(p, sender, receiver, l_begin, l_end, made, &P, &mw, &ma, &max_pair_tiles);
+  const bool single = p->few_rows;
+  hf_status s = make_xfer(p, sender, receiver, l_begin, l_end, made, single, &P, &mw, &ma,
+                          &max_pair_tiles);
   if (s != HF_OK) return s;
   P.stall = stall ? 1 : 0;
-  const size_t smem = smem_bytes(stage_b_bytes(p->BN, p->single), P.stages_a, P.stages_b);
+  const size_t smem = smem_bytes(stage_b_bytes(p->BN, single), P.stages_a, P.stages_b);
   auto go = [&](auto kern) {
-    return launch_pairs(kern, p->single, max_pair_tiles, smem, stream, mw, ma, P);
+    return launch_pairs(kern, single, max_pair_tiles, smem, stream, mw, ma, P);
   };
   using Bf = __nv_bfloat16;
   if (d.dtype == HF_F32)
     return p->gather ? go(transfer_kernel<float, kCopiedRows, 2>)
                      : go(transfer_kernel<float, kBuiltRows, 2>);
-  if (p->single) return go(transfer_kernel<Bf, kCopiedRows, 0, false>);
+  if (single) return go(transfer_kernel<Bf, kCopiedRows, 0, false>);
   if (made)
     return p->pam ? go(transfer_kernel<Bf, kMadeRows, 1>) : go(transfer_kernel<Bf, kMadeRows, 0>);
   if (p->pam)
@@ -2013,18 +2015,31 @@ hf_status launch_transfer(hf_plan_s* p, const void* sender, void* receiver, cuda
 }
 
 bool batch_compatible(const hf_plan_s* const* plans, int n) {
-  if (plans[0]->made) return false;  // operand passes of their own
-  for (int i = 1; i < n; ++i)
-    if (plans[i]->desc.dtype != plans[0]->desc.dtype || plans[i]->gather != plans[0]->gather ||
-        plans[i]->split != plans[0]->split || plans[i]->staged != plans[0]->staged ||
-        plans[i]->pam != plans[0]->pam || plans[i]->wide != plans[0]->wide ||
-        plans[i]->made || plans[i]->single != plans[0]->single)
+  const hf_plan_s* first = nullptr;  // plans without receiver tokens have no tiles
+  for (int i = 0; i < n; ++i) {
+    const hf_plan_s* const p = plans[i];
+    if (p->T_r == 0) continue;
+    if (!first) first = p;
+    if (p->made)  // operand passes of their own
       return false;
+    if (p->desc.dtype != first->desc.dtype || p->gather != first->gather ||
+        p->split != first->split || p->staged != first->staged || p->pam != first->pam ||
+        p->wide != first->wide)
+      return false;
+  }
   return true;
 }
 
 hf_status launch_transfer_batch(hf_plan_s* const* plans, const void* const* senders,
                                 void* const* receivers, int n, cudaStream_t stream) {
+  const hf_plan_s* first = nullptr;
+  bool single = true;  // a plan with few rows may run in pairs, not the other way round
+  for (int i = 0; i < n; ++i) {
+    if (plans[i]->T_r == 0) continue;
+    if (!first) first = plans[i];
+    single = single && plans[i]->few_rows;
+  }
+  if (!first) return HF_OK;
   BatchParams* B = new BatchParams();
   std::memset(B, 0, sizeof(*B));
   int64_t tiles = 0;
@@ -2033,7 +2048,7 @@ hf_status launch_transfer_batch(hf_plan_s* const* plans, const void* const* send
     hf_plan_s* p = plans[i];
     if (p->T_r == 0) continue;
     int64_t mt = 0;
-    const hf_status s = make_xfer(p, senders[i], receivers[i], 0, p->desc.L_r, false, &B->P[k],
+    const hf_status s = make_xfer(p, senders[i], receivers[i], 0, p->desc.L_r, false, single, &B->P[k],
                                   &B->maps[k], &B->maps_a[k], &mt);
     if (s != HF_OK) {
       delete B;
@@ -2043,12 +2058,8 @@ hf_status launch_transfer_batch(hf_plan_s* const* plans, const void* const* send
     max_bn = std::max(max_bn, p->BN);
     ++k;
   }
-  if (k == 0) {
-    delete B;
-    return HF_OK;
-  }
   int sa = 0, sb = 0, lag = 0;
-  const int stage_b = stage_b_bytes(max_bn, plans[0]->single);
+  const int stage_b = stage_b_bytes(max_bn, single);
   pick_rings(stage_b, &sa, &sb, &lag);
   for (int i = 0; i < k; ++i) {
     B->P[i].stages_a = sa;
@@ -2059,16 +2070,16 @@ hf_status launch_transfer_batch(hf_plan_s* const* plans, const void* const* send
   B->stage_b_stride = stage_b;
   const size_t smem = smem_bytes(stage_b, sa, sb);
   hf_status s;
-  if (plans[0]->single)
+  if (single)
     s = launch_batch_typed<__nv_bfloat16, kCopiedRows, 0, false>(*B, tiles, smem, stream);
-  else if (plans[0]->desc.dtype == HF_F32)
-    s = plans[0]->gather ? launch_batch_typed<float, kCopiedRows, 2>(*B, tiles, smem, stream)
+  else if (first->desc.dtype == HF_F32)
+    s = first->gather ? launch_batch_typed<float, kCopiedRows, 2>(*B, tiles, smem, stream)
                          : launch_batch_typed<float, kBuiltRows, 2>(*B, tiles, smem, stream);
-  else if (plans[0]->pam)
-    s = plans[0]->gather ? launch_batch_typed<__nv_bfloat16, kCopiedRows, 1>(*B, tiles, smem, stream)
+  else if (first->pam)
+    s = first->gather ? launch_batch_typed<__nv_bfloat16, kCopiedRows, 1>(*B, tiles, smem, stream)
                          : launch_batch_typed<__nv_bfloat16, kBuiltRows, 1>(*B, tiles, smem, stream);
   else
-    s = plans[0]->gather ? launch_batch_typed<__nv_bfloat16, kCopiedRows, 0>(*B, tiles, smem, stream)
+    s = first->gather ? launch_batch_typed<__nv_bfloat16, kCopiedRows, 0>(*B, tiles, smem, stream)
                          : launch_batch_typed<__nv_bfloat16, kBuiltRows, 0>(*B, tiles, smem, stream);
   delete B;
   return s;

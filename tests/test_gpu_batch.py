@@ -3,6 +3,8 @@
 direction must equal, bit for bit, its own hf_transfer (the same tiles, the
 same code), and match the fp64 oracle within the parity tolerance."""
 
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -36,6 +38,42 @@ def test_message_round_batch_matches_single_transfers_and_oracle():
     for c, ref in zip(cases, single):
         assert torch.equal(c.job.receiver, ref), c.w.name
         c.check_parity()
+
+
+def _captured_nodes(cases):
+    """Number of launches of one batch of the cases, as a capture records them."""
+    g = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(g):
+        B.transfer_batch([c.job.plan for c in cases], [c.sender for c in cases],
+                         [c.job.receiver for c in cases], torch.cuda.current_stream())
+    nodes = ctypes.c_size_t(0)
+    cudart = ctypes.CDLL(f"libcudart.so.{torch.version.cuda.split('.')[0]}")
+    assert cudart.cudaGraphGetNodes(ctypes.c_void_p(g.raw_cuda_graph()), None,
+                                    ctypes.byref(nodes)) == 0
+    return nodes.value
+
+
+def test_batch_of_short_long_and_empty_directions():
+    """Short messages alone would take single-CTA tiles; beside longer ones, and
+    beside a direction without tokens, all run in one launch."""
+    ws = [W.llama_to_qwen25(400).with_(L_s=4, L_r=3), W.llama_to_ministral(700).with_(L_s=4, L_r=3),
+          W.llama_to_qwen25(90).with_(L_s=4, L_r=3, align_mode="same_index")]
+    cases = [Case(w, sentinel=SENTINEL).run() for w in ws]
+    single = [c.job.receiver.clone() for c in cases]
+    empty = Case(W.llama_to_ministral(5).with_(L_s=4, L_r=3))
+    empty.job.desc._r[1] = 0  # no receiver token
+    empty.job.make_plan()
+    empty.job.receiver.fill_(SENTINEL)
+    cases.insert(1, empty)
+    for c in cases:
+        c.job.receiver.fill_(SENTINEL)
+    B.transfer_batch([c.job.plan for c in cases], [c.sender for c in cases],
+                     [c.job.receiver for c in cases])
+    torch.cuda.synchronize()
+    for c, ref in zip([c for c in cases if c is not empty], single):
+        assert torch.equal(c.job.receiver, ref), c.w.name
+    assert (empty.job.receiver == SENTINEL).all()
+    assert _captured_nodes(cases) == 1
 
 
 def test_batch_mixing_operand_paths():

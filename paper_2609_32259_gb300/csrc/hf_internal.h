@@ -65,13 +65,16 @@ struct WorkspaceLayout {
   int x_layers, made;
 };
 
-// Receiver tokens up to which copied bf16 rows take single-CTA tiles.  With 512
-// receiver tokens or fewer about 150 distinct rows at most are to be expected
-// with Token Alignment: a pair's 256-row tile is then mostly padding, and the
-// maps, read once, are what bounds the transfer (256 tokens, Ministral ->
+// Copied bf16 rows may take single-CTA tiles where at most kSingleRows distinct
+// rows, one such tile's, are to be expected: in as many tokens on either side, and
+// with Token Alignment, where about a quarter of the receiver's rows are distinct,
+// in kSingleTokens receiver tokens.  A pair's 256-row tile is then mostly padding,
+// and the maps, read once, are what bounds the transfer (256 tokens, Ministral ->
 // Llama-shaped, whole step: 104 us with pairs, 95 us single, of which the maps'
-// bytes take 60; six directions of 160 tokens 418 and 378 us).
-constexpr int64_t kSingleRows = 512;
+// bytes take 60).  With a second block of rows every map is read twice: same-index
+// Llama -> Ministral-shaped, 192 tokens 128 us in pairs, 146 single, 512 tokens 195
+// and 226; Token Alignment, 512 tokens (129 distinct) 138 and 156.
+constexpr int64_t kSingleRows = 128, kSingleTokens = 400;
 
 // Bytes of made operand rows to aim at: receiver layers per launch, so that
 // a launch's last round of tiles is a small part of it.

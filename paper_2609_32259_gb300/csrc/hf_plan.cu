@@ -860,7 +860,9 @@ hf_status plan_build(const hf_plan_desc* desc, void* d_workspace, size_t workspa
   p->made = workspace_bytes >= lay.total_made ? lay.made : 0;
   p->x_rows = lay.x_rows;
   p->x_layers = lay.x_layers;
-  p->few_rows = p->gather && !p->pam && desc->dtype == HF_BF16 && p->T_r <= kSingleRows;
+  p->few_rows = p->gather && !p->pam && desc->dtype == HF_BF16 &&
+                (std::min(p->T_s, p->T_r) <= kSingleRows ||
+                 (desc->align_mode == HF_ALIGN_TA && p->T_r <= kSingleTokens));
   const bool one_entry = path.one_entry;
   // one-entry rows (Token Alignment, same-index, sender rows of pooling
   // after the map) have at most two (term, entry) pairs per segment, both

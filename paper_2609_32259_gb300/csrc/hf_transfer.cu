@@ -37,7 +37,7 @@
 // (pam_epilogue).  Plans whose rows the builders compute use wide tiles:
 // two 256-column blocks per tile in the two accumulators, so each built A
 // stage feeds twice the MMAs.
-// Transfers of few distinct rows (kSingleRows) take tiles of 128 rows x 256
+// Transfers of few distinct rows (kSingleRows, single_fills) take tiles of 128 rows x 256
 // columns on single CTAs (kPair = false): the same roles without a pair.
 // Pipeline hand-offs use mbarriers with bounded waits; nothing traps.
 #include <algorithm>
@@ -1937,6 +1937,16 @@ hf_status launch_batch_typed(const BatchParams& B, int64_t max_pair_tiles, size_
 
 }  // namespace
 
+// Whether `tiles` tiles of one block of rows each are sooner done by single CTAs.
+// A CTA alone takes about 1.7 times as long for a tile as a pair (a round of six
+// directions, 1,376 tiles, 418 us in pairs and 378 single: 19 and 10 rounds of
+// tiles), so it is the number of rounds that counts: 320 tiles, 5 and 3 rounds,
+// 127.7 and 129.7 us; 112 tiles, 2 and 1 rounds, 66 and 60.
+static bool single_fills(int64_t tiles) {
+  const int64_t sms = device_sm_count(), pairs = std::max<int64_t>(1, sms / 2);
+  return 17 * ((tiles + sms - 1) / sms) < 10 * ((tiles + pairs - 1) / pairs);
+}
+
 static hf_status transfer_layers(hf_plan_s* p, const void* sender, void* receiver,
                                  cudaStream_t stream, int l_begin, int l_end, bool made,
                                  bool stall) {
@@ -1962,7 +1972,8 @@ static hf_status transfer_layers(hf_plan_s* p, const void* sender, void* receive
   XferParams P;
   CUtensorMap mw, ma = {};
   int64_t max_pair_tiles = 0;
-  const bool single = p->few_rows;
+  const bool single =
+      p->few_rows && single_fills(2LL * (l_end - l_begin) * (p->d_r / p->BN));
   hf_status s = make_xfer(p, sender, receiver, l_begin, l_end, made, single, &P, &mw, &ma,
                           &max_pair_tiles);
   if (s != HF_OK) return s;
@@ -2034,12 +2045,15 @@ hf_status launch_transfer_batch(hf_plan_s* const* plans, const void* const* send
                                 void* const* receivers, int n, cudaStream_t stream) {
   const hf_plan_s* first = nullptr;
   bool single = true;  // a plan with few rows may run in pairs, not the other way round
+  int64_t maps = 0;
   for (int i = 0; i < n; ++i) {
     if (plans[i]->T_r == 0) continue;
     if (!first) first = plans[i];
     single = single && plans[i]->few_rows;
+    maps += 2LL * plans[i]->desc.L_r * (plans[i]->d_r / plans[i]->BN);
   }
   if (!first) return HF_OK;
+  single = single && single_fills(maps);
   BatchParams* B = new BatchParams();
   std::memset(B, 0, sizeof(*B));
   int64_t tiles = 0;

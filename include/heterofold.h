@@ -348,10 +348,11 @@ hf_status hf_transfer_host(hf_plan plan, const void* h_sender_kv, void* d_sender
  * multi-agent round sends each message to receivers of other model
  * families; Appendix "HiddenBench Evaluation").  Direction i is
  * hf_transfer(plans[i], sender_kv[i], receiver_kv[i]).  When all plans
- * share the dtype and the operand path (one-entry alignment rows with
- * one-layer segments, or not), the directions run in one launch of the
- * transfer kernel over all their tiles; otherwise each direction's kernel
- * runs on a stream of a per-device pool forked from `stream` (created on
+ * with receiver tokens share the dtype and the operand path (one-entry
+ * alignment rows with one-layer segments, or not) and none makes its computed
+ * map input rows in a pass of its own (see hf_transfer), the directions run in
+ * one launch of the transfer kernel over all their tiles; otherwise each
+ * direction's launches run on a stream of a per-device pool forked from `stream` (created on
  * the first such call on a device).  `stream` is ordered after all of them.
  * n in [0, 16]; a plan appears at most once; the receiver caches must not
  * overlap.  Asynchronous.

@@ -218,8 +218,9 @@ hf_status launch_transfer(hf_plan_s* p, const void* sender, void* receiver, cuda
 hf_status launch_operands(const hf_plan_s* p, const void* sender, cudaStream_t stream, int l_begin,
                           int l_end);
 // Several plans in one launch: they must share the dtype, the operand path
-// and where the pooling happens (batch_compatible); n <= kMaxBatch.
-bool batch_compatible(const hf_plan_s* const* plans, int n);
+// and where the pooling happens, and make no operand rows (batch_compatible);
+// n <= kMaxBatch.
+bool batch_compatible(const hf_plan_s* const* plans, int n, cudaStream_t stream);
 hf_status launch_transfer_batch(hf_plan_s* const* plans, const void* const* senders,
                                 void* const* receivers, int n, cudaStream_t stream);
 

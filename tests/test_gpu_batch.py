@@ -92,11 +92,10 @@ def test_batch_mixing_operand_paths():
         assert torch.equal(c.job.receiver, ref), c.w.name
 
 
-def test_batch_of_built_operand_rows():
-    """Directions whose operand rows the loader warps build (layers blended
-    per sender token, overlap pooling after the map; a Qwen2.5-shaped
-    receiver is one 512-column wide tile) in one launch: each equals its
-    single transfer and the oracle."""
+def test_batch_of_computed_operand_rows():
+    """Directions with computed operand rows (layers blended per sender token,
+    overlap pooling after the map), each with its own pass that makes them: each
+    equals its single transfer and the oracle."""
     ws = [W.llama_to_ministral(700).with_(L_s=5, L_r=4, layer_mode="interp",
                                           align_mode="overlap_mean"),
           W.llama_to_qwen25(500).with_(L_s=6, L_r=3, layer_mode="interp",
@@ -113,6 +112,61 @@ def test_batch_of_built_operand_rows():
     for c, ref in zip(cases, single):
         assert torch.equal(c.job.receiver, ref), c.w.name
         c.check_parity()
+
+
+BUILT = {
+    # staged blends in wide tiles, pooling after the map
+    "overlap_interp": [W.llama_to_ministral(700).with_(L_s=5, L_r=4, layer_mode="interp",
+                                                       align_mode="overlap_mean"),
+                       W.llama_to_qwen25(500).with_(L_s=6, L_r=3, layer_mode="interp",
+                                                    align_mode="overlap_mean")],
+    # staged blends, one row per distinct alignment row, paged and not
+    "interp": [W.llama_to_ministral(400).with_(L_s=5, L_r=4, layer_mode="interp"),
+               W.qwen25_to_llama_batched(n_req=2, lo=80, hi=300, seed=61).with_(
+                   L_s=4, L_r=3, layer_mode="interp")],
+    # rows built in registers: keys rotated back, pooling before the map
+    "rotated": [W.llama_to_ministral(300).with_(L_s=4, L_r=3, sender_k_rotated=True),
+                W.llama_to_qwen25(150).with_(L_s=4, L_r=3, sender_k_rotated=True)],
+    "pooled_knorm": [W.llama_to_ministral(300).with_(L_s=4, L_r=3, align_mode="overlap_mean",
+                                                     knorm=True, sender_k_rotated=True),
+                     W.llama_to_qwen25(150).with_(L_s=4, L_r=3, align_mode="overlap_mean",
+                                                  knorm=True, sender_k_rotated=True)],
+}
+
+
+def _without_room(job):
+    """Makes the plan in a workspace without room for made operand rows (an fp32
+    plan's: those make none)."""
+    dtype, job.desc.c.dtype = job.desc.c.dtype, B.DTYPES["f32"]
+    job.workspace = torch.empty(B.plan_workspace_size(job.desc), dtype=torch.uint8, device="cuda")
+    job.desc.c.dtype = dtype
+    job.make_plan()
+
+
+@pytest.mark.parametrize("name", sorted(BUILT))
+def test_batch_of_built_operand_rows(name):
+    """Directions whose operand rows the loader warps build, in one launch: in
+    workspaces without room for made rows, and captured."""
+    cases = [Case(w, sentinel=SENTINEL).run() for w in BUILT[name]]
+    single = [c.job.receiver.clone() for c in cases]
+    args = ([c.sender for c in cases], [c.job.receiver for c in cases])
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        B.transfer_batch([c.job.plan for c in cases], *args, torch.cuda.current_stream())
+    assert _captured_nodes(cases) == 1
+    plans = [c.job.plan for c in cases]  # the graph's
+    for c in cases:
+        c.job.plan = None
+        _without_room(c.job)
+    for launch in (g.replay, lambda: B.transfer_batch([c.job.plan for c in cases], *args)):
+        for c in cases:
+            c.job.receiver.fill_(SENTINEL)
+        launch()
+        torch.cuda.synchronize()
+        for c, ref in zip(cases, single):
+            assert c.job.device_status() == 0
+            assert torch.equal(c.job.receiver, ref), c.w.name
+    del plans
 
 
 def test_batch_mixing_layer_tables():

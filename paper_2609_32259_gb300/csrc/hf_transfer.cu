@@ -2020,9 +2020,9 @@ hf_status launch_transfer(hf_plan_s* p, const void* sender, void* receiver, cuda
   else
     HF_CUDA_TRY(cudaEventCreateWithFlags(&p->x_done, cudaEventDisableTiming), "operand rows' event");
   const hf_status s = transfer_layers(p, sender, receiver, stream, l_begin, l_end, true, stall);
-  if (s != HF_OK) return s;
+  // also when a launch failed: those before it still use the rows
   HF_CUDA_TRY(cudaEventRecord(p->x_done, stream), "record the operand rows' event");
-  return HF_OK;
+  return s;
 }
 
 bool batch_compatible(const hf_plan_s* const* plans, int n, cudaStream_t stream) {

@@ -279,21 +279,23 @@ def launches_per_step(w, pool_before_map=False):
     return align + plan + 1
 
 
-def step_launches(w, tok, pool_before_map=False, round_built=False):
+def step_launches(w, tok, pool_before_map=False, round_built=False, captured=False):
     """Kernel launches of one hf_align_build + hf_plan_create + hf_transfer: up
     to 32,768 tokens a side and 64 requests the alignment and the plan are one
-    launch each; bf16 operand rows that are computed are made by a pass before
-    each transfer launch, for as many receiver layers as 512 MB hold."""
+    launch each; bf16 operand rows that are computed are made before each
+    transfer launch, outside of captures, for as many receiver layers as 512 MB
+    hold: by one pass, or two where rotated keys and computed values differ."""
     n = launches_per_step(w, pool_before_map)
     if max(tok.T_r, tok.T_s) <= 32768 and w.n_req <= 64:
         n = 3
-    if w.dtype == "bf16" and not _copied_operands(w, pool_before_map):
+    if w.dtype == "bf16" and not captured and not _copied_operands(w, pool_before_map):
         one_role = _copied_operands(w.with_(sender_k_rotated=False), pool_before_map) and \
             w.align_mode != "overlap_mean"
         rows = tok.T_s if _pool_after_map(w, pool_before_map) else tok.T_r
         layer = (1 if one_role else 2) * max(rows, 1) * w.K * (2 if round_built else 4)
         if layer <= 4 << 29:
-            n += 2 * -(-w.L_r // min(w.L_r, max(1, (1 << 29) // layer))) - 1
+            passes = 2 if w.sender_k_rotated and not one_role else 1
+            n += (passes + 1) * -(-w.L_r // min(w.L_r, max(1, (1 << 29) // layer))) - 1
     return n
 
 
@@ -580,7 +582,8 @@ def run_ours(args):
                "sample": (f"{samp.n_rows} contiguous receiver rows x {w.L_r} layers x K/V "
                           f"of {w.name} (dense fp64 numpy oracle as written)")}
 
-    launches = step_launches(w, tok, args.pool_before_map, args.round_built_operands)
+    launches = step_launches(w, tok, args.pool_before_map, args.round_built_operands,
+                             captured=args.graph)
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world,
         "steps": args.steps, "warmup": args.warmup, "ms_per_step": step_ms,

@@ -48,3 +48,18 @@ def test_single_rank_aggregate():
     import bench
     value, out = bench.aggregate([4.0], 1000, 1)
     assert out == [4.0] and value == pytest.approx(1000 / 4e-3)
+
+
+@pytest.mark.parametrize("over,launches", [
+    (dict(), 3),                                                # align, plan, transfer
+    (dict(layer_mode="interp"), 4),                             # and a pass that makes the rows
+    (dict(sender_k_rotated=True), 4),                           # keys only: values are copies
+    (dict(sender_k_rotated=True, layer_mode="interp"), 5),      # keys and values by a pass each
+    (dict(align_mode="overlap_mean", knorm=True), 4)])
+def test_step_launches(over, launches):
+    import bench
+    from paper_2609_32259_gb300 import workloads as W
+    w = W.llama_to_ministral(300).with_(**over)
+    tok = W.tokens(w)
+    assert bench.step_launches(w, tok) == launches
+    assert bench.step_launches(w, tok, captured=True) == 3

@@ -269,6 +269,11 @@ hf_status gemm_f32(cudaStream_t s, const GemmWork& wk, int M, int N, int K, floa
                    int64_t b_j, float beta, float* C, int64_t ldc, const float* Cin = nullptr,
                    float diag = 0.f);
 
+// Tensor map of [n][rows][cols] bf16 with boxes of box_rows x 32 columns of one
+// matrix, in the 64-byte swizzle.
+hf_status bf16_strip_map(CUtensorMap* map, const void* base, uint64_t n, uint64_t rows,
+                         uint64_t cols, uint32_t box_rows);
+
 // Triangular factor of the symmetric positive definite n x n matrix W
 // (row-major, leading dimension ld, n a multiple of kFactorBlock; the blocks on
 // and above the diagonal are read): W = L L^T.  On return row i holds
@@ -277,11 +282,6 @@ hf_status gemm_f32(cudaStream_t s, const GemmWork& wk, int M, int N, int K, floa
 // n_upper.  Tt: kFactorBlock^2 floats; planes: tri_factor_planes_bytes(n).  A
 // pivot that is not above *thr sets *flag (cleared before) and the result is
 // of no use.
-// Tensor map of [n][rows][cols] bf16 with boxes of box_rows x 32 columns of one
-// matrix, in the 64-byte swizzle.
-hf_status bf16_strip_map(CUtensorMap* map, const void* base, uint64_t n, uint64_t rows,
-                         uint64_t cols, uint32_t box_rows);
-
 // Up to two matrices are factored side by side: a chain of latencies each.
 constexpr int kFactorBlock = 128;
 size_t tri_factor_planes_bytes(int n);

@@ -106,7 +106,6 @@ struct XferParams {
   // [x_rows][K] per layer of this launch and role) it holds for those tiles only.
   int split, n_batoms;  // n_batoms: B atoms (map atoms of K) per tile
   int made, made_roles;
-  const void* x;
   int64_t x_rows;
   int staged;  // split one-entry rows built by build_rows_staged
   // wide tiles (operand rows built by the loader warps, which bound those
@@ -802,19 +801,13 @@ __device__ __forceinline__ void gather_rows(const XferParams* Ps, const DirTable
       return static_cast<int64_t>(ld_dep(&lsegs->layer[s2][0]) * 2 + c) * P.s_rows;
     };
     auto seg_base = [&](int s2) -> int64_t { return seg_row(s2) * P.d_s; };
+    // rows that follow one another: their first one in maps_a, for this warp
+    const bool bulk = kBulk && (kl.made || (kRows == kCopiedRows && !P.srow));
     int64_t sbase = 0, snext = 0;
-    // made rows are whole operand rows: one base, and the residuals a plane on
-    const int64_t width = kl.made ? static_cast<int64_t>(P.n_batoms) * kBK : P.d_s;
-    const int64_t plane = P.x_rows * width;
-    if (kl.made) {
-      const int at = (l - P.l0) * P.made_roles + (P.made_roles == 2 ? c : 0);
-      sender = reinterpret_cast<const T*>(P.x) + at * (kl.split ? 2 : 1) * plane;
-    } else {
+    if (!bulk) {
       sbase = seg_base(0);
       if (n_seg > 1) snext = seg_base(1);
     }
-    // rows that follow one another: their first one in maps_a, for this warp
-    const bool bulk = kBulk && (kl.made || (kRows == kCopiedRows && !P.srow));
     int64_t first_row = 0, brow = 0;  // brow: the segment's first sender row
     bool any_row = false;
     if (bulk) {
@@ -826,7 +819,7 @@ __device__ __forceinline__ void gather_rows(const XferParams* Ps, const DirTable
         k0 = static_cast<int64_t>(m) * kTileRows + row0 + slab * 32;
         any_row = k0 < U;
       }
-      if (kl.made) {
+      if (kl.made) {  // planes of whole operand rows, the residuals' after the values'
         const int at = (l - P.l0) * P.made_roles + (P.made_roles == 2 ? c : 0);
         k0 += at * (kl.split ? 2 : 1) * P.x_rows;
       }
@@ -845,14 +838,14 @@ __device__ __forceinline__ void gather_rows(const XferParams* Ps, const DirTable
       int64_t kr;  // sender-cache row
       if (pam_on<kPam>(P)) {
         const int k = pam_token(P, m, row0, r);
-        kr = P.srow && !kl.made ? ld_dep(P.srow + k) : k;
+        kr = P.srow ? ld_dep(P.srow + k) : k;
         live |= 1u << i;
       } else {
         const int u = m * kTileRows + row0 + r;
-        kr = kl.made ? min(u, U - 1) : P.ucol[min(u, U - 1)];
+        kr = P.ucol[min(u, U - 1)];
         live |= (u < U ? 1u : 0u) << i;
       }
-      roff[i] = kr * width + ch * kPerChunk;
+      roff[i] = kr * P.d_s + ch * kPerChunk;
       doff[i] = static_cast<uint32_t>(r * 128 + ((ch ^ (r & 7)) << 4));
     }
     int seg = 0, kin = 0;  // segment of the next atom, and the atom within it
@@ -904,14 +897,10 @@ __device__ __forceinline__ void gather_rows(const XferParams* Ps, const DirTable
       for (int a = 0; a < kAtoms; ++a) {
         if (a < na) {
           const T* base = sender + sbase + kin * kBK;
-          if (kl.split && a == 1) base += plane - kBK;  // the residuals of the same atom
 #pragma unroll
           for (int i = 0; i < 8; ++i)
             if (live >> i & 1u) cp_async_16(sa + a * kAtomABytes + doff[i], base + roff[i]);
-          ++kin;
-          if (kl.made) {
-            if (kl.split && a == 1) --kin;
-          } else if (kin == P.atoms_per_seg) {
+          if (++kin == P.atoms_per_seg) {
             kin = 0;
             ++seg;
             sbase = snext;
@@ -1905,7 +1894,6 @@ hf_status make_xfer(hf_plan_s* p, const void* sender, void* receiver, int l_begi
   P.n_batoms = n_atoms;
   P.made = made ? p->made : 0;
   P.made_roles = p->made == 3 ? 2 : 1;
-  P.x = made ? ws + p->lay.xbuf : nullptr;
   P.x_rows = p->x_rows;
   P.atoms_per_seg = p->d_s / bk;
   P.BN = p->BN;

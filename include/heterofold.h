@@ -406,6 +406,7 @@ hf_status hf_transfer_noalloc(const hf_plan_desc* desc, const void* sender_kv,
  * d_W_final: device, like d_W (may be d_W itself: folded in place);
  *            rounded once to `dtype`.
  * d_b_final: device float[n_maps][d_R] (may be d_b).
+ * Infinities and NaN come out as plain fp32 sums give them.
  * rank 4, 8, 16 or 32 (the paper uses 16); K even; d_W, d_W_final and
  * d_B 16-byte aligned.  Asynchronous on `stream`.
  */

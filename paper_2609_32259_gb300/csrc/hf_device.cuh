@@ -266,6 +266,12 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
+// Orders this thread's accesses through the generic and the async proxy, in any
+// memory.
+__device__ __forceinline__ void fence_proxy_async_all() {
+  asm volatile("fence.proxy.async;" ::: "memory");
+}
+
 // ---------------------------------------------------------------------------
 // cp.async.bulk (shared -> global copies of whole rows by the copy engine)
 // ---------------------------------------------------------------------------

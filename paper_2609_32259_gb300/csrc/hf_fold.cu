@@ -257,6 +257,12 @@ constexpr int kMmaCols = 32;            // columns of W per unit of work
 constexpr int kMmaRows = 1024;          // d_R at most: 64 rows per warp
 constexpr int kTStride = kMmaCols + 8;  // padded row of T: 80 bytes, no bank twice
 constexpr int kPartStride = kMmaCols + 4;
+constexpr int kMmaUnits = 8192;         // units of one CTA at most
+// What sums of split products cannot give: an infinity times a part that is zero is
+// NaN, and so is the residual of a value that rounds to an infinity in bf16.
+// Columns whose T is not finite or above this, and maps with a G above it, take
+// fp32 arithmetic (products of the rest stay below 2^124).
+constexpr float kMmaRange = 0x1p60f;
 
 __device__ __forceinline__ void mma_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0,
                                           uint32_t b1) {
@@ -294,8 +300,45 @@ struct FoldMmaSmem {
   __nv_bfloat16 w[2][kMmaRows][kMmaCols];
   float part[kMmaWarps][16][kPartStride];
   __nv_bfloat16 t[3][16][kTStride];
+  float tf[16][kMmaCols];   // fold_plain_columns' T
+  unsigned plain[2];        // columns that fold_plain_columns does: this unit's, the next one's
+  unsigned redo[kMmaUnits]; // and every unit's of this CTA
 };
 static_assert(kMmaCols == 32, "the 64-byte swizzle is over rows of 32");
+
+__device__ __forceinline__ bool above(float x, float limit) { return !(fabsf(x) <= limit); }
+
+// The columns `mask` of the strip at column k0 of one map, whose W_final still is
+// W, with plain fp32 sums in fold_kernel's order.  All threads of the CTA.
+__device__ __forceinline__ void fold_plain_columns(FoldMmaSmem& sm, __nv_bfloat16* Wf, const float* B,
+                                                   const float* G, int d_r, int64_t K, int rank,
+                                                   int64_t k0, unsigned mask) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool mine = mask >> lane & 1u;
+  __nv_bfloat16* const col = Wf + k0 + lane;
+  __syncthreads();
+  if (mine && warp < rank) {
+    float t = 0.f;
+#pragma unroll 1
+    for (int s = 0; s < kFoldSlices; ++s) {
+      float acc = 0.f;
+#pragma unroll 1
+      for (int m = s; m < d_r; m += kFoldSlices)
+        acc = fmaf(B[static_cast<int64_t>(m) * rank + warp], __bfloat162float(col[m * K]), acc);
+      t += acc;
+    }
+    sm.tf[warp][lane] = t;
+  }
+  __syncthreads();
+  if (!mine) return;
+#pragma unroll 1
+  for (int n = warp; n < d_r; n += kMmaWarps) {
+    float v = __bfloat162float(col[n * K]);
+#pragma unroll 1
+    for (int r = 0; r < rank; ++r) v = fmaf(G[static_cast<int64_t>(r) * d_r + n], sm.tf[r][lane], v);
+    col[n * K] = __float2bfloat16_rn(v);
+  }
+}
 
 // A persistent CTA takes a run of units (map, 32 columns).  Warp w owns rows 16
 // steps w .. of W (steps <= 4 blocks of 16): it alone copies them in, works on
@@ -314,9 +357,12 @@ static_assert(kMmaCols == 32, "the 64-byte swizzle is over rows of 32");
 // rate allows 5.6K.  With the rows written out by the threads a unit took 13K
 // (4.1K of them in those stores; 80 maps of 1,024 x 3,072: 358 us, 254 now).
 // Step 1 of a unit before step 3 of the one before it exposed the copies.
+// Columns that need fp32 arithmetic (kMmaRange) leave as they came and are done
+// after the run: any of it inside the loop cost 55 us, the looking costs 1.
 __global__ void __launch_bounds__(32 * kMmaWarps)
     fold_mma_kernel(const __nv_bfloat16* W, const float* __restrict__ Bm,
-                    const float* __restrict__ Gm, const __grid_constant__ CUtensorMap map_out,
+                    const float* __restrict__ Gm, __nv_bfloat16* Wf,
+                    const __grid_constant__ CUtensorMap map_out,
                     int n_maps, int d_r, int64_t K, int rank, int steps) {
   extern __shared__ __align__(1024) uint8_t fold_smem[];
   FoldMmaSmem& sm = *reinterpret_cast<FoldMmaSmem*>(fold_smem);
@@ -348,6 +394,9 @@ __global__ void __launch_bounds__(32 * kMmaWarps)
     fold_cp_commit();
   };
   load(u0);
+  if (tid < 2) sm.plain[tid] = 0;
+  bool big_g = false;    // this thread's part of G has a value above kMmaRange
+  unsigned any = 0;      // columns left to fold_plain_columns
   uint32_t bf[4][3][4];  // B^T, rank x 16 rows per step, split
   uint32_t gf[4][3][4];  // G^T, 16 rows x rank per step, split
   int map_now = -1;
@@ -360,6 +409,7 @@ __global__ void __launch_bounds__(32 * kMmaWarps)
     auto& w = sm.w[buf];
     if (map != map_now) {
       map_now = map;
+      big_g = false;
       const float* const B = Bm + static_cast<int64_t>(map) * d_r * rank;
       const float* const G = Gm + static_cast<int64_t>(map) * rank * d_r;
       auto at_b = [&](int n, int r) { return n < d_r && r < rank ? __ldg(B + n * rank + r) : 0.f; };
@@ -374,7 +424,12 @@ __global__ void __launch_bounds__(32 * kMmaWarps)
           split3(at_b(c, r), at_b(c + 1, r), &bf[s][0][i], &bf[s][1][i], &bf[s][2][i]);
           // G^T: W row g (+8), rank columns 2t (+8)
           const int n = row0 + 16 * s + g + 8 * (i & 1), q = 2 * t + 8 * (i >> 1);
-          split3(at_g(n, q), at_g(n, q + 1), &gf[s][0][i], &gf[s][1][i], &gf[s][2][i]);
+          float g0 = at_g(n, q), g1 = at_g(n, q + 1);
+          if (above(g0, kMmaRange) || above(g1, kMmaRange)) {
+            big_g = true;
+            g0 = g1 = 0.f;
+          }
+          split3(g0, g1, &gf[s][0][i], &gf[s][1][i], &gf[s][2][i]);
         }
       }
     }
@@ -407,12 +462,16 @@ __global__ void __launch_bounds__(32 * kMmaWarps)
       __syncwarp();
       load(u + 1);
     }
-    __syncthreads();
+    const bool big_map = __syncthreads_or(big_g);
     {
       // step 2
+      if (tid == 0) sm.plain[buf ^ 1] = 0;
       float x = 0.f;  // T[warp][lane]
 #pragma unroll
       for (int q = 0; q < kMmaWarps; ++q) x += sm.part[q][warp][lane];
+      const unsigned redo =
+          __ballot_sync(0xffffffffu, warp < rank && (big_map || above(x, kMmaRange)));
+      if (redo && lane == 0) atomicOr(&sm.plain[buf], redo);
       const __nv_bfloat16 h0 = __float2bfloat16_rn(x);
       x -= __bfloat162float(h0);
       const __nv_bfloat16 h1 = __float2bfloat16_rn(x);
@@ -421,6 +480,14 @@ __global__ void __launch_bounds__(32 * kMmaWarps)
       sm.t[2][warp][lane] = __float2bfloat16_rn(x - __bfloat162float(h1));
     }
     __syncthreads();
+    const unsigned plain = sm.plain[buf];
+    if (tid == 0) sm.redo[u - u0] = plain;
+    any |= plain;
+    if (plain) {  // without T these columns leave as they came
+      if (plain >> lane & 1u)
+        sm.t[0][warp][lane] = sm.t[1][warp][lane] = sm.t[2][warp][lane] = __nv_bfloat16(0.f);
+      __syncthreads();
+    }
     {
       // step 3
 #pragma unroll
@@ -461,6 +528,19 @@ __global__ void __launch_bounds__(32 * kMmaWarps)
   if (lane == 0) {
     bulk_store_wait_read();
     bulk_store_wait_all();
+  }
+  if (any) {
+    fence_proxy_async_all();
+    __syncthreads();  // the strips have been written
+#pragma unroll 1
+    for (int64_t u = u0; u < u1; ++u) {
+      const int64_t map = u / per_map, k0 = (u - map * per_map) * kMmaCols;
+      unsigned mask = sm.redo[u - u0];
+      if (K - k0 < kMmaCols) mask &= (1u << (K - k0)) - 1u;
+      if (mask)
+        fold_plain_columns(sm, Wf + map * d_r * K, Bm + map * d_r * rank, Gm + map * rank * d_r, d_r,
+                           K, rank, k0, mask);
+    }
   }
 }
 
@@ -559,13 +639,14 @@ hf_status launch_fold(int n_maps, int d_r, int64_t K, int rank, const void* W, c
                                      static_cast<int>(sizeof(FoldMmaSmem))),
                 "hf_fold: shared memory size");
     const int64_t units = n_maps * ((K + kMmaCols - 1) / kMmaCols);
-    const int grid = static_cast<int>(std::min<int64_t>(units, device_sm_count()));
+    const int grid = static_cast<int>(std::max<int64_t>(
+        std::min<int64_t>(units, device_sm_count()), (units + kMmaUnits - 1) / kMmaUnits));
     const int steps = (d_r + 16 * kMmaWarps - 1) / (16 * kMmaWarps);
     CUtensorMap map_out;
     s = bf16_strip_map(&map_out, Wf, n_maps, d_r, K, 16 * steps);
     if (s != HF_OK) return s;
     fold_mma_kernel<<<grid, 32 * kMmaWarps, sizeof(FoldMmaSmem), stream>>>(
-        static_cast<const __nv_bfloat16*>(W), B, G, map_out, n_maps, d_r, K, rank, steps);
+        static_cast<const __nv_bfloat16*>(W), B, G, static_cast<__nv_bfloat16*>(Wf), map_out, n_maps, d_r, K, rank, steps);
     HF_CUDA_TRY(cudaGetLastError(), "hf_fold: launch");
   } else
   switch (rank) {

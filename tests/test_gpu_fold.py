@@ -149,3 +149,39 @@ def test_fold_infinity_stays_in_its_column():
     assert not torch.isfinite(got[:, 3, cols]).any()
     got[:, :, cols] = clean[:, :, cols]
     assert torch.equal(got, clean)
+
+
+@pytest.mark.parametrize("d_R,rank,in_place", [(1000, 8, True), (128, 16, False), (270, 4, True)])
+def test_fold_keeps_infinities(d_R, rank, in_place):
+    """Infinities and NaN of W, factors that are exact in bf16 (whose residual parts
+    are zero) and factors that overflow bf16: the tensor-core form gives infinities,
+    NaN and finite values where the fp32 form does."""
+    dev = torch.device("cuda")
+    n_maps, K = 3, 40 * 152 + 8  # a last strip of eight columns
+    g = torch.Generator(device="cpu").manual_seed(d_R)
+    Wm = (torch.randn((n_maps, d_R, K), generator=g) / np.sqrt(K)).to(torch.bfloat16)
+    Bm, Gm = _factors(n_maps, d_R, rank, 6, "cpu")
+    Bm[0, 3], Gm[0] = 0.5, Gm[0].abs()  # one sign: infinite, not NaN
+    Bm[1, 3] = Bm[1, 3].to(torch.bfloat16).float()
+    Bm[2, 5], Gm[2, 0, 7] = 3.4e38, 3.4e38  # infinite when rounded to bf16
+    Wm[2, 5], Wm[2, :, ::3] = 2.0**-120, 2.0**-120
+    for m in range(2):
+        Wm[m, 3, 1::50] = float("inf")
+        Wm[m, 3, 7::50] = -float("inf")
+        Wm[m, d_R - 1, 11::50] = float("nan")
+    Wm, Bm, Gm = Wm.to(dev), Bm.to(dev), Gm.to(dev)
+    b = torch.zeros((n_maps, d_R), device=dev)
+    got = Wm.clone() if in_place else torch.empty_like(Wm)
+    plain, bf = torch.empty(Wm.shape, device=dev), torch.empty_like(b)
+    B.fold("bf16", got if in_place else Wm, b, Bm, Gm, got, bf)
+    B.fold("f32", Wm.float(), b, Bm, Gm, plain, bf)
+    torch.cuda.synchronize()
+    plain = plain.to(torch.bfloat16)
+    assert torch.isposinf(got[0, :, 1::50]).all() and torch.isneginf(got[0, :, 7::50]).all()
+    assert torch.equal(torch.isnan(got), torch.isnan(plain))
+    inf = torch.isinf(plain)
+    assert torch.equal(torch.isinf(got), inf) and torch.equal(got[inf], plain[inf])
+    finite = torch.isfinite(plain)
+    diff = (got[finite].double() - plain[finite].double()).abs()
+    # both are rounded once: at most a bf16 ulp apart, beside the fp32 sums
+    assert (diff <= 2.0**-7 * plain[finite].double().abs() + 1e-6).all()

@@ -45,8 +45,11 @@ def _results(w, extra, **opts):
     return out
 
 
-# one CTA up to 4,096 tokens, eight above, the passes above 32,768
-SIZES = [(1,), (4093,), (4097,), (32760,), (130, 1, 5000), tuple([37] * 64)]
+# one CTA up to 1,024 tokens on the longer side (here the receiver's), eight above,
+# four rows a thread above 8,192, the passes above 32,768; requests that start and end
+# inside one thread's rows
+SIZES = [(1,), (1024,), (1025,), (300, 1, 2, 500), (4093,), (4097,), (8192,), (8193,), (32760,),
+         (32768,), (130, 1, 5000), (3, 1, 9000, 2, 1, 1, 3, 700, 1, 2), tuple([37] * 64)]
 FORMS = {
     "ta": {}, "ta_paged": dict(paged=True), "ta_span": dict(span_gap=11),
     "ta_rotated": dict(sender_k_rotated=True), "same_index": dict(align_mode="same_index"),

@@ -288,7 +288,8 @@ def step_launches(w, tok, pool_before_map=False, round_built=False, captured=Fal
     n = launches_per_step(w, pool_before_map)
     if max(tok.T_r, tok.T_s) <= 32768 and w.n_req <= 64:
         n = 3
-    if w.dtype == "bf16" and not captured and not _copied_operands(w, pool_before_map):
+    if (w.dtype == "bf16" and not captured and not _copied_operands(w, pool_before_map)
+            and _made_rows_pay(w, tok, pool_before_map, round_built)):
         one_role = _copied_operands(w.with_(sender_k_rotated=False), pool_before_map) and \
             w.align_mode != "overlap_mean"
         rows = tok.T_s if _pool_after_map(w, pool_before_map) else tok.T_r
@@ -297,6 +298,24 @@ def step_launches(w, tok, pool_before_map=False, round_built=False, captured=Fal
             passes = 2 if w.sender_k_rotated and not one_role else 1
             n += (passes + 1) * -(-w.L_r // min(w.L_r, max(1, (1 << 29) // layer))) - 1
     return n
+
+
+def _made_rows_pay(w, tok, pool_before_map, round_built):
+    """The library's rule for computed rows (made_rows_pay of hf_plan.cu)."""
+    passes = w.d_r // (512 if w.d_r % 512 == 0 else 256 if w.d_r % 256 == 0 else 128)
+    if w.sender_k_rotated or passes > 2:
+        return True
+    after = _pool_after_map(w, pool_before_map)
+    rows = (tok.T_s if after else min(tok.T_s, tok.T_r) if w.align_mode == "same_index"
+            else tok.T_r * 28 // 100 if w.align_mode == "ta" else tok.T_r)
+    staged = (after or w.align_mode != "overlap_mean") and not round_built
+    small = rows * w.K <= 16000000
+    if passes == 2:
+        return small or not staged
+    tiles = 2 * w.L_r * -(-rows // 256)
+    rounds = -(-tiles // 76)
+    return small if not staged else 2 * tiles <= 76 or (
+        w.K <= 1024 and rounds <= 3 and 4 * tiles <= 3 * 76 * rounds)
 
 
 def _copied_operands(w, pool_before_map=False):

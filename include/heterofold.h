@@ -267,8 +267,8 @@ typedef struct hf_plan_s* hf_plan;
 /* Bytes of device workspace hf_plan_create needs for this descriptor.  For
  * bf16 plans whose map input rows are computed (interpolated or weighted
  * layers, pooling before the map, sender_k_rotated) they include room for
- * those rows, at most 512 MB or one receiver layer's: hf_transfer makes them
- * in a pass of their own.  Where one layer's would take over 2 GiB, in a
+ * those rows where that is the faster way, at most 512 MB or one receiver
+ * layer's: hf_transfer makes them in a pass of their own.  Where one layer's would take over 2 GiB, in a
  * workspace without that room (as many bytes as the same plan in fp32 needs)
  * and in captured transfers, the transfer kernel computes them itself, slower,
  * to the same bits. */

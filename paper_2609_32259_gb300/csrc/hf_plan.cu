@@ -47,6 +47,39 @@ struct OperandPath {
   int made;  // roles whose rows a pass of their own makes (hf_plan_s::made)
   int64_t K;
 };
+
+// Whether computed rows are sooner made by a pass of their own than built by the
+// loader warps, which build a row once for every 512 columns (d_R a multiple of 512)
+// or BN columns of the receiver: once up to d_R = 512.  Transfers alone, made and
+// built, rows distinct, 8 layers: rotated keys 4 to 6 times faster made; three passes
+// and more 1.2 to 2.2 times (d_R 2,048, K 1,024, 16K rows 1.64 and 2.45 ms).  Blends
+// (one sender token, two bf16 parts: staged by cp.async) in two passes (d_R 1,024):
+// 8K rows 0.54 and 0.63 ms at K 1,024, 1.56 and 1.61 at 3,072, but 3.42 and 3.06 at
+// 6,144.  In one pass only while the tiles leave half of the SM pairs idle (d_R 512, K
+// 3,072, 512 rows 0.094 and 0.133 ms, 1,024 rows 0.158 and 0.135, 16K rows 2.62 and
+// 1.61) or, up to K = 1,024, in at most three rounds, a quarter of the last idle
+// (28 layers, 566 rows 168 tiles, 1.27 times faster made, 352 rows 1.30; but 720 rows
+// 0.93, and 906 rows, 224 tiles, 0.99).  Pooled rows, built in registers, in one pass: 4K rows 0.63 and 0.73 ms (d_R
+// 512, K 3,072), 7.5K rows 1.58 and 1.49.
+bool made_rows_pay(const hf_plan_desc& d, const OperandPath& o) {
+  const int64_t d_r = static_cast<int64_t>(d.H_r) * d.D_r;
+  const int64_t passes = d_r % 512 == 0 ? d_r / 512 : d_r / (d_r % 256 == 0 ? 256 : 128);
+  if (d.sender_k_rotated == 1 || passes > 2) return true;
+  const int64_t T_s = d.s_tok_ptr[d.n_req], T_r = d.r_tok_ptr[d.n_req];
+  // distinct rows to be expected: with Token Alignment a quarter or so
+  const int64_t rows = o.pam                                   ? T_s
+                       : d.align_mode == HF_ALIGN_SAME_INDEX ? std::min(T_s, T_r)
+                       : d.align_mode == HF_ALIGN_TA         ? T_r * 28 / 100
+                                                             : T_r;
+  const bool staged = o.one_entry && o.split, small = rows * o.K <= 16000000;
+  if (passes == 2) return !staged || small;
+  const int64_t pairs = 76, tiles = 2 * d.L_r * ((rows + 255) / 256);
+  const int64_t rounds = (tiles + pairs - 1) / pairs;
+  return !staged ? small
+                 : 2 * tiles <= pairs ||
+                       (o.K <= 1024 && rounds <= 3 && 4 * tiles <= 3 * pairs * rounds);
+}
+
 OperandPath operand_path(const hf_plan_desc& d) {
   OperandPath o{};
   // hf_plan_workspace_size has not validated the descriptor, and gives one that
@@ -77,7 +110,7 @@ OperandPath operand_path(const hf_plan_desc& d) {
   const bool copies = one_layer_segments && o.one_entry;  // values, and keys if not rotated
   o.gather = copies && !unrot;
   o.split = !o.gather && d.dtype == HF_BF16 && d.round_built_operands == 0;
-  if (!o.gather && d.dtype == HF_BF16 && o.K > 0) o.made = copies ? 1 : 3;
+  if (!o.gather && d.dtype == HF_BF16 && o.K > 0 && made_rows_pay(d, o)) o.made = copies ? 1 : 3;
   return o;
 }
 

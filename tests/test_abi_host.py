@@ -118,6 +118,44 @@ def test_workspace_size_of_refused_descriptors(B, over):
     assert st in (B.HF_ERR_INVALID_ARGUMENT, B.HF_ERR_UNSUPPORTED)
 
 
+@pytest.mark.parametrize("over,made", [
+    # d_R 512, blends: half of the 76 SM pairs (16 tiles a block of 256 rows), or K up to
+    # 1,024, at most three rounds of tiles and a quarter of the last idle
+    (dict(), True), (dict(L_r=19, tokens=256), True), (dict(L_r=29, tokens=256), False),
+    (dict(tokens=768), True), (dict(tokens=769), False), (dict(tokens=1025), True),
+    (dict(L_r=58, tokens=256), False), (dict(L_r=57, tokens=256), True), (dict(L_r=85, tokens=256), True),
+    (dict(L_r=86, tokens=256), False), (dict(L_r=10, tokens=3000), False),
+    (dict(H_s=16, tokens=512), True), (dict(H_s=16, tokens=513), False),
+    (dict(align_mode="ta", tokens=1828), True), (dict(align_mode="ta", tokens=2747), False),
+    (dict(align_mode="overlap_mean"), True), (dict(align_mode="overlap_mean", tokens=769), False),
+    # d_R 1,024: rows x K up to 16 M
+    (dict(H_r=8, tokens=15625), True), (dict(H_r=8, tokens=15626), False),
+    (dict(H_r=6, tokens=15626), True),                                  # three passes
+    (dict(round_built_operands=True, tokens=15625), True),              # rounded once
+    (dict(round_built_operands=True, tokens=15626), False),
+    (dict(align_mode="overlap_mean", pool_before_map=True, tokens=15625), True),
+    (dict(align_mode="overlap_mean", pool_before_map=True, tokens=15626), False),
+    (dict(align_mode="overlap_mean", pool_before_map=True, H_r=8, tokens=15626), True),
+    (dict(sender_k_rotated=True, theta_s=1e4, tokens=15626), True)])
+def test_room_for_made_rows_follows_their_rule(B, over, made):
+    import bench
+    from paper_2609_32259_gb300 import workloads as W
+    over = dict(over)
+    T, lr = over.pop("tokens", 512), over.get("L_r", 8)
+    kw = dict(L_s=16, H_s=8, D_s=128, L_r=lr, H_r=4, D_r=128, layer_mode="interp",
+              align_mode="same_index", s_tok_ptr=[0, T], r_tok_ptr=[0, T], r=np.ones((lr, 2)))
+    kw.update(over)
+    base = B.plan_workspace_size(_desc(B, **dict(kw, dtype="f32")))
+    assert (B.plan_workspace_size(_desc(B, **kw)) > base) == made
+    # bench.py counts the launches by the same rule
+    w = W.llama_to_ministral(T).with_(
+        layer_mode="interp", L_s=16, H_s=kw["H_s"], L_r=lr, H_r=kw["H_r"], align_mode=kw["align_mode"],
+        sender_k_rotated=kw.get("sender_k_rotated", False))
+    tok = W.Tokens(*(np.array([0, T], np.int32),) * 2, np.zeros(T), np.zeros(T))
+    assert bench._made_rows_pay(w, tok, kw.get("pool_before_map", False),
+                                kw.get("round_built_operands", False)) == made
+
+
 def test_workspace_grows_with_tokens(B):
     a = B.plan_workspace_size(_desc(B, r_tok_ptr=[0, 6]))
     b = B.plan_workspace_size(_desc(B, r_tok_ptr=[0, 60000]))

@@ -32,6 +32,8 @@ BATCH = W.qwen25_to_llama_batched(n_req=3, lo=30, hi=400, seed=5).with_(L_s=4, L
 CASES = {
     "interp_one_token": (L(1, layer_mode="interp"), {}),
     "interp_129": (L(129, layer_mode="interp"), {}),
+    "interp_one_wide_tile": (L(600, H_r=4, layer_mode="interp"), {}),
+    "pooled_one_wide_tile": (L(300, H_r=4, align_mode="overlap_mean"), dict(pool_before_map=True)),
     "interp_same_index": (L(517, layer_mode="interp", align_mode="same_index"), {}),
     "interp_overlap": (L(700, layer_mode="interp", align_mode="overlap_mean"), {}),
     "interp_round_once": (L(300, layer_mode="interp"), dict(round_built_operands=True)),

@@ -5,7 +5,7 @@
 //   W_final = W + G^T T            (element [n][k] += sum_r G[r][n] T[r][k])
 //   b_final = b + (b B) G.
 // Two forms.  fold_mma_kernel (bf16 maps, rank <= 16, d_R <= 1,024, K a multiple
-// of 8) reads W once: the 4 rank FLOP per element outweigh the memory time on
+// of 8, where it is the faster: see launch_fold) reads W once: the 4 rank FLOP per element outweigh the memory time on
 // the fp32 ALUs, so both contractions run on the warp-level tensor
 // instructions, with every fp32 factor split exactly into three bf16 parts and
 // the products above 2^-23 kept (a rank of 16 is one 16-deep step: too thin for
@@ -629,19 +629,26 @@ hf_status launch_fold(int n_maps, int d_r, int64_t K, int rank, const void* W, c
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   hf_status s = HF_OK;
-  // the tensor-core form where its units fit; in fp32 the maps need more than
-  // bf16 products of an exact W, and two 16-deep steps of rank 32 more registers
-  // than a warp's share of B and G leaves
-  const bool mma = sizeof(T) == 2 && (rank == 4 || rank == 8 || rank == 16) && d_r <= kMmaRows &&
-                   K % 8 == 0 && sizeof(FoldMmaSmem) <= static_cast<size_t>(optin);
+  // the tensor-core form where its units fit and its chain of steps, about as long for
+  // few rows and a low rank as for many, is the shorter way (tensor-core and fp32 form,
+  // K 3,072, 80 maps: rank 16, d_R 1,024 253 and 484 us, 192 119 and 124, 128 118 and 98;
+  // rank 8, 1,024 249 and 299, 640 206 and 194; rank 4, 1,024 248 and 243, 256 124 and
+  // 71; one map of 1,024 x 3,072, rank 4: 14 and 26); in fp32 the maps need more than
+  // bf16 products of an exact W, and two 16-deep steps of rank 32 more registers than
+  // a warp's share of B and G leaves
+  const int64_t units = n_maps * ((K + kMmaCols - 1) / kMmaCols);
+  const int steps = (d_r + 16 * kMmaWarps - 1) / (16 * kMmaWarps);
+  static constexpr int kLeast[4] = {3072, 4608, 6144, 7040};  // rank d_R, by steps
+  const bool fits = sizeof(T) == 2 && (rank == 4 || rank == 8 || rank == 16) && d_r <= kMmaRows &&
+                    K % 8 == 0 && sizeof(FoldMmaSmem) <= static_cast<size_t>(optin);
+  const bool mma =
+      fits && rank * d_r >= (units <= device_sm_count() ? 768 : kLeast[steps - 1]);
   if (mma) {
     HF_CUDA_TRY(cudaFuncSetAttribute(fold_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      static_cast<int>(sizeof(FoldMmaSmem))),
                 "hf_fold: shared memory size");
-    const int64_t units = n_maps * ((K + kMmaCols - 1) / kMmaCols);
     const int grid = static_cast<int>(std::max<int64_t>(
         std::min<int64_t>(units, device_sm_count()), (units + kMmaUnits - 1) / kMmaUnits));
-    const int steps = (d_r + 16 * kMmaWarps - 1) / (16 * kMmaWarps);
     CUtensorMap map_out;
     s = bf16_strip_map(&map_out, Wf, n_maps, d_r, K, 16 * steps);
     if (s != HF_OK) return s;

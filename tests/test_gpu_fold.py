@@ -59,7 +59,10 @@ def test_fold_matches_oracle(dtype, in_place):
 # units than SMs; a d_R, a K and a rank past it (the other form).
 @pytest.mark.parametrize("n_maps,d_R,K,rank", [
     (1, 1, 8, 4), (3, 270, 40, 8), (2, 1024, 104, 16), (1, 1008, 3080, 16), (9, 128, 1024, 16),
-    (1, 1040, 64, 16), (2, 64, 36, 16), (2, 64, 64, 32)])
+    (1, 1040, 64, 16), (2, 64, 36, 16), (2, 64, 64, 32),
+    # both sides of the rule: one round of units, and several for one to four blocks of rows
+    (1, 191, 4096, 4), (1, 192, 4096, 4), (1, 192, 4904, 4), (9, 191, 1024, 16), (9, 192, 1024, 16),
+    (5, 287, 2000, 16), (5, 288, 2000, 16), (3, 768, 2056, 8), (3, 880, 2056, 8), (3, 879, 2056, 8)])
 def test_fold_bf16_units(n_maps, d_R, K, rank):
     dev = torch.device("cuda")
     g = torch.Generator(device="cpu").manual_seed(d_R + K)
@@ -151,13 +154,14 @@ def test_fold_infinity_stays_in_its_column():
     assert torch.equal(got, clean)
 
 
-@pytest.mark.parametrize("d_R,rank,in_place", [(1000, 8, True), (128, 16, False), (270, 4, True)])
-def test_fold_keeps_infinities(d_R, rank, in_place):
+@pytest.mark.parametrize("d_R,rank,K,in_place", [
+    (1000, 8, 6088, True), (256, 16, 6088, False), (300, 16, 6088, True), (270, 4, 1288, False)])
+def test_fold_keeps_infinities(d_R, rank, K, in_place):
     """Infinities and NaN of W, factors that are exact in bf16 (whose residual parts
     are zero) and factors that overflow bf16: the tensor-core form gives infinities,
     NaN and finite values where the fp32 form does."""
     dev = torch.device("cuda")
-    n_maps, K = 3, 40 * 152 + 8  # a last strip of eight columns
+    n_maps = 3  # a last strip of eight columns each
     g = torch.Generator(device="cpu").manual_seed(d_R)
     Wm = (torch.randn((n_maps, d_R, K), generator=g) / np.sqrt(K)).to(torch.bfloat16)
     Bm, Gm = _factors(n_maps, d_R, rank, 6, "cpu")

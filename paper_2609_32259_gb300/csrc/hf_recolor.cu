@@ -664,11 +664,22 @@ hf_status recolor_typed(int64_t N, int dx, int dy, const void* Xv, const void* Y
     HF_CUDA_TRY(cudaGetLastError(), "hf_recolor_fit: ridge launch");
     return HF_OK;
   };
-  auto extract = [&](const float* S, int rows, int cols, int mode, float* out) {
+  auto extract_ld = [&](const float* S, int64_t ld, int rows, int cols, int mode, float* out) {
     rc_extract_kernel<<<dim3((cols + 255) / 256, std::min(rows, 1024)), 256, 0, s>>>(
-        S, L.F, rows, cols, mode, out);
+        S, ld, rows, cols, mode, out);
+  };
+  auto extract = [&](const float* S, int rows, int cols, int mode, float* out) {
+    extract_ld(S, L.F, rows, cols, mode, out);
   };
   if ((st = moments()) != HF_OK) return st;
+  // no pivot is below the ridge but for rounding: with a larger one the roots are not
+  // to be expected, and taking the moments again (2.5 ms of a fit of 32,768 x 3,072 ->
+  // 1,024 with roots, 20.5 ms) is dearer than these copies only then
+  const bool kept = reg < 2.f * kPivot;
+  if (kept) {
+    extract(G, dx, dx, 0, F(L.p1));
+    extract(GY, dy, dy, 0, F(L.p2));
+  }
   HF_CUDA_TRY(cudaMemsetAsync(flag, 0, sizeof(int32_t), s), "clear");
   HF_CUDA_TRY(cudaMemsetAsync(F(L.sy_h), 0, sizeof(float) * dy * dy, s), "clear");
   const TriProblem tri[2] = {
@@ -683,9 +694,13 @@ hf_status recolor_typed(int64_t N, int dx, int dy, const void* Xv, const void* Y
   int it1 = 1, it2 = 1, it3 = 0;
   const int64_t left_i = weak ? dx : 1, left_k = weak ? 1 : dx;  // left root: symmetric, or L^{-T}
   if (weak) {
-    if ((st = moments()) != HF_OK) return st;
-    extract(G, dx, dx, 1, F(L.sz));
-    extract(GY, dy, dy, 1, F(L.sy));
+    if (!kept) {
+      if ((st = moments()) != HF_OK) return st;
+      extract(G, dx, dx, 0, F(L.p1));
+      extract(GY, dy, dy, 0, F(L.p2));
+    }
+    extract_ld(F(L.p1), dx, dx, dx, 1, F(L.sz));
+    extract_ld(F(L.p2), dy, dy, dy, 1, F(L.sy));
     extract(G + L.np, dx, dy, 0, F(L.szy));
     if ((st = ns_sqrt(s, h, F(L.sz), dx, reg, F(L.p1), F(L.p2), F(L.p3), F(L.p4), nullptr,
                       F(L.sz_ih), dscr, &it1)) != HF_OK)

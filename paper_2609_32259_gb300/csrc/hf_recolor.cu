@@ -62,12 +62,11 @@ __device__ __forceinline__ float ld(const float* p) { return *p; }
 // Column sums of w [X | Y] and, from X, sum w and sum w |x|^2, in two passes.
 // rc_stats_kernel: a warp takes every eighth row of the block's slice and
 // 32 V columns per read, four reads of two rows in flight; one fp32 sum takes at
-// most 128 values (GB300's fp64 rate is a small fraction of fp32's): a column's
-// rows of a slice, up to 67 M samples, and kStatRows rows of the squares, and
-// the block's partial sums go out as fp64; rc_stats_sum_kernel adds the slices.
+// most 128 values, the rows of a slice, up to 67 M samples (GB300's fp64 rate is a
+// small fraction of fp32's), the squares of a row's 4 V values being summed before,
+// and the block's partial sums go out as fp64; rc_stats_sum_kernel adds the slices.
 // Bounded by reading X and Y once.  (fp64 atomics in the place of the partial
 // sums took 0.36 ms for 0.27 GB.)
-constexpr int kStatRows = 16;
 inline int stat_slices(int64_t N) {
   const int64_t fill = std::min<int64_t>((N + 63) / 64, 128);
   return static_cast<int>(std::min<int64_t>(std::max(fill, (N + 1023) / 1024), 65535));
@@ -90,39 +89,35 @@ __global__ void __launch_bounds__(256)
   const T* const M = is_x ? X : Y;
   const int64_t per = (N + gridDim.y - 1) / gridDim.y;
   const int64_t n0 = blockIdx.y * per, n1 = min(N, n0 + per);
-  float s[4 * V], wt = 0.f;
-  double dq = 0.0;
+  float s[4 * V], q = 0.f, wt = 0.f;
 #pragma unroll
   for (int i = 0; i < 4 * V; ++i) s[i] = 0.f;
-#pragma unroll 1
-  for (int64_t m0 = n0 + warp; m0 < n1; m0 += 8 * kStatRows) {
-    const int64_t m1 = min(n1, m0 + 8 * kStatRows);
-    float q = 0.f;
 #pragma unroll 2
-    for (int64_t n = m0; n < m1; n += 8) {
-      const float wn = w[n];
-      const T* row = M + n * d;
-      StatVec<T, V> v[4];
+  for (int64_t n = n0 + warp; n < n1; n += 8) {
+    const float wn = w[n];
+    const T* row = M + n * d;
+    StatVec<T, V> v[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int c = b0 + (lane + 32 * i) * V;  // d is a multiple of V
-        if (c < d)
-          v[i] = *reinterpret_cast<const StatVec<T, V>*>(row + c);
-        else
-          for (int k = 0; k < V; ++k) v[i].x[k] = T(0.f);
-      }
-#pragma unroll
-      for (int i = 0; i < 4 * V; ++i) {
-        const float x = ld(&v[i / V].x[i % V]), wv = wn * x;
-        s[i] += wv;
-        q = fmaf(wv, x, q);
-      }
-      wt += wn;
+    for (int i = 0; i < 4; ++i) {
+      const int c = b0 + (lane + 32 * i) * V;  // d is a multiple of V
+      if (c < d)
+        v[i] = *reinterpret_cast<const StatVec<T, V>*>(row + c);
+      else
+        for (int k = 0; k < V; ++k) v[i].x[k] = T(0.f);
     }
-    dq += q;
+    float row_q = 0.f;
+#pragma unroll
+    for (int i = 0; i < 4 * V; ++i) {
+      const float x = ld(&v[i / V].x[i % V]), wv = wn * x;
+      s[i] += wv;
+      row_q = fmaf(wv, x, row_q);
+    }
+    q += row_q;
+    wt += wn;
   }
 #pragma unroll
   for (int i = 0; i < 4 * V; ++i) sums[warp][(lane + 32 * (i / V)) * V + i % V] = s[i];
+  double dq = q;
   for (int o = 16; o > 0; o >>= 1) dq += __shfl_xor_sync(0xffffffffu, dq, o);
   if (lane == 0) {
     ss[warp] = dq;

@@ -111,9 +111,10 @@ def test_recolor_recovers_an_exact_rotation():
 
 
 def test_recolor_statistics_of_many_samples():
-    """8 M samples of one weight: no fp32 sum takes more than 128 values, so the
-    sums of w and of w x^2 are each within 128 2^-24 (equal weights round the same
-    way every time: sums of 8 M / 1,024 values come out 8e-5 off)."""
+    """8 M samples of one weight: no fp32 sum takes more than 128 values (of up to
+    eight squares each), so the sums of w and of w x^2 are within 136 2^-24 (equal
+    weights round the same way every time: sums of 8 M / 1,024 values come out 8e-5
+    off)."""
     N = 8_000_000
     g = torch.Generator(device="cuda").manual_seed(3)
     X = torch.randn((N, 16), generator=g, device="cuda")
@@ -121,7 +122,7 @@ def test_recolor_statistics_of_many_samples():
     w = torch.full((N,), 0.6, device="cuda")
     _, _, r = _fit("f32", X, Y, w, 1e-3)
     r_ref = float(X.double().square().mean().sqrt())
-    assert abs(r - r_ref) <= 128 * 2.0**-24 * r_ref
+    assert abs(r - r_ref) <= 136 * 2.0**-24 * r_ref
 
 
 # Ridges from just above the smallest accepted pivot (1e-4 of the mean eigenvalue)

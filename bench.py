@@ -309,7 +309,7 @@ def _made_rows_pay(w, tok, pool_before_map, round_built):
     rows = (tok.T_s if after else min(tok.T_s, tok.T_r) if w.align_mode == "same_index"
             else tok.T_r * 28 // 100 if w.align_mode == "ta" else tok.T_r)
     staged = (after or w.align_mode != "overlap_mean") and not round_built
-    small = rows * w.K <= 16000000
+    small = rows * w.K <= (5000000 if w.align_mode == "ta" else 16000000)
     if passes == 2:
         return small or not staged
     tiles = 2 * w.L_r * -(-rows // 256)

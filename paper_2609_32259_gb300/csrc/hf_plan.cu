@@ -55,7 +55,8 @@ struct OperandPath {
 // and more 1.2 to 2.2 times (d_R 2,048, K 1,024, 16K rows 1.64 and 2.45 ms).  Blends
 // (one sender token, two bf16 parts: staged by cp.async) in two passes (d_R 1,024):
 // 8K rows 0.54 and 0.63 ms at K 1,024, 1.56 and 1.61 at 3,072, but 3.42 and 3.06 at
-// 6,144.  In one pass only while the tiles leave half of the SM pairs idle (d_R 512, K
+// 6,144; with Token Alignment and K 1,024, 40 layers, 4.2K rows 1.84 and 1.91 ms, 6.1K
+// 2.94 and 2.77.  In one pass only while the tiles leave half of the SM pairs idle (d_R 512, K
 // 3,072, 512 rows 0.094 and 0.133 ms, 1,024 rows 0.158 and 0.135, 16K rows 2.62 and
 // 1.61) or, up to K = 1,024, in at most three rounds, a quarter of the last idle
 // (28 layers, 566 rows 168 tiles, 1.27 times faster made, 352 rows 1.30; but 720 rows
@@ -71,7 +72,8 @@ bool made_rows_pay(const hf_plan_desc& d, const OperandPath& o) {
                        : d.align_mode == HF_ALIGN_SAME_INDEX ? std::min(T_s, T_r)
                        : d.align_mode == HF_ALIGN_TA         ? T_r * 28 / 100
                                                              : T_r;
-  const bool staged = o.one_entry && o.split, small = rows * o.K <= 16000000;
+  const bool staged = o.one_entry && o.split;
+  const bool small = rows * o.K <= (d.align_mode == HF_ALIGN_TA ? 5000000 : 16000000);
   if (passes == 2) return !staged || small;
   const int64_t pairs = 76, tiles = 2 * d.L_r * ((rows + 255) / 256);
   const int64_t rounds = (tiles + pairs - 1) / pairs;

@@ -128,8 +128,9 @@ def test_workspace_size_of_refused_descriptors(B, over):
     (dict(H_s=16, tokens=512), True), (dict(H_s=16, tokens=513), False),
     (dict(align_mode="ta", tokens=1828), True), (dict(align_mode="ta", tokens=2747), False),
     (dict(align_mode="overlap_mean"), True), (dict(align_mode="overlap_mean", tokens=769), False),
-    # d_R 1,024: rows x K up to 16 M
+    # d_R 1,024: rows x K up to 16 M, 5 M with Token Alignment
     (dict(H_r=8, tokens=15625), True), (dict(H_r=8, tokens=15626), False),
+    (dict(H_r=8, align_mode="ta", tokens=17438), True), (dict(H_r=8, align_mode="ta", tokens=17443), False),
     (dict(H_r=6, tokens=15626), True),                                  # three passes
     (dict(round_built_operands=True, tokens=15625), True),              # rounded once
     (dict(round_built_operands=True, tokens=15626), False),
